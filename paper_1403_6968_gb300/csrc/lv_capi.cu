@@ -159,7 +159,6 @@ struct linview_program {
   void* V1 = nullptr;   // input right factor, column-major n x r_max
   void* Mr = nullptr;   // T_i^T V blocks in reverse order, p x k r_max
   void* TVpart = nullptr;  // row-block partial sums of those products
-  int64_t tv_cap = 0;      // columns x p the partial sets hold (k r p <= tv_cap)
   void* Gpanel = nullptr;
   void* Dh = nullptr;   // hybrid strategy: dense deltas D_{i-1}, D_i (2 x n x p, ld ldD)
   int64_t ldD = 0;
@@ -168,7 +167,7 @@ struct linview_program {
   void* Xar[2] = {nullptr, nullptr};  // n x r_max k, column-major (fs)
   void* Yar[2] = {nullptr, nullptr};  // p x r_max k, column-major (ld p)
   void* What = nullptr;               // n x Rcap, column-major (fs)
-  void* XtV = nullptr;                // (r_max k) x Rcap
+  void* XtV = nullptr;                // (r_max k) x Rcap (FP64)
   int ie_s = 0, ie_Ls = 0, ie_NT = 0;  // skip step s (k/2 for EXP), log2 s, number of T views
   void* Tfull = nullptr;  // T_0 .. T_k recomputed for the adjoint (exponential / skip)
   int64_t ldTf = 0;
@@ -1402,8 +1401,6 @@ static bool iter_exp(const linview_program* p) {
 static linview_status iter_sk_create(linview_program* p, const void* const* inputs,
                                      const int64_t* lds, int on_dev, cudaStream_t s);
 
-constexpr int64_t kTvCap = 16384;  // k r p of the one-pass M_i products
-
 static linview_status iter_create(linview_program* p, const void* const* inputs,
                                   const int64_t* lds, int on_dev, cudaStream_t s) {
   if (iter_exp(p)) return iter_sk_create(p, inputs, lds, on_dev, s);
@@ -1432,12 +1429,9 @@ static linview_status iter_create(linview_program* p, const void* const* inputs,
   LV_TRY(dalloc(p, (size_t)p->fs * p->Rcap * p->elem, &p->Kar, s));
   LV_TRY(dalloc(p, (size_t)p->fs * p->d.r_max * p->elem, &p->V1, s));
   LV_TRY(dalloc(p, (size_t)pp * p->Rcap * p->elem, &p->Mr, s));
-  // partial sets of M_i = T_i^T V for all views (one pass over the T panel),
-  // when small: k r_max p <= 16384 per row block
-  if ((int64_t)p->Rcap * pp <= kTvCap) {
-    p->tv_cap = (int64_t)p->Rcap * pp;
-    LV_TRY(dalloc(p, (size_t)panel_tv_blocks((int)n) * p->tv_cap * p->elem, &p->TVpart, s));
-  }
+  // partial sets of M_i = T_i^T V (one pass over the T panel for all views)
+  LV_TRY(dalloc(p, (size_t)tdot_work_elems((int)n, (int)(k * pp), p->d.r_max, p->sms) * p->elem,
+                &p->TVpart, s));
   const PassGeom g = fused_geom(p->elem, (int)n, p->sms);
   p->part_cs = p->fs;
   p->xp_s = (int64_t)kMaxFusedR * p->part_cs;
@@ -1458,6 +1452,30 @@ static linview_status iter_create(linview_program* p, const void* const* inputs,
   return iter_reeval(p, s);
 }
 
+// M blocks (p x w column-major, ld p; the newest view first) = T_i^T F for kv
+// panels of p columns side by side at A (ld lda), F n x w with column stride fs.
+template <typename T>
+static linview_status panel_tdot(linview_program* p, const T* A, int64_t lda, const T* F, int w,
+                                 int kv, T* M, cudaStream_t s) {
+  TdotOp<T> o{A, lda, F, p->fs, (int)p->d.n, (int)p->d.p, kv, w, M, p->d.p,
+              static_cast<T*>(p->TVpart)};
+  ProfScope ps(p, s, 0.0);
+  LV_CUDA(launch_tdot<T>(o, p->sms, s));
+  p->all_launches++;  // the partial sums
+  return LINVIEW_OK;
+}
+
+// rank-w update of one n x p panel, Q += K M^T (K n x w with column stride fs, M
+// p x w with ld p; accumulate = false: Q = K M^T)
+template <typename T>
+static linview_status panel_rank(linview_program* p, void* Q, int64_t ldq, const T* K, const T* M,
+                                 int w, cudaStream_t s, bool accumulate = true) {
+  ProfScope ps(p, s, 0.0);
+  LV_CUDA(launch_outer<T>(static_cast<T*>(Q), ldq, K, p->fs, M, p->d.p, (int)p->d.n, (int)p->d.p, 1,
+                          w, accumulate, p->sms, s));
+  return LINVIEW_OK;
+}
+
 // Appendix B: U_1 = U, V_1 = T_0^T V, U_i = [U, A U_{i-1} + U (V^T U_{i-1})],
 // V_i = [T_{i-1}^T V, V_{i-1}], dT_i = U_i V_i^T.  U_i's blocks are the
 // Krylov blocks K_a = A'^a U (A' = A + U V^T); each step adds only the
@@ -1474,10 +1492,10 @@ static linview_status panel_update(linview_program* p, char* Tp, const T* K, con
   const int n = (int)p->d.n;
   const int64_t pp = p->d.p;
   const int64_t fs = p->fs;
-  if (panel_update_fits(k, r, sizeof(T))) {
+  if (outer_fits(k * r, sizeof(T))) {
     ProfScope ps(p, s, 0.0);
-    LV_CUDA(launch_panel_update<T>(reinterpret_cast<T*>(Tp), p->ldT, K, fs, M, pp, n, (int)pp, k,
-                                   r, s));
+    LV_CUDA(launch_outer<T>(reinterpret_cast<T*>(Tp) + pp, p->ldT, K, fs, M, pp, n, (int)pp, k, r,
+                            true, p->sms, s));
     return LINVIEW_OK;
   }
   for (int i = 1; i <= k; ++i) {
@@ -1502,18 +1520,8 @@ static linview_status iter_propagate(linview_program* p, int r, cudaStream_t s) 
   View& a = p->views[0];
   const PassGeom g = fused_geom(sizeof(T), n, p->sms);
   // M_i = T_i^T V (old T_i), stored at block k-1-i so that [M_{i-1} .. M_0]
-  // is one contiguous p x (i r) slab: one pass over the T panel (partials
-  // per row block) when its partial sets fit, else one batched GEMM launch
-  // (column-major view: T_i is p x n (ld ldT) at panel block i, V is n x r (ld fs))
-  if (p->TVpart && (int64_t)k * r * pp <= p->tv_cap) {
-    ProfScope ps(p, s, 0.0);
-    LV_CUDA(launch_panel_tv<T>(reinterpret_cast<const T*>(Tp), p->ldT, V1, fs,
-                               static_cast<T*>(p->TVpart), M, pp, n, (int)pp, k, r, s));
-    p->all_launches++;  // the partial sums
-  } else {
-    LV_TRY(gemm_cm_own(p, false, false, pp, r, n, 1.0, Tp, p->ldT, V1, fs, 0.0,
-                       M + (int64_t)(k - 1) * r * pp, pp, s, k, pp, 0, -(int64_t)r * pp));
-  }
+  // is one contiguous p x (i r) slab: one pass over the T panel
+  LV_TRY(panel_tdot<T>(p, reinterpret_cast<const T*>(Tp), p->ldT, V1, r, k, M, s));
   if (k >= 2) {
     {
       ProfScope ps(p, s, 0.0);
@@ -1583,9 +1591,7 @@ static linview_status iter_propagate_b(linview_program* p, int rb, cudaStream_t 
   }
   // T_i += [K_0 .. K_{i-1}] [V_b .. V_b]^T for every i (every M block is V_b)
   LV_TRY(panel_update<T>(p, Tp, K, M, k, rb, true, s));
-  // B += U_b V_b^T (column-major B^T, p x n)
-  LV_TRY(gemm_cm_own(p, false, true, pp, n, rb, 1.0, M, pp, K, fs, 1.0, p->Bm, p->ldB, s));
-  return LINVIEW_OK;
+  return panel_rank<T>(p, p->Bm, p->ldB, K, M, rb, s);  // B += U_b V_b^T
 }
 
 // Hybrid strategy (Sec. 4.3; App. B, hybrid linear model): the change of
@@ -1630,8 +1636,7 @@ static linview_status iter_propagate_hybrid(linview_program* p, int r, bool b_up
     T* ti = reinterpret_cast<T*>(Tp + (size_t)i * pp * sizeof(T));
     const T* tprev = reinterpret_cast<const T*>(Tp + (size_t)(i - 1) * pp * sizeof(T));
     if (!b_update)  // W^T = T'_{i-1}^T V (T'_{i-1} is already refreshed)
-      LV_TRY(gemm_cm_own(p, false, false, pp, r, n, 1.0, tprev, p->ldT, V1, fs, 0.0, W, pp, s));
-    double beta = 0.0;
+      LV_TRY(panel_tdot<T>(p, tprev, p->ldT, V1, r, 1, W, s));
     if (i >= 2) {  // D_i = A D_{i-1}
       if (sizeof(T) == 4 && view_panel_fits<T>(p, a, (int)pp)) {  // a few columns
         LV_TRY(view_panel_product<T>(p, a, false, dp, p->ldD, (int)pp, nullptr, 0, dc, p->ldD, s));
@@ -1640,15 +1645,14 @@ static linview_status iter_propagate_hybrid(linview_program* p, int r, bool b_up
                        0, dc, p->ldD, s, p->hyA ? &hy : nullptr, a_split));
         a_split = true;
       }
-      beta = 1.0;
     }
-    // D_i^T += W U^T  (the rank-r term)
-    LV_TRY(gemm_cm_own(p, false, true, pp, n, r, 1.0, W, pp, K, fs, beta, dc, p->ldD, s));
+    // D_i += U W^T (the rank-r term; D_1 is that term alone)
+    LV_TRY(panel_rank<T>(p, dc, p->ldD, K, W, r, s, i >= 2));
     ProfScope ps(p, s, 0.0);
     LV_CUDA(launch_axpy_rows<T>(ti, p->ldT, dc, p->ldD, T(1), (int)n, (int)pp, s));
   }
-  if (b_update)  // B += U_b V_b^T (column-major B^T, p x n)
-    LV_TRY(gemm_cm_own(p, false, true, pp, n, r, 1.0, W, pp, K, fs, 1.0, p->Bm, p->ldB, s));
+  if (b_update)  // B += U_b V_b^T
+    LV_TRY(panel_rank<T>(p, p->Bm, p->ldB, K, W, r, s));
   else
     LV_TRY(run_update<T>(p, a, K, V1, r, s));
   return LINVIEW_OK;
@@ -1813,7 +1817,9 @@ static linview_status iter_sk_create(linview_program* p, const void* const* inpu
     LV_TRY(dalloc(p, (size_t)p->fs * ck * p->elem, &p->Xar[i], s));
     LV_TRY(dalloc(p, (size_t)pp * ck * p->elem, &p->Yar[i], s));
   }
-  LV_TRY(dalloc(p, (size_t)ck * p->Rcap * p->elem, &p->XtV, s));
+  LV_TRY(dalloc(p, (size_t)ck * p->Rcap * sizeof(double), &p->XtV, s));
+  LV_TRY(dalloc(p, (size_t)tdot_work_elems((int)n, (int)pp, p->Rcap, p->sms) * p->elem, &p->TVpart,
+                s));
   LV_TRY(dalloc(p, (size_t)pp * p->d.r_max * p->elem, &p->Mr, s));  // V_b of an update to B
   const PassGeom g = fused_geom(p->elem, (int)n, p->sms);
   p->part_cs = p->fs;
@@ -1847,25 +1853,44 @@ static linview_status iter_sk_step(linview_program* p, int cur, View& tj, const 
   const int n = (int)p->d.n;
   const int64_t pp = p->d.p;
   const int64_t fs = p->fs;
-  const int mode = exact_mode(p);
   const View& b = p->views[p->ie_NT + 1];
   T* Xc = static_cast<T*>(p->Xar[cur]);
   T* Yc = static_cast<T*>(p->Yar[cur]);
   T* Xn = static_cast<T*>(p->Xar[cur ^ 1]);
   T* Yn = static_cast<T*>(p->Yar[cur ^ 1]);
-  T* XtV = static_cast<T*>(p->XtV);
-  // first block of Y_i (column-major p x rh): T_j^T V_h + Y_j (X_j^T V_h)
-  LV_TRY(gemm_cm_own(p, false, false, pp, rh, n, 1.0, tj.ptr, tj.ld, Vh, fs, 0.0, Yn, pp, s));
-  LV_TRY(gemm_cm_own(p, true, false, c, rh, n, 1.0, Xc, fs, Vh, fs, 0.0, XtV, c, s));
-  LV_TRY(gemm_cm_own(p, false, false, pp, rh, c, 1.0, Yc, pp, XtV, c, 1.0, Yn, pp, s));
-  if (with_b) {  // + B^T (W^_h - V_h) (W^_h in the What arena; dS_1 = 0)
-    LV_TRY(gemm_cm_own(p, false, false, pp, rh, n, 1.0, b.ptr, b.ld, p->What, fs, 1.0, Yn, pp, s));
-    LV_TRY(gemm_cm_own(p, false, false, pp, rh, n, -1.0, b.ptr, b.ld, Vh, fs, 1.0, Yn, pp, s));
+  double* XtV = static_cast<double*>(p->XtV);
+  // X_j^T V_h (c x rh): FP32 factors in double-float (row-major), FP64 ones on
+  // the CUDA-core GEMM (column-major)
+  if constexpr (sizeof(T) == 4) {
+    ProfScope ps(p, s, 0.0);
+    LV_CUDA(launch_cross_gram(Xc, Vh, fs, n, c, rh, p->Cpart, XtV, s));
+    p->all_launches++;
+  } else {
+    LV_TRY(gemm_cm_own(p, true, false, c, rh, n, 1.0, Xc, fs, Vh, fs, 0.0, XtV, c, s));
+  }
+  // first block of Y_i (column-major p x rh): T_j^T V_h + Y_j (X_j^T V_h), and
+  // with_b + B^T (W^_h - V_h) (W^_h in the What arena; dS_1 = 0)
+  TdotOp<T> o{static_cast<const T*>(tj.ptr), tj.ld, Vh, fs, n, (int)pp, 1, rh, Yn, pp,
+              static_cast<T*>(p->TVpart)};
+  if (with_b) {
+    o.A1 = static_cast<const T*>(b.ptr);
+    o.lda1 = b.ld;
+    o.F1 = static_cast<const T*>(p->What);
+  }
+  o.Yc = Yc;
+  o.ldy = pp;
+  o.ny = c;
+  o.S = XtV;
+  o.s_t = sizeof(T) == 4 ? rh : 1;
+  o.s_c = sizeof(T) == 4 ? 1 : c;
+  {
+    ProfScope ps(p, s, 0.0);
+    LV_CUDA(launch_tdot<T>(o, p->sms, s));
+    p->all_launches++;
   }
   LV_CUDA(cudaMemcpyAsync(Yn + (int64_t)rh * pp, Yc, sizeof(T) * pp * c, cudaMemcpyDeviceToDevice,
                           s));
-  // T_j += X_j Y_j^T  (column-major T_j^T, p x n)
-  LV_TRY(gemm_cm_own(p, false, true, pp, n, c, 1.0, Yc, pp, Xc, fs, 1.0, tj.ptr, tj.ld, s));
+  LV_TRY(panel_rank<T>(p, tj.ptr, tj.ld, Xc, Yc, c, s));  // T_j += X_j Y_j^T
   // X_i = [U_h, P_h X_j] from the old P_h
   const PassGeom g = fused_geom(sizeof(T), n, p->sms);
   LV_TRY(run_products_update<T>(p, ph, c, Xc, nullptr, nullptr, nullptr, s));
@@ -1892,8 +1917,8 @@ static linview_status iter_sk_propagate(linview_program* p, int r, cudaStream_t 
   int cur = 0;
   // X_1 = U_1, Y_1 = T_0^T V_1
   LV_CUDA(cudaMemcpyAsync(p->Xar[0], U, sizeof(T) * fs * r, cudaMemcpyDeviceToDevice, s));
-  LV_TRY(gemm_cm_own(p, false, false, pp, r, n, 1.0, t0.ptr, t0.ld, V + (int64_t)(p->Rcap - r) * fs,
-                 fs, 0.0, p->Yar[0], pp, s));
+  LV_TRY(panel_tdot<T>(p, static_cast<const T*>(t0.ptr), t0.ld, V + (int64_t)(p->Rcap - r) * fs, r,
+                       1, static_cast<T*>(p->Yar[0]), s));
   for (int l = 0; l < Ls; ++l) {  // exponential part: T_2h from T_h, h = 2^l < s
     const int rh = r << l;
     T* Vh = V + (int64_t)(p->Rcap - rh) * fs;
@@ -1946,8 +1971,8 @@ static linview_status iter_sk_propagate(linview_program* p, int r, cudaStream_t 
   }
   // T_k += X_k Y_k^T, then P_s and S'_s
   View& tk = ie_T(p, NT - 1);
-  LV_TRY(gemm_cm_own(p, false, true, pp, n, (int64_t)r * k, 1.0, p->Yar[cur], pp, p->Xar[cur], fs,
-                 1.0, tk.ptr, tk.ld, s));
+  LV_TRY(panel_rank<T>(p, tk.ptr, tk.ld, static_cast<const T*>(p->Xar[cur]),
+                       static_cast<const T*>(p->Yar[cur]), r * k, s));
   LV_TRY(run_update<T>(p, ie_P(p, Ls), U, Vs, rs, s));
   if (Ls >= 1) LV_TRY(run_update<T>(p, ie_S(p, Ls), U, Wh, rs, s));
   return LINVIEW_OK;
@@ -1968,7 +1993,6 @@ static linview_status iter_sk_step_b(linview_program* p, int cur, int c, int rb,
   const int n = (int)p->d.n;
   const int64_t pp = p->d.p;
   const int64_t fs = p->fs;
-  const int mode = exact_mode(p);
   const T* Ub = static_cast<const T*>(p->Uar);
   const T* Vb = static_cast<const T*>(p->Mr);
   T* Xc = static_cast<T*>(p->Xar[cur]);
@@ -1977,8 +2001,7 @@ static linview_status iter_sk_step_b(linview_program* p, int cur, int c, int rb,
   T* Yn = static_cast<T*>(p->Yar[cur ^ 1]);
   T* tmp = static_cast<T*>(p->What);
   const PassGeom g = fused_geom(sizeof(T), n, p->sms);
-  // T_j += X_j Y_j^T
-  LV_TRY(gemm_cm_own(p, false, true, pp, n, c, 1.0, Yc, pp, Xc, fs, 1.0, tj.ptr, tj.ld, s));
+  LV_TRY(panel_rank<T>(p, tj.ptr, tj.ld, Xc, Yc, c, s));  // T_j += X_j Y_j^T
   // [P X_j | P U_b] in one products pass over P
   LV_CUDA(cudaMemcpyAsync(Xc + (int64_t)c * fs, Ub, sizeof(T) * fs * rb, cudaMemcpyDeviceToDevice,
                           s));
@@ -2026,11 +2049,11 @@ static linview_status iter_sk_propagate_b(linview_program* p, int rb, cudaStream
     c += rb;
   }
   View& tk = ie_T(p, NT - 1);
-  LV_TRY(gemm_cm_own(p, false, true, pp, n, c, 1.0, p->Yar[cur], pp, p->Xar[cur], fs, 1.0, tk.ptr,
-                 tk.ld, s));
-  // B += U_b V_b^T (column-major B^T, p x n)
-  LV_TRY(gemm_cm_own(p, false, true, pp, n, rb, 1.0, p->Mr, pp, p->Uar, fs, 1.0, p->Bm, p->ldB, s));
-  return LINVIEW_OK;
+  LV_TRY(panel_rank<T>(p, tk.ptr, tk.ld, static_cast<const T*>(p->Xar[cur]),
+                       static_cast<const T*>(p->Yar[cur]), c, s));
+  // B += U_b V_b^T
+  return panel_rank<T>(p, p->Bm, p->ldB, static_cast<const T*>(p->Uar),
+                       static_cast<const T*>(p->Mr), rb, s);
 }
 
 // ---------------------------------------------------------------------------

@@ -104,29 +104,29 @@ __device__ __forceinline__ void df_add(float& hi, float& lo, float x, float xe) 
   lo = __fadd_rn(lo, __fadd_rn(err, xe));
 }
 
-// FP32 programs: per-block partials of C = V^T U in double-float.  GB300's
+// FP32 programs: per-block partials of C = V^T U (rv x r) in double-float.  GB300's
 // FP64 pipe is narrow, so the FP64-grade sums use FP32 arithmetic; every
 // block of 256 threads takes one 32-row tile per step.
 __global__ void __launch_bounds__(kThreads) gram_df_kernel(const float* __restrict__ V,
                                                            const float* __restrict__ U,
-                                                           int64_t fs, int n, int r,
+                                                           int64_t fs, int n, int rv, int r,
                                                            float2* Cpart) {
   __shared__ float Vs[kGramRows][kGramMaxR + 1];
   __shared__ float Us[kGramRows][kGramMaxR + 1];
   const int tid = threadIdx.x;
   const int G = gridDim.x;
-  const int ne = r * r;
+  const int ne = rv * r;
   float hi[kGramPerThread], lo[kGramPerThread];
 #pragma unroll
   for (int i = 0; i < kGramPerThread; ++i) hi[i] = lo[i] = 0.f;
   for (int t0 = blockIdx.x * kGramRows; t0 < n; t0 += G * kGramRows) {
     const int nr = min(kGramRows, n - t0);
-    for (int idx = tid; idx < kGramRows * r; idx += kThreads) {
+    for (int idx = tid; idx < kGramRows * max(rv, r); idx += kThreads) {
       const int c = idx / kGramRows;
       const int j = idx % kGramRows;
       const bool ok = j < nr;
-      Vs[j][c] = ok ? V[(int64_t)c * fs + t0 + j] : 0.f;
-      Us[j][c] = ok ? U[(int64_t)c * fs + t0 + j] : 0.f;
+      if (c < rv) Vs[j][c] = ok ? V[(int64_t)c * fs + t0 + j] : 0.f;
+      if (c < r) Us[j][c] = ok ? U[(int64_t)c * fs + t0 + j] : 0.f;
     }
     __syncthreads();
 #pragma unroll
@@ -173,7 +173,7 @@ __global__ void gram_reduce_kernel(const float2* __restrict__ Cpart, int G, int 
   }
   if (lane == 0) {
     const double sum = (double)h + (double)l;
-    if (!isfinite(sum)) atomicOr(status, kStatusNonFinite);
+    if (status && !isfinite(sum)) atomicOr(status, kStatusNonFinite);
     C[e] = sum;
     if (Cdf) {  // the same sum as a normalised FP32 pair
       const float hh = __fadd_rn(h, l);
@@ -190,13 +190,29 @@ cudaError_t launch_gram(const T* V, const T* U, int64_t fs, int n, int r, double
   const int G = gram_grid(n);
   if constexpr (std::is_same<T, float>::value) {
     float2* part = reinterpret_cast<float2*>(Cpart);
-    gram_df_kernel<<<G, kThreads, 0, s>>>(V, U, fs, n, r, part);
+    gram_df_kernel<<<G, kThreads, 0, s>>>(V, U, fs, n, r, r, part);
     const int ne = r * r;
     const int warps_per_block = kThreads / 32;
     gram_reduce_kernel<<<(ne + warps_per_block - 1) / warps_per_block, kThreads, 0, s>>>(
         part, G, ne, C, status, Cdf);
   } else {
     gram_f64_kernel<<<G, kThreads, 0, s>>>(V, U, fs, n, r, Cpart, ticket, C, status);
+  }
+  return cudaGetLastError();
+}
+
+cudaError_t launch_cross_gram(const float* X, const float* V, int64_t fs, int n, int rx, int rv,
+                              double* Cpart, double* C, cudaStream_t s) {
+  if (rv < 1 || rv > kGramMaxR || rx < 1) return cudaErrorInvalidValue;
+  const int G = gram_grid(n);
+  float2* part = reinterpret_cast<float2*>(Cpart);
+  for (int c0 = 0; c0 < rx; c0 += kGramMaxR) {
+    const int w = rx - c0 < kGramMaxR ? rx - c0 : kGramMaxR;
+    gram_df_kernel<<<G, kThreads, 0, s>>>(X + (int64_t)c0 * fs, V, fs, n, w, rv, part);
+    const int ne = w * rv;
+    const int warps_per_block = kThreads / 32;
+    gram_reduce_kernel<<<(ne + warps_per_block - 1) / warps_per_block, kThreads, 0, s>>>(
+        part, G, ne, C + (int64_t)c0 * rv, nullptr, nullptr);
   }
   return cudaGetLastError();
 }
@@ -572,168 +588,6 @@ cudaError_t launch_bounded_wait_probe(uint64_t limit_ns, unsigned* status,
   return cudaGetLastError();
 }
 
-// T panel update of the linear iteration model, all views in one launch:
-// T_i += [K_0 .. K_{i-1}] [M blocks]^T for i = 1..k, i.e.
-//   T_i(j, q) = Tp[j ldT + i p + q] += sum_{t < i r} K[t fs + j] M[((k - i) r + t) ldm + q]
-// (App. B, linear model: view i takes the first i Krylov blocks and the i
-// newest M blocks).  A CTA takes 16 rows j and 64 columns q of every view;
-// the 16 x k r Krylov rows and the k r x 64 slice of M are staged in shared
-// memory once for all k views.  A thread owns 4 adjacent columns of one row
-// (one broadcast K load and one 128-bit M load per 4 FMAs) and loads the T
-// entries of 8 views at once before it updates them.  Sums over t in
-// increasing order, in T.
-constexpr int kPanelRows = 16, kPanelQ = 64;
-
-template <typename T>
-__global__ void __launch_bounds__(256)
-    panel_update_kernel(T* Tp, int64_t ldT, const T* K, int64_t fs, const T* M, int64_t ldm,
-                        int n, int p, int k, int r) {
-  extern __shared__ __align__(16) unsigned char panel_sm[];
-  const int KR = k * r;
-  T* Ks = reinterpret_cast<T*>(panel_sm);  // [kPanelRows][KR]
-  T* Ms = Ks + kPanelRows * KR;            // [KR][kPanelQ]
-  const int j0 = blockIdx.x * kPanelRows, q0 = blockIdx.y * kPanelQ;
-  for (int e = threadIdx.x; e < kPanelRows * KR; e += blockDim.x) {
-    const int jr = e % kPanelRows, t = e / kPanelRows;  // coalesced down a Krylov column
-    Ks[jr * KR + t] = (j0 + jr < n) ? K[(int64_t)t * fs + j0 + jr] : T(0);
-  }
-  for (int e = threadIdx.x; e < KR * kPanelQ; e += blockDim.x) {
-    const int q = e % kPanelQ, t = e / kPanelQ;
-    Ms[t * kPanelQ + q] = (q0 + q < p) ? M[(int64_t)t * ldm + q0 + q] : T(0);
-  }
-  __syncthreads();
-  const int jr = threadIdx.x / 16, qa = 4 * (threadIdx.x % 16);
-  const int j = j0 + jr;
-  if (j >= n || q0 + qa >= p) return;
-  const int nq = (p - q0 - qa) < 4 ? p - q0 - qa : 4;  // columns of this thread in the view
-  const T* kr = Ks + jr * KR;
-  T* trow = Tp + (int64_t)j * ldT + q0 + qa;
-  constexpr int VB = 8;  // views per group: their T loads are in flight together
-  for (int i0 = 1; i0 <= k; i0 += VB) {
-    T tv[VB][4];
-#pragma unroll
-    for (int v = 0; v < VB; ++v)
-#pragma unroll
-      for (int c = 0; c < 4; ++c)
-        if (i0 + v <= k && c < nq) tv[v][c] = trow[(int64_t)(i0 + v) * p + c];
-#pragma unroll
-    for (int v = 0; v < VB; ++v) {
-      const int i = i0 + v;
-      if (i > k) break;
-      const T* mi = Ms + (k - i) * r * kPanelQ + qa;
-      T a0 = 0, a1 = 0, a2 = 0, a3 = 0;
-      for (int t = 0; t < i * r; ++t) {
-        const T kv = kr[t];
-        const T* mt = mi + t * kPanelQ;
-        a0 += kv * mt[0];
-        a1 += kv * mt[1];
-        a2 += kv * mt[2];
-        a3 += kv * mt[3];
-      }
-      const T av[4] = {a0, a1, a2, a3};
-#pragma unroll
-      for (int c = 0; c < 4; ++c)
-        if (c < nq) trow[(int64_t)i * p + c] = tv[v][c] + av[c];
-    }
-  }
-}
-
-// M_i = T_i^T V of the linear iteration model, all views in one pass over
-// the T panel (App. B: V_{i+1} = [T_i^T V_1, V_i]): for i < k, c < r, q < p,
-//   M[((k - 1 - i) r + c) ldm + q] = sum_j Tp[j ldT + i p + q] V[c fs + j],
-// as partial sums over blocks of ``rows`` rows (part[b][col][q], column
-// stride p) that launch_sum_partials adds in block order.  A thread owns
-// column q of one view (4 views per CTA, grid z over the views); V's rows of
-// the block are staged in shared memory (r <= 8).
-template <typename T>
-__global__ void __launch_bounds__(256)
-    panel_tv_kernel(const T* Tp, int64_t ldT, const T* V, int64_t fs, T* part, int n, int p,
-                    int k, int r, int rows) {
-  extern __shared__ __align__(16) unsigned char tv_sm[];
-  T* Vs = reinterpret_cast<T*>(tv_sm);  // [rows][8]
-  const int j0 = blockIdx.x * rows, q0 = blockIdx.y * 64;
-  for (int e = threadIdx.x; e < rows * r; e += blockDim.x) {
-    const int jr = e % rows, c = e / rows;
-    Vs[jr * 8 + c] = (j0 + jr < n) ? V[(int64_t)c * fs + j0 + jr] : T(0);
-  }
-  __syncthreads();
-  const int q = q0 + (int)(threadIdx.x % 64);
-  const int i = (int)blockIdx.z * 4 + (int)(threadIdx.x / 64);
-  if (q >= p || i >= k) return;
-  const int nr = (n - j0 < rows) ? n - j0 : rows;
-  T* pb = part + (int64_t)blockIdx.x * k * r * p;
-  {
-    T acc[8] = {};
-    const T* tcol = Tp + (int64_t)j0 * ldT + (int64_t)i * p + q;
-#pragma unroll 8
-    for (int jr = 0; jr < nr; ++jr) {
-      const T t = tcol[(int64_t)jr * ldT];
-#pragma unroll
-      for (int c = 0; c < 8; ++c) acc[c] += t * Vs[jr * 8 + c];
-    }
-    for (int c = 0; c < r; ++c) pb[((int64_t)(k - 1 - i) * r + c) * p + q] = acc[c];
-  }
-}
-
-// blocks of about n / 128 rows (at least 64, at most 768, so that V's staged
-// rows stay within 48 KB of shared memory in FP64)
-int panel_tv_blocks(int n) {
-  int rows = (n + 127) / 128;
-  rows = rows < 64 ? 64 : (rows + 7) / 8 * 8;
-  if (rows > 768) rows = 768;
-  return (n + rows - 1) / rows;
-}
-
-template <typename T>
-cudaError_t launch_panel_tv(const T* Tp, int64_t ldT, const T* V, int64_t fs, T* part, T* M,
-                            int64_t ldm, int n, int p, int k, int r, cudaStream_t s) {
-  if (r < 1 || r > 8 || k < 1 || p < 1) return cudaErrorInvalidValue;
-  const int nb = panel_tv_blocks(n);
-  const int rows = (n + nb - 1) / nb;
-  const dim3 grid((unsigned)nb, (unsigned)((p + 63) / 64), (unsigned)((k + 3) / 4));
-  panel_tv_kernel<T><<<grid, 256, sizeof(T) * (size_t)rows * 8, s>>>(Tp, ldT, V, fs, part, n, p,
-                                                                     k, r, rows);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  return launch_sum_partials<T>(part, nb, (int64_t)k * r * p, p, p, k * r, M, ldm, s);
-}
-
-// largest dynamic shared memory a block of this device may opt in to
-static int smem_optin_max() {
-  static const int v = [] {
-    int dev = 0, b = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&b, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
-      (void)cudaGetLastError();
-      return 49152;
-    }
-    return b;
-  }();
-  return v;
-}
-
-bool panel_update_fits(int k, int r, size_t elem_bytes) {
-  return elem_bytes * (size_t)(kPanelRows + kPanelQ) * (size_t)k * (size_t)r <=
-         (size_t)smem_optin_max();
-}
-
-template <typename T>
-cudaError_t launch_panel_update(T* Tp, int64_t ldT, const T* K, int64_t fs, const T* M,
-                                int64_t ldm, int n, int p, int k, int r, cudaStream_t s) {
-  if (n <= 0 || p <= 0 || k < 1 || r < 1) return cudaSuccess;
-  if (!panel_update_fits(k, r, sizeof(T))) return cudaErrorInvalidValue;
-  const size_t smem = sizeof(T) * (size_t)(kPanelRows + kPanelQ) * k * r;
-  if (smem > 49152) {  // opt in once, to the device's limit
-    static const cudaError_t configured = cudaFuncSetAttribute(
-        panel_update_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin_max());
-    if (configured != cudaSuccess) return configured;
-  }
-  const dim3 grid((unsigned)((n + kPanelRows - 1) / kPanelRows),
-                  (unsigned)((p + kPanelQ - 1) / kPanelQ));
-  panel_update_kernel<T><<<grid, 256, smem, s>>>(Tp, ldT, K, fs, M, ldm, n, p, k, r);
-  return cudaGetLastError();
-}
-
 #define LV_INST(T)                                                                              \
   template cudaError_t launch_gram<T>(const T*, const T*, int64_t, int, int, double*, unsigned*, \
                                       double*, unsigned*, cudaStream_t, float2*);               \
@@ -747,11 +601,7 @@ cudaError_t launch_panel_update(T* Tp, int64_t ldT, const T* K, int64_t fs, cons
   template cudaError_t launch_axpy_rows<T>(T*, int64_t, const T*, int64_t, T, int, int,           \
                                            cudaStream_t);                                       \
   template cudaError_t launch_scale_copy<T>(T*, int64_t, const T*, int64_t, T, int, int,          \
-                                            cudaStream_t);                                      \
-  template cudaError_t launch_panel_update<T>(T*, int64_t, const T*, int64_t, const T*, int64_t, \
-                                              int, int, int, int, cudaStream_t);                \
-  template cudaError_t launch_panel_tv<T>(const T*, int64_t, const T*, int64_t, T*, T*, int64_t, \
-                                          int, int, int, int, cudaStream_t);
+                                            cudaStream_t);
 LV_INST(float)
 LV_INST(double)
 

@@ -169,6 +169,10 @@ cudaError_t launch_gram(const T* V, const T* U, int64_t fs, int n, int r, double
                         unsigned* ticket, double* C, unsigned* status, cudaStream_t s,
                         float2* Cdf = nullptr);
 int gram_grid(int n);
+// C (rx x rv, FP64, row-major) = X^T V over n rows (FP32 factors, double-float
+// sums; rv <= 64, any rx in blocks of 64), no status check.
+cudaError_t launch_cross_gram(const float* X, const float* V, int64_t fs, int n, int rx, int rv,
+                              double* Cpart, double* C, cudaStream_t s);
 
 struct AssembleParams {
   int n, r_h;             // rows, current factor width
@@ -219,21 +223,40 @@ cudaError_t launch_axpy_rows(T* y, int64_t ldy, const T* x, int64_t ldx, T alpha
 template <typename T>
 cudaError_t launch_scale_copy(T* y, int64_t ldy, const T* x, int64_t ldx, T alpha, int rows,
                               int cols, cudaStream_t s);  // y = alpha x
-// Linear-model T panel update, all k views in one launch: T_i(j, q) =
-// Tp[j ldT + i p + q] += sum_{t < i r} K[t fs + j] M[((k - i) r + t) ldm + q]
-// (one launch for all views; its shared memory, (16 + 64) k r elements, must fit
-// the device's opt-in limit: panel_update_fits)
+// Products of n x p panels with narrow factors (lv_panel.cu).
+// M[((k - 1 - i) w + c) ldm + q] = sum_j A0[j lda0 + i p + q] F0[c fs + j] for
+// i < k, c < w <= 64, q < p; optionally + sum_j A1[j lda1 + i p + q] (F1 - F0)[c fs +
+// j] and + sum_{t < ny} Yc[t ldy + i p + q] S[t s_t + c s_c].  ``work`` holds
+// tdot_work_elems(n, k p, w) elements.
 template <typename T>
-cudaError_t launch_panel_update(T* Tp, int64_t ldT, const T* K, int64_t fs, const T* M,
-                                int64_t ldm, int n, int p, int k, int r, cudaStream_t s);
-bool panel_update_fits(int k, int r, size_t elem_bytes);
-// M[((k - 1 - i) r + c) ldm + q] = sum_j Tp[j ldT + i p + q] V[c fs + j] for
-// i < k, c < r <= 8, q < p, through panel_tv_blocks(n) partial sets in
-// ``part`` (panel_tv_blocks(n) x k r p elements)
-int panel_tv_blocks(int n);
+struct TdotOp {
+  const T* A0;
+  int64_t lda0;
+  const T* F0;
+  int64_t fs;
+  int n, p, k, w;
+  T* M;
+  int64_t ldm;
+  T* work;
+  const T* A1 = nullptr;
+  int64_t lda1 = 0;
+  const T* F1 = nullptr;
+  const T* Yc = nullptr;
+  int64_t ldy = 0;
+  int ny = 0;
+  const double* S = nullptr;
+  int64_t s_t = 0, s_c = 0;
+};
+int64_t tdot_work_elems(int n, int cols, int w, int num_sms);
 template <typename T>
-cudaError_t launch_panel_tv(const T* Tp, int64_t ldT, const T* V, int64_t fs, T* part, T* M,
-                            int64_t ldm, int n, int p, int k, int r, cudaStream_t s);
+cudaError_t launch_tdot(const TdotOp<T>& o, int num_sms, cudaStream_t s);
+// T_i(j, q) = T1[j ldT + (i - 1) p + q] += sum_{t < i r} K[t fs + j] M[((k - i) r + t) ldm
+// + q] for i = 1 .. k (k = 1: one panel, rank r); accumulate = false overwrites.
+// The staged factors must fit shared memory: outer_fits(k r).
+template <typename T>
+cudaError_t launch_outer(T* T1, int64_t ldT, const T* K, int64_t fs, const T* M, int64_t ldm, int n,
+                         int p, int k, int r, bool accumulate, int num_sms, cudaStream_t s);
+bool outer_fits(int kr, size_t elem_bytes);
 
 // OLS pieces (lv_ols.cu).
 template <typename T>
