@@ -85,8 +85,10 @@ typedef enum {
   LINVIEW_REEVAL_TF32 = 2,    /* comparison: one TF32 tensor-core pass (cuBLAS; ~1e-3 relative) */
   LINVIEW_REEVAL_BF16X9 = 3,  /* comparison: FP32 emulated by nine BF16 products (cuBLAS) */
   LINVIEW_REEVAL_FP64 = 4,    /* FP64 programs: the library's FP64 GEMM on the CUDA cores */
-  LINVIEW_REEVAL_TC3 = 5      /* FP32 programs: the library's tcgen05 GEMM in split TF32
-                                 (three TF32 products per operand pair, FP32 accuracy) */
+  LINVIEW_REEVAL_TC3 = 5      /* FP32 programs: the library's tcgen05 GEMM on split operands
+                                 (three FP16 products of scaled 11-bit halves per
+                                 operand pair, or three TF32 products where the
+                                 operands' range asks for it; FP32 accuracy) */
 } linview_reeval_mode;
 
 typedef struct {
@@ -145,7 +147,7 @@ typedef struct {
  * X_R^T X_R of every row block, on the side stream next to the Woodbury
  * passes); a correction is then one Newton-Schulz step for the inverse of Z,
  * W <- W + W (I - Z W), with the residual I - Z W in double-float and W (I - Z W)
- * on the split-TF32 GEMM, followed by beta = W X^T Y.  The step squares the
+ * on the split-operand GEMM, followed by beta = W X^T Y.  The step squares the
  * error of W in the residual sense (W - Z^-1 -> -(W - Z^-1) Z (W - Z^-1)), so
  * a W that has drifted by rounding returns to FP32 rounding of Z^-1 without
  * the re-evaluation's FP64 X^T X over all m rows.  Other kinds or FP64 OLS
@@ -380,8 +382,8 @@ linview_status linview_level_pass(int precision, int64_t n, void* P, int64_t ldp
  *   (ld >= M); B is K x N (ld >= N), or N x K when tb (ld >= K).  beta = 0
  *   ignores C's old contents.  M = 0 or N = 0 is an empty product (OK, no
  *   pointer is read); K >= 1.
- *  precision LINVIEW_F32: the tcgen05 split-TF32 GEMM (near-FP32 accuracy,
- *   three TF32 products per operand pair, FP32 accumulation) when M >= 128,
+ *  precision LINVIEW_F32: the tcgen05 split-operand GEMM (near-FP32 accuracy,
+ *   three FP16 or TF32 products per operand pair, FP32 accumulation) when M >= 128,
  *   N >= 8 and K >= 128, else the CUDA-core GEMM in FP32; LINVIEW_F64: the
  *   FP64 CUDA-core GEMM.
  * Temporary device memory (split operands, partial sums) is allocated

@@ -182,6 +182,8 @@ struct linview_program {
   int64_t gwork_elems = 0;
   float* hyA = nullptr;  // split rows of the old A (n x tc_split_ld(n))
   float* hyB = nullptr;  // split rows of D_{i-1}^T (p x tc_split_ld(n))
+  unsigned* hyW = nullptr;  // ... and their words (tc_words(n, p, n))
+  float* hyP = nullptr;     // ... and the pieces of its cut tiles
   // OLS: X (m x n), Y (m x p) on the device; views W, beta, X^T Y, X
   void* Xd = nullptr;
   int64_t ldX = 0;
@@ -592,12 +594,7 @@ static linview_status gemm_rm(linview_program* p, bool ta, bool tb, int64_t M, i
   return gemm_cm(p, tb, ta, N, M, K, alpha, B, ldb, A, lda, beta, C, ldc, s, mode);
 }
 
-// accurate arithmetic for the internal small GEMMs of the incremental path
-static int exact_mode(const linview_program* p) {
-  return p->elem == 8 ? LINVIEW_REEVAL_FP64 : LINVIEW_REEVAL_FP32;
-}
-
-// the program's re-evaluation arithmetic: the library's own GEMM (split-TF32
+// the program's re-evaluation arithmetic: the library's own GEMM (split-operand
 // tensor cores for FP32, FP64 CUDA cores for FP64) unless a library
 // comparison mode was selected
 static int reeval_mode(const linview_program* p) {
@@ -684,12 +681,13 @@ static void tfree(linview_program* p, void* ptr, size_t bytes_in, cudaStream_t s
 }
 
 // Split-operand scratch of the tensor-core GEMM: rows of A_s, then of B_s,
-// then room for the K parts of a split product.
-constexpr int64_t kTcWorkFloats = int64_t(4) << 20;  // 16 MB
+// their words, then room for the pieces of tiles cut along K.
 struct TcScratch {
   float* a = nullptr;
   float* b = nullptr;
   float* work = nullptr;
+  int64_t work_floats = 0;
+  unsigned* words = nullptr;  // [flag (4 words) | words of A | words of B]
   int64_t a_rows = 0, b_rows = 0, K = 0;
   void* block = nullptr;  // temporary block owned by this scratch (null: borrowed)
   size_t bytes = 0;
@@ -699,6 +697,9 @@ struct TcScratch {
     if (block) tfree(p, block, bytes, s);
   }
 };
+static int64_t tc_words(int64_t a_rows, int64_t b_rows, int64_t K) {
+  return 4 + tc_split_words(a_rows, K) + tc_split_words(b_rows, K);
+}
 
 // Temporary split scratch for products with up to a_rows x K and b_rows x K
 // operands (FP32 programs; FP64 programs take the CUDA-core path and get none).
@@ -708,19 +709,24 @@ static linview_status tc_scratch(linview_program* p, TcScratch* sc, int64_t a_ro
   const int64_t ld = tc_split_ld(K);
   const size_t abytes = (size_t)alloc_bytes(a_rows * ld * 4);
   const size_t bbytes = (size_t)alloc_bytes(b_rows * ld * 4);
-  const size_t bytes = abytes + bbytes + (size_t)kTcWorkFloats * 4;
+  const size_t wbytes = (size_t)alloc_bytes(tc_words(a_rows, b_rows, K) * 4);
+  sc->work_floats = tc_work_floats(a_rows, b_rows, K, p->sms);
+  const size_t bytes = abytes + bbytes + wbytes + (size_t)sc->work_floats * 4;
   void* blk = nullptr;
   LV_TRY(talloc(p, bytes, &blk, s));
+  char* at = static_cast<char*>(blk);
   sc->block = blk;
   sc->bytes = bytes;
   sc->p = p;
   sc->s = s;
-  sc->a = static_cast<float*>(blk);
-  sc->b = reinterpret_cast<float*>(static_cast<char*>(blk) + abytes);
-  sc->work = reinterpret_cast<float*>(static_cast<char*>(blk) + abytes + bbytes);
+  sc->a = reinterpret_cast<float*>(at);
+  sc->b = reinterpret_cast<float*>(at + abytes);
+  sc->words = reinterpret_cast<unsigned*>(at + abytes + bbytes);
+  sc->work = reinterpret_cast<float*>(at + abytes + bbytes + wbytes);
   sc->a_rows = a_rows;
   sc->b_rows = b_rows;
   sc->K = K;
+  LV_CUDA(cudaMemsetAsync(sc->words, 0, sizeof(unsigned), s));  // no operand needs TF32 yet
   return LINVIEW_OK;
 }
 
@@ -734,31 +740,30 @@ static bool tc_eligible(const linview_program* p, const TcScratch* sc, int64_t M
 
 // D (M x N, row-major, ldd) = alpha sum_k a(m, k) b(n, k) + beta C (C row-major,
 // ldc; may be D; beta == 0 ignores it), with a = rows of op(A) (M x K) and b =
-// rows of op(B)^T (N x K).  FP32 with scratch: split TF32 on the tensor cores
-// (a_ready / b_ready: the scratch already holds that operand's split rows);
+// rows of op(B)^T (N x K).  FP32 with scratch: split operands on the tensor cores
+// (a_ready / b_ready: the scratch already holds that operand's split rows;
+// reverse: visit K from its end, for every other product with the same A);
 // otherwise the CUDA-core GEMM in the program's arithmetic.
 static linview_status gemm_ab(linview_program* p, int64_t M, int64_t N, int64_t K, double alpha,
                               Opnd a, Opnd b, double beta, const void* C, int64_t ldc, void* D,
                               int64_t ldd, cudaStream_t s, TcScratch* sc = nullptr,
-                              bool a_ready = false, bool b_ready = false) {
+                              bool a_ready = false, bool b_ready = false,
+                              bool reverse = false) {
   if (M <= 0 || N <= 0) return LINVIEW_OK;
   const int e = p->elem;
   if (tc_eligible(p, sc, M, N, K)) {
-    const int64_t ld = tc_split_ld(K);
-    if (!a_ready) {
-      LV_CUDA(launch_split_rows(static_cast<const float*>(a.p), a.rs, a.cs, (int)M, (int)K, sc->a,
-                                ld, s));
-      p->all_launches++;
+    const TcOperand ta{static_cast<const float*>(a.p), a.rs, a.cs, (int)M, (int)K, sc->a,
+                       sc->words + 4};
+    const TcOperand tb{static_cast<const float*>(b.p), b.rs, b.cs, (int)N, (int)K, sc->b,
+                       sc->words + 4 + tc_split_words(sc->a_rows, sc->K)};
+    if (!a_ready || !b_ready) {
+      LV_CUDA(launch_tc_split(a_ready ? nullptr : &ta, b_ready ? nullptr : &tb, sc->words, s));
+      p->all_launches += 2;
     }
-    if (!b_ready) {
-      LV_CUDA(launch_split_rows(static_cast<const float*>(b.p), b.rs, b.cs, (int)N, (int)K, sc->b,
-                                ld, s));
-      p->all_launches++;
-    }
-    LV_CUDA(launch_tc_gemm(sc->a, sc->b, (int)M, (int)N, (int)K, static_cast<float*>(D), ldd,
+    LV_CUDA(launch_tc_gemm(ta, tb, sc->words, static_cast<float*>(D), ldd,
                            static_cast<const float*>(C), ldc, (float)alpha, (float)beta, p->sms,
-                           p->status, s, sc->work, sc->work ? kTcWorkFloats : 0));
-    p->all_launches++;
+                           p->status, s, sc->work, sc->work_floats, reverse));
+    p->all_launches += 2;
     return LINVIEW_OK;
   }
   if (beta != 0.0 && C != D)
@@ -1387,7 +1392,7 @@ static linview_status iter_reeval(linview_program* p, cudaStream_t s) {
                                        static_cast<float*>(ti), p->ldT, s));
     } else {  // T_i = A T_{i-1} + B, A's rows split once
       LV_TRY(gemm_ab(p, n, pp, n, 1.0, rows_of(a.ptr, a.ld), cols_of(tp, p->ldT), 1.0, p->Bm,
-                     p->ldB, ti, p->ldT, s, &sc, i > 1));
+                     p->ldB, ti, p->ldT, s, &sc, i > 1, false, i % 2 == 0));
     }
   }
   return LINVIEW_OK;
@@ -1447,6 +1452,10 @@ static linview_status iter_create(linview_program* p, const void* const* inputs,
       p->hyA = static_cast<float*>(t);
       LV_TRY(dalloc(p, (size_t)pp * tc_split_ld(n) * 4, &t, s));
       p->hyB = static_cast<float*>(t);
+      LV_TRY(dalloc(p, (size_t)tc_words(n, pp, n) * 4, &t, s));
+      p->hyW = static_cast<unsigned*>(t);
+      LV_TRY(dalloc(p, (size_t)tc_work_floats(n, pp, n, p->sms) * 4, &t, s));
+      p->hyP = static_cast<float*>(t);
     }
   }
   return iter_reeval(p, s);
@@ -1510,7 +1519,6 @@ static linview_status panel_update(linview_program* p, char* Tp, const T* K, con
 template <typename T>
 static linview_status iter_propagate(linview_program* p, int r, cudaStream_t s) {
   const int n = (int)p->d.n;
-  const int64_t pp = p->d.p;
   const int k = p->d.k;
   const int64_t fs = p->fs;
   T* K = static_cast<T*>(p->Kar);
@@ -1604,7 +1612,7 @@ static linview_status iter_propagate_b(linview_program* p, int rb, cudaStream_t 
 // D_{i-1}; then A += U V^T.  For dB = U_b V_b^T (U_b in K_0, V_b in the first
 // block of M; A unchanged):  D_1 = U_b V_b^T,  D_i = A D_{i-1} + U_b V_b^T,
 // and B += U_b V_b^T.  Each step is one n x n x p product with A (the own
-// split-TF32 GEMM, or one products pass over A when p is a few columns), the
+// split-operand GEMM, or one products pass over A when p is a few columns), the
 // rank-r term and T_i += D_i.  Column-major views:
 // T_i^T, D_i^T are p x n (ld ldT, ldD), A's row-major storage is A^T.
 template <typename T>
@@ -1612,7 +1620,6 @@ static linview_status iter_propagate_hybrid(linview_program* p, int r, bool b_up
                                             cudaStream_t s) {
   const int64_t n = p->d.n, pp = p->d.p;
   const int k = p->d.k;
-  const int64_t fs = p->fs;
   const T* K = static_cast<const T*>(p->Kar);
   const T* V1 = static_cast<const T*>(p->V1);
   T* W = static_cast<T*>(p->Mr);  // p x r: (V^T T'_{i-1})^T, or V_b for dB
@@ -1625,6 +1632,10 @@ static linview_status iter_propagate_hybrid(linview_program* p, int r, bool b_up
   if (p->hyA) {
     hy.a = p->hyA;
     hy.b = p->hyB;
+    hy.words = p->hyW;
+    hy.work = p->hyP;
+    hy.work_floats = tc_work_floats(n, pp, n, p->sms);
+    LV_CUDA(cudaMemsetAsync(p->hyW, 0, sizeof(unsigned), s));
     hy.a_rows = n;
     hy.b_rows = pp;
     hy.K = n;
@@ -1642,7 +1653,7 @@ static linview_status iter_propagate_hybrid(linview_program* p, int r, bool b_up
         LV_TRY(view_panel_product<T>(p, a, false, dp, p->ldD, (int)pp, nullptr, 0, dc, p->ldD, s));
       } else {
         LV_TRY(gemm_ab(p, n, pp, n, 1.0, rows_of(a.ptr, a.ld), cols_of(dp, p->ldD), 0.0, nullptr,
-                       0, dc, p->ldD, s, p->hyA ? &hy : nullptr, a_split));
+                       0, dc, p->ldD, s, p->hyA ? &hy : nullptr, a_split, false, i % 2 == 0));
         a_split = true;
       }
     }
@@ -1906,7 +1917,6 @@ static linview_status iter_sk_step(linview_program* p, int cur, View& tj, const 
 template <typename T>
 static linview_status iter_sk_propagate(linview_program* p, int r, cudaStream_t s) {
   const int n = (int)p->d.n;
-  const int64_t pp = p->d.p;
   const int k = p->d.k, sk = p->ie_s, Ls = p->ie_Ls, NT = p->ie_NT;
   const int64_t fs = p->fs;
   T* U = static_cast<T*>(p->Uar);
@@ -2034,7 +2044,6 @@ static linview_status iter_sk_step_b(linview_program* p, int cur, int c, int rb,
 
 template <typename T>
 static linview_status iter_sk_propagate_b(linview_program* p, int rb, cudaStream_t s) {
-  const int n = (int)p->d.n;
   const int64_t pp = p->d.p;
   const int Ls = p->ie_Ls, NT = p->ie_NT;
   const int64_t fs = p->fs;
@@ -2334,7 +2343,7 @@ static linview_status ols_history_push(linview_program* p, int kr, cudaStream_t 
 }
 
 // Newton-Schulz correction of an FP32 OLS program: R = I - Z W (double-float),
-// W <- W + W R (split-TF32 GEMM; W R is small, so its FP32-level error is far
+// W <- W + W R (split-operand GEMM; W R is small, so its FP32-level error is far
 // below W's rounding); then one step of iterative refinement of beta against
 // the normal equations, r = X^T Y - Z beta (double-float, X^T Y as pairs),
 // beta <- beta + W r.  (beta = W X^T Y from the corrected W would lose about
@@ -3039,7 +3048,7 @@ static linview_status adjoint_iteration(linview_program* p, const void* Gk, int6
                                          reinterpret_cast<float*>(ti), ldT, s));
       else
         LV_TRY(gemm_ab(p, n, pp, n, 1.0, rows_of(a.ptr, a.ld), cols_of(tp, ldT), 1.0, p->Bm,
-                       p->ldB, ti, ldT, s, &sc, i > 1));
+                       p->ldB, ti, ldT, s, &sc, i > 1, false, i % 2 == 0));
     }
   }
   // G_k = seed; G_i = A^T G_{i+1}
@@ -3065,7 +3074,7 @@ static linview_status adjoint_iteration(linview_program* p, const void* Gk, int6
                                        nullptr, 0, static_cast<float*>(gi), p->ldG, s));
     } else {
       LV_TRY(gemm_ab(p, n, pp, n, 1.0, cols_of(a.ptr, a.ld), cols_of(gn, p->ldG), 0.0, nullptr,
-                     0, gi, p->ldG, s, &sc, at_split));
+                     0, gi, p->ldG, s, &sc, at_split, false, i % 2 == 0));
       at_split = true;
     }
   }
@@ -3080,17 +3089,13 @@ static linview_status adjoint_iteration(linview_program* p, const void* Gk, int6
                      dT0, ld_dT0, s, &sc, at_split));
   }
   if (dB) {
-    LV_CUDA(cudaMemcpy2DAsync(dB, ld_dB * e, G, p->ldG * e, pp * e, n, cudaMemcpyDeviceToDevice, s));
-    for (int i = 2; i <= k; ++i) {
-      void* gi = G + (size_t)(i - 1) * pp * e;
-      if (e == 4)
-        LV_CUDA(launch_axpy_rows<float>(static_cast<float*>(dB), ld_dB, static_cast<float*>(gi),
-                                        p->ldG, 1.0f, (int)n, (int)pp, s));
-      else
-        LV_CUDA(launch_axpy_rows<double>(static_cast<double*>(dB), ld_dB,
-                                         static_cast<double*>(gi), p->ldG, 1.0, (int)n, (int)pp, s));
-      p->all_launches++;
-    }
+    if (e == 4)
+      LV_CUDA(launch_panel_sum<float>(reinterpret_cast<const float*>(G), p->ldG,
+                                      static_cast<float*>(dB), ld_dB, (int)n, (int)pp, k, s));
+    else
+      LV_CUDA(launch_panel_sum<double>(reinterpret_cast<const double*>(G), p->ldG,
+                                       static_cast<double*>(dB), ld_dB, (int)n, (int)pp, k, s));
+    p->all_launches++;
   }
   if (dA) {
     // dA = [G_1 .. G_k] [T_0 .. T_{k-1}]^T, one product with inner dimension k p

@@ -5,34 +5,45 @@
 // iteration's n x n x p products (T_i = A T_{i-1} + B, the hybrid strategy's
 // D_i = A D_{i-1}) and the small factor products of the general form.
 //
-//  * tc_gemm_kernel<BN> (FP32): D = A_s B_s^T (+ beta C) on tcgen05 in split
-//    TF32.  Every FP32 operand value x is split as x = hi + lo with hi = x
-//    rounded to nearest TF32 and lo = x - hi (exact in FP32) rounded to nearest
-//    TF32 in turn (so the tensor cores' handling of the low mantissa bits does
-//    not matter and the split carries no one-sided bias);
-//    A B^T ~= hi(A) hi(B)^T + lo(A) hi(B)^T + hi(A) lo(B)^T (the dropped
-//    lo lo^T term is ~2^-22 relative): near-FP32 accuracy, where one TF32
-//    product alone gives ~5e-4.  The operands are split
-//    beforehand by split_rows_kernel into K-major rows [hi(x) | lo(x)] (which
-//    also transposes where the product needs the other operand layout).
-//    Tiles of 128 x BN outputs (BN = 256, 128 or 64), K chunks of 32 values
-//    (one 128-byte swizzle atom); a persistent grid of one CTA per SM walks the
-//    tiles in groups of 8 row blocks (the A and B chunks a wave reads stay in
-//    L2).  Per CTA: warp 0 streams A and B chunks with TMA into an S-stage ring,
-//    one thread of warp 1 issues 12 MMAs per chunk (3 products x 4 K steps of
-//    8) into one of two BN-column FP32 accumulators in tensor memory, and the
-//    epilogue warps read the other accumulator back (tcgen05.ld).  The tensor
+//  * tc_gemm_kernel<BN> (FP32): D = A B^T (+ beta C) on tcgen05 from operands
+//    split into two 11-bit halves, x = hi + lo, and three products,
+//    A B^T ~= lo(A) hi(B)^T + hi(A) lo(B)^T + hi(A) hi(B)^T (the dropped lo lo^T
+//    term is ~2^-22 relative): near-FP32 accuracy, where one TF32 product alone
+//    gives ~5e-4.  The halves are FP16 by default (tcgen05 kind::f16, twice the
+//    rate and half the bytes of TF32): each run of 64 values of an operand row is
+//    scaled by a power of two that takes its largest entry to [2^14, 2^15), so
+//    that every entry down to 2^-17 of the run's largest keeps the 22 bits of a
+//    TF32 pair and a smaller one is off by at most 2^-40 of the largest; a run is
+//    one K chunk of the MMAs, whose result the epilogue scales back exactly as it
+//    adds it up.  Operands for which that is not enough (many small entries
+//    side by side, e.g. columns of very different scale), whose scale is out of
+//    the exponent's comfortable range, or that hold infinities or NaN are found
+//    while they are split, and such a product runs on TF32 halves instead (same
+//    kernel, kind::tf32; hi = x rounded to nearest
+//    TF32, lo = x - hi rounded in turn).  Operands are K-major rows [hi | lo]
+//    (the split also transposes where the product needs the other layout).
+//    CTA pairs (cta_group::2) compute tiles of 256 x BN outputs (BN = 256, 128 or
+//    64), each CTA holding 128 rows of A and half of B's rows, in K chunks of
+//    one 128-byte swizzle atom (64 FP16 or 32 TF32 values); a persistent grid
+//    walks the tiles in groups of 8 row blocks (the A and B chunks a wave reads
+//    stay in L2).  Per CTA: warp 0 streams its A and B chunks with TMA into an
+//    S-stage ring, one thread of the pair's first CTA issues 12 MMAs per chunk
+//    (3 products x 4 K steps of 32 bytes) into one of two BN-column FP32
+//    accumulators in tensor memory, and the epilogue warps read the other
+//    accumulator back (tcgen05.ld).  The tensor
 //    cores accumulate with round-toward-zero, a bias that grows with the number
 //    of accumulation steps (measured 7.9e-6 relative at K = 1000, ~6e-5 at
 //    K = 8192 if the whole K were accumulated in tensor memory), so the MMAs
-//    accumulate only segments of kSegChunks chunks into a fresh accumulator
-//    (each chunk's two small correction products first, while the accumulator
-//    is small), and the epilogue warps add each segment's result into FP32
+//    accumulate only one chunk into a fresh accumulator
+//    (its two small correction products first, while the accumulator
+//    is small), and the epilogue warps add each chunk's result into FP32
 //    registers (round to nearest), 128 columns per thread (8 epilogue warps
-//    for 256-column tiles, 4 otherwise); after the tile's last segment they
-//    add beta C and store D.
+//    for 256-column tiles, 4 otherwise); after the tile's last chunk they
+//    scale back, add beta C and store D.  Single CTAs on 128 x 256 tiles would
+//    read 96 bytes of shared memory per clock for the FP16 products and twice
+//    the operand bytes from L2; the pair halves B's share of both.
 //    Every wait is bounded; an expired wait latches LINVIEW_ETIMEOUT and the
-//    CTA drains its copies and MMAs and frees its tensor memory.
+//    pair drains its copies and MMAs and frees its tensor memory.
 //  * gemm_simt_kernel<T>: C = alpha op(A) op(B) + beta C with arbitrary
 //    strides on the CUDA cores (64 x 64 tiles, 4 x 4 outputs per thread), with
 //    a deterministic split of long inner dimensions (partials summed in a
@@ -40,6 +51,7 @@
 //    no fast FP64 tensor path) and the small FP32 factor products.
 #include <cuda_runtime.h>
 #include <cudaTypedefs.h>
+#include <cuda_fp16.h>
 
 #include "lv_device.cuh"
 #include "lv_internal.h"
@@ -48,42 +60,46 @@ namespace lv {
 
 namespace {
 
-constexpr int kGBM = 128;       // tile rows (MMA M)
+constexpr int kGBM = 256;       // tile rows (MMA M, 128 per CTA of the pair)
 constexpr int kGroupM = 8;      // row blocks per raster group
-#ifndef LV_GEMM_SEG_CHUNKS
-#define LV_GEMM_SEG_CHUNKS 1
-#endif
-// K chunks of 32 accumulated in tensor memory per segment (compile-time tuning)
-constexpr int kSegChunks = LV_GEMM_SEG_CHUNKS;
 
 template <int BN>
 struct GShape {
-  static constexpr uint32_t AHalf = kGBM * 128;           // one half (hi or lo) of an A chunk
-  static constexpr uint32_t BHalf = BN * 128;
-  static constexpr uint32_t StageBytes = 2 * AHalf + 2 * BHalf;
-  static constexpr int S = BN == 256 ? 2 : (BN == 128 ? 3 : 4);
+  static constexpr uint32_t AHalf = 128 * 128;            // one half (hi or lo) of a CTA's A chunk
+  static constexpr uint32_t BHalf = BN / 2 * 128;         // ... of its B chunk
+  static constexpr uint32_t StageBytes = 2 * AHalf + 2 * BHalf;  // 64, 48, 40 KB
+  static constexpr int S = BN == 256 ? 3 : (BN == 128 ? 4 : 5);
   static constexpr uint32_t OffBar = S * StageBytes;
-  static constexpr uint32_t SmemBytes = OffBar + 256 + 1024;  // + alignment slack
-  static constexpr uint32_t TmemCols = 2 * BN;                // two accumulators
+  static constexpr int NB = 512 / BN;                         // accumulators (all of tensor memory)
+  static constexpr uint32_t TmemCols = 512;
   static constexpr int CW = BN < 128 ? BN : 128;              // columns per epilogue thread
   static constexpr int NE = 4 * (BN / CW);                    // epilogue warps
-  static constexpr int Threads = 64 + 32 * NE;
-  // instruction descriptor: D F32, A/B TF32, both K-major, N = BN, M = 128
-  static constexpr uint32_t Idesc = (1u << 4) | (2u << 7) | (2u << 10) |
-                                    ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(kGBM >> 4) << 24);
+  static constexpr uint32_t OffScale = OffBar + 512;          // [NE][CW] column factors of a chunk
+  static constexpr uint32_t SmemBytes = OffScale + NE * CW * 4 + 1024;  // + alignment slack
+  // warps 0-3: copies, MMAs, two idle; then the epilogue
+  static constexpr int Threads = 128 + 32 * NE;
+  // With eight epilogue warps (BN = 256) a thread has 168 registers, too few for
+  // 128 sums and the 64 accumulator columns in flight: the first four warps hand
+  // theirs over (40 x 128 + 224 x 256 <= 168 x 384).
+  static constexpr bool Rebalance = NE == 8;
+  // instruction descriptor: D F32, A and B K-major, N = BN, M = 256; the operand
+  // type fields are 0 (F16) or 2 (TF32)
+  static constexpr uint32_t Idesc16 =
+      (1u << 4) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(kGBM >> 4) << 24);
+  static constexpr uint32_t Idesc32 = Idesc16 | (2u << 7) | (2u << 10);
 };
 static_assert(GShape<256>::SmemBytes <= 232448 && GShape<128>::SmemBytes <= 232448 &&
                   GShape<64>::SmemBytes <= 232448,
               "shared memory per CTA");
 
 struct GBars {
-  uint64_t full[4], empty[4];
-  uint64_t acc_full[2], acc_empty[2];
+  uint64_t full[5], empty[5];
+  uint64_t acc_full[8], acc_empty[8];
   uint64_t drain;
   uint32_t tmem_base;
   int abort;
 };
-static_assert(sizeof(GBars) <= 256, "barrier block");
+static_assert(sizeof(GBars) <= 512, "barrier block");
 
 // shared-memory descriptor of a K-major operand in 128-byte swizzled rows,
 // 8-row groups 1024 bytes apart (the layout TMA writes with SWIZZLE_128B)
@@ -97,20 +113,31 @@ __device__ __forceinline__ uint64_t g_desc(uint32_t saddr) {
   return d;
 }
 
+template <bool F16>
 __device__ __forceinline__ void g_mma(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc,
                                       uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
-      : "memory");
+  if constexpr (F16)
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
+        : "memory");
+  else
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
+        : "memory");
 }
 
+// arrive on ``bar`` of both CTAs of the pair once every MMA issued so far is done
 __device__ __forceinline__ void g_commit(uint64_t* bar) {
   asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-          smem_u32(bar))
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 "
+      "[%0], %1;" ::"r"(smem_u32(bar)),
+      "h"((uint16_t)3)
       : "memory");
 }
 
@@ -121,17 +148,39 @@ __device__ __forceinline__ void g_fence_after() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
-__device__ __forceinline__ void g_tmem_ld16(uint32_t taddr, float (&v)[16]) {
-  uint32_t r[16];
+__device__ __forceinline__ uint32_t cta_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+// cluster-window address of a barrier of the pair's first CTA
+__device__ __forceinline__ uint32_t lead_bar(uint64_t* bar) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(a) : "r"(smem_u32(bar)));
+  return a;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+// TMA box into this CTA's shared memory, completing bytes on a barrier of the pair
+__device__ __forceinline__ void g_tma(void* dst, const void* tmap, int x, int y, uint32_t bar) {
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, "
-      "%11, %12, %13, %14, %15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-        "=r"(r[14]), "=r"(r[15])
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%2, %3}], [%4];" ::"r"(smem_u32(dst)),
+      "l"(reinterpret_cast<uint64_t>(tmap)), "r"(x), "r"(y), "r"(bar)
+      : "memory");
+}
+__device__ __forceinline__ void g_arrive_lead(uint32_t bar) {
+  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar)
+               : "memory");
+}
+
+// 32 columns of this warp's 32 lanes (complete after g_tmem_wait_ld)
+__device__ __forceinline__ void g_tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr));
-#pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
 __device__ __forceinline__ void g_tmem_wait_ld() {
@@ -140,10 +189,21 @@ __device__ __forceinline__ void g_tmem_wait_ld() {
 
 __device__ __forceinline__ bool g_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
                                        unsigned* status) {
+  if (mbar_try_wait(bar, parity)) return true;
   if (*abort_flag) return false;
   if (mbar_wait_bounded(bar, parity, status)) return true;
   *abort_flag = 1;
   return false;
+}
+// one lane of a converged warp
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(p));
+  return p != 0;
 }
 
 // tile t of the raster: groups of kGroupM row blocks, column blocks within
@@ -157,162 +217,276 @@ __device__ __forceinline__ void g_tile(long long t, int mt, int nt, int& mb, int
   nb = rem / gm;
 }
 
-// D (M x N, row-major, ldd) = alpha A_s B_s^T + beta C over inner length K (nk
-// chunks of 32); A_s / B_s: split rows [hi | lo] of length 2 kp (tensor maps
-// tmA: box 32 x 128, tmB: box 32 x BN, both 128-byte swizzle).
+__device__ __forceinline__ float pow2f(int e) { return __int_as_float((127 + e) << 23); }  // |e| <= 126
+
+// Work of one CTA pair: whole tiles pair, pair + npairs, .. < dp, then its range of
+// the chunk sequence of the tiles left over, which would leave most pairs idle as
+// whole tiles (their last wave).  A tile's pieces are numbered range + cut tile
+// (both grow along the sequence, so the numbers are distinct) and go to that
+// slot of the work buffer, unless one range covers the tile.
+struct GWork {
+  long long t, pos, end;
+  int npairs, dp, nk, pair;
+  int tile, kb, ke, slot;  // current piece; slot < 0: a whole tile
+  __device__ GWork(int pair_, int npairs_, int dp_, int cut, int tiles, int nk_)
+      : t(pair_), pos(0), end(0), npairs(npairs_), dp(dp_), nk(nk_), pair(pair_) {
+    if (pair < cut) {
+      const long long W = (long long)(tiles - dp) * nk;
+      pos = W * pair / cut;
+      end = W * (pair + 1) / cut;
+    }
+  }
+  __device__ bool next() {
+    if (t < dp) {
+      tile = (int)t;
+      kb = 0;
+      ke = nk;
+      slot = -1;
+      t += npairs;
+      return true;
+    }
+    if (pos >= end) return false;
+    const int r = (int)(pos / nk);
+    tile = dp + r;
+    kb = (int)(pos - (long long)r * nk);
+    ke = (int)(end - pos < nk - kb ? kb + (end - pos) : nk);
+    slot = kb == 0 && ke == nk ? -1 : pair + r;
+    pos += ke - kb;
+    return true;
+  }
+};
+
+struct GMaps {
+  CUtensorMap a16, b16, a32, b32;
+};
+struct GArgs {
+  int M, N, kp16, kp32;
+  float* D;
+  int64_t ldd;
+  const float* C;
+  int64_t ldc;
+  float alpha, beta;
+  int vec_ok;
+  int reverse;    // visit the K chunks last to first
+  int dp;         // tiles computed whole; the others are cut into ``cut`` equal ranges
+  int cut;        // of K chunks, one per CTA pair
+  float* work;    // [range + cut tile][256][BN] partial sums of the tiles cut
+  const float* sa;      // factors of A's and B's runs of 64: [chunk][row], strides pa, pb
+  const float* sb;
+  int64_t pa, pb;
+  unsigned* fmta;       // format of each split buffer, written here for later products
+  unsigned* fmtb;
+  const unsigned* flag;
+  unsigned* status;
+};
+
+// D (M x N, row-major, ldd) = alpha A B^T + beta C over the split rows [hi | lo]
+// (FP16: halves kp16 long; TF32: kp32 long).
 template <int BN>
-__global__ void __launch_bounds__(GShape<BN>::Threads, 1)
-    tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                   int M, int N, int nk, int kp, float* __restrict__ D, int64_t ldd,
-                   const float* __restrict__ C, int64_t ldc, float alpha, float beta, int vec_ok,
-                   int ksplit, float* __restrict__ work, unsigned* status) {
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GShape<BN>::Threads, 1)
+    tc_gemm_kernel(const __grid_constant__ GMaps maps, const GArgs a) {
   using Sh = GShape<BN>;
-  constexpr int S = Sh::S, CW = Sh::CW, NE = Sh::NE;
+  constexpr int S = Sh::S, CW = Sh::CW, NE = Sh::NE, NB = Sh::NB;
   extern __shared__ __align__(1024) unsigned char g_smem_raw[];
   const uint32_t raw = smem_u32(g_smem_raw);
   unsigned char* base = g_smem_raw + (((raw + 1023u) & ~1023u) - raw);
   GBars* bars = reinterpret_cast<GBars*>(base + Sh::OffBar);
   volatile int* abort_flag = &bars->abort;
+  unsigned* status = a.status;
   const int tid = threadIdx.x;
   const int warp = tid >> 5;
   const int lane = tid & 31;
-  const int mt = (M + kGBM - 1) / kGBM;
-  const int nt = (N + BN - 1) / BN;
-  // work items: (tile, K part); a split K (ksplit > 1) sends each part's
-  // product to work[part] and a second kernel sums the parts in order
-  const long long tiles = (long long)mt * nt;
-  const long long T = tiles * ksplit;
+  const uint32_t rank = cta_rank();
+  const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
 
   if (tid == 0) {
-    prefetch_tmap(&tmA);
-    prefetch_tmap(&tmB);
     for (int i = 0; i < S; ++i) {
       mbar_init(&bars->full[i], 1);
       mbar_init(&bars->empty[i], 1);
     }
-    for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < NB; ++i) {
       mbar_init(&bars->acc_full[i], 1);
-      mbar_init(&bars->acc_empty[i], NE);  // one arrival per epilogue warp
+      mbar_init(&bars->acc_empty[i], 2 * NE);  // one arrival per epilogue warp of the pair
     }
     mbar_init(&bars->drain, 1);
     bars->abort = 0;
     fence_mbar_init();
   }
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(&bars->tmem_base)),
                  "r"(Sh::TmemCols)
                  : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
   g_fence_before();
   __syncthreads();
+  cluster_sync();
   g_fence_after();
   const uint32_t tmem = bars->tmem_base;
+  griddep_wait();  // the splits
+  griddep_launch_dependents();
+  const bool f16 = *a.flag == 0u;
+  const int kc_len = f16 ? 64 : 32;
+  const int kp = f16 ? a.kp16 : a.kp32;
+  const int nk = kp / kc_len;
+  const int mt = (a.M + kGBM - 1) / kGBM;
+  const int nt = (a.N + BN - 1) / BN;
+  GWork work(pair, npairs, a.dp, a.cut, mt * nt, nk);
+  auto chunk = [&](int kc) { return a.reverse ? nk - 1 - kc : kc; };
+  if (blockIdx.x == 0 && tid == 0) {  // the buffers' format, for later products on the same split
+    *a.fmta = f16 ? 0u : 1u;
+    *a.fmtb = f16 ? 0u : 1u;
+  }
 
-  if (warp == 0) {
-    // ---------------- producer ----------------
-    if (lane == 0) {
-      long long g = 0;
-      for (long long t = blockIdx.x; t < T && !*abort_flag; t += gridDim.x) {
+  if (warp < 4) {
+    if constexpr (Sh::Rebalance) asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
+    if (warp == 0 && lane == 0) {
+      // ---------------- producer (each CTA its own half) ----------------
+      const CUtensorMap* ma = f16 ? &maps.a16 : &maps.a32;
+      const CUtensorMap* mb_ = f16 ? &maps.b16 : &maps.b32;
+      prefetch_tmap(ma);
+      prefetch_tmap(mb_);
+      const uint32_t lead_full = lead_bar(&bars->full[0]);
+      int st = 0;
+      uint32_t phase = 0;      // of the ring's current round
+      long long loaded = 0;    // chunks requested
+      while (!*abort_flag && work.next()) {
         int mb, nb;
-        g_tile(t % tiles, mt, nt, mb, nb);
-        const int ks = (int)(t / tiles);
-        const int kb = (int)((long long)nk * ks / ksplit), ke = (int)((long long)nk * (ks + 1) / ksplit);
-        for (int kc = kb; kc < ke; ++kc, ++g) {
-          const int st = (int)(g % S);
-          const long long use = g / S;
-          if (use >= 1 && !g_wait(&bars->empty[st], (uint32_t)((use - 1) & 1), abort_flag, status))
-            break;
+        g_tile(work.tile, mt, nt, mb, nb);
+        const int arow = mb * kGBM + (int)rank * 128, brow = nb * BN + (int)rank * (BN / 2);
+        for (int kc = work.kb; kc < work.ke; ++kc, ++loaded) {
+          if (loaded >= S && !g_wait(&bars->empty[st], phase ^ 1u, abort_flag, status)) break;
+          const int x = chunk(kc) * kc_len;
           unsigned char* sb = base + st * Sh::StageBytes;
-          mbar_arrive_expect_tx(&bars->full[st], Sh::StageBytes);
-          tma_load_2d(sb, &tmA, kc * 32, mb * kGBM, &bars->full[st]);
-          tma_load_2d(sb + Sh::AHalf, &tmA, kp + kc * 32, mb * kGBM, &bars->full[st]);
-          tma_load_2d(sb + 2 * Sh::AHalf, &tmB, kc * 32, nb * BN, &bars->full[st]);
-          tma_load_2d(sb + 2 * Sh::AHalf + Sh::BHalf, &tmB, kp + kc * 32, nb * BN,
-                      &bars->full[st]);
+          // the first CTA's barrier counts both CTAs' bytes
+          const uint32_t fb = lead_full + st * 8;
+          if (rank == 0) mbar_arrive_expect_tx(&bars->full[st], 2 * Sh::StageBytes);
+          g_tma(sb, ma, x, arow, fb);
+          g_tma(sb + Sh::AHalf, ma, kp + x, arow, fb);
+          g_tma(sb + 2 * Sh::AHalf, mb_, x, brow, fb);
+          g_tma(sb + 2 * Sh::AHalf + Sh::BHalf, mb_, kp + x, brow, fb);
+          if (++st == S) {
+            st = 0;
+            phase ^= 1u;
+          }
         }
       }
-      if (*abort_flag) {
+      if (*abort_flag && rank == 0) {
         // the stages loaded last may still be in flight: wait (bounded) for them
-        const long long first = g > S ? g - S : 0;
-        for (long long j = first; j < g; ++j)
+        const long long first = loaded > S ? loaded - S : 0;
+        for (long long j = first; j < loaded; ++j)
           mbar_wait_bounded(&bars->full[j % S], (uint32_t)((j / S) & 1), nullptr);
       }
     }
-  } else if (warp == 1) {
-    // ---------------- MMA issuer ----------------
-    if (lane == 0) {
-      long long g = 0, gs = 0;  // chunks and segments consumed
+    if (warp == 1 && rank == 0) {
+      // ---------------- MMA issuer (first CTA of the pair) ----------------
+      // The whole warp walks the chunks and one elected lane issues, so that the
+      // descriptors and counters are warp-uniform: with the loop inside a
+      // lane-0 branch every MMA took about 35 ns to issue and a chunk at least
+      // 0.70 us whatever its width (4096^3 in 64-column tiles 626 us, now 449).
+      int st = 0, buf = 0;
+      uint32_t phase = 0, aphase = 0;
+      bool first_round = true;  // the accumulators have not been used yet
+      const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+      const uint64_t d0 = g_desc(smem_u32(base));
       bool ok = true;
-      for (long long t = blockIdx.x; t < T && ok && !*abort_flag; t += gridDim.x) {
-        const int ks = (int)(t / tiles);
-        const int kb = (int)((long long)nk * ks / ksplit), ke = (int)((long long)nk * (ks + 1) / ksplit);
-        const int nseg = (ke - kb + kSegChunks - 1) / kSegChunks;
-        for (int sg = 0; sg < nseg && ok; ++sg, ++gs) {
-          const int buf = (int)(gs & 1);
-          const long long ause = gs >> 1;
-          if (ause >= 1 &&
-              !g_wait(&bars->acc_empty[buf], (uint32_t)((ause - 1) & 1), abort_flag, status)) {
+      while (ok && !*abort_flag && work.next()) {
+        for (int kc = work.kb; kc < work.ke; ++kc) {
+          if ((!first_round && !g_wait(&bars->acc_empty[buf], aphase ^ 1u, abort_flag, status)) ||
+              !g_wait(&bars->full[st], phase, abort_flag, status))
+            ok = false;
+          if (!__all_sync(0xffffffffu, ok)) {
             ok = false;
             break;
           }
           g_fence_after();
-          const uint32_t d = tmem + buf * BN;
-          const int kc0 = kb + sg * kSegChunks;
-          const int kc1 = kc0 + kSegChunks < ke ? kc0 + kSegChunks : ke;
-          for (int kc = kc0; kc < kc1; ++kc, ++g) {
-            const int st = (int)(g % S);
-            if (!g_wait(&bars->full[st], (uint32_t)((g / S) & 1), abort_flag, status)) {
-              ok = false;
-              break;
-            }
-            g_fence_after();
-            const uint32_t a_hi = smem_u32(base + st * Sh::StageBytes);
-            const uint32_t a_lo = a_hi + Sh::AHalf;
-            const uint32_t b_hi = a_hi + 2 * Sh::AHalf;
-            const uint32_t b_lo = b_hi + Sh::BHalf;
+          if (elect_one()) {
+            const uint32_t d = tm + buf * BN;
+            const uint64_t a_hi = d0 + (uint32_t)st * (Sh::StageBytes >> 4);
+            const uint64_t a_lo = a_hi + (Sh::AHalf >> 4);
+            const uint64_t b_hi = a_hi + (2 * Sh::AHalf >> 4);
+            const uint64_t b_lo = b_hi + (Sh::BHalf >> 4);
             // lo(A) hi(B), hi(A) lo(B), then hi(A) hi(B)
-            const uint32_t pa[3] = {a_lo, a_hi, a_hi};
-            const uint32_t pb[3] = {b_hi, b_lo, b_hi};
-            const bool first = kc == kc0;
+            const uint64_t pa[3] = {a_lo, a_hi, a_hi};
+            const uint64_t pb[3] = {b_hi, b_lo, b_hi};
+            if (f16) {
 #pragma unroll
-            for (int pr = 0; pr < 3; ++pr) {
+              for (int pr = 0; pr < 3; ++pr)
 #pragma unroll
-              for (int kk = 0; kk < 4; ++kk)  // K = 8 per MMA: 32 bytes of a 128-byte row
-                g_mma(d, g_desc(pa[pr] + kk * 32), g_desc(pb[pr] + kk * 32), Sh::Idesc,
-                      (!first || pr != 0 || kk != 0) ? 1u : 0u);
+                for (int kk = 0; kk < 4; ++kk)  // 32 bytes of a 128-byte row per MMA
+                  g_mma<true>(d, pa[pr] + kk * 2, pb[pr] + kk * 2, Sh::Idesc16,
+                              (pr != 0 || kk != 0) ? 1u : 0u);
+            } else {
+#pragma unroll
+              for (int pr = 0; pr < 3; ++pr)
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk)
+                  g_mma<false>(d, pa[pr] + kk * 2, pb[pr] + kk * 2, Sh::Idesc32,
+                               (pr != 0 || kk != 0) ? 1u : 0u);
             }
             g_commit(&bars->empty[st]);
+            g_commit(&bars->acc_full[buf]);
           }
-          if (!ok) break;
-          g_commit(&bars->acc_full[buf]);
+          __syncwarp();
+          if (++st == S) {
+            st = 0;
+            phase ^= 1u;
+          }
+          if (++buf == NB) {
+            buf = 0;
+            aphase ^= 1u;
+            first_round = false;
+          }
         }
       }
       // every MMA issued has completed before the tensor memory is freed
-      g_commit(&bars->drain);
-      mbar_wait_bounded(&bars->drain, 0, status);
+      if (elect_one()) g_commit(&bars->drain);
+      __syncwarp();
     }
+    // both CTAs: the MMAs' arrivals have reached this CTA's barriers
+    if (warp == 1 && lane == 0) mbar_wait_bounded(&bars->drain, 0, status);
   } else {
-    // ---------------- epilogue (warps 2 .. 2 + NE - 1) ----------------
-    const int ew = warp - 2;
+    // ---------------- epilogue (warps 4 .. 4 + NE - 1) ----------------
+    if constexpr (Sh::Rebalance) asm volatile("setmaxnreg.inc.sync.aligned.u32 224;");
+    const int ew = warp - 4;
     const int quarter = warp & 3;     // tensor-memory lanes 32*quarter .. +31
     const int cpart = ew >> 2;        // column part: columns cpart*CW .. +CW-1
     const int row = quarter * 32 + lane;
-    long long gs = 0;
+    float* cs = reinterpret_cast<float*>(base + Sh::OffScale) + ew * CW;
+    const uint32_t ae = lead_bar(&bars->acc_empty[0]);
+    int buf = 0;
+    uint32_t aphase = 0;
     bool ok = true;
-    for (long long t = blockIdx.x; t < T && ok; t += gridDim.x) {
+    while (ok && work.next()) {
       int mb, nb;
-      g_tile(t % tiles, mt, nt, mb, nb);
-      const int ks = (int)(t / tiles);
-      const int kb = (int)((long long)nk * ks / ksplit), ke = (int)((long long)nk * (ks + 1) / ksplit);
-      const int nseg = (ke - kb + kSegChunks - 1) / kSegChunks;
-      float acc[CW];
+      g_tile(work.tile, mt, nt, mb, nb);
+      const int grow = mb * kGBM + (int)rank * 128 + row;
+      const int gc0 = nb * BN + cpart * CW;
+      // the chunk's factors, loaded one chunk ahead: this thread's row, and four
+      // columns a lane to be shared with the warp
+      const bool has_row = f16 && grow < a.M, has_col = f16 && 4 * lane < CW && gc0 + 4 * lane < a.pb;
+      const float* sa = a.sa + grow;
+      const float* sb = a.sb + gc0 + 4 * lane;
+      auto row_factor = [&](int kc) { return has_row ? __ldg(sa + chunk(kc) * a.pa) : 1.f; };
+      auto col_factors = [&](int kc) {
+        return has_col ? __ldg(reinterpret_cast<const float4*>(sb + chunk(kc) * a.pb))
+                       : make_float4(1.f, 1.f, 1.f, 1.f);
+      };
+      float fr_next = row_factor(work.kb);
+      float4 fc_next = col_factors(work.kb);
+      float2 acc[CW / 2];
 #pragma unroll
-      for (int c = 0; c < CW; ++c) acc[c] = 0.f;
-      for (int sg = 0; sg < nseg; ++sg, ++gs) {
-        const int buf = (int)(gs & 1);
-        const bool w = g_wait(&bars->acc_full[buf], (uint32_t)((gs >> 1) & 1), abort_flag, status);
+      for (int c = 0; c < CW / 2; ++c) acc[c] = make_float2(0.f, 0.f);
+      for (int kc = work.kb; kc < work.ke; ++kc) {
+        const float2 fr2 = make_float2(fr_next, fr_next);
+        __syncwarp();
+        if (4 * lane < CW) reinterpret_cast<float4*>(cs)[lane] = fc_next;
+        if (kc + 1 < work.ke) {
+          fr_next = row_factor(kc + 1);
+          fc_next = col_factors(kc + 1);
+        }
+        const bool w = g_wait(&bars->acc_full[buf], aphase, abort_flag, status);
         if (!__all_sync(0xffffffffu, w)) {  // tcgen05.ld is warp-collective
           ok = false;
           break;
@@ -320,91 +494,243 @@ __global__ void __launch_bounds__(GShape<BN>::Threads, 1)
         g_fence_after();
         const uint32_t ta = tmem + ((uint32_t)(quarter * 32) << 16) + buf * BN + cpart * CW;
 #pragma unroll
-        for (int q = 0; q < CW / 16; ++q) {
-          float v[16];
-          g_tmem_ld16(ta + q * 16, v);
+        for (int q = 0; q < CW / 64; ++q) {  // 64 columns in flight
+          uint32_t v[2][32];
+          g_tmem_ld32(ta + q * 64, v[0]);
+          g_tmem_ld32(ta + q * 64 + 32, v[1]);
           g_tmem_wait_ld();
+          if (q == CW / 64 - 1) {  // all read: the accumulator is free
+            g_fence_before();
+            __syncwarp();
+            if (lane == 0) g_arrive_lead(ae + buf * 8);
+          }
 #pragma unroll
-          for (int e = 0; e < 16; ++e) acc[q * 16 + e] += v[e];
+          for (int e = 0; e < 16; ++e) {
+            // the factors are powers of two: one rounding, in the addition
+            const float4 f = reinterpret_cast<const float4*>(cs)[q * 16 + e];
+            const uint32_t* x = &v[e / 8][e % 8 * 4];
+            float2& a0 = acc[q * 32 + 2 * e];
+            float2& a1 = acc[q * 32 + 2 * e + 1];
+            a0 = __ffma2_rn(__fmul2_rn(make_float2(__uint_as_float(x[0]), __uint_as_float(x[1])),
+                                       make_float2(f.x, f.y)), fr2, a0);
+            a1 = __ffma2_rn(__fmul2_rn(make_float2(__uint_as_float(x[2]), __uint_as_float(x[3])),
+                                       make_float2(f.z, f.w)), fr2, a1);
+          }
         }
-        g_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&bars->acc_empty[buf]);  // the accumulator is free
+        if (++buf == NB) {
+          buf = 0;
+          aphase ^= 1u;
+        }
       }
       if (!ok) break;
-      const int grow = mb * kGBM + row;
-      const int gc0 = nb * BN + cpart * CW;
-      if (ksplit > 1) {  // this K part's product, to be summed by gemm_parts_kernel
-        if (grow < M && gc0 < N) {
-          float* wrow = work + ((int64_t)ks * M + grow) * N + gc0;
+      if (grow < a.M && gc0 < a.N) {
+        if (work.slot >= 0) {  // a piece of a tile, to be summed by gemm_parts_kernel
+          float4* wrow = reinterpret_cast<float4*>(
+              a.work + ((int64_t)work.slot * kGBM + rank * 128 + row) * BN + cpart * CW);
 #pragma unroll
-          for (int j = 0; j < CW; ++j)
-            if (gc0 + j < N) wrow[j] = acc[j];
-        }
-      } else if (grow < M && gc0 < N) {
-        float* drow = D + (int64_t)grow * ldd + gc0;
-        const float* crow = (C && beta != 0.f) ? C + (int64_t)grow * ldc + gc0 : nullptr;
-        if (vec_ok && gc0 + CW <= N) {
-#pragma unroll
-          for (int j = 0; j < CW / 4; ++j) {
-            float4 o = make_float4(alpha * acc[4 * j], alpha * acc[4 * j + 1],
-                                   alpha * acc[4 * j + 2], alpha * acc[4 * j + 3]);
-            if (crow) {
-              const float4 c = *reinterpret_cast<const float4*>(crow + 4 * j);
-              o.x += beta * c.x;
-              o.y += beta * c.y;
-              o.z += beta * c.z;
-              o.w += beta * c.w;
-            }
-            *reinterpret_cast<float4*>(drow + 4 * j) = o;
-          }
+          for (int j = 0; j < CW / 4; ++j)
+            wrow[j] = make_float4(acc[2 * j].x, acc[2 * j].y, acc[2 * j + 1].x, acc[2 * j + 1].y);
         } else {
+          float* drow = a.D + (int64_t)grow * a.ldd + gc0;
+          const float* crow = (a.C && a.beta != 0.f) ? a.C + (int64_t)grow * a.ldc + gc0 : nullptr;
+          if (a.vec_ok && gc0 + CW <= a.N) {
 #pragma unroll
-          for (int j = 0; j < CW; ++j) {
-            if (gc0 + j < N) drow[j] = alpha * acc[j] + (crow ? beta * crow[j] : 0.f);
+            for (int j = 0; j < CW / 4; ++j) {
+              float4 o = make_float4(a.alpha * acc[2 * j].x, a.alpha * acc[2 * j].y,
+                                     a.alpha * acc[2 * j + 1].x, a.alpha * acc[2 * j + 1].y);
+              if (crow) {
+                const float4 c = *reinterpret_cast<const float4*>(crow + 4 * j);
+                o.x += a.beta * c.x;
+                o.y += a.beta * c.y;
+                o.z += a.beta * c.z;
+                o.w += a.beta * c.w;
+              }
+              *reinterpret_cast<float4*>(drow + 4 * j) = o;
+            }
+          } else {
+#pragma unroll
+            for (int j = 0; j < CW; ++j) {
+              if (gc0 + j < a.N)
+                drow[j] = a.alpha * (j & 1 ? acc[j / 2].y : acc[j / 2].x) +
+                          (crow ? a.beta * crow[j] : 0.f);
+            }
           }
         }
       }
+      __syncwarp();
     }
   }
   g_fence_before();
   __syncthreads();
+  cluster_sync();  // neither CTA leaves while the other's MMAs or copies use its memory
   if (warp == 1) {
     g_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem),
                  "r"(Sh::TmemCols)
                  : "memory");
   }
 }
 
-// Split rows: element (i, k) of the source, X[i * rs + k * cs] (i < rows,
-// k < K), goes to dst row i as hi at column k and lo at column kp + k (kp =
-// rup(K, 32)); columns K .. kp - 1 of both halves are zero.  32 x 32 tiles
-// through shared memory, read along whichever source index has unit stride.
-__global__ void __launch_bounds__(256) split_rows_kernel(const float* __restrict__ X, int64_t rs,
-                                                         int64_t cs, int rows, int K, int kp,
-                                                         float* __restrict__ dst, int64_t ldd) {
-  __shared__ float tile[32][33];
-  const int k0 = blockIdx.x * 32, i0 = blockIdx.y * 32;
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 8 warps
-  const bool k_fast = cs == 1;
-  for (int j = ty; j < 32; j += 8) {
-    const int il = k_fast ? j : tx, kl = k_fast ? tx : j;
-    const int i = i0 + il, k = k0 + kl;
-    tile[il][kl] = (i < rows && k < K) ? X[(int64_t)i * rs + (int64_t)k * cs] : 0.f;
+// ---------------------------------------------------------------- operand split
+// Element (i, k) of op(X) is X[i * rs + k * cs] with rs or cs == 1.
+struct SplitOp {
+  const float* X;
+  int64_t rs, cs;
+  int rows, K;
+  unsigned char* dst;
+  float* sc;        // factors of the runs of 64, [run][row] with stride ``pitch``
+  int64_t pitch;
+  unsigned* fmt;    // 0: FP16 rows, 1: TF32 rows
+  int vec;          // rows of X start on 16-byte units
+  int blocks;       // CTAs of this operand in the launch at hand
+};
+struct SplitPair {
+  SplitOp o[2];
+  unsigned* flag;
+};
+
+// FP16 halves: tiles of 64 rows x 128 k (two runs), rows of 2 kp halves [hi | lo]
+// (kp = rup(K, 64), zero past K), one pass over the operand: eight lanes hold a
+// run and find its largest entry by shuffles.  An entry y = 2^sh x with 0 < |y| <
+// 2^-2 has fewer than 22 bits; eight of them among 32 neighbours of a row or of a
+// column of a tile (dense data without such structure has none), a scale outside
+// 2^-60 .. 2^60 or a non-finite entry sets the flag that sends the product to TF32.
+// 8192 x 8192: 101 us transposed, 93 us not, 4 bytes read and 4 written per entry
+// (floor 79); TF32 halves (8 written) took 196 us.
+constexpr int kSpR = 64, kSpK = 128, kSmallCount = 8;
+__global__ void __launch_bounds__(256) split_f16_kernel(const __grid_constant__ SplitPair sp) {
+  __shared__ float tile[kSpK][kSpR + 1];
+  __shared__ int rowcnt[kSpR][kSpK / 32], colcnt[kSpR / 32][kSpK];
+  const bool second = (int)blockIdx.x >= sp.o[0].blocks;
+  const SplitOp& o = sp.o[second];
+  const int b = blockIdx.x - (second ? sp.o[0].blocks : 0);
+  const int kp = (o.K + 63) / 64 * 64;
+  const int kb = (kp + kSpK - 1) / kSpK, ib = (o.rows + kSpR - 1) / kSpR;
+  // neighbouring CTAs read neighbouring memory
+  const int i0 = (o.cs == 1 ? b / kb : b % ib) * kSpR, k0 = (o.cs == 1 ? b % kb : b / ib) * kSpK;
+  const int tid = threadIdx.x;
+  griddep_wait();
+  griddep_launch_dependents();
+  if (b == 0 && tid == 0) *o.fmt = 0u;
+  (&rowcnt[0][0])[tid] = 0;
+  (&colcnt[0][0])[tid] = 0;
+  if (o.cs != 1) {  // transpose: 16 lanes read 64 rows of one k
+    const int il = 4 * (tid & 15);
+#pragma unroll
+    for (int u = 0; u < kSpK / 16; ++u) {
+      const int kl = u * 16 + (tid >> 4), k = k0 + kl, i = i0 + il;
+      float v[4] = {0.f, 0.f, 0.f, 0.f};
+      if (k < o.K) {
+        const float* col = o.X + (int64_t)k * o.cs + i;
+        if (o.vec && i + 4 <= o.rows) {
+          const float4 x = *reinterpret_cast<const float4*>(col);
+          v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+        } else {
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            if (i + e < o.rows) v[e] = col[e];
+        }
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) tile[kl][il + e] = v[e];
+    }
   }
   __syncthreads();
-  for (int j = ty; j < 32; j += 8) {
-    const int i = i0 + j, k = k0 + tx;
-    if (i >= rows || k >= kp) continue;
-    const float x = tile[j][tx];
-    // round to nearest TF32 (ties away from zero): add half of the dropped
-    // 13-bit field, then clear it; x - hi is exact
-    const float hi = __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xFFFFE000u);
-    const float r = x - hi;
-    float* d = dst + (int64_t)i * ldd;
-    d[k] = hi;
-    d[kp + k] = __uint_as_float((__float_as_uint(r) + 0x1000u) & 0xFFFFE000u);
+  bool bad = false;
+#pragma unroll
+  for (int u = 0; u < kSpR * kSpK / (8 * 256); ++u) {
+    const int idx = u * 256 + tid;
+    const int il = idx / (kSpK / 8), kl = idx % (kSpK / 8) * 8;
+    const int i = i0 + il, k = k0 + kl;
+    const bool in = i < o.rows && k < kp;
+    float x[8];
+    if (o.cs == 1) {
+      const float* row = o.X + (int64_t)i * o.rs + k;
+      if (in && o.vec && k + 8 <= o.K) {
+        const float4 p = reinterpret_cast<const float4*>(row)[0];
+        const float4 q = reinterpret_cast<const float4*>(row)[1];
+        x[0] = p.x; x[1] = p.y; x[2] = p.z; x[3] = p.w;
+        x[4] = q.x; x[5] = q.y; x[6] = q.z; x[7] = q.w;
+      } else {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) x[e] = in && k + e < o.K ? row[e] : 0.f;
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < 8; ++e) x[e] = tile[kl + e][il];  // zeros past the operand
+    }
+    unsigned mx = 0;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) mx = max(mx, __float_as_uint(x[e]) & 0x7fffffffu);
+#pragma unroll
+    for (int d = 1; d < 8; d <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, d));
+    int sh = mx ? 14 - ((int)(mx >> 23) - 127) : 0;
+    bad |= sh > 60 || sh < -60;  // (non-finite: sh = -114)
+    sh = min(60, max(-60, sh));
+    const float sc = pow2f(sh);
+    __align__(16) __half hi[8], lo[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const float y = x[e] * sc;
+      hi[e] = __float2half_rn(y);
+      lo[e] = __float2half_rn(y - __half2float(hi[e]));
+      if (y != 0.f && fabsf(y) < 0.25f) {
+        atomicAdd(&rowcnt[il][(kl + e) / 32], 1);
+        atomicAdd(&colcnt[il / 32][kl + e], 1);
+      }
+    }
+    if (in) {
+      __half* d = reinterpret_cast<__half*>(o.dst) + (int64_t)i * 2 * kp + k;
+      *reinterpret_cast<uint4*>(d) = *reinterpret_cast<const uint4*>(hi);
+      *reinterpret_cast<uint4*>(d + kp) = *reinterpret_cast<const uint4*>(lo);
+      if (kl % 64 == 0) o.sc[(int64_t)(k / 64) * o.pitch + i] = pow2f(-sh);
+    }
+  }
+  __syncthreads();
+  bad |= (&rowcnt[0][0])[tid] >= kSmallCount || (&colcnt[0][0])[tid] >= kSmallCount;
+  if (__syncthreads_or(bad) && tid == 0) atomicOr(sp.flag, 1u);
+}
+
+// TF32 halves, only when the flag is set (else the kernel returns at once) and
+// the buffer does not hold them already: rows of 2 kp floats [hi | lo], kp =
+// rup(K, 32).  32 x 32 tiles through shared memory, read along whichever source
+// index has unit stride.
+__global__ void __launch_bounds__(256) split_tf32_kernel(const __grid_constant__ SplitPair sp) {
+  griddep_wait();
+  griddep_launch_dependents();
+  if (*sp.flag == 0u) return;
+  __shared__ float tile[32][33];
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 8 warps
+#pragma unroll 1
+  for (int w = 0; w < 2; ++w) {
+    const SplitOp& o = sp.o[w];
+    if (*o.fmt != 0u) continue;
+    const int kp = (o.K + 31) / 32 * 32;
+    const int kb = kp / 32;
+    const long long tiles = (long long)kb * ((o.rows + 31) / 32);
+    const bool k_fast = o.cs == 1;
+    for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {
+      const int k0 = (int)(t % kb) * 32, i0 = (int)(t / kb) * 32;
+      __syncthreads();
+      for (int j = ty; j < 32; j += 8) {
+        const int il = k_fast ? j : tx, kl = k_fast ? tx : j;
+        const int i = i0 + il, k = k0 + kl;
+        tile[il][kl] = (i < o.rows && k < o.K) ? o.X[(int64_t)i * o.rs + (int64_t)k * o.cs] : 0.f;
+      }
+      __syncthreads();
+      for (int j = ty; j < 32; j += 8) {
+        const int i = i0 + j, k = k0 + tx;
+        if (i >= o.rows) continue;
+        const float x = tile[j][tx];
+        // round to nearest TF32 (ties away from zero): add half of the dropped
+        // 13-bit field, then clear it; x - hi is exact
+        const float hi = __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xFFFFE000u);
+        const float r = x - hi;
+        float* d = reinterpret_cast<float*>(o.dst) + (int64_t)i * 2 * kp;
+        d[k] = hi;
+        d[kp + k] = __uint_as_float((__float_as_uint(r) + 0x1000u) & 0xFFFFE000u);
+      }
+    }
   }
 }
 
@@ -531,90 +857,226 @@ __global__ void gemm_reduce_kernel(int M, int N, int splits, int batch, T alpha,
   }
 }
 
-// D = alpha sum_q work[q] + beta C (the K parts of a split product, summed in order)
-__global__ void gemm_parts_kernel(int M, int N, int parts, const float* __restrict__ work,
-                                  float alpha, float beta, const float* C, int64_t ldc, float* D,
-                                  int64_t ldd) {
-  const int64_t total = (int64_t)M * N;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    float acc = work[e];
-    for (int q = 1; q < parts; ++q) acc += work[(int64_t)q * total + e];
-    const int m = (int)(e / N), n = (int)(e - (int64_t)m * N);
-    float o = alpha * acc;
-    if (C && beta != 0.f) o += beta * C[(int64_t)m * ldc + n];
-    D[(int64_t)m * ldd + n] = o;
+// D = alpha (pieces) + beta C for the tiles cut along K: a CTA adds 16 rows of one
+// tile, the pieces in their order along K.
+template <int BN>
+__global__ void __launch_bounds__(256) gemm_parts_kernel(const GArgs a, int tiles) {
+  griddep_wait();
+  griddep_launch_dependents();
+  const int r = blockIdx.x;
+  const int nk = *a.flag == 0u ? a.kp16 / 64 : a.kp32 / 32;
+  const long long W = (long long)(tiles - a.dp) * nk, lo = (long long)r * nk, hi = lo + nk;
+  // ranges that meet the tile: W c / cut < hi and W (c + 1) / cut > lo
+  int c0 = (int)(lo * a.cut / W), c1;
+  while (c0 > 0 && W * c0 / a.cut > lo) --c0;
+  while (W * (c0 + 1) / a.cut <= lo) ++c0;
+  c1 = c0;
+  while (W * (c1 + 1) / a.cut < hi) ++c1;
+  if (c0 == c1) return;  // computed whole
+  int mb, nb;
+  g_tile(a.dp + r, (a.M + kGBM - 1) / kGBM, (a.N + BN - 1) / BN, mb, nb);
+  for (int e = threadIdx.x; e < 16 * BN / 4; e += 256) {
+    const int row = blockIdx.y * 16 + e / (BN / 4), col = e % (BN / 4) * 4;
+    const int m = mb * kGBM + row, n = nb * BN + col;
+    if (m >= a.M || n >= a.N) continue;
+    const float* w = a.work + ((int64_t)(c0 + r) * kGBM + row) * BN + col;
+    float4 s = *reinterpret_cast<const float4*>(w);
+#pragma unroll 4
+    for (int c = c0 + 1; c <= c1; ++c) {
+      const float4 x =
+          *reinterpret_cast<const float4*>(w + (int64_t)(c - c0) * kGBM * BN);
+      s.x += x.x;
+      s.y += x.y;
+      s.z += x.z;
+      s.w += x.w;
+    }
+    const float v[4] = {s.x, s.y, s.z, s.w};
+    for (int j = 0; j < 4 && n + j < a.N; ++j) {
+      float o = a.alpha * v[j];
+      if (a.C && a.beta != 0.f) o += a.beta * a.C[(int64_t)m * a.ldc + n + j];
+      a.D[(int64_t)m * a.ldd + n + j] = o;
+    }
   }
 }
 
 template <int BN>
-cudaError_t launch_tc_gemm_t(const CUtensorMap& tmA, const CUtensorMap& tmB, int M, int N, int nk,
-                             int kp, float* D, int64_t ldd, const float* C, int64_t ldc,
-                             float alpha, float beta, int vec_ok, int num_sms, float* work,
-                             int64_t work_floats, unsigned* status, cudaStream_t s) {
+cudaError_t launch_tc_gemm_t(const GMaps& maps, const GArgs& a, int num_sms, cudaStream_t s) {
   using Sh = GShape<BN>;
-  static const cudaError_t configured = cudaFuncSetAttribute(
-      tc_gemm_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::SmemBytes);
+  static const cudaError_t configured = [] {
+    cudaFuncAttributes at;
+    cudaError_t e = cudaFuncGetAttributes(&at, tc_gemm_kernel<BN>);
+    // the registers handed over must be there, or setmaxnreg would wait forever
+    if (e == cudaSuccess && Sh::Rebalance && at.numRegs * Sh::Threads < 40 * 128 + 224 * 256)
+      e = cudaErrorInvalidConfiguration;
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(tc_gemm_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)Sh::SmemBytes);
+  }();
   if (configured != cudaSuccess) return configured;
-  const long long tiles = (long long)((M + kGBM - 1) / kGBM) * ((N + BN - 1) / BN);
-  // too few tiles to fill the SMs: split K (each part at least 16 chunks of 32)
-  int ksplit = 1;
-  if (work) {
-    while (tiles * (ksplit + 1) <= num_sms && nk / (ksplit + 1) >= 16 &&
-           (int64_t)(ksplit + 1) * M * N <= work_floats)
-      ++ksplit;
+  const int tiles = ((a.M + kGBM - 1) / kGBM) * ((a.N + BN - 1) / BN);
+  const int busy = a.dp > a.cut ? a.dp : a.cut;
+  const int pairs = busy < num_sms / 2 ? busy : num_sms / 2;
+  const cudaError_t e =
+      launch_pdl(tc_gemm_kernel<BN>, 2 * pairs, Sh::Threads, Sh::SmemBytes, s, maps, a);
+  if (e != cudaSuccess || tiles == a.dp) return e;
+  return launch_pdl(gemm_parts_kernel<BN>, dim3(tiles - a.dp, kGBM / 16), 256, 0, s, a, tiles);
+}
+
+// FP16 operand rows [hi | lo]: 64-value boxes (128 bytes), 128-byte swizzle
+bool make_tmap_f16(CUtensorMap* out, const void* base, int64_t cols, int64_t rows, int box_rows) {
+  static const PFN_cuTensorMapEncodeTiled_v12000 encode = []() {
+    cudaDriverEntryPointQueryResult q;
+    void* fn = nullptr;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault,
+                                         &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess)
+      fn = nullptr;
+    return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
+  }();
+  if (!encode) return false;
+  cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
+  cuuint64_t strides[1] = {(cuuint64_t)(cols * 2)};
+  cuuint32_t box[2] = {64u, (cuuint32_t)box_rows};
+  cuuint32_t estr[2] = {1, 1};
+  return encode(out, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void*>(base), dims, strides,
+                box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+SplitOp split_op(const TcOperand* t) {
+  SplitOp o{};
+  if (!t) return o;
+  o.X = t->X;
+  o.rs = t->rs;
+  o.cs = t->cs;
+  o.rows = t->rows;
+  o.K = t->K;
+  o.dst = reinterpret_cast<unsigned char*>(t->buf);
+  o.fmt = t->words;
+  o.sc = reinterpret_cast<float*>(t->words + 4);
+  o.pitch = (t->rows + 3) / 4 * 4;
+  o.vec = (t->cs == 1 ? t->rs : t->cs) % 4 == 0 && reinterpret_cast<uintptr_t>(t->X) % 16 == 0;
+  return o;
+}
+
+// Tile width of a product of nk chunks, the tiles computed whole (full waves of
+// CTA pairs) and the number of ranges the others are cut into (0: all whole).  The
+// modelled time is the longest pair's chunks times the width's chunk time (1.03,
+// 0.62, 0.50 us at 256, 128, 64 columns: 4096^3 in 265, 278, 449 us), 7 us of
+// start and end, and for cut tiles a launch and their pieces written and read.
+// It lies within 4 us of the best of the six choices at 1024^3 (64 columns, whole:
+// 13 us), 2048^3 (256, whole: 40), 3001 x 1025 x 5003 (256, cut: 76 + 12),
+// 4096 x 128 x 4096 (128, cut: 21 + 5), 8192 x 64 x 8192 (64, cut: 57 + 6) and
+// 300 x 40 x 5000 (64, cut: 9 + 7, whole: 38).
+void gemm_plan(int M, int N, int nk, int num_sms, int64_t work_floats, GArgs& a, int* bn_out) {
+  const int pairs = num_sms / 2;
+  const long long mt = (M + kGBM - 1) / kGBM;
+  double best = 1e30;
+  for (int bn = 256; bn >= 64; bn /= 2) {
+    const double chunk = bn == 256 ? 1.03 : (bn == 128 ? 0.62 : 0.50);
+    const long long tiles = mt * ((N + bn - 1) / bn);
+    for (int c = 0; c < 2; ++c) {
+      long long left = c ? tiles % pairs : 0;
+      int cut = (int)(left * nk / 4 < pairs ? left * nk / 4 : pairs);  // at least four chunks each
+      if (c && (cut <= left || (left + cut) * kGBM * bn > work_floats)) continue;
+      double t = 7.0 + (double)((tiles - left + pairs - 1) / pairs) * nk * chunk;
+      if (cut)
+        t += (double)((left * nk + cut - 1) / cut) * chunk + 3.5 +
+             (double)(left + cut) * (kGBM * bn) * 8.0 / 6e6;
+      if (t < best) {
+        best = t;
+        *bn_out = bn;
+        a.dp = (int)(tiles - left);
+        a.cut = cut;
+      }
+    }
   }
-  const long long T = tiles * ksplit;
-  const int grid = (int)(T < num_sms ? T : num_sms);
-  tc_gemm_kernel<BN><<<grid, Sh::Threads, Sh::SmemBytes, s>>>(
-      tmA, tmB, M, N, nk, kp, D, ldd, C, ldc, alpha, beta, vec_ok, ksplit, work, status);
-  if (ksplit == 1) return cudaGetLastError();
-  const int64_t total = (int64_t)M * N;
-  const int blocks = (int)((total + 255) / 256 < 4096 ? (total + 255) / 256 : 4096);
-  gemm_parts_kernel<<<blocks, 256, 0, s>>>(M, N, ksplit, work, alpha, beta, C, ldc, D, ldd);
-  return cudaGetLastError();
 }
 
 }  // namespace
 
 int64_t tc_split_ld(int64_t K) { return 2 * ((K + 31) / 32 * 32); }
-
-cudaError_t launch_split_rows(const float* X, int64_t rs, int64_t cs, int rows, int K, float* dst,
-                              int64_t ldd, cudaStream_t s) {
-  if (rows <= 0 || K <= 0) return cudaSuccess;
-  const int kp = (K + 31) / 32 * 32;
-  if (ldd < 2 * kp) return cudaErrorInvalidValue;
-  dim3 grid(kp / 32, (rows + 31) / 32);
-  split_rows_kernel<<<grid, 256, 0, s>>>(X, rs, cs, rows, K, kp, dst, ldd);
-  return cudaGetLastError();
+int64_t tc_work_floats(int64_t a_rows, int64_t b_rows, int64_t K, int num_sms) {
+  const int64_t pairs = num_sms / 2, nk = (K + 63) / 64;
+  int64_t most = 0;
+  for (int bn = 256; bn >= 64; bn /= 2) {
+    int64_t left = (a_rows + kGBM - 1) / kGBM * ((b_rows + bn - 1) / bn);
+    left = left < pairs ? left : pairs;
+    const int64_t cut = left * nk / 4 < pairs ? left * nk / 4 : pairs;
+    most = most > (left + cut) * kGBM * bn ? most : (left + cut) * kGBM * bn;
+  }
+  return most;
+}
+int64_t tc_split_words(int64_t rows, int64_t K) {
+  return 4 + (rows + 3) / 4 * 4 * ((K + 63) / 64);
 }
 
-cudaError_t launch_tc_gemm(const float* As, const float* Bs, int M, int N, int K, float* D,
+cudaError_t launch_tc_split(const TcOperand* a, const TcOperand* b, unsigned* flag,
+                            cudaStream_t s) {
+  SplitPair sp{};
+  sp.flag = flag;
+  const TcOperand* in[2] = {a, b};
+  for (int w = 0; w < 2; ++w) {
+    if (!in[w]) continue;
+    if (in[w]->rows <= 0 || in[w]->K <= 0) return cudaErrorInvalidValue;
+    // TMA sources (rows are 128-byte multiples) and 128-bit loads of the factors
+    if ((reinterpret_cast<uintptr_t>(in[w]->buf) | reinterpret_cast<uintptr_t>(in[w]->words)) & 15)
+      return cudaErrorInvalidValue;
+    sp.o[w] = split_op(in[w]);
+    sp.o[w].blocks = ((sp.o[w].rows + kSpR - 1) / kSpR) *
+                     (((sp.o[w].K + 63) / 64 * 64 + kSpK - 1) / kSpK);
+  }
+  return launch_pdl(split_f16_kernel, sp.o[0].blocks + sp.o[1].blocks, 256, 0, s, sp);
+}
+
+cudaError_t launch_tc_gemm(const TcOperand& a, const TcOperand& b, unsigned* flag, float* D,
                            int64_t ldd, const float* C, int64_t ldc, float alpha, float beta,
                            int num_sms, unsigned* status, cudaStream_t s, float* work,
-                           int64_t work_floats) {
-  if (M <= 0 || N <= 0 || K <= 0) return cudaErrorInvalidValue;
-  const int64_t ld = tc_split_ld(K);
-  const int kp = (int)(ld / 2);
-  const int nk = kp / 32;
-  // the split buffers are TMA sources: 16-byte aligned bases (rows are 128-byte multiples)
-  if ((reinterpret_cast<uintptr_t>(As) | reinterpret_cast<uintptr_t>(Bs)) & 15)
-    return cudaErrorInvalidValue;
-  const int BN = N >= 192 ? 256 : (N > 64 ? 128 : 64);
-  CUtensorMap tmA, tmB;
-  if (!make_tmap_sw128(&tmA, As, ld, M, ld, kGBM) || !make_tmap_sw128(&tmB, Bs, ld, N, ld, BN))
+                           int64_t work_floats, bool reverse) {
+  const int M = a.rows, N = b.rows, K = a.K;
+  if (M <= 0 || N <= 0 || K <= 0 || b.K != K) return cudaErrorInvalidValue;
+  SplitPair sp{};
+  sp.flag = flag;
+  sp.o[0] = split_op(&a);
+  sp.o[1] = split_op(&b);
+  const cudaError_t es = launch_pdl(split_tf32_kernel, 2 * num_sms, 256, 0, s, sp);
+  if (es != cudaSuccess) return es;
+  GArgs g{};
+  g.M = M;
+  g.N = N;
+  g.kp16 = (K + 63) / 64 * 64;
+  g.kp32 = (int)(tc_split_ld(K) / 2);
+  int bn = 256;
+  gemm_plan(M, N, g.kp16 / 64, num_sms, work ? work_floats : 0, g, &bn);
+  g.reverse = reverse ? 1 : 0;
+  GMaps maps;
+  if (!make_tmap_f16(&maps.a16, a.buf, 2 * g.kp16, M, 128) ||
+      !make_tmap_f16(&maps.b16, b.buf, 2 * g.kp16, N, bn / 2) ||
+      !make_tmap_sw128(&maps.a32, a.buf, 2 * g.kp32, M, 2 * g.kp32, 128) ||
+      !make_tmap_sw128(&maps.b32, b.buf, 2 * g.kp32, N, 2 * g.kp32, bn / 2))
     return cudaErrorInvalidValue;
   const bool c_used = C != nullptr && beta != 0.f;
-  const int vec_ok = (ldd % 4 == 0) && (reinterpret_cast<uintptr_t>(D) % 16 == 0) &&
-                     (!c_used || (ldc % 4 == 0 && reinterpret_cast<uintptr_t>(C) % 16 == 0));
-  if (BN == 256)
-    return launch_tc_gemm_t<256>(tmA, tmB, M, N, nk, kp, D, ldd, C, ldc, alpha, beta, vec_ok,
-                                 num_sms, work, work_floats, status, s);
-  if (BN == 128)
-    return launch_tc_gemm_t<128>(tmA, tmB, M, N, nk, kp, D, ldd, C, ldc, alpha, beta, vec_ok,
-                                 num_sms, work, work_floats, status, s);
-  return launch_tc_gemm_t<64>(tmA, tmB, M, N, nk, kp, D, ldd, C, ldc, alpha, beta, vec_ok,
-                              num_sms, work, work_floats, status, s);
+  g.D = D;
+  g.ldd = ldd;
+  g.C = C;
+  g.ldc = ldc;
+  g.alpha = alpha;
+  g.beta = beta;
+  g.vec_ok = (ldd % 4 == 0) && (reinterpret_cast<uintptr_t>(D) % 16 == 0) &&
+             (!c_used || (ldc % 4 == 0 && reinterpret_cast<uintptr_t>(C) % 16 == 0));
+  g.work = work;
+  g.sa = sp.o[0].sc;
+  g.sb = sp.o[1].sc;
+  g.pa = sp.o[0].pitch;
+  g.pb = sp.o[1].pitch;
+  g.fmta = a.words;
+  g.fmtb = b.words;
+  g.flag = flag;
+  g.status = status;
+  if (bn == 256) return launch_tc_gemm_t<256>(maps, g, num_sms, s);
+  if (bn == 128) return launch_tc_gemm_t<128>(maps, g, num_sms, s);
+  return launch_tc_gemm_t<64>(maps, g, num_sms, s);
 }
 
 static int gemm_simt_splits(int M, int N, int K, int batch, int num_sms, int64_t work_elems) {

@@ -118,22 +118,38 @@ cudaError_t launch_tc_update(const CUtensorMap& tmP, const CUtensorMap& tmA,
                              int num_sms, unsigned* status, cudaStream_t s);
 
 // Own dense GEMMs (lv_gemm.cu).
-// Split-TF32 operand rows: rows x tc_split_ld(K) floats, row i = [hi | lo]
-// (each half rup(K, 32) long, zero past K).
+// A split operand of the tensor-core GEMM: element (i, k) of op(X) at X[i * rs +
+// k * cs] (rs or cs == 1), its split rows in ``buf`` (rows x tc_split_ld(K) floats,
+// 16-byte aligned; FP16 rows take half of it) and in ``words`` (tc_split_words(rows,
+// K), 16-byte aligned) the buffer's format and the factors of its runs.  X stays
+// readable for as long as products use the split: a product that has to fall back
+// to TF32 splits it again.
+struct TcOperand {
+  const float* X;
+  int64_t rs, cs;
+  int rows, K;
+  float* buf;
+  unsigned* words;
+};
 int64_t tc_split_ld(int64_t K);
-// Split the rows of op(X) (element (i, k) at X[i * rs + k * cs], rs or cs == 1)
-// into dst (ldd >= tc_split_ld(K)).
-cudaError_t launch_split_rows(const float* X, int64_t rs, int64_t cs, int rows, int K, float* dst,
-                              int64_t ldd, cudaStream_t s);
-// D (M x N, row-major, ldd) = alpha A_s B_s^T + beta C on the tensor cores
-// (split TF32, FP32 accumulation), A_s / B_s split rows of inner length K
-// (16-byte aligned).  C may alias D (beta == 0 ignores it).  ``work``
-// (work_floats floats, may be null): room for the K parts of a product with
-// too few tiles to fill the SMs (split K, parts summed in a fixed order).
-cudaError_t launch_tc_gemm(const float* As, const float* Bs, int M, int N, int K, float* D,
+int64_t tc_split_words(int64_t rows, int64_t K);
+// floats of ``work`` below that let every product with up to these sizes cut tiles
+int64_t tc_work_floats(int64_t a_rows, int64_t b_rows, int64_t K, int num_sms);
+// Split a and b (either may be null).  ``flag`` (one word, zeroed by the caller
+// before the first split of a scratch) is set when an operand needs TF32; it
+// stays set, so all later products on the scratch take TF32.
+cudaError_t launch_tc_split(const TcOperand* a, const TcOperand* b, unsigned* flag,
+                            cudaStream_t s);
+// D (M x N, row-major, ldd) = alpha A B^T + beta C on the tensor cores (split
+// FP16 or TF32, FP32 accumulation) of split operands with M and N rows.  C may
+// alias D (beta == 0 ignores it).  ``work`` (work_floats floats, 16-byte aligned, may
+// be null): room for the pieces of tiles that several CTA pairs share along K
+// (summed in a fixed order).  ``reverse`` visits K from its end: a product that
+// follows another one with the same A then starts on the part still in L2.
+cudaError_t launch_tc_gemm(const TcOperand& a, const TcOperand& b, unsigned* flag, float* D,
                            int64_t ldd, const float* C, int64_t ldc, float alpha, float beta,
                            int num_sms, unsigned* status, cudaStream_t s, float* work = nullptr,
-                           int64_t work_floats = 0);
+                           int64_t work_floats = 0, bool reverse = false);
 // C (M x N) = alpha A B + beta C on the CUDA cores, A(m, k) = A[m a_rs + k a_cs],
 // B(k, n) = B[k b_rs + n b_cs], C(m, n) = C[m c_rs + n c_cs]; long inner
 // dimensions are split over ``work`` (work_elems elements, may be null) and
@@ -257,6 +273,10 @@ template <typename T>
 cudaError_t launch_outer(T* T1, int64_t ldT, const T* K, int64_t fs, const T* M, int64_t ldm, int n,
                          int p, int k, int r, bool accumulate, int num_sms, cudaStream_t s);
 bool outer_fits(int kr, size_t elem_bytes);
+// out(j, q) = sum_{i < k} A[j lda + i p + q], in order
+template <typename T>
+cudaError_t launch_panel_sum(const T* A, int64_t lda, T* out, int64_t ldo, int n, int p, int k,
+                             cudaStream_t s);
 
 // OLS pieces (lv_ols.cu).
 template <typename T>
