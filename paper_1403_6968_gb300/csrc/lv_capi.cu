@@ -909,6 +909,21 @@ static View& pview(linview_program* p, int l) { return p->views[l]; }
 // S'_h for the power view of index l >= 1 (h = 2^l, or the skip view l)
 static View& sview(linview_program* p, int l) { return p->views[p->npv + l - 1]; }
 
+// S'_2 = P_2 + A (S'_{2h} = P_h S'_h + S'_h at h = 1, where P_1 S'_1 = A A is P_2)
+static linview_status first_sums_view(linview_program* p, const View& a, const View& p2,
+                                      const View& s2, cudaStream_t s) {
+  if (p->elem == 4)
+    LV_CUDA(launch_add_views<float>(static_cast<const float*>(p2.ptr),
+                                    static_cast<const float*>(a.ptr), static_cast<float*>(s2.ptr),
+                                    s2.rows, s2.ld, s));
+  else
+    LV_CUDA(launch_add_views<double>(static_cast<const double*>(p2.ptr),
+                                     static_cast<const double*>(a.ptr),
+                                     static_cast<double*>(s2.ptr), s2.rows, s2.ld, s));
+  p->all_launches++;
+  return LINVIEW_OK;
+}
+
 // Linear model (Section 3.3): P_i = P_{i-1} A, i = 2..k (views i-1), and
 // S'_k = P_1 + ... + P_k (view k) for sums programs.
 static linview_status linear_reeval(linview_program* p, cudaStream_t s) {
@@ -978,7 +993,10 @@ static linview_status skip_reeval(linview_program* p, cudaStream_t s) {
     // S'_{2h} = P_h S'_h + S'_h up to s (S'_1 = A), then S'_i = P_s S'_{i-s} + S'_s
     for (int l = 0; l < Ls; ++l) {
       View& sh = (l == 0) ? pview(p, 0) : sview(p, l);
-      LV_TRY(prod(pview(p, l), sh, &sh, sview(p, l + 1), false));
+      if (l == 0 && !lib)
+        LV_TRY(first_sums_view(p, sh, pview(p, 1), sview(p, 1), s));
+      else
+        LV_TRY(prod(pview(p, l), sh, &sh, sview(p, l + 1), false));
     }
     View& ss = (Ls == 0) ? pview(p, 0) : sview(p, Ls);
     for (int i = 2; i <= p->d.k / p->d.skip; ++i) {
@@ -1024,8 +1042,10 @@ static linview_status powers_reeval(linview_program* p, cudaStream_t s) {
     View& c = pview(p, l + 1);
     LV_TRY(gemm_ab(p, n, n, n, 1.0, rows_of(ph.ptr, ph.ld), cols_of(ph.ptr, ph.ld), 0.0, nullptr,
                    0, c.ptr, c.ld, s, &sc));
-    if (sums) {
-      View& sh = (l == 0) ? pview(p, 0) : sview(p, l);
+    if (sums && l == 0) {
+      LV_TRY(first_sums_view(p, ph, c, sview(p, 1), s));
+    } else if (sums) {
+      View& sh = sview(p, l);
       View& s2 = sview(p, l + 1);
       LV_TRY(gemm_ab(p, n, n, n, 1.0, rows_of(ph.ptr, ph.ld), cols_of(sh.ptr, sh.ld), 1.0, sh.ptr,
                      sh.ld, s2.ptr, s2.ld, s, &sc, /*a_ready=*/true));
@@ -1749,8 +1769,11 @@ static linview_status iter_sk_reeval(linview_program* p, cudaStream_t s) {
     } else {
       LV_TRY(gemm_ab(p, n, n, n, 1.0, rows_of(ph.ptr, ph.ld), cols_of(ph.ptr, ph.ld), 0.0,
                      nullptr, 0, p2.ptr, p2.ld, s, &sc));
-      LV_TRY(gemm_ab(p, n, n, n, 1.0, rows_of(ph.ptr, ph.ld), cols_of(sh.ptr, sh.ld), 1.0,
-                     sh.ptr, sh.ld, s2.ptr, s2.ld, s, &sc, /*a_ready=*/true));
+      if (l == 1)
+        LV_TRY(first_sums_view(p, sh, p2, s2, s));
+      else
+        LV_TRY(gemm_ab(p, n, n, n, 1.0, rows_of(ph.ptr, ph.ld), cols_of(sh.ptr, sh.ld), 1.0,
+                       sh.ptr, sh.ld, s2.ptr, s2.ld, s, &sc, /*a_ready=*/true));
     }
   }
   const View& b = p->views[p->ie_NT + 1];

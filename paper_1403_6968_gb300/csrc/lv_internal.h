@@ -233,6 +233,10 @@ cudaError_t launch_sum_partials(const T* part, int blocks, int64_t block_stride,
                                 int n, int r, T* out, int64_t out_cs, cudaStream_t s);
 
 // Elementwise helpers.
+// out = x + y, rows x ld elements each (views of one layout)
+template <typename T>
+cudaError_t launch_add_views(const T* x, const T* y, T* out, int64_t rows, int64_t ld,
+                             cudaStream_t s);
 template <typename T>
 cudaError_t launch_axpy_rows(T* y, int64_t ldy, const T* x, int64_t ldx, T alpha, int rows,
                              int cols, cudaStream_t s);  // y += alpha x (row-major blocks)
