@@ -107,6 +107,7 @@ __device__ __forceinline__ void df_add(float& hi, float& lo, float x, float xe) 
 // FP32 programs: per-block partials of C = V^T U (rv x r) in double-float.  GB300's
 // FP64 pipe is narrow, so the FP64-grade sums use FP32 arithmetic; every
 // block of 256 threads takes one 32-row tile per step.
+template <bool RECT>
 __global__ void __launch_bounds__(kThreads) gram_df_kernel(const float* __restrict__ V,
                                                            const float* __restrict__ U,
                                                            int64_t fs, int n, int rv, int r,
@@ -115,18 +116,18 @@ __global__ void __launch_bounds__(kThreads) gram_df_kernel(const float* __restri
   __shared__ float Us[kGramRows][kGramMaxR + 1];
   const int tid = threadIdx.x;
   const int G = gridDim.x;
-  const int ne = rv * r;
+  const int ne = RECT ? rv * r : r * r;
   float hi[kGramPerThread], lo[kGramPerThread];
 #pragma unroll
   for (int i = 0; i < kGramPerThread; ++i) hi[i] = lo[i] = 0.f;
   for (int t0 = blockIdx.x * kGramRows; t0 < n; t0 += G * kGramRows) {
     const int nr = min(kGramRows, n - t0);
-    for (int idx = tid; idx < kGramRows * max(rv, r); idx += kThreads) {
+    for (int idx = tid; idx < kGramRows * (RECT ? max(rv, r) : r); idx += kThreads) {
       const int c = idx / kGramRows;
       const int j = idx % kGramRows;
       const bool ok = j < nr;
-      if (c < rv) Vs[j][c] = ok ? V[(int64_t)c * fs + t0 + j] : 0.f;
-      if (c < r) Us[j][c] = ok ? U[(int64_t)c * fs + t0 + j] : 0.f;
+      if (!RECT || c < rv) Vs[j][c] = ok ? V[(int64_t)c * fs + t0 + j] : 0.f;
+      if (!RECT || c < r) Us[j][c] = ok ? U[(int64_t)c * fs + t0 + j] : 0.f;
     }
     __syncthreads();
 #pragma unroll
@@ -190,7 +191,7 @@ cudaError_t launch_gram(const T* V, const T* U, int64_t fs, int n, int r, double
   const int G = gram_grid(n);
   if constexpr (std::is_same<T, float>::value) {
     float2* part = reinterpret_cast<float2*>(Cpart);
-    gram_df_kernel<<<G, kThreads, 0, s>>>(V, U, fs, n, r, r, part);
+    gram_df_kernel<false><<<G, kThreads, 0, s>>>(V, U, fs, n, r, r, part);
     const int ne = r * r;
     const int warps_per_block = kThreads / 32;
     gram_reduce_kernel<<<(ne + warps_per_block - 1) / warps_per_block, kThreads, 0, s>>>(
@@ -208,7 +209,7 @@ cudaError_t launch_cross_gram(const float* X, const float* V, int64_t fs, int n,
   float2* part = reinterpret_cast<float2*>(Cpart);
   for (int c0 = 0; c0 < rx; c0 += kGramMaxR) {
     const int w = rx - c0 < kGramMaxR ? rx - c0 : kGramMaxR;
-    gram_df_kernel<<<G, kThreads, 0, s>>>(X + (int64_t)c0 * fs, V, fs, n, w, rv, part);
+    gram_df_kernel<true><<<G, kThreads, 0, s>>>(X + (int64_t)c0 * fs, V, fs, n, w, rv, part);
     const int ne = w * rv;
     const int warps_per_block = kThreads / 32;
     gram_reduce_kernel<<<(ne + warps_per_block - 1) / warps_per_block, kThreads, 0, s>>>(
