@@ -195,17 +195,6 @@ __device__ __forceinline__ bool g_wait(uint64_t* bar, uint32_t parity, volatile 
   *abort_flag = 1;
   return false;
 }
-// one lane of a converged warp
-__device__ __forceinline__ bool elect_one() {
-  uint32_t p;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "elect.sync _|p, 0xffffffff;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(p));
-  return p != 0;
-}
-
 // tile t of the raster: groups of kGroupM row blocks, column blocks within
 __device__ __forceinline__ void g_tile(long long t, int mt, int nt, int& mb, int& nb) {
   const long long per_group = (long long)kGroupM * nt;

@@ -138,6 +138,7 @@ static_assert(sizeof(TcBars) <= 512, "barrier block");
 
 __device__ __forceinline__ bool tc_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
                                         unsigned* status) {
+  if (mbar_try_wait(bar, parity)) return true;
   if (*abort_flag) return false;
   if (mbar_wait_bounded(bar, parity, status)) return true;
   *abort_flag = 1;
@@ -250,47 +251,51 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
-    if (lane == 0) {
-      int cur_rb = -1, a_loads = 0, issued = 0;
-      for (int i = 0; i < ntile && !*abort_flag; ++i) {
-        const long long t = t0 + i;
-        const int rb = (int)(t / ncb);
-        const int buf = i & 1, use = i >> 1;
-        if (rb != cur_rb) {
-          if (!tc_wait(&bars->a_full, a_loads & 1, abort_flag, status)) break;
-          ++a_loads;
-          cur_rb = rb;
-        }
-        if (!tc_wait(&bars->b_full[buf], use & 1, abort_flag, status)) break;
-        if (use >= 1 && !tc_wait(&bars->acc_empty[buf], (use - 1) & 1, abort_flag, status)) break;
-        tc_fence_after();
-        const uint32_t d = tmem + buf * BN;
-        const uint32_t a0 = smem_u32(base + Sh::OffA);
-        const uint32_t b0 = smem_u32(base + Sh::OffB + buf * Sh::BBytes);
+    // the whole warp walks the tiles, one elected lane issues (inside a lane-0
+    // branch the descriptors are rebuilt in vector registers, 35 ns per MMA)
+    const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+    const uint64_t a0 = sw128_desc(smem_u32(base + Sh::OffA));
+    const uint64_t b00 = sw128_desc(smem_u32(base + Sh::OffB));
+    int left = 0;  // tiles left in the current row block
+    int a_loads = 0, issued = 0;
+    for (int i = 0; i < ntile; ++i) {
+      const int buf = i & 1, use = i >> 1;
+      bool ok = !*abort_flag;
+      if (left == 0) {
+        left = ncb - (int)((t0 + i) % ncb);
+        ok = ok && tc_wait(&bars->a_full, a_loads & 1, abort_flag, status);
+        ++a_loads;
+      }
+      --left;
+      ok = ok && tc_wait(&bars->b_full[buf], use & 1, abort_flag, status) &&
+           (use < 1 || tc_wait(&bars->acc_empty[buf], (use - 1) & 1, abort_flag, status));
+      if (!__all_sync(0xffffffffu, ok)) break;
+      tc_fence_after();
+      if (elect_one()) {
+        const uint32_t d = tm + buf * BN;
+        const uint64_t b0 = b00 + (uint32_t)buf * (Sh::BBytes >> 4);
         // (A half, B half): hi*hi, lo*hi, hi*lo; each over the H chunks of a half
         constexpr int kPairA[3] = {0, 1, 0};
         constexpr int kPairB[3] = {0, 0, 1};
 #pragma unroll
-        for (int pr = 0; pr < 3; ++pr) {
+        for (int pr = 0; pr < 3; ++pr)
 #pragma unroll
-          for (int hk = 0; hk < H; ++hk) {
+          for (int hk = 0; hk < H; ++hk)
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk) {  // K = 8 per MMA: 32 bytes of a 128-byte row
-              const uint64_t ad = sw128_desc(a0 + (kPairA[pr] * H + hk) * kBM * 128 + kk * 32);
-              const uint64_t bd = sw128_desc(b0 + (kPairB[pr] * H + hk) * BN * 128 + kk * 32);
-              tc_mma(d, ad, bd, Sh::Idesc, (pr | hk | kk) != 0 ? 1u : 0u);
-            }
-          }
-        }
+            for (int kk = 0; kk < 4; ++kk)  // K = 8 per MMA: 32 bytes of a 128-byte row
+              tc_mma(d, a0 + ((kPairA[pr] * H + hk) * kBM * 8 + kk * 2),
+                     b0 + ((kPairB[pr] * H + hk) * BN * 8 + kk * 2), Sh::Idesc,
+                     (pr | hk | kk) != 0 ? 1u : 0u);
         tc_commit(&bars->b_empty[buf]);
         tc_commit(&bars->acc_full[buf]);
-        issued = i + 1;
       }
-      if (*abort_flag && issued > 0) {
-        // the MMAs issued must finish before the TMEM is freed
-        const int j = issued - 1;
-        mbar_wait_bounded(&bars->acc_full[j & 1], (j >> 1) & 1, nullptr);
-      }
+      __syncwarp();
+      issued = i + 1;
+    }
+    if (issued < ntile && issued > 0 && lane == 0) {
+      // aborted: the MMAs issued must finish before the TMEM is freed
+      const int j = issued - 1;
+      mbar_wait_bounded(&bars->acc_full[j & 1], (j >> 1) & 1, nullptr);
     }
   } else {
     // ---------------- epilogue (warps 2..5) ----------------
@@ -604,46 +609,48 @@ __global__ void __launch_bounds__(kTpThreads, 1)
           mbar_wait_bounded(&bars->full[j % S], (uint32_t)((j / S) & 1), nullptr);
     }
   } else if (warp == 1) {
-    // ---------------- MMA issuer ----------------
-    if (lane == 0) {
-      long long g = 0, issued = 0;
-      for (long long c = c0; c < c1 && !*abort_flag;) {
-        int ot, part, kb0, kb1;
-        segment(c, ot, kb0, kb1, part);
-        c += kb1 - kb0;
-        for (int kb = kb0; kb < kb1; ++kb, ++g) {
-          const int st = (int)(g % S);
-          const long long use = g / S;
-          const int buf = (int)(g & 1);
-          const long long bu = g >> 1;
-          if (!tc_wait(&bars->split[st], (uint32_t)(use & 1), abort_flag, status)) break;
-          if (bu >= 1 && !tc_wait(&bars->acc_empty[buf], (uint32_t)((bu - 1) & 1), abort_flag, status))
-            break;
-          tc_fence_after();
-          const uint32_t d = tmem + buf * (2 * RP);
-          const uint32_t s0 = smem_u32(base + st * Sh::StageBytes);
-          const uint32_t a_hi = TR ? s0 + Sh::PBytes : s0;
-          const uint32_t a_lo = s0 + Sh::PBytes + Sh::HiBytes;
-          const uint32_t b_hi = a_lo + Sh::LoBytes;  // 2 RP rows: hi(B), then lo(B)
-          // per K step of 8 (32 bytes of each 128-byte row): hi(A) [hi(B) |
-          // lo(B)] over 2 RP columns, then lo(A) hi(B) into the first RP: the
-          // three products of the split in two MMAs, the wider one filling
-          // the tensor pipe better than three of width RP
+    // ---------------- MMA issuer (whole warp, one elected lane issues) ----------------
+    const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+    const uint64_t s00 = sw128_desc(smem_u32(base));
+    const long long chunks = c1 - c0;
+    int st = 0;
+    uint32_t phase = 0;
+    long long g = 0;
+    for (; g < chunks; ++g) {
+      const int buf = (int)(g & 1);
+      const long long bu = g >> 1;
+      const bool ok =
+          !*abort_flag && tc_wait(&bars->split[st], phase, abort_flag, status) &&
+          (bu < 1 || tc_wait(&bars->acc_empty[buf], (uint32_t)((bu - 1) & 1), abort_flag, status));
+      if (!__all_sync(0xffffffffu, ok)) break;
+      tc_fence_after();
+      if (elect_one()) {
+        const uint32_t d = tm + buf * (2 * RP);
+        const uint64_t s0 = s00 + (uint32_t)st * (Sh::StageBytes >> 4);
+        const uint64_t a_hi = TR ? s0 + (Sh::PBytes >> 4) : s0;
+        const uint64_t a_lo = s0 + ((Sh::PBytes + Sh::HiBytes) >> 4);
+        const uint64_t b_hi = a_lo + (Sh::LoBytes >> 4);  // 2 RP rows: hi(B), then lo(B)
+        // per K step of 8 (32 bytes of each 128-byte row): hi(A) [hi(B) |
+        // lo(B)] over 2 RP columns, then lo(A) hi(B) into the first RP: the
+        // three products of the split in two MMAs, the wider one filling
+        // the tensor pipe better than three of width RP
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk) {
-            tc_mma(d, sw128_desc(a_hi + kk * 32), sw128_desc(b_hi + kk * 32), Sh::IdescW,
-                   kk != 0 ? 1u : 0u);
-            tc_mma(d, sw128_desc(a_lo + kk * 32), sw128_desc(b_hi + kk * 32), Sh::IdescN, 1u);
-          }
-          tc_commit(&bars->empty[st]);
-          tc_commit(&bars->acc_full[buf]);
-          issued = g + 1;
+        for (int kk = 0; kk < 4; ++kk) {
+          tc_mma(d, a_hi + kk * 2, b_hi + kk * 2, Sh::IdescW, kk != 0 ? 1u : 0u);
+          tc_mma(d, a_lo + kk * 2, b_hi + kk * 2, Sh::IdescN, 1u);
         }
+        tc_commit(&bars->empty[st]);
+        tc_commit(&bars->acc_full[buf]);
       }
-      if (*abort_flag && issued > 0) {
-        const long long j = issued - 1;  // the MMAs issued finish before the TMEM is freed
-        mbar_wait_bounded(&bars->acc_full[j & 1], (uint32_t)((j >> 1) & 1), nullptr);
+      __syncwarp();
+      if (++st == S) {
+        st = 0;
+        phase ^= 1u;
       }
+    }
+    if (g < chunks && g > 0 && lane == 0) {
+      const long long j = g - 1;  // aborted: the MMAs issued finish before the TMEM is freed
+      mbar_wait_bounded(&bars->acc_full[j & 1], (uint32_t)((j >> 1) & 1), nullptr);
     }
   } else if (warp < 6) {
     // ---------------- split (warps 2..5, 128 threads) ----------------
