@@ -513,7 +513,7 @@ static linview_status run_products_update(linview_program* p, const View& v, int
     // Y = P^T V on the tensor cores, one read of P each, K split in ``parts``
     const int n = (int)v.rows;
     const int parts = tp_parts(n, p->sms);  // partial sets the pass writes
-    if (allow_tc && p->tpF && v.square && r > kMaxProductR && parts <= p->xslots &&
+    if (allow_tc && p->tpF && v.square && r > tp_min_r(n) && parts <= p->xslots &&
         (!want_y || parts <= p->yslots) && (v.ld * 4) % 16 == 0 && p->fs % 64 == 0) {
       const double nn = (double)n * (double)n * sizeof(float);
       for (int c0 = 0; c0 < r; c0 += kMaxTcR) {
@@ -1086,7 +1086,7 @@ static bool powers_uses_tc(const linview_program_desc& d) {
 // CUDA-core products pass: the tensor-core products pass
 static bool powers_uses_tp(const linview_program_desc& d) {
   return d.precision == LINVIEW_F32 && d.model == LINVIEW_MODEL_EXP &&
-         (int64_t)d.r_max * (d.k / 2) > kMaxProductR;
+         (int64_t)d.r_max * (d.k / 2) > tp_min_r(d.n);
 }
 
 // Device bytes powers_create allocates (with the buffers every program has),

@@ -105,6 +105,13 @@ cudaError_t launch_tc_products(bool transpose, const float* P, int64_t ldp, cons
                                int64_t fs, float* Fsplit, int n, int r, float* out, int64_t ps,
                                int64_t cs, int parts, int num_sms, unsigned* status,
                                cudaStream_t s);
+// Blocks wider than this run on the tensor-core products pass, two passes over the
+// view and two splits of the factor; narrower ones on the CUDA cores in one pass.
+// The CUDA-core pass is bound by its issue slots at 9 - 16 columns: n = 8192 145 us
+// against 59 + 59 + 4, n = 4096 43 against 19 + 19 + 4 (an update of A^16 at rank 2:
+// 217 -> 215 us, rank 4: 286 -> 277), n = 3000 27 against 12 + 12 + 3 (150 -> 153,
+// 200 -> 196), n = 2048 15 against 8 + 9 + 3 (106 -> 110, 141 -> 143).
+inline int tp_min_r(int64_t n) { return n >= 3500 ? kMaxFusedR : kMaxProductR; }
 // partial sets the products pass writes for an n x n view (<= kTpMaxParts)
 int tp_parts(int n, int num_sms);
 // Tensor-core update pass P += U W^T (FP32 view, 17 <= r <= 64 factor

@@ -33,6 +33,8 @@
 #include <cuda_runtime.h>
 #include <cudaTypedefs.h>
 
+#include <type_traits>
+
 #include "lv_device.cuh"
 #include "lv_internal.h"
 
@@ -458,28 +460,37 @@ __global__ void __launch_bounds__(256) tc_split_kernel(const float* __restrict__
 // few CTAs, whose sums land in consecutive partials of the output (Xpart /
 // Ypart layout: partial stride ps, column stride cs), summed by the
 // assembly.  Warps: 0 TMA producer, 1 TMEM allocation and
-// MMA issue, 2-5 split, 6-9 epilogue.  The pass is bound by shared-memory
+// MMA issue, then the split, the epilogue and (Y) a producer of factor chunks.  The pass is bound by shared-memory
 // traffic (the TMA writes, the split, and the tensor pipe reading each A
 // tile three times), not by HBM.  Every mbarrier wait is bounded: an expired
 // wait latches LINVIEW_ETIMEOUT, stops the CTA's loops, drains the copies and
 // MMAs in flight and frees the TMEM.
-constexpr int kTpThreads = 320;
-constexpr int kTpMaxStages = 5;
+constexpr int kTpMaxStages = 6;
 
+// X: stages of [P box | lo(P) | factor chunk].  Y: a ring of R raw slabs of P, which
+// the split warps free as soon as they have read them, and a ring of S stages
+// [hi | lo | factor chunk] that the MMAs free; with the slab in the stage only
+// three stages fit and a slab's load, split and MMAs ran in near lockstep (73 us at
+// n = 8192, 32 columns; 61 us now, with eight split warps instead of four).
 template <bool TR, int RP>
 struct TpShape {
   static constexpr uint32_t PBytes = kBM * 128;            // 128 x 32 FP32 (X) / 4 boxes 32 x 32 (Y)
-  static constexpr uint32_t HiBytes = TR ? kBM * 128 : 0;  // Y: transposed hi (X: the loaded box)
+  static constexpr uint32_t HiBytes = kBM * 128;           // Y: transposed hi; X: the loaded box
   static constexpr uint32_t LoBytes = kBM * 128;
   static constexpr uint32_t BBytes = 2 * RP * 128;         // factor chunk: hi rows, then lo rows
-  static constexpr uint32_t StageBytes = PBytes + HiBytes + LoBytes + BBytes;
-  static constexpr int S = (int)((221184u / StageBytes) < (uint32_t)kTpMaxStages
-                                     ? (221184u / StageBytes) : (uint32_t)kTpMaxStages);
-  static constexpr uint32_t OffBar = S * StageBytes;
+  static constexpr uint32_t StageBytes = HiBytes + LoBytes + BBytes;
+  static constexpr int S = TR ? 3 : (RP == 16 ? 6 : (RP == 32 ? 5 : 4));
+  static constexpr int R = TR ? (RP == 64 ? 4 : 6) : 0;    // raw slabs (Y)
+  static constexpr uint32_t OffRaw = S * StageBytes;
+  static constexpr uint32_t OffBar = OffRaw + R * PBytes;
+  static constexpr int NS = TR ? 8 : 4;                    // split warps
+  // warps: 0 P loads, 1 MMA, NS split, 4 epilogue, (Y) one for the factor loads
+  static constexpr int Threads = 32 * (2 + NS + 4 + (TR ? 1 : 0));
   static constexpr uint32_t SmemBytes = OffBar + 512 + 1024;
   // a chunk accumulator holds hi(A) [hi(B) | lo(B)] in 2 RP columns (with
-  // lo(A) hi(B) added to the first RP); two of them
-  static constexpr uint32_t TmemCols = 4 * RP;
+  // lo(A) hi(B) added to the first RP); NB of them
+  static constexpr int NB = RP == 64 ? 4 : 8;
+  static constexpr uint32_t TmemCols = NB * 2 * RP;
   static constexpr uint32_t IdescW = (1u << 4) | (2u << 7) | (2u << 10) |
                                      ((uint32_t)(2 * RP >> 3) << 17) | ((uint32_t)(kBM >> 4) << 24);
   static constexpr uint32_t IdescN = (1u << 4) | (2u << 7) | (2u << 10) |
@@ -487,11 +498,14 @@ struct TpShape {
 };
 static_assert(TpShape<false, 64>::SmemBytes <= 232448 && TpShape<true, 64>::SmemBytes <= 232448,
               "shared memory per CTA");
-static_assert(TpShape<true, 64>::S >= 3 && TpShape<false, 64>::S >= 4, "pipeline depth");
+static_assert(TpShape<true, 32>::SmemBytes <= 232448 && TpShape<false, 32>::SmemBytes <= 232448 &&
+                  TpShape<true, 16>::SmemBytes <= 232448 && TpShape<false, 16>::SmemBytes <= 232448,
+              "shared memory per CTA");
 
 struct TpBars {
   uint64_t full[kTpMaxStages], split[kTpMaxStages], empty[kTpMaxStages];
-  uint64_t acc_full[2], acc_empty[2];
+  uint64_t raw_free[kTpMaxStages], b_full[kTpMaxStages];  // Y only
+  uint64_t acc_full[8], acc_empty[8];
   uint32_t tmem_base;
   int abort;
 };
@@ -511,12 +525,13 @@ __device__ __forceinline__ uint32_t sw128_off(int row, int chunk) {
 }
 
 template <bool TR, int RP>
-__global__ void __launch_bounds__(kTpThreads, 1)
+__global__ void __launch_bounds__(TpShape<TR, RP>::Threads, 1)
     tc_products_kernel(const __grid_constant__ CUtensorMap tmP, const __grid_constant__ CUtensorMap tmF,
                        float* out, int64_t ps, int64_t cs, int n, int r_out, int parts,
                        unsigned* status) {
   using Sh = TpShape<TR, RP>;
-  constexpr int S = Sh::S;
+  constexpr int S = Sh::S, R = TR ? Sh::R : Sh::S, NS = Sh::NS, NB = Sh::NB;
+  // R: slots of the P ring
   extern __shared__ __align__(1024) unsigned char tp_smem_raw[];
   const uint32_t raw = smem_u32(tp_smem_raw);
   unsigned char* base = tp_smem_raw + (((raw + 1023u) & ~1023u) - raw);
@@ -551,12 +566,14 @@ __global__ void __launch_bounds__(kTpThreads, 1)
   if (tid == 0) {
     prefetch_tmap(&tmP);
     prefetch_tmap(&tmF);
-    for (int i = 0; i < S; ++i) {
+    for (int i = 0; i < kTpMaxStages; ++i) {
       mbar_init(&bars->full[i], 1);
-      mbar_init(&bars->split[i], 4);  // one arrival per split warp
+      mbar_init(&bars->split[i], NS);  // one arrival per split warp
       mbar_init(&bars->empty[i], 1);
+      mbar_init(&bars->raw_free[i], NS);
+      mbar_init(&bars->b_full[i], 1);
     }
-    for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < NB; ++i) {
       mbar_init(&bars->acc_full[i], 1);
       mbar_init(&bars->acc_empty[i], 4);  // one arrival per epilogue warp
     }
@@ -584,29 +601,56 @@ __global__ void __launch_bounds__(kTpThreads, 1)
         segment(c, ot, kb0, kb1, part);
         c += kb1 - kb0;
         for (int kb = kb0; kb < kb1 && !*abort_flag; ++kb, ++g) {
-          const int st = (int)(g % S);
-          const long long use = g / S;
-          if (use >= 1 && !tc_wait(&bars->empty[st], (uint32_t)((use - 1) & 1), abort_flag, status))
+          const int st = (int)(g % R);
+          const long long use = g / R;
+          if (use >= 1 && !tc_wait(TR ? &bars->raw_free[st] : &bars->empty[st],
+                                   (uint32_t)((use - 1) & 1), abort_flag, status))
             break;
-          unsigned char* sb = base + st * Sh::StageBytes;
           fence_proxy_async();
-          mbar_arrive_expect_tx(&bars->full[st], Sh::PBytes + Sh::BBytes);
           if constexpr (!TR) {
+            unsigned char* sb = base + st * Sh::StageBytes;
+            mbar_arrive_expect_tx(&bars->full[st], Sh::PBytes + Sh::BBytes);
             tma_load_2d(sb, &tmP, kb * 32, ot * kBM, &bars->full[st]);
+            unsigned char* bb = sb + Sh::HiBytes + Sh::LoBytes;
+            tma_load_2d(bb, &tmF, kb * 32, 0, &bars->full[st]);
+            tma_load_2d(bb + RP * 128, &tmF, kb * 32, 64, &bars->full[st]);
           } else {
+            unsigned char* sb = base + Sh::OffRaw + st * Sh::PBytes;
+            mbar_arrive_expect_tx(&bars->full[st], Sh::PBytes);
 #pragma unroll
             for (int b = 0; b < 4; ++b)
               tma_load_2d(sb + b * 4096, &tmP, ot * kBM + 32 * b, kb * 32, &bars->full[st]);
           }
-          unsigned char* bb = sb + Sh::PBytes + Sh::HiBytes + Sh::LoBytes;
-          tma_load_2d(bb, &tmF, kb * 32, 0, &bars->full[st]);
-          tma_load_2d(bb + RP * 128, &tmF, kb * 32, 64, &bars->full[st]);
           issued = g + 1;
         }
       }
       if (*abort_flag)  // the loads issued land before the CTA exits (bounded)
+        for (long long j = (issued > R ? issued - R : 0); j < issued; ++j)
+          mbar_wait_bounded(&bars->full[j % R], (uint32_t)((j / R) & 1), nullptr);
+    }
+  } else if (TR && warp == 2 + NS + 4) {
+    // ---------------- factor chunks (Y) ----------------
+    if (lane == 0) {
+      long long g = 0, issued = 0;
+      for (long long c = c0; c < c1 && !*abort_flag;) {
+        int ot, part, kb0, kb1;
+        segment(c, ot, kb0, kb1, part);
+        c += kb1 - kb0;
+        for (int kb = kb0; kb < kb1 && !*abort_flag; ++kb, ++g) {
+          const int st = (int)(g % S);
+          const long long use = g / S;
+          if (use >= 1 && !tc_wait(&bars->empty[st], (uint32_t)((use - 1) & 1), abort_flag, status))
+            break;
+          unsigned char* bb = base + st * Sh::StageBytes + Sh::HiBytes + Sh::LoBytes;
+          mbar_arrive_expect_tx(&bars->b_full[st], Sh::BBytes);
+          tma_load_2d(bb, &tmF, kb * 32, 0, &bars->b_full[st]);
+          tma_load_2d(bb + RP * 128, &tmF, kb * 32, 64, &bars->b_full[st]);
+          issued = g + 1;
+        }
+      }
+      if (*abort_flag)
         for (long long j = (issued > S ? issued - S : 0); j < issued; ++j)
-          mbar_wait_bounded(&bars->full[j % S], (uint32_t)((j / S) & 1), nullptr);
+          mbar_wait_bounded(&bars->b_full[j % S], (uint32_t)((j / S) & 1), nullptr);
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer (whole warp, one elected lane issues) ----------------
@@ -617,18 +661,19 @@ __global__ void __launch_bounds__(kTpThreads, 1)
     uint32_t phase = 0;
     long long g = 0;
     for (; g < chunks; ++g) {
-      const int buf = (int)(g & 1);
-      const long long bu = g >> 1;
+      const int buf = (int)(g % NB);
+      const long long bu = g / NB;
       const bool ok =
           !*abort_flag && tc_wait(&bars->split[st], phase, abort_flag, status) &&
+          (!TR || tc_wait(&bars->b_full[st], phase, abort_flag, status)) &&
           (bu < 1 || tc_wait(&bars->acc_empty[buf], (uint32_t)((bu - 1) & 1), abort_flag, status));
       if (!__all_sync(0xffffffffu, ok)) break;
       tc_fence_after();
       if (elect_one()) {
         const uint32_t d = tm + buf * (2 * RP);
         const uint64_t s0 = s00 + (uint32_t)st * (Sh::StageBytes >> 4);
-        const uint64_t a_hi = TR ? s0 + (Sh::PBytes >> 4) : s0;
-        const uint64_t a_lo = s0 + ((Sh::PBytes + Sh::HiBytes) >> 4);
+        const uint64_t a_hi = s0;
+        const uint64_t a_lo = s0 + (Sh::HiBytes >> 4);
         const uint64_t b_hi = a_lo + (Sh::LoBytes >> 4);  // 2 RP rows: hi(B), then lo(B)
         // per K step of 8 (32 bytes of each 128-byte row): hi(A) [hi(B) |
         // lo(B)] over 2 RP columns, then lo(A) hi(B) into the first RP: the
@@ -650,10 +695,10 @@ __global__ void __launch_bounds__(kTpThreads, 1)
     }
     if (g < chunks && g > 0 && lane == 0) {
       const long long j = g - 1;  // aborted: the MMAs issued finish before the TMEM is freed
-      mbar_wait_bounded(&bars->acc_full[j & 1], (uint32_t)((j >> 1) & 1), nullptr);
+      mbar_wait_bounded(&bars->acc_full[j % NB], (uint32_t)((j / NB) & 1), nullptr);
     }
-  } else if (warp < 6) {
-    // ---------------- split (warps 2..5, 128 threads) ----------------
+  } else if (warp < 2 + NS) {
+    // ---------------- split (warps 2 .. 2 + NS - 1) ----------------
     const int st_tid = tid - 64;
     long long g = 0;
     bool ok = true;
@@ -662,16 +707,17 @@ __global__ void __launch_bounds__(kTpThreads, 1)
       segment(c, ot, kb0, kb1, part);
       c += kb1 - kb0;
       for (int kb = kb0; kb < kb1; ++kb, ++g) {
-        const int st = (int)(g % S);
-        const long long use = g / S;
-        ok = tc_wait(&bars->full[st], (uint32_t)(use & 1), abort_flag, status);
+        const int st = (int)(g % S), rs = (int)(g % R);
+        ok = tc_wait(&bars->full[rs], (uint32_t)((g / R) & 1), abort_flag, status) &&
+             (!TR || g < S ||
+              tc_wait(&bars->empty[st], (uint32_t)((g / S - 1) & 1), abort_flag, status));
         if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
-        unsigned char* sb = base + st * Sh::StageBytes;
+        unsigned char* sb = TR ? base + Sh::OffRaw + rs * Sh::PBytes : base + st * Sh::StageBytes;
         if constexpr (!TR) {
           // the loaded box is hi(P) as the tensor pipe reads it; lo beside it
           // (same swizzled offsets)
           const float4* pv = reinterpret_cast<const float4*>(sb);
-          float4* lv = reinterpret_cast<float4*>(sb + Sh::PBytes);
+          float4* lv = reinterpret_cast<float4*>(sb + Sh::HiBytes);
 #pragma unroll
           for (int q = 0; q < (int)(Sh::PBytes / 16) / 128; ++q) {
             const int f = st_tid + q * 128;
@@ -684,11 +730,10 @@ __global__ void __launch_bounds__(kTpThreads, 1)
           // 128 rows j x 32 i; a thread moves 4 x 4 blocks (4 i, 4 j): the 8
           // threads of a group take distinct (i-block, j-block mod 8) pairs,
           // which fall in distinct 16-byte chunks on both sides
-          unsigned char* hi = sb + Sh::PBytes;
+          unsigned char* hi = base + st * Sh::StageBytes;
           unsigned char* lo = hi + Sh::HiBytes;
-#pragma unroll
-          for (int it = 0; it < 2; ++it) {
-            const int grp = (st_tid >> 3) + 16 * it;  // 0..31
+          {
+            const int grp = st_tid >> 3;  // 0..31
             const int k8 = st_tid & 7;
             const int ib = k8;                                       // rows 4 ib .. 4 ib + 3
             const int jb = 8 * (grp & 3) + ((k8 + (grp >> 2)) & 7);  // columns 4 jb .. + 3
@@ -715,11 +760,14 @@ __global__ void __launch_bounds__(kTpThreads, 1)
         }
         fence_proxy_async();  // generic-proxy writes, read next by the tensor cores
         __syncwarp();
-        if (lane == 0) mbar_arrive(&bars->split[st]);
+        if (lane == 0) {
+          mbar_arrive(&bars->split[st]);
+          if constexpr (TR) mbar_arrive(&bars->raw_free[rs]);
+        }
       }
     }
   } else {
-    // ---------------- epilogue (warps 6..9) ----------------
+    // ---------------- epilogue (four warps) ----------------
     const int quarter = warp & 3;  // TMEM lanes 32 quarter .. + 31
     const int row = quarter * 32 + lane;
     long long g = 0;
@@ -732,8 +780,8 @@ __global__ void __launch_bounds__(kTpThreads, 1)
 #pragma unroll
       for (int c = 0; c < RP; ++c) acc[c] = 0.f;
       for (int kb = kb0; kb < kb1; ++kb, ++g) {
-        const int buf = (int)(g & 1);
-        const long long bu = g >> 1;
+        const int buf = (int)(g % NB);
+        const long long bu = g / NB;
         ok = tc_wait(&bars->acc_full[buf], (uint32_t)(bu & 1), abort_flag, status);
         if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
         tc_fence_after();
@@ -870,7 +918,7 @@ static cudaError_t launch_tp_t(const CUtensorMap& tmP, const CUtensorMap& tmF, f
       tc_products_kernel<TR, RP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::SmemBytes);
   if (configured != cudaSuccess) return configured;
   const int grid = (int)tp_grid(n, num_sms);
-  tc_products_kernel<TR, RP><<<grid, kTpThreads, Sh::SmemBytes, s>>>(tmP, tmF, out, ps, cs, n,
+  tc_products_kernel<TR, RP><<<grid, Sh::Threads, Sh::SmemBytes, s>>>(tmP, tmF, out, ps, cs, n,
                                                                      r_out, parts, status);
   return cudaGetLastError();
 }
@@ -881,7 +929,7 @@ cudaError_t launch_tc_products(bool transpose, const float* P, int64_t ldp, cons
                                cudaStream_t s) {
   if (r < 1 || r > kMaxTcR || parts != tp_parts(n, num_sms) || fs % 64 || fs < n)
     return cudaErrorInvalidValue;
-  const int rp = r <= 32 ? 32 : 64;
+  const int rp = r <= 16 ? 16 : (r <= 32 ? 32 : 64);
   const int64_t tot = (int64_t)rp * n;
   tp_split_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(F, fs, n, r, rp, Fsplit);
   CUtensorMap tmP, tmF;
@@ -890,11 +938,15 @@ cudaError_t launch_tc_products(bool transpose, const float* P, int64_t ldp, cons
   if (!make_tmap_sw128(&tmP, P, n, n, ldp, transpose ? 32 : 128) ||
       !make_tmap_sw128(&tmF, Fsplit, n, 128, fs, rp))
     return cudaErrorInvalidValue;
-  if (transpose)
-    return rp == 32 ? launch_tp_t<true, 32>(tmP, tmF, out, ps, cs, n, r, parts, num_sms, status, s)
-                    : launch_tp_t<true, 64>(tmP, tmF, out, ps, cs, n, r, parts, num_sms, status, s);
-  return rp == 32 ? launch_tp_t<false, 32>(tmP, tmF, out, ps, cs, n, r, parts, num_sms, status, s)
-                  : launch_tp_t<false, 64>(tmP, tmF, out, ps, cs, n, r, parts, num_sms, status, s);
+  auto run = [&](auto tr) {
+    constexpr bool TR = decltype(tr)::value;
+    if (rp == 16)
+      return launch_tp_t<TR, 16>(tmP, tmF, out, ps, cs, n, r, parts, num_sms, status, s);
+    if (rp == 32)
+      return launch_tp_t<TR, 32>(tmP, tmF, out, ps, cs, n, r, parts, num_sms, status, s);
+    return launch_tp_t<TR, 64>(tmP, tmF, out, ps, cs, n, r, parts, num_sms, status, s);
+  };
+  return transpose ? run(std::true_type{}) : run(std::false_type{});
 }
 
 }  // namespace lv
