@@ -216,7 +216,8 @@ struct linview_program {
   int* solver_info = nullptr;
   int64_t ols_chunk = 0;
   // CUDA graphs of the per-update propagation (powers/sums), one per rank,
-  // replayed on a program-owned stream joined to the caller's stream
+  // captured on a program-owned stream and replayed on the caller's stream (joining
+  // two streams by events around each replay idled the GPU for a few us per update)
   bool use_graphs = true;
   cudaStream_t gstream = nullptr;
   // side stream of a propagation: the sums-view updates run there, forked
@@ -224,7 +225,9 @@ struct linview_program {
   cudaStream_t side = nullptr;
   cudaEvent_t side_fork_ev = nullptr, side_join_ev = nullptr;
   bool side_pending = false;
-  cudaEvent_t gev_in = nullptr, gev_out = nullptr;
+  // stream of the factor cores of wide levels (core_fork)
+  cudaStream_t core = nullptr;
+  cudaEvent_t core_fork_ev = nullptr, core_join_ev = nullptr;
   struct Rec {
     cudaEvent_t e0, e1;
     int kind;
@@ -1235,6 +1238,38 @@ static linview_status sums_update(linview_program* p, View& sv, const T* U, cons
   return sums_update_on<T>(p, sv, U, Vh, rh, r, side, 1);
 }
 
+// The factor core C_h = V_h^T U_h of a wide level reads only factors and is read
+// only by the assembly: it runs on a stream of its own next to the level's passes
+// (two launches, 5 - 15 us by width, off the chain), forked from s here and joined by
+// core_join before the assembly.  Under profiling everything stays on s.
+template <typename T>
+static linview_status core_fork(linview_program* p, const T* V, const T* U, int rh,
+                                cudaStream_t s) {
+  cudaStream_t cs = s;
+  if (!p->prof) {
+    if (!p->core) {
+      LV_CUDA(cudaStreamCreateWithFlags(&p->core, cudaStreamNonBlocking));
+      LV_CUDA(cudaEventCreateWithFlags(&p->core_fork_ev, cudaEventDisableTiming));
+      LV_CUDA(cudaEventCreateWithFlags(&p->core_join_ev, cudaEventDisableTiming));
+    }
+    LV_CUDA(cudaEventRecord(p->core_fork_ev, s));
+    LV_CUDA(cudaStreamWaitEvent(p->core, p->core_fork_ev, 0));
+    cs = p->core;
+  }
+  {
+    ProfScope ps(p, cs, 0.0);
+    LV_CUDA((launch_gram<T>(V, U, p->fs, (int)p->d.n, rh, p->Cpart, p->ticket, p->C, p->status,
+                            cs)));
+  }
+  if (cs != s) LV_CUDA(cudaEventRecord(p->core_join_ev, cs));
+  return LINVIEW_OK;
+}
+
+static linview_status core_join(linview_program* p, cudaStream_t s) {
+  if (!p->prof) LV_CUDA(cudaStreamWaitEvent(s, p->core_join_ev, 0));
+  return LINVIEW_OK;
+}
+
 // Exponential-model levels l = 0 .. nlev-1 (h = 2^l, Appendix A): the level
 // pass on P_h (P_h U_h, P_h^T V_h from the old view, P_h += U_h V_h^T; for
 // r_h <= kMaxFusedR the same pass yields the partials of C_h = V_h^T U_h),
@@ -1251,15 +1286,13 @@ static linview_status exp_levels(linview_program* p, int r, int nlev, bool sums,
     const int rh = r << l;
     T* Vh = V + (int64_t)(p->Rcap - rh) * fs;
     const bool fused = rh <= kMaxFusedR;
-    if (!fused) {
-      ProfScope ps(p, s, 0.0);
-      LV_CUDA((launch_gram<T>(Vh, U, fs, n, rh, p->Cpart, p->ticket, p->C, p->status, s)));
-    }
+    if (!fused) LV_TRY(core_fork<T>(p, Vh, U, rh, s));
     // sums: S'_h += U_h (V_h K_h^T)^T, the suffix block sums taken in the pass
     // (side stream, concurrent with the level pass)
     if (sums && l >= 1) LV_TRY(sums_update<T>(p, sview(p, l), U, Vh, rh, r, s));
     LV_TRY(run_products_update<T>(p, pview(p, l), rh, U, Vh, U, Vh, s,
                                   fused ? p->Cpart : nullptr, /*allow_tc=*/true));
+    if (!fused) LV_TRY(core_join(p, s));
     AssembleParams a{};
     a.status = p->status;
     a.n = n;
@@ -1307,10 +1340,8 @@ static linview_status krylov_levels(linview_program* p, int bw, int nsteps, int 
     const int rh = j * bw;
     T* Vj = V + (int64_t)(p->Rcap - rh) * fs;
     View& Q = p->views[view0 + j - 1];
-    {  // C = V_j^T U_j (its first bw columns are V_j^T U_base)
-      ProfScope ps(p, s, 0.0);
-      LV_CUDA((launch_gram<T>(Vj, U, fs, n, rh, p->Cpart, p->ticket, p->C, p->status, s)));
-    }
+    // C = V_j^T U_j (its first bw columns are V_j^T U_base)
+    LV_TRY(core_fork<T>(p, Vj, U, rh, s));
     bool rev = false;
     LV_TRY(run_products_update<T>(p, Q, bw, U, Vb, nullptr, nullptr, s, nullptr, false, &rev));
     LV_TRY(run_update<T>(p, Q, U, Vj, rh, s, 0, 0, rev));
@@ -1319,6 +1350,7 @@ static linview_status krylov_levels(linview_program* p, int bw, int nsteps, int 
     // (S'_1 is A itself: no sums view for power index 0)
     if (sums_r > 0 && view0 + j - 1 >= 1)
       LV_TRY(sums_update<T>(p, sview(p, view0 + j - 1), U, Vj, rh, sums_r, s));
+    LV_TRY(core_join(p, s));
     AssembleParams a{};
     a.status = p->status;
     a.n = n;
@@ -1551,12 +1583,10 @@ static linview_status iter_propagate(linview_program* p, int r, cudaStream_t s) 
   // is one contiguous p x (i r) slab: one pass over the T panel
   LV_TRY(panel_tdot<T>(p, reinterpret_cast<const T*>(Tp), p->ldT, V1, r, k, M, s));
   if (k >= 2) {
-    {
-      ProfScope ps(p, s, 0.0);
-      LV_CUDA((launch_gram<T>(V1, K, fs, n, r, p->Cpart, p->ticket, p->C, p->status, s)));
-    }
+    LV_TRY(core_fork<T>(p, V1, K, r, s));
     // X = A K_0 on the old A, A += K_0 V^T in the same pass
     LV_TRY(run_fused<T>(p, a, kModeXU, r, K, nullptr, K, V1, p->Xpart, p->Ypart, s));
+    LV_TRY(core_join(p, s));
     AssembleParams as{};
     as.status = p->status;
     as.n = n;
@@ -2548,12 +2578,13 @@ void linview_destroy(linview_program* p) {
   for (auto& ge : p->graphs) cudaGraphExecDestroy(ge.exec);
   for (cudaEvent_t e : p->ev_pool) cudaEventDestroy(e);
   for (cudaEvent_t e : p->gev_pool) cudaEventDestroy(e);
-  if (p->gev_in) cudaEventDestroy(p->gev_in);
-  if (p->gev_out) cudaEventDestroy(p->gev_out);
   if (p->gstream) cudaStreamDestroy(p->gstream);
   if (p->side_fork_ev) cudaEventDestroy(p->side_fork_ev);
   if (p->side_join_ev) cudaEventDestroy(p->side_join_ev);
   if (p->side) cudaStreamDestroy(p->side);
+  if (p->core_fork_ev) cudaEventDestroy(p->core_fork_ev);
+  if (p->core_join_ev) cudaEventDestroy(p->core_join_ev);
+  if (p->core) cudaStreamDestroy(p->core);
   if (p->blas) cublasDestroy(p->blas);
   if (p->solver) cusolverDnDestroy(p->solver);
   delete p;
@@ -2773,8 +2804,6 @@ static linview_status capture_graph(linview_program* p, int r, bool inst,
 static linview_status graphs_for(linview_program* p, int r, bool inst, std::vector<size_t>* idx) {
   if (!p->gstream) {
     LV_CUDA(cudaStreamCreateWithFlags(&p->gstream, cudaStreamNonBlocking));
-    LV_CUDA(cudaEventCreateWithFlags(&p->gev_in, cudaEventDisableTiming));
-    LV_CUDA(cudaEventCreateWithFlags(&p->gev_out, cudaEventDisableTiming));
   }
   idx->clear();
   for (size_t i = 0; i < p->graphs.size(); ++i)
@@ -2801,11 +2830,7 @@ static linview_status graph_propagate(linview_program* p, int r, cudaStream_t s)
     pick = idx[p->prof_rr[r]++ % idx.size()];
   }
   linview_program::GraphEntry& ge = p->graphs[pick];
-  LV_CUDA(cudaEventRecord(p->gev_in, s));
-  LV_CUDA(cudaStreamWaitEvent(p->gstream, p->gev_in, 0));
-  LV_CUDA(cudaGraphLaunch(ge.exec, p->gstream));
-  LV_CUDA(cudaEventRecord(p->gev_out, p->gstream));
-  LV_CUDA(cudaStreamWaitEvent(s, p->gev_out, 0));
+  LV_CUDA(cudaGraphLaunch(ge.exec, s));
   ge.replayed = true;
   p->all_launches += ge.launches;
   return LINVIEW_OK;
@@ -2854,18 +2879,17 @@ static linview_status apply_b_delta(linview_program* p, int r, const void* U, in
   // U_b into Krylov block K_0 (linear model) or the U arena (exponential and
   // skip models); V_b into M (p x rank)
   void* ub_dst = iter_exp(p) ? p->Uar : p->Kar;
-  if (p->elem == 4) {
-    LV_CUDA(launch_rm_to_cm<float>(static_cast<const float*>(u), ldu, static_cast<float*>(ub_dst),
-                                   p->fs, (int)n, r, s));
-    LV_CUDA(launch_rm_to_cm<float>(static_cast<const float*>(v), ldv, static_cast<float*>(p->Mr),
-                                   pp, (int)pp, r, s));
-  } else {
-    LV_CUDA(launch_rm_to_cm<double>(static_cast<const double*>(u), ldu,
-                                    static_cast<double*>(ub_dst), p->fs, (int)n, r, s));
-    LV_CUDA(launch_rm_to_cm<double>(static_cast<const double*>(v), ldv,
-                                    static_cast<double*>(p->Mr), pp, (int)pp, r, s));
-  }
-  p->all_launches += 2;
+  if (p->elem == 4)
+    LV_CUDA(launch_ingest_pair<float>(static_cast<const float*>(u), ldu,
+                                      static_cast<float*>(ub_dst), p->fs, (int)n,
+                                      static_cast<const float*>(v), ldv,
+                                      static_cast<float*>(p->Mr), pp, (int)pp, r, s));
+  else
+    LV_CUDA(launch_ingest_pair<double>(static_cast<const double*>(u), ldu,
+                                       static_cast<double*>(ub_dst), p->fs, (int)n,
+                                       static_cast<const double*>(v), ldv,
+                                       static_cast<double*>(p->Mr), pp, (int)pp, r, s));
+  p->all_launches++;
   LV_TRY(propagate(p, kKeyB + r, s));
   return after_update(p, s);
 }
@@ -2902,18 +2926,17 @@ linview_status linview_apply_delta(linview_program* p, int input_id, int64_t ran
     ldu = r;
     ldv = r;
   }
-  if (p->elem == 4) {
-    LV_CUDA(launch_rm_to_cm<float>(static_cast<const float*>(u), ldu, static_cast<float*>(u_dst(p)),
-                                   p->fs, (int)n, r, s));
-    LV_CUDA(launch_rm_to_cm<float>(static_cast<const float*>(v), ldv,
-                                   static_cast<float*>(v_dst(p, r)), p->fs, (int)n, r, s));
-  } else {
-    LV_CUDA(launch_rm_to_cm<double>(static_cast<const double*>(u), ldu,
-                                    static_cast<double*>(u_dst(p)), p->fs, (int)n, r, s));
-    LV_CUDA(launch_rm_to_cm<double>(static_cast<const double*>(v), ldv,
-                                    static_cast<double*>(v_dst(p, r)), p->fs, (int)n, r, s));
-  }
-  p->all_launches += 2;
+  if (p->elem == 4)
+    LV_CUDA(launch_ingest_pair<float>(static_cast<const float*>(u), ldu,
+                                      static_cast<float*>(u_dst(p)), p->fs, (int)n,
+                                      static_cast<const float*>(v), ldv,
+                                      static_cast<float*>(v_dst(p, r)), p->fs, (int)n, r, s));
+  else
+    LV_CUDA(launch_ingest_pair<double>(static_cast<const double*>(u), ldu,
+                                       static_cast<double*>(u_dst(p)), p->fs, (int)n,
+                                       static_cast<const double*>(v), ldv,
+                                       static_cast<double*>(v_dst(p, r)), p->fs, (int)n, r, s));
+  p->all_launches++;
   LV_TRY(propagate(p, r, s));
   return after_update(p, s);
 }
@@ -2928,13 +2951,17 @@ linview_status linview_apply_row_delta(linview_program* p, int input_id, int64_t
   if (on_device) LV_TRY(check_dev_ptr(v, p->device, "v"));
   LV_CUDA(cudaSetDevice(p->device));
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  LV_CUDA(cudaMemcpyAsync(v_dst(p, 1), v, n * p->elem,
-                          on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
-  if (p->elem == 4) {
-    LV_CUDA(launch_unit_column<float>(static_cast<float*>(u_dst(p)), (int)n, (int)row, s));
-  } else {
-    LV_CUDA(launch_unit_column<double>(static_cast<double*>(u_dst(p)), (int)n, (int)row, s));
-  }
+  if (!on_device)
+    LV_CUDA(cudaMemcpyAsync(v_dst(p, 1), v, n * p->elem, cudaMemcpyHostToDevice, s));
+  const void* vd = on_device ? v : nullptr;
+  if (p->elem == 4)
+    LV_CUDA(launch_ingest_row<float>(static_cast<float*>(u_dst(p)),
+                                     static_cast<float*>(v_dst(p, 1)),
+                                     static_cast<const float*>(vd), (int)n, (int)row, s));
+  else
+    LV_CUDA(launch_ingest_row<double>(static_cast<double*>(u_dst(p)),
+                                      static_cast<double*>(v_dst(p, 1)),
+                                      static_cast<const double*>(vd), (int)n, (int)row, s));
   p->all_launches += 1;
   LV_TRY(propagate(p, 1, s));
   return after_update(p, s);

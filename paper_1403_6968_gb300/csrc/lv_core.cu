@@ -37,6 +37,8 @@ __global__ void __launch_bounds__(kThreads) gram_f64_kernel(const double* __rest
                                                             int64_t fs, int n, int r,
                                                             double* Cpart, unsigned* ticket,
                                                             double* C, unsigned* status) {
+  griddep_wait();
+  griddep_launch_dependents();
   __shared__ double Vs[kGramRows][kGramMaxR + 1];
   __shared__ double Us[kGramRows][kGramMaxR + 1];
   __shared__ bool last;
@@ -112,6 +114,8 @@ __global__ void __launch_bounds__(kThreads) gram_df_kernel(const float* __restri
                                                            const float* __restrict__ U,
                                                            int64_t fs, int n, int rv, int r,
                                                            float2* Cpart) {
+  griddep_wait();
+  griddep_launch_dependents();
   __shared__ float Vs[kGramRows][kGramMaxR + 1];
   __shared__ float Us[kGramRows][kGramMaxR + 1];
   const int tid = threadIdx.x;
@@ -158,6 +162,8 @@ __global__ void __launch_bounds__(kThreads) gram_df_kernel(const float* __restri
 // in order, then a fixed butterfly combines the lanes (lane 0's sum is kept).
 __global__ void gram_reduce_kernel(const float2* __restrict__ Cpart, int G, int ne, double* C,
                                    unsigned* status, float2* Cdf) {
+  griddep_wait();
+  griddep_launch_dependents();
   const int e = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
   const int lane = threadIdx.x & 31;
   if (e >= ne) return;  // warp-uniform
@@ -191,13 +197,14 @@ cudaError_t launch_gram(const T* V, const T* U, int64_t fs, int n, int r, double
   const int G = gram_grid(n);
   if constexpr (std::is_same<T, float>::value) {
     float2* part = reinterpret_cast<float2*>(Cpart);
-    gram_df_kernel<false><<<G, kThreads, 0, s>>>(V, U, fs, n, r, r, part);
+    LV_LAUNCH(launch_pdl(gram_df_kernel<false>, G, kThreads, 0, s, V, U, fs, n, r, r, part));
     const int ne = r * r;
     const int warps_per_block = kThreads / 32;
-    gram_reduce_kernel<<<(ne + warps_per_block - 1) / warps_per_block, kThreads, 0, s>>>(
-        part, G, ne, C, status, Cdf);
+    LV_LAUNCH(launch_pdl(gram_reduce_kernel, (ne + warps_per_block - 1) / warps_per_block, kThreads,
+        0, s, part, G, ne, C, status, Cdf));
   } else {
-    gram_f64_kernel<<<G, kThreads, 0, s>>>(V, U, fs, n, r, Cpart, ticket, C, status);
+    LV_LAUNCH(launch_pdl(gram_f64_kernel, G, kThreads, 0, s, V, U, fs, n, r, Cpart, ticket, C,
+        status));
   }
   return cudaGetLastError();
 }
@@ -209,11 +216,12 @@ cudaError_t launch_cross_gram(const float* X, const float* V, int64_t fs, int n,
   float2* part = reinterpret_cast<float2*>(Cpart);
   for (int c0 = 0; c0 < rx; c0 += kGramMaxR) {
     const int w = rx - c0 < kGramMaxR ? rx - c0 : kGramMaxR;
-    gram_df_kernel<true><<<G, kThreads, 0, s>>>(X + (int64_t)c0 * fs, V, fs, n, w, rv, part);
+    LV_LAUNCH(launch_pdl(gram_df_kernel<true>, G, kThreads, 0, s, X + (int64_t)c0 * fs, V, fs, n, w,
+        rv, part));
     const int ne = w * rv;
     const int warps_per_block = kThreads / 32;
-    gram_reduce_kernel<<<(ne + warps_per_block - 1) / warps_per_block, kThreads, 0, s>>>(
-        part, G, ne, C + (int64_t)c0 * rv, nullptr, nullptr);
+    LV_LAUNCH(launch_pdl(gram_reduce_kernel, (ne + warps_per_block - 1) / warps_per_block, kThreads,
+        0, s, part, G, ne, C + (int64_t)c0 * rv, nullptr, nullptr));
   }
   return cudaGetLastError();
 }
@@ -331,10 +339,12 @@ __global__ void __launch_bounds__(kThreads) assemble_kernel(const AssembleParams
   if (Yp) static_cast<T*>(a.Ynew)[(int64_t)c * a.fs + j] = ys;
 }
 
-// The same assembly for wide blocks (r_out >= 8): there are enough outputs
+// The same assembly for wide blocks (r_out >= 8) where there are enough outputs
 // to fill the GPU with one thread per (j, c), which then sums all partials
 // itself (CTA = 256 rows of one column; the C_h column is summed once per
-// CTA).  Same fixed orders as above within a thread's sums.
+// CTA).  Same fixed orders as above within a thread's sums.  Small views have few
+// outputs and many row ranges (n = 1000: 127 partial sets): below n = 4096 with more
+// than 24 sets the warps of a CTA share them (n = 1000, 12 columns: 15.5 -> ASM_NEW us).
 template <typename T>
 __global__ void __launch_bounds__(kThreads) assemble_wide_kernel(const AssembleParams a) {
   __shared__ T Cc[kMaxAsmR];
@@ -385,7 +395,8 @@ cudaError_t launch_assemble(const AssembleParams& a, cudaStream_t s) {
   if (a.r_h > kMaxAsmR) return cudaErrorInvalidValue;
   const int ro = a.r_out > 0 ? a.r_out : a.r_h;
   cudaError_t e;
-  if (ro >= 8) {
+  const int sets = a.gC + (a.Ypart ? a.gR : 0);
+  if (ro >= 8 && (sets <= 24 || a.n >= 4096)) {
     const dim3 grid((unsigned)((a.n + kThreads - 1) / kThreads), (unsigned)ro);
     e = launch_pdl(assemble_wide_kernel<T>, grid, kThreads, 0, s, a);
   } else {
@@ -404,6 +415,8 @@ constexpr int kChunk = 16;  // independent loads issued together
 template <typename T>
 __global__ void suffix_sums_kernel(const T* __restrict__ V, T* __restrict__ W, int64_t fs, int n,
                                    int width, int r_in) {
+  griddep_wait();
+  griddep_launch_dependents();
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (int64_t)n * r_in) return;
   int c, j;
@@ -434,13 +447,15 @@ template <typename T>
 cudaError_t launch_suffix_sums(const T* V, T* W, int64_t fs, int n, int width, int r_in,
                                cudaStream_t s) {
   const int64_t tot = (int64_t)n * r_in;
-  suffix_sums_kernel<T><<<(unsigned)((tot + kThreads - 1) / kThreads), kThreads, 0, s>>>(
-      V, W, fs, n, width, r_in);
+  LV_LAUNCH(launch_pdl(suffix_sums_kernel<T>, (unsigned)((tot + kThreads - 1) / kThreads), kThreads,
+      0, s, V, W, fs, n, width, r_in));
   return cudaGetLastError();
 }
 
 template <typename T>
 __global__ void rm_to_cm_kernel(const T* src, int64_t ld, T* dst, int64_t fs, int rows, int cols) {
+  griddep_wait();
+  griddep_launch_dependents();
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (int64_t)rows * cols) return;
   int c, j;
@@ -453,26 +468,59 @@ cudaError_t launch_rm_to_cm(const T* src, int64_t ld, T* dst, int64_t fs, int ro
                             cudaStream_t s) {
   const int64_t tot = (int64_t)rows * cols;
   if (tot == 0) return cudaSuccess;
-  rm_to_cm_kernel<T><<<(unsigned)((tot + kThreads - 1) / kThreads), kThreads, 0, s>>>(
-      src, ld, dst, fs, rows, cols);
+  LV_LAUNCH(launch_pdl(rm_to_cm_kernel<T>, (unsigned)((tot + kThreads - 1) / kThreads), kThreads, 0,
+      s, src, ld, dst, fs, rows, cols));
   return cudaGetLastError();
 }
 
+// Ingest of an update's factors in one launch: two row-major blocks into
+// column-major storage, and e_row with a copy of v.
 template <typename T>
-__global__ void unit_column_kernel(T* dst, int n, int row) {
+__global__ void ingest_pair_kernel(const T* U, int64_t ldu, T* du, int nu, const T* V, int64_t ldv,
+                                   T* dv, int nv, int64_t fsu, int64_t fsv, int cols) {
+  griddep_wait();
+  griddep_launch_dependents();
+  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t tu = (int64_t)nu * cols;
+  int c, j;
+  if (idx < tu) {
+    split_index(idx, nu, c, j);
+    du[(int64_t)c * fsu + j] = U[(int64_t)j * ldu + c];
+  } else if (idx < tu + (int64_t)nv * cols) {
+    split_index(idx - tu, nv, c, j);
+    dv[(int64_t)c * fsv + j] = V[(int64_t)j * ldv + c];
+  }
+}
+
+template <typename T>
+cudaError_t launch_ingest_pair(const T* U, int64_t ldu, T* du, int64_t fsu, int nu, const T* V,
+                               int64_t ldv, T* dv, int64_t fsv, int nv, int cols, cudaStream_t s) {
+  const int64_t tot = (int64_t)(nu + nv) * cols;
+  return launch_pdl(ingest_pair_kernel<T>, (unsigned)((tot + kThreads - 1) / kThreads), kThreads, 0,
+                    s, U, ldu, du, nu, V, ldv, dv, nv, fsu, fsv, cols);
+}
+
+template <typename T>
+__global__ void ingest_row_kernel(T* du, T* dv, const T* v, int n, int row) {
+  griddep_wait();
+  griddep_launch_dependents();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j < n) dst[j] = (j == row) ? T(1) : T(0);
+  if (j >= n) return;
+  du[j] = (j == row) ? T(1) : T(0);
+  if (v) dv[j] = v[j];
 }
 
 template <typename T>
-cudaError_t launch_unit_column(T* dst, int n, int row, cudaStream_t s) {
-  unit_column_kernel<T><<<(n + kThreads - 1) / kThreads, kThreads, 0, s>>>(dst, n, row);
-  return cudaGetLastError();
+cudaError_t launch_ingest_row(T* du, T* dv, const T* v, int n, int row, cudaStream_t s) {
+  return launch_pdl(ingest_row_kernel<T>, (n + kThreads - 1) / kThreads, kThreads, 0, s, du, dv, v,
+                    n, row);
 }
 
 template <typename T>
 __global__ void sum_partials_kernel(const T* part, int blocks, int64_t bs, int64_t cs, int n,
                                     int r, T* out, int64_t ocs) {
+  griddep_wait();
+  griddep_launch_dependents();
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (int64_t)n * r) return;
   int c, j;
@@ -488,6 +536,8 @@ __global__ void sum_partials_kernel(const T* part, int blocks, int64_t bs, int64
 // passes leave a few dozen partials per entry).
 __global__ void sum_partials_f32_kernel(const float* part, int blocks, int64_t bs, int64_t cs,
                                         int n, int r, float* out, int64_t ocs) {
+  griddep_wait();
+  griddep_launch_dependents();
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (int64_t)n * r) return;
   int c, j;
@@ -519,17 +569,19 @@ cudaError_t launch_sum_partials(const T* part, int blocks, int64_t block_stride,
   if (tot == 0) return cudaSuccess;
   const unsigned grid = (unsigned)((tot + kThreads - 1) / kThreads);
   if constexpr (sizeof(T) == 4)
-    sum_partials_f32_kernel<<<grid, kThreads, 0, s>>>(part, blocks, block_stride, cs, n, r, out,
-                                                      out_cs);
+    LV_LAUNCH(launch_pdl(sum_partials_f32_kernel, grid, kThreads, 0, s, part, blocks, block_stride,
+        cs, n, r, out, out_cs));
   else
-    sum_partials_kernel<T><<<grid, kThreads, 0, s>>>(part, blocks, block_stride, cs, n, r, out,
-                                                      out_cs);
+    LV_LAUNCH(launch_pdl(sum_partials_kernel<T>, grid, kThreads, 0, s, part, blocks, block_stride,
+        cs, n, r, out, out_cs));
   return cudaGetLastError();
 }
 
 template <typename T>
 __global__ void axpy_rows_kernel(T* y, int64_t ldy, const T* x, int64_t ldx, T alpha, int rows,
                                  int cols) {
+  griddep_wait();
+  griddep_launch_dependents();
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (int64_t)rows * cols) return;
   int i, c;
@@ -542,14 +594,16 @@ cudaError_t launch_axpy_rows(T* y, int64_t ldy, const T* x, int64_t ldx, T alpha
                              int cols, cudaStream_t s) {
   const int64_t tot = (int64_t)rows * cols;
   if (tot == 0) return cudaSuccess;
-  axpy_rows_kernel<T><<<(unsigned)((tot + kThreads - 1) / kThreads), kThreads, 0, s>>>(
-      y, ldy, x, ldx, alpha, rows, cols);
+  LV_LAUNCH(launch_pdl(axpy_rows_kernel<T>, (unsigned)((tot + kThreads - 1) / kThreads), kThreads,
+      0, s, y, ldy, x, ldx, alpha, rows, cols));
   return cudaGetLastError();
 }
 
 template <typename T>
 __global__ void scale_copy_kernel(T* y, int64_t ldy, const T* x, int64_t ldx, T alpha, int rows,
                                   int cols) {
+  griddep_wait();
+  griddep_launch_dependents();
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (int64_t)rows * cols) return;
   int i, c;
@@ -562,8 +616,8 @@ cudaError_t launch_scale_copy(T* y, int64_t ldy, const T* x, int64_t ldx, T alph
                               int cols, cudaStream_t s) {
   const int64_t tot = (int64_t)rows * cols;
   if (tot == 0) return cudaSuccess;
-  scale_copy_kernel<T><<<(unsigned)((tot + kThreads - 1) / kThreads), kThreads, 0, s>>>(
-      y, ldy, x, ldx, alpha, rows, cols);
+  LV_LAUNCH(launch_pdl(scale_copy_kernel<T>, (unsigned)((tot + kThreads - 1) / kThreads), kThreads,
+      0, s, y, ldy, x, ldx, alpha, rows, cols));
   return cudaGetLastError();
 }
 
@@ -629,7 +683,9 @@ cudaError_t launch_bounded_wait_probe(uint64_t limit_ns, unsigned* status,
   template cudaError_t launch_suffix_sums<T>(const T*, T*, int64_t, int, int, int, cudaStream_t); \
   template cudaError_t launch_rm_to_cm<T>(const T*, int64_t, T*, int64_t, int, int,               \
                                           cudaStream_t);                                        \
-  template cudaError_t launch_unit_column<T>(T*, int, int, cudaStream_t);                        \
+  template cudaError_t launch_ingest_row<T>(T*, T*, const T*, int, int, cudaStream_t);           \
+  template cudaError_t launch_ingest_pair<T>(const T*, int64_t, T*, int64_t, int, const T*,      \
+                                             int64_t, T*, int64_t, int, int, cudaStream_t);      \
   template cudaError_t launch_add_views<T>(const T*, const T*, T*, int64_t, int64_t,             \
                                            cudaStream_t);                                       \
   template cudaError_t launch_sum_partials<T>(const T*, int, int64_t, int64_t, int, int, T*,      \

@@ -11,11 +11,11 @@ namespace lv {
 // Launch ``k`` with programmatic stream serialisation (the kernel calls
 // griddep_wait() before it reads what earlier kernels of the stream wrote).
 template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*k)(KArgs...), dim3 grid, unsigned block, size_t smem,
+cudaError_t launch_pdl(void (*k)(KArgs...), dim3 grid, dim3 block, size_t smem,
                        cudaStream_t s, Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
-  cfg.blockDim = dim3(block);
+  cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -25,6 +25,13 @@ cudaError_t launch_pdl(void (*k)(KArgs...), dim3 grid, unsigned block, size_t sm
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, k, args...);
 }
+
+// return a failed launch's error from a launcher
+#define LV_LAUNCH(expr)                    \
+  do {                                     \
+    const cudaError_t e_ = (expr);         \
+    if (e_ != cudaSuccess) return e_;      \
+  } while (0)
 
 constexpr int kThreads = 256;   // threads per pass CTA
 constexpr int kBatch = 8;       // rows per pipeline stage = TMA box height = warps per CTA
@@ -230,9 +237,13 @@ cudaError_t launch_suffix_sums(const T* V, T* W, int64_t fs, int n, int width, i
 template <typename T>
 cudaError_t launch_rm_to_cm(const T* src, int64_t ld, T* dst, int64_t fs, int rows, int cols,
                             cudaStream_t s);
-// e_row as one column (column-major, n rows).
+// Ingest of an update in one launch: U (nu x cols, row-major) and V (nv x cols) into
+// column-major storage; or e_row into du with a copy of v (may be null: du only) in dv.
 template <typename T>
-cudaError_t launch_unit_column(T* dst, int n, int row, cudaStream_t s);
+cudaError_t launch_ingest_pair(const T* U, int64_t ldu, T* du, int64_t fsu, int nu, const T* V,
+                               int64_t ldv, T* dv, int64_t fsv, int nv, int cols, cudaStream_t s);
+template <typename T>
+cudaError_t launch_ingest_row(T* du, T* dv, const T* v, int n, int row, cudaStream_t s);
 
 // Sum of column-major partial blocks: out[c][j] = sum_b part[b][c][j].
 template <typename T>

@@ -25,6 +25,8 @@ namespace lv {
 template <typename T>
 __global__ void gather_rows_kernel(const T* X, int64_t ldx, const int64_t* rows, int k, int n,
                                    T* dst, int64_t ts, int64_t js) {
+  griddep_wait();
+  griddep_launch_dependents();
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (int64_t)k * n) return;
   int t, j;
@@ -36,6 +38,8 @@ __global__ void gather_rows_kernel(const T* X, int64_t ldx, const int64_t* rows,
 template <typename T>
 __global__ void scatter_rows_kernel(T* X, int64_t ldx, const int64_t* rows, int k, int n,
                                     const T* src, int64_t ts) {
+  griddep_wait();
+  griddep_launch_dependents();
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (int64_t)k * n) return;
   int t, j;
@@ -59,6 +63,8 @@ size_t core_inverse_smem(int kk) { return sizeof(double) * ((size_t)4 * kk * kk 
 
 __global__ void __launch_bounds__(kInvTx * kInvTy)
     core_inverse_kernel(const double* S, int kk, int kpos, double* Minv, unsigned* status) {
+  griddep_wait();
+  griddep_launch_dependents();
   extern __shared__ double inv_sm[];
   const int w = 2 * kk;
   double* cur = inv_sm;           // kk x w
@@ -384,6 +390,8 @@ __device__ __forceinline__ float ns_product(const float* A, const float* B, floa
 
 __global__ void __launch_bounds__(kCoreThreads)
     core_inverse_df_kernel(const float2* S, int kk, int kpos, float2* Minv, unsigned* status) {
+  griddep_wait();
+  griddep_launch_dependents();
   extern __shared__ __align__(16) unsigned char core_sm[];
   __shared__ float wsum[kCoreThreads / 32];
   const int tid = threadIdx.x;
@@ -490,6 +498,8 @@ __global__ void __launch_bounds__(kCoreThreads)
 // is even).
 __global__ void wu_f64_kernel(const double* G, int64_t fs, int n, int kk, const double* Minv,
                               double* Wu) {
+  griddep_wait();
+  griddep_launch_dependents();
   __shared__ double ms[64][2];
   const int c = 2 * blockIdx.y;
   for (int e = threadIdx.x; e < kk; e += blockDim.x) {
@@ -516,6 +526,8 @@ __global__ void wu_f64_kernel(const double* G, int64_t fs, int n, int kk, const 
 constexpr int kWuCols = 4;
 __global__ void wu_df_kernel(const float* G, int64_t fs, int n, int kk, const float2* Minv,
                              float* Wu) {
+  griddep_wait();
+  griddep_launch_dependents();
   __shared__ df2 ms[64][kWuCols];
   const int c0 = kWuCols * blockIdx.y;
   for (int e = threadIdx.x; e < kk * kWuCols; e += blockDim.x) {
@@ -545,6 +557,8 @@ __global__ void wu_df_kernel(const float* G, int64_t fs, int n, int kk, const fl
 template <typename T>
 __global__ void xty_update_kernel(T* xty, int64_t ld, T* xtyc, int64_t fs, const T* U, int n,
                                   int p, int k, const T* Yr) {
+  griddep_wait();
+  griddep_launch_dependents();
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (int64_t)n * p) return;
   int j, c;
@@ -565,6 +579,8 @@ __global__ void xty_update_kernel(T* xty, int64_t ld, T* xtyc, int64_t fs, const
 constexpr int kRowCols = 4;
 __global__ void xty_update_df_kernel(float* xty, float* xtyl, int64_t ld, float* xtyc, int64_t fs,
                                      const float* U, int n, int p, int k, const float* Yr) {
+  griddep_wait();
+  griddep_launch_dependents();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   const int c0 = blockIdx.y * kRowCols;
   if (j >= n) return;
@@ -601,6 +617,8 @@ __global__ void xty_update_df_kernel(float* xty, float* xtyl, int64_t ld, float*
 template <typename T>
 __global__ void __launch_bounds__(256) wtc_kernel(const T* Wu, const T* Cc, int64_t fs, int n,
                                                   int kk, int p, T* H) {
+  griddep_wait();
+  griddep_launch_dependents();
   __shared__ double part[8];
   const int c2 = blockIdx.x % kk, c = blockIdx.x / kk;
   const T* a = Wu + (int64_t)c2 * fs;
@@ -627,6 +645,8 @@ __global__ void __launch_bounds__(256) wtc_kernel(const T* Wu, const T* Cc, int6
 template <typename T>
 __global__ void beta_update_kernel(T* beta, int64_t ld, const T* G, int64_t fs, int n, int p,
                                    int k, const T* Yr, const T* H) {
+  griddep_wait();
+  griddep_launch_dependents();
   extern __shared__ __align__(16) unsigned char beta_sm[];
   T* Ys = reinterpret_cast<T*>(beta_sm);  // k x kRowCols
   T* Hs = Ys + k * kRowCols;              // 2k x kRowCols
@@ -912,8 +932,8 @@ template <typename T>
 cudaError_t launch_gather_rows(const T* X, int64_t ldx, const int64_t* rows, int k, int n, T* dst,
                                int64_t ts, int64_t js, cudaStream_t s) {
   if ((int64_t)k * n == 0) return cudaSuccess;
-  gather_rows_kernel<T><<<blocks_for((int64_t)k * n), kThreads, 0, s>>>(X, ldx, rows, k, n, dst,
-                                                                        ts, js);
+  LV_LAUNCH(launch_pdl(gather_rows_kernel<T>, blocks_for((int64_t)k * n), kThreads, 0, s, X, ldx,
+      rows, k, n, dst, ts, js));
   return cudaGetLastError();
 }
 
@@ -921,8 +941,8 @@ template <typename T>
 cudaError_t launch_scatter_rows(T* X, int64_t ldx, const int64_t* rows, int k, int n,
                                 const T* src, int64_t ts, cudaStream_t s) {
   if ((int64_t)k * n == 0) return cudaSuccess;
-  scatter_rows_kernel<T><<<blocks_for((int64_t)k * n), kThreads, 0, s>>>(X, ldx, rows, k, n, src,
-                                                                         ts);
+  LV_LAUNCH(launch_pdl(scatter_rows_kernel<T>, blocks_for((int64_t)k * n), kThreads, 0, s, X, ldx,
+      rows, k, n, src, ts));
   return cudaGetLastError();
 }
 
@@ -933,8 +953,8 @@ cudaError_t launch_core_inverse(const double* S, int kk, int kpos, double* Minv,
       cudaFuncSetAttribute(core_inverse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)core_inverse_smem(64));
   if (configured != cudaSuccess) return configured;
-  core_inverse_kernel<<<1, dim3(kInvTx, kInvTy), core_inverse_smem(kk), s>>>(S, kk, kpos, Minv,
-                                                                           status);
+  LV_LAUNCH(launch_pdl(core_inverse_kernel, 1, dim3(kInvTx, kInvTy), core_inverse_smem(kk), s, S,
+      kk, kpos, Minv, status));
   return cudaGetLastError();
 }
 
@@ -945,22 +965,24 @@ cudaError_t launch_core_inverse_df(const float2* S, int kk, int kpos, float2* Mi
       cudaFuncSetAttribute(core_inverse_df_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)core_df_smem(64));
   if (configured != cudaSuccess) return configured;
-  core_inverse_df_kernel<<<1, kCoreThreads, core_df_smem(kk), s>>>(S, kk, kpos, Minv, status);
+  LV_LAUNCH(launch_pdl(core_inverse_df_kernel, 1, kCoreThreads, core_df_smem(kk), s, S, kk, kpos,
+      Minv, status));
   return cudaGetLastError();
 }
 
 cudaError_t launch_wu(const double* G, int64_t fs, int n, int kk, const double* Minv, double* Wu,
                       cudaStream_t s) {
   if (kk < 2 || kk > 64 || (kk & 1)) return cudaErrorInvalidValue;
-  wu_f64_kernel<<<dim3(blocks_for(n), kk / 2), kThreads, 0, s>>>(G, fs, n, kk, Minv, Wu);
+  LV_LAUNCH(launch_pdl(wu_f64_kernel, dim3(blocks_for(n), kk / 2), kThreads, 0, s, G, fs, n, kk,
+      Minv, Wu));
   return cudaGetLastError();
 }
 
 cudaError_t launch_wu(const float* G, int64_t fs, int n, int kk, const float2* Minv, float* Wu,
                       cudaStream_t s) {
   if (kk < 2 || kk > 64 || (kk & 1)) return cudaErrorInvalidValue;
-  wu_df_kernel<<<dim3(blocks_for(n), (kk + kWuCols - 1) / kWuCols), kThreads, 0, s>>>(G, fs, n,
-                                                                                      kk, Minv, Wu);
+  LV_LAUNCH(launch_pdl(wu_df_kernel, dim3(blocks_for(n), (kk + kWuCols - 1) / kWuCols), kThreads, 0,
+      s, G, fs, n, kk, Minv, Wu));
   return cudaGetLastError();
 }
 
@@ -968,10 +990,10 @@ template <typename T>
 cudaError_t launch_beta_update(T* beta, int64_t ld, const T* G, const T* Wu, const T* Cc,
                                int64_t fs, int n, int p, int k, const T* Yr, T* H,
                                cudaStream_t s) {
-  wtc_kernel<T><<<(unsigned)(2 * k * p), 256, 0, s>>>(Wu, Cc, fs, n, 2 * k, p, H);
-  beta_update_kernel<T>
-      <<<dim3(blocks_for(n), (p + kRowCols - 1) / kRowCols), kThreads,
-         sizeof(T) * 3 * k * kRowCols, s>>>(beta, ld, G, fs, n, p, k, Yr, H);
+  LV_LAUNCH(launch_pdl(wtc_kernel<T>, (unsigned)(2 * k * p), 256, 0, s, Wu, Cc, fs, n, 2 * k, p,
+      H));
+  LV_LAUNCH(launch_pdl(beta_update_kernel<T>, dim3(blocks_for(n), (p + kRowCols - 1) / kRowCols),
+      kThreads, sizeof(T) * 3 * k * kRowCols, s, beta, ld, G, fs, n, p, k, Yr, H));
   return cudaGetLastError();
 }
 
@@ -979,11 +1001,11 @@ template <typename T>
 cudaError_t launch_xty_update(T* xty, int64_t ld, T* xtyc, int64_t fs, const T* U, int n, int p,
                               int k, const T* Yr, cudaStream_t s, T* xtyl) {
   if constexpr (sizeof(T) == 4)
-    xty_update_df_kernel<<<dim3(blocks_for(n), (p + kRowCols - 1) / kRowCols), kThreads, 0, s>>>(
-        xty, xtyl, ld, xtyc, fs, U, n, p, k, Yr);
+    LV_LAUNCH(launch_pdl(xty_update_df_kernel, dim3(blocks_for(n), (p + kRowCols - 1) / kRowCols),
+        kThreads, 0, s, xty, xtyl, ld, xtyc, fs, U, n, p, k, Yr));
   else
-    xty_update_kernel<T><<<blocks_for((int64_t)n * p), kThreads, 0, s>>>(xty, ld, xtyc, fs, U, n,
-                                                                         p, k, Yr);
+    LV_LAUNCH(launch_pdl(xty_update_kernel<T>, blocks_for((int64_t)n * p), kThreads, 0, s, xty, ld,
+        xtyc, fs, U, n, p, k, Yr));
   return cudaGetLastError();
 }
 

@@ -204,6 +204,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = bars->tmem_base;
+  griddep_wait();  // the factors' split and whatever wrote the view
+  griddep_launch_dependents();
 
   if (warp == 0) {
     // ---------------- producer ----------------
@@ -406,6 +408,8 @@ __global__ void __launch_bounds__(256) tc_split_kernel(const float* __restrict__
                                                        int n, int r, int half,
                                                        float* __restrict__ Acat,
                                                        float* __restrict__ Bcat) {
+  griddep_wait();
+  griddep_launch_dependents();
   __shared__ float su[64][33], sw[64][33];
   const int row0 = blockIdx.x * 32;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 8 warps
@@ -591,6 +595,8 @@ __global__ void __launch_bounds__(TpShape<TR, RP>::Threads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = bars->tmem_base;
+  griddep_wait();  // the factors' split and whatever wrote the view
+  griddep_launch_dependents();
 
   if (warp == 0) {
     // ---------------- producer ----------------
@@ -827,6 +833,8 @@ __global__ void __launch_bounds__(TpShape<TR, RP>::Threads, 1)
 // column-major (column stride fs), n rows.
 __global__ void tp_split_kernel(const float* __restrict__ Fin, int64_t fs, int n, int r, int rp,
                                 float* __restrict__ F) {
+  griddep_wait();
+  griddep_launch_dependents();
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (int64_t)rp * n) return;
   const int c = (int)(idx / n), i = (int)(idx % n);
@@ -877,7 +885,8 @@ static cudaError_t launch_tc_t(const CUtensorMap& tmP, const CUtensorMap& tmA,
   if (configured != cudaSuccess) return configured;
   const long long T = (long long)((n + kBM - 1) / kBM) * ((n + Sh::BN - 1) / Sh::BN);
   const int grid = (int)(T < num_sms ? T : num_sms);
-  tc_update_kernel<RP><<<grid, kTcThreads, Sh::SmemBytes, s>>>(tmP, tmA, tmB, P, ldp, n, status);
+  LV_LAUNCH(launch_pdl(tc_update_kernel<RP>, grid, kTcThreads, Sh::SmemBytes, s, tmP, tmA, tmB, P,
+      ldp, n, status));
   return cudaGetLastError();
 }
 
@@ -887,7 +896,8 @@ cudaError_t launch_tc_update(const CUtensorMap& tmP, const CUtensorMap& tmA,
                              int num_sms, unsigned* status, cudaStream_t s) {
   if (r < 1 || r > kMaxTcR) return cudaErrorInvalidValue;
   const int half = r <= 32 ? 32 : 64;
-  tc_split_kernel<<<(n + 31) / 32, 256, 0, s>>>(U, W, fs, n, r, half, Acat, Bcat);
+  LV_LAUNCH(launch_pdl(tc_split_kernel, (n + 31) / 32, 256, 0, s, U, W, fs, n, r, half, Acat,
+      Bcat));
   if (half == 32) return launch_tc_t<32>(tmP, tmA, tmB, P, ldp, n, num_sms, status, s);
   return launch_tc_t<64>(tmP, tmA, tmB, P, ldp, n, num_sms, status, s);
 }
@@ -918,8 +928,8 @@ static cudaError_t launch_tp_t(const CUtensorMap& tmP, const CUtensorMap& tmF, f
       tc_products_kernel<TR, RP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::SmemBytes);
   if (configured != cudaSuccess) return configured;
   const int grid = (int)tp_grid(n, num_sms);
-  tc_products_kernel<TR, RP><<<grid, Sh::Threads, Sh::SmemBytes, s>>>(tmP, tmF, out, ps, cs, n,
-                                                                     r_out, parts, status);
+  LV_LAUNCH(launch_pdl(tc_products_kernel<TR, RP>, grid, Sh::Threads, Sh::SmemBytes, s, tmP, tmF,
+      out, ps, cs, n, r_out, parts, status));
   return cudaGetLastError();
 }
 
@@ -931,7 +941,8 @@ cudaError_t launch_tc_products(bool transpose, const float* P, int64_t ldp, cons
     return cudaErrorInvalidValue;
   const int rp = r <= 16 ? 16 : (r <= 32 ? 32 : 64);
   const int64_t tot = (int64_t)rp * n;
-  tp_split_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(F, fs, n, r, rp, Fsplit);
+  LV_LAUNCH(launch_pdl(tp_split_kernel, (unsigned)((tot + 255) / 256), 256, 0, s, F, fs, n, r, rp,
+      Fsplit));
   CUtensorMap tmP, tmF;
   // P: boxes of 32 columns x 128 rows (X) or 32 x 32 (Y); F: 32 columns of
   // K x rp factor rows (hi at row 0, lo at row 64)
