@@ -2263,7 +2263,16 @@ static linview_status ols_create(linview_program* p, const void* const* inputs,
   p->part_cs = p->fs;
   const int64_t width = (kk > pp) ? kk : pp;
   p->xp_s = rup(width, kMaxFusedR) * p->part_cs;
-  LV_TRY(dalloc(p, (size_t)g.gC * p->xp_s * p->elem, &p->Xpart, s));
+  // wide blocks (FP32): G = W U on the tensor cores where that is faster (32 columns:
+  // n = 4096 2 + 20 us and 6 sets to sum against 32 and 38 sets; a whole update at
+  // n = 2048 107 -> 99 us, n = 4096 112 -> 98)
+  const bool tp = p->elem == 4 && kk > kMaxProductR && n >= 2048;
+  const int64_t xsets = tp && g.gC < kTpMaxParts ? kTpMaxParts : g.gC;
+  LV_TRY(dalloc(p, (size_t)xsets * p->xp_s * p->elem, &p->Xpart, s));
+  if (tp) {
+    LV_TRY(dalloc(p, sizeof(float) * 128 * p->fs, &t, s));
+    p->tpF = static_cast<float*>(t);
+  }
   // FP32: G = W U by column sums, up to kMaxColSumR columns per pass, one
   // partial per row block
   const int64_t ycols = p->elem == 4 ? rup(kk < kMaxColSumR ? kk : kMaxColSumR, kMaxFusedR)
@@ -2300,36 +2309,47 @@ static linview_status ols_propagate_t(linview_program* p, int kr, cudaStream_t s
   View& w = p->views[kOlsW];
   const PassGeom g = fused_geom(sizeof(T), n, p->sms);
   // U = [X'_R^T, X_R^T]: the old rows become the kr columns after the new ones
-  LV_CUDA(launch_gather_rows<T>(static_cast<const T*>(p->Xd), p->ldX, p->rows_d, kr, n,
-                                U + (int64_t)kr * fs, fs, 1, s));
-  LV_CUDA(launch_gather_rows<T>(static_cast<const T*>(p->Yd), p->ldY, p->rows_d, kr, pp,
-                                static_cast<T*>(p->Yr), pp, 1, s));
-  p->all_launches += 2;
-  // X's rows and X^T Y read only U and Y_R: a side stream, next to the
-  // Woodbury passes and the core, joined before the beta refresh that reads
-  // the new X^T Y
+  LV_CUDA(launch_exchange_rows<T>(static_cast<T*>(p->Xd), p->ldX, static_cast<const T*>(p->Yd),
+                                  p->ldY, p->rows_d, kr, n, pp, U, fs, static_cast<T*>(p->Yr), s));
+  p->all_launches++;
+  // X^T Y reads only U and Y_R: a side stream, next to the Woodbury passes and
+  // the core, which goes on with the beta refresh once Wu is there
+  cudaStream_t side = nullptr;
+  LV_TRY(side_fork(p, s, &side));
   {
-    cudaStream_t side = nullptr;
-    LV_TRY(side_fork(p, s, &side));
-    LV_CUDA(launch_scatter_rows<T>(static_cast<T*>(p->Xd), p->ldX, p->rows_d, kr, n, U, fs,
-                                   side));
     View& xty0 = p->views[kOlsXtY];
     T* xtyl = nullptr;
     if constexpr (sizeof(T) == 4) xtyl = p->XtYl;
     LV_CUDA(launch_xty_update<T>(static_cast<T*>(xty0.ptr), xty0.ld, static_cast<T*>(p->XtYc),
                                  fs, U, n, pp, kr, static_cast<const T*>(p->Yr), side, xtyl));
-    p->all_launches += 2;
+    p->all_launches++;
   }
   if constexpr (sizeof(T) == 4) {
-    // G = W U = W^T U (W is symmetric): column sums of a pass over W, which
-    // need no cross-lane reductions, up to 32 columns per read of W
-    for (int c0 = 0; c0 < kk; c0 += kMaxColSumR) {
-      const int wd = (kk - c0 < kMaxColSumR) ? kk - c0 : kMaxColSumR;
-      LV_TRY(run_fused<T>(p, w, kModeY, wd, nullptr, U + (int64_t)c0 * fs, nullptr, nullptr,
-                          p->Xpart, p->Ypart, s));
+    if (p->tpF && kk > kMaxProductR) {
+      // wide blocks: one tensor-core products pass
+      const int parts = tp_parts(n, p->sms);
+      {
+        ProfScope ps(p, s, (double)n * (double)n * sizeof(float), 1);
+        LV_CUDA(launch_tc_products(false, static_cast<const float*>(w.ptr), w.ld,
+                                   reinterpret_cast<const float*>(U), fs, p->tpF, n, kk,
+                                   static_cast<float*>(p->Xpart), p->xp_s, p->part_cs, parts,
+                                   p->sms, p->status, s));
+        p->all_launches++;  // the split kernel
+      }
       ProfScope ps(p, s, 0.0);
-      LV_CUDA(launch_sum_partials<T>(static_cast<T*>(p->Ypart), g.gR, p->yp_q, p->part_cs, n, wd,
-                                     G + (int64_t)c0 * fs, fs, s));
+      LV_CUDA(launch_sum_partials<T>(static_cast<T*>(p->Xpart), parts, p->xp_s, p->part_cs, n, kk, G,
+                                     fs, s));
+    } else {
+      // G = W U = W^T U (W is symmetric): column sums of a pass over W, which
+      // need no cross-lane reductions, up to 32 columns per read of W
+      for (int c0 = 0; c0 < kk; c0 += kMaxColSumR) {
+        const int wd = (kk - c0 < kMaxColSumR) ? kk - c0 : kMaxColSumR;
+        LV_TRY(run_fused<T>(p, w, kModeY, wd, nullptr, U + (int64_t)c0 * fs, nullptr, nullptr,
+                            p->Xpart, p->Ypart, s));
+        ProfScope ps(p, s, 0.0);
+        LV_CUDA(launch_sum_partials<T>(static_cast<T*>(p->Ypart), g.gR, p->yp_q, p->part_cs, n, wd,
+                                       G + (int64_t)c0 * fs, fs, s));
+      }
     }
   } else {
     // G = W U (row sums, one read of W per 8 columns)
@@ -2353,26 +2373,38 @@ static linview_status ols_propagate_t(linview_program* p, int kr, cudaStream_t s
     else
       LV_CUDA(launch_core_inverse(p->C, kk, kr, p->Minv, p->status, s));
   }
+  // the update W += G Wu^T goes to the tensor cores from 17 columns on
+  const bool presplit = sizeof(T) == 4 && p->tcA && kk > kMaxProductR;
   {
     ProfScope ps(p, s, 0.0);
     if constexpr (sizeof(T) == 4)
-      LV_CUDA(launch_wu(G, fs, n, kk, reinterpret_cast<const float2*>(p->Minv), Wu, s));
+      LV_CUDA(launch_wu(G, fs, n, kk, reinterpret_cast<const float2*>(p->Minv), Wu,
+                        presplit ? p->tcA : nullptr, presplit ? p->tcB : nullptr, s));
     else
       LV_CUDA(launch_wu(G, fs, n, kk, p->Minv, Wu, s));
   }
-  // W' = W + G Wu^T = W - G M^{-1} G^T
-  LV_TRY(run_update<T>(p, w, G, Wu, kk, s));
-  LV_TRY(side_join(p, s));  // the new X rows and X^T Y
-  // beta' = beta + (G_1 - G_2) Y_R + G (Wu^T C'): from the factors, no pass over W
+  // beta' = beta + (G_1 - G_2) Y_R + G (Wu^T C'): from the factors, no pass over
+  // W, so it runs beside W' = W + G Wu^T = W - G M^{-1} G^T (14 us at 2k = 32)
+  LV_CUDA(cudaEventRecord(p->side_fork_ev, s));
+  LV_CUDA(cudaStreamWaitEvent(side, p->side_fork_ev, 0));
   View& beta = p->views[kOlsBeta];
   {
-    ProfScope ps(p, s, 0.0);
+    ProfScope ps(p, side, 0.0);
     LV_CUDA(launch_beta_update<T>(static_cast<T*>(beta.ptr), beta.ld, G, Wu,
                                   static_cast<const T*>(p->XtYc), fs, n, pp, kr,
-                                  static_cast<const T*>(p->Yr), static_cast<T*>(p->Hols), s));
+                                  static_cast<const T*>(p->Yr), static_cast<T*>(p->Hols), side));
   }
   p->all_launches += 2;
-  return LINVIEW_OK;
+  if (presplit) {
+    ProfScope ps(p, s, 2.0 * (double)n * (double)n * sizeof(T), 2);
+    LV_CUDA(launch_tc_update(w.tmap_tc, p->tmA, p->tmB, static_cast<float*>(w.ptr), w.ld, p->tcA,
+                             p->tcB, reinterpret_cast<const float*>(G),
+                             reinterpret_cast<const float*>(Wu), fs, n, kk, p->sms, p->status, s,
+                             /*presplit=*/true));
+  } else {
+    LV_TRY(run_update<T>(p, w, G, Wu, kk, s));
+  }
+  return side_join(p, s);  // X^T Y and beta
 }
 
 // Z += X'_R^T X'_R - X_R^T X_R for the Newton-Schulz correction, deferred:

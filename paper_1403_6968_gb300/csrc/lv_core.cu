@@ -344,7 +344,7 @@ __global__ void __launch_bounds__(kThreads) assemble_kernel(const AssembleParams
 // itself (CTA = 256 rows of one column; the C_h column is summed once per
 // CTA).  Same fixed orders as above within a thread's sums.  Small views have few
 // outputs and many row ranges (n = 1000: 127 partial sets): below n = 4096 with more
-// than 24 sets the warps of a CTA share them (n = 1000, 12 columns: 15.5 -> ASM_NEW us).
+// than 24 sets the warps of a CTA share them (n = 1000, 12 columns: 15.5 -> 7 us).
 template <typename T>
 __global__ void __launch_bounds__(kThreads) assemble_wide_kernel(const AssembleParams a) {
   __shared__ T Cc[kMaxAsmR];
@@ -562,12 +562,50 @@ __global__ void sum_partials_f32_kernel(const float* part, int blocks, int64_t b
   out[(int64_t)c * ocs + j] = __fadd_rn(hi, lo);
 }
 
+// The same sums with many sets: a CTA takes 32 rows of one column and its warps share
+// the sets (warp w those congruent to w mod 8, then the warps in order), so the chain
+// of dependent load rounds is an eighth (128 sets of 8 columns, n = 1024: 6.8 -> 3.5 us).
+__global__ void __launch_bounds__(kThreads)
+    sum_partials_shared_kernel(const float* part, int blocks, int64_t bs, int64_t cs, int n,
+                               float* out, int64_t ocs) {
+  griddep_wait();
+  griddep_launch_dependents();
+  __shared__ float2 ps[kThreads];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int j = blockIdx.x * 32 + lane, c = blockIdx.y;
+  float hi = 0.f, lo = 0.f;
+  if (j < n) {
+    const float* src = part + (int64_t)c * cs + j;
+    for (int b0 = w; b0 < blocks; b0 += 64) {  // eight loads in flight, added in order
+      float x[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) x[i] = b0 + 8 * i < blocks ? src[(int64_t)(b0 + 8 * i) * bs] : 0.f;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) df_add(hi, lo, x[i], 0.f);
+    }
+  }
+  ps[threadIdx.x] = make_float2(hi, lo);
+  __syncthreads();
+  if (w != 0 || j >= n) return;
+#pragma unroll
+  for (int i = 1; i < kThreads / 32; ++i) {
+    const float2 x = ps[32 * i + lane];
+    df_add(hi, lo, x.x, x.y);
+  }
+  out[(int64_t)c * ocs + j] = __fadd_rn(hi, lo);
+}
+
 template <typename T>
 cudaError_t launch_sum_partials(const T* part, int blocks, int64_t block_stride, int64_t cs, int n,
                                 int r, T* out, int64_t out_cs, cudaStream_t s) {
   const int64_t tot = (int64_t)n * r;
   if (tot == 0) return cudaSuccess;
   const unsigned grid = (unsigned)((tot + kThreads - 1) / kThreads);
+  if constexpr (sizeof(T) == 4) {
+    if (blocks >= 12)
+      return launch_pdl(sum_partials_shared_kernel, dim3((unsigned)((n + 31) / 32), (unsigned)r),
+                        kThreads, 0, s, part, blocks, block_stride, cs, n, out, out_cs);
+  }
   if constexpr (sizeof(T) == 4)
     LV_LAUNCH(launch_pdl(sum_partials_f32_kernel, grid, kThreads, 0, s, part, blocks, block_stride,
         cs, n, r, out, out_cs));

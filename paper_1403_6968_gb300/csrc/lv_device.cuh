@@ -189,6 +189,19 @@ __device__ __forceinline__ void split_index(int64_t idx, int d, int& q, int& r) 
   }
 }
 
+// Columns c0 .. c0 + 3 of row i of a split factor of the tensor-core update pass
+// (128 columns: hi = the top 19 bits in 0 .. 63, lo in 64 .. 127).
+__device__ __forceinline__ void tc_split_store4(float* cat, int64_t i, int c0,
+                                                const float (&x)[4]) {
+  float h[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) h[q] = __uint_as_float(__float_as_uint(x[q]) & 0xFFFFE000u);
+  float* d = cat + i * 128 + c0;
+  *reinterpret_cast<float4*>(d) = make_float4(h[0], h[1], h[2], h[3]);
+  *reinterpret_cast<float4*>(d + 64) =
+      make_float4(x[0] - h[0], x[1] - h[1], x[2] - h[2], x[3] - h[3]);
+}
+
 // Programmatic dependent launch: a kernel launched with programmatic stream
 // serialisation may start while the kernel before it drains; griddep_wait()
 // blocks until that kernel has completed and its writes are visible, and

@@ -122,14 +122,15 @@ inline int tp_min_r(int64_t n) { return n >= 3500 ? kMaxFusedR : kMaxProductR; }
 // partial sets the products pass writes for an n x n view (<= kTpMaxParts)
 int tp_parts(int n, int num_sms);
 // Tensor-core update pass P += U W^T (FP32 view, 17 <= r <= 64 factor
-// columns, split TF32): splits U, W into the scratch, then one persistent
+// columns, split TF32): splits U, W into the scratch (presplit: already there), then one persistent
 // launch over 128 x 64 tiles.  tmP:
 // make_tmap_sw128 over the view P (box rows 128, row stride ldp); tmA / tmB:
 // over A_cat (128 columns, box rows 128) / B_cat (128 columns, box rows 32).
 cudaError_t launch_tc_update(const CUtensorMap& tmP, const CUtensorMap& tmA,
                              const CUtensorMap& tmB, float* P, int64_t ldp, float* Acat,
                              float* Bcat, const float* U, const float* W, int64_t fs, int n, int r,
-                             int num_sms, unsigned* status, cudaStream_t s);
+                             int num_sms, unsigned* status, cudaStream_t s,
+                             bool presplit = false);
 
 // Own dense GEMMs (lv_gemm.cu).
 // A split operand of the tensor-core GEMM: element (i, k) of op(X) at X[i * rs +
@@ -301,12 +302,11 @@ cudaError_t launch_panel_sum(const T* A, int64_t lda, T* out, int64_t ldo, int n
                              cudaStream_t s);
 
 // OLS pieces (lv_ols.cu).
+// Row block exchange: U's column k + t = the old row rows[t] of X, X takes U's column t
+// (the new row), Yr's row t = the row rows[t] of Y.
 template <typename T>
-cudaError_t launch_gather_rows(const T* X, int64_t ldx, const int64_t* rows, int k, int n, T* dst,
-                               int64_t ts, int64_t js, cudaStream_t s);
-template <typename T>
-cudaError_t launch_scatter_rows(T* X, int64_t ldx, const int64_t* rows, int k, int n,
-                                const T* src, int64_t ts, cudaStream_t s);
+cudaError_t launch_exchange_rows(T* X, int64_t ldx, const T* Y, int64_t ldy, const int64_t* rows,
+                                 int k, int n, int p, T* U, int64_t fs, T* Yr, cudaStream_t s);
 // Minv = (diag(+1 x kpos, -1 x (kk - kpos)) + S)^{-1}, kk <= 64: FP64
 // programs in FP64 (S and Minv kk x kk doubles); FP32 programs in
 // double-float on the FP32 pipe (S and Minv kk x kk float2 pairs).
@@ -317,8 +317,9 @@ cudaError_t launch_core_inverse_df(const float2* S, int kk, int kpos, float2* Mi
 // Wu = -G Minv (FP64 core for double views, double-float core for float views)
 cudaError_t launch_wu(const double* G, int64_t fs, int n, int kk, const double* Minv, double* Wu,
                       cudaStream_t s);
+// (Acat, Bcat: also the split of G and Wu for launch_tc_update's presplit form; may be null)
 cudaError_t launch_wu(const float* G, int64_t fs, int n, int kk, const float2* Minv, float* Wu,
-                      cudaStream_t s);
+                      float* Acat, float* Bcat, cudaStream_t s);
 // Newton-Schulz correction of FP32 OLS programs: Z = X^T X as double-float
 // pairs (Zh, Zl; n x n, row-major ldz, a multiple of 64 with zero padding)
 cudaError_t launch_z_from_lower(const double* L, int64_t ldl, int n, float* Zh, float* Zl,

@@ -21,31 +21,41 @@
 
 namespace lv {
 
-// dst[t * ts + j * js] = X[rows[t] * ldx + j]
+// A row block's exchange in one launch: the old row rows[t] of X becomes column k + t of
+// U (its column t holds the new row), X takes the new row, and row rows[t] of Y goes to
+// Yr.  Every element of X is read and written by one thread (the rows are distinct).
 template <typename T>
-__global__ void gather_rows_kernel(const T* X, int64_t ldx, const int64_t* rows, int k, int n,
-                                   T* dst, int64_t ts, int64_t js) {
+__global__ void exchange_rows_kernel(T* X, int64_t ldx, const T* Y, int64_t ldy,
+                                     const int64_t* rows, int k, int n, int p, T* U, int64_t fs,
+                                     T* Yr) {
   griddep_wait();
   griddep_launch_dependents();
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (int64_t)k * n) return;
   int t, j;
-  split_index(idx, n, t, j);
-  dst[t * ts + j * js] = X[rows[t] * ldx + j];
+  if (idx < (int64_t)k * n) {
+    split_index(idx, n, t, j);
+    T* x = X + rows[t] * ldx + j;
+    U[(int64_t)(k + t) * fs + j] = *x;
+    *x = U[(int64_t)t * fs + j];
+  } else if (idx < (int64_t)k * (n + p)) {
+    split_index(idx - (int64_t)k * n, p, t, j);
+    Yr[(int64_t)t * p + j] = Y[rows[t] * ldy + j];
+  }
 }
 
-// X[rows[t] * ldx + j] = src[t * ts + j]
 template <typename T>
-__global__ void scatter_rows_kernel(T* X, int64_t ldx, const int64_t* rows, int k, int n,
-                                    const T* src, int64_t ts) {
-  griddep_wait();
-  griddep_launch_dependents();
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (int64_t)k * n) return;
-  int t, j;
-  split_index(idx, n, t, j);
-  X[rows[t] * ldx + j] = src[t * ts + j];
+cudaError_t launch_exchange_rows(T* X, int64_t ldx, const T* Y, int64_t ldy, const int64_t* rows,
+                                 int k, int n, int p, T* U, int64_t fs, T* Yr, cudaStream_t s) {
+  const int64_t tot = (int64_t)k * (n + p);
+  return launch_pdl(exchange_rows_kernel<T>, (unsigned)((tot + kThreads - 1) / kThreads), kThreads,
+                    0, s, X, ldx, Y, ldy, rows, k, n, p, U, fs, Yr);
 }
+template cudaError_t launch_exchange_rows<float>(float*, int64_t, const float*, int64_t,
+                                                 const int64_t*, int, int, int, float*, int64_t,
+                                                 float*, cudaStream_t);
+template cudaError_t launch_exchange_rows<double>(double*, int64_t, const double*, int64_t,
+                                                  const int64_t*, int, int, int, double*, int64_t,
+                                                  double*, cudaStream_t);
 
 // Minv = (diag(c) + S)^{-1} for the kk x kk FP64 matrix S (row-major, kk <=
 // 64) with c = (+1 x kpos, -1 x (kk - kpos)): Gauss-Jordan elimination with
@@ -523,9 +533,12 @@ __global__ void wu_f64_kernel(const double* G, int64_t fs, int n, int kk, const 
 // FP32 G entry and a core pair is accumulated as a pair (df_acc) and the sum
 // is rounded once to FP32.  A thread computes four columns c = 4 blockIdx.y
 // .. + 3 of one row j (kk is even; a trailing pair is masked).
+// With Acat, the factors also go to the split rows of the tensor-core update (G to Acat,
+// Wu to Bcat; the grid covers its 32 or 64 columns, zero past kk): one launch less on
+// the chain.
 constexpr int kWuCols = 4;
 __global__ void wu_df_kernel(const float* G, int64_t fs, int n, int kk, const float2* Minv,
-                             float* Wu) {
+                             float* Wu, float* Acat, float* Bcat) {
   griddep_wait();
   griddep_launch_dependents();
   __shared__ df2 ms[64][kWuCols];
@@ -541,14 +554,30 @@ __global__ void wu_df_kernel(const float* G, int64_t fs, int n, int kk, const fl
   df2 acc[kWuCols];
 #pragma unroll
   for (int q = 0; q < kWuCols; ++q) acc[q] = {0.f, 0.f};
-  for (int c2 = 0; c2 < kk; ++c2) {
-    const float g = G[(int64_t)c2 * fs + j];
+  for (int c2 = 0; c2 < kk; c2 += 8) {  // eight loads in flight
+    float g[8];
 #pragma unroll
-    for (int q = 0; q < kWuCols; ++q) df_acc(acc[q], ms[c2][q], g);
+    for (int u = 0; u < 8; ++u) g[u] = c2 + u < kk ? G[(int64_t)(c2 + u) * fs + j] : 0.f;
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (c2 + u < kk) {
+#pragma unroll
+        for (int q = 0; q < kWuCols; ++q) df_acc(acc[q], ms[c2 + u][q], g[u]);
+      }
   }
+  float w[kWuCols];
 #pragma unroll
-  for (int q = 0; q < kWuCols; ++q)
-    if (c0 + q < kk) Wu[(int64_t)(c0 + q) * fs + j] = __fadd_rn(acc[q].hi, acc[q].lo);
+  for (int q = 0; q < kWuCols; ++q) {
+    w[q] = c0 + q < kk ? __fadd_rn(acc[q].hi, acc[q].lo) : 0.f;
+    if (c0 + q < kk) Wu[(int64_t)(c0 + q) * fs + j] = w[q];
+  }
+  if (Acat) {
+    float g[kWuCols];
+#pragma unroll
+    for (int q = 0; q < kWuCols; ++q) g[q] = c0 + q < kk ? G[(int64_t)(c0 + q) * fs + j] : 0.f;
+    tc_split_store4(Acat, j, c0, g);
+    tc_split_store4(Bcat, j, c0, w);
+  }
 }
 
 // X^T Y += (X'_R - X_R)^T Y_R.  U holds X'_R^T in columns [0, k) and X_R^T in
@@ -928,24 +957,6 @@ __global__ void from_double_kernel(const double* src, int64_t lds, T* dst, int64
 
 static unsigned blocks_for(int64_t tot) { return (unsigned)((tot + kThreads - 1) / kThreads); }
 
-template <typename T>
-cudaError_t launch_gather_rows(const T* X, int64_t ldx, const int64_t* rows, int k, int n, T* dst,
-                               int64_t ts, int64_t js, cudaStream_t s) {
-  if ((int64_t)k * n == 0) return cudaSuccess;
-  LV_LAUNCH(launch_pdl(gather_rows_kernel<T>, blocks_for((int64_t)k * n), kThreads, 0, s, X, ldx,
-      rows, k, n, dst, ts, js));
-  return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t launch_scatter_rows(T* X, int64_t ldx, const int64_t* rows, int k, int n,
-                                const T* src, int64_t ts, cudaStream_t s) {
-  if ((int64_t)k * n == 0) return cudaSuccess;
-  LV_LAUNCH(launch_pdl(scatter_rows_kernel<T>, blocks_for((int64_t)k * n), kThreads, 0, s, X, ldx,
-      rows, k, n, src, ts));
-  return cudaGetLastError();
-}
-
 cudaError_t launch_core_inverse(const double* S, int kk, int kpos, double* Minv, unsigned* status,
                                 cudaStream_t s) {
   if (kk < 1 || kk > 64) return cudaErrorInvalidValue;
@@ -979,10 +990,11 @@ cudaError_t launch_wu(const double* G, int64_t fs, int n, int kk, const double* 
 }
 
 cudaError_t launch_wu(const float* G, int64_t fs, int n, int kk, const float2* Minv, float* Wu,
-                      cudaStream_t s) {
+                      float* Acat, float* Bcat, cudaStream_t s) {
   if (kk < 2 || kk > 64 || (kk & 1)) return cudaErrorInvalidValue;
-  LV_LAUNCH(launch_pdl(wu_df_kernel, dim3(blocks_for(n), (kk + kWuCols - 1) / kWuCols), kThreads, 0,
-      s, G, fs, n, kk, Minv, Wu));
+  const int cols = Acat ? (kk <= 32 ? 32 : 64) : kk;
+  LV_LAUNCH(launch_pdl(wu_df_kernel, dim3(blocks_for(n), (cols + kWuCols - 1) / kWuCols), kThreads,
+                       0, s, G, fs, n, kk, Minv, Wu, Acat, Bcat));
   return cudaGetLastError();
 }
 
@@ -1035,10 +1047,6 @@ cudaError_t launch_from_double(const double* src, int64_t lds, T* dst, int64_t l
 }
 
 #define LV_OLS_INST(T)                                                                           \
-  template cudaError_t launch_gather_rows<T>(const T*, int64_t, const int64_t*, int, int, T*,     \
-                                             int64_t, int64_t, cudaStream_t);                    \
-  template cudaError_t launch_scatter_rows<T>(T*, int64_t, const int64_t*, int, int, const T*,    \
-                                              int64_t, cudaStream_t);                            \
   template cudaError_t launch_beta_update<T>(T*, int64_t, const T*, const T*, const T*, int64_t,  \
                                              int, int, int, const T*, T*, cudaStream_t);         \
   template cudaError_t launch_xty_update<T>(T*, int64_t, T*, int64_t, const T*, int, int, int,    \

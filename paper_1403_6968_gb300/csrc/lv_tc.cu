@@ -893,10 +893,11 @@ static cudaError_t launch_tc_t(const CUtensorMap& tmP, const CUtensorMap& tmA,
 cudaError_t launch_tc_update(const CUtensorMap& tmP, const CUtensorMap& tmA,
                              const CUtensorMap& tmB, float* P, int64_t ldp, float* Acat,
                              float* Bcat, const float* U, const float* W, int64_t fs, int n, int r,
-                             int num_sms, unsigned* status, cudaStream_t s) {
+                             int num_sms, unsigned* status, cudaStream_t s, bool presplit) {
   if (r < 1 || r > kMaxTcR) return cudaErrorInvalidValue;
   const int half = r <= 32 ? 32 : 64;
-  LV_LAUNCH(launch_pdl(tc_split_kernel, (n + 31) / 32, 256, 0, s, U, W, fs, n, r, half, Acat,
+  if (!presplit)
+    LV_LAUNCH(launch_pdl(tc_split_kernel, (n + 31) / 32, 256, 0, s, U, W, fs, n, r, half, Acat,
       Bcat));
   if (half == 32) return launch_tc_t<32>(tmP, tmA, tmB, P, ldp, n, num_sms, status, s);
   return launch_tc_t<64>(tmP, tmA, tmB, P, ldp, n, num_sms, status, s);
