@@ -180,8 +180,8 @@ struct linview_program {
   // persistent split operands of the tensor-core GEMM
   void* gwork = nullptr;
   int64_t gwork_elems = 0;
-  float* hyA = nullptr;  // split rows of the old A (n x tc_split_ld(n))
-  float* hyB = nullptr;  // split rows of D_{i-1}^T (p x tc_split_ld(n))
+  float* hyA = nullptr;  // split blocks of the old A
+  float* hyB = nullptr;  // split blocks of D_{i-1}^T
   unsigned* hyW = nullptr;  // ... and their words (tc_words(n, p, n))
   float* hyP = nullptr;     // ... and the pieces of its cut tiles
   // OLS: X (m x n), Y (m x p) on the device; views W, beta, X^T Y, X
@@ -709,9 +709,8 @@ static int64_t tc_words(int64_t a_rows, int64_t b_rows, int64_t K) {
 static linview_status tc_scratch(linview_program* p, TcScratch* sc, int64_t a_rows, int64_t b_rows,
                                  int64_t K, cudaStream_t s) {
   if (p->elem != 4 || a_rows < 128) return LINVIEW_OK;  // such products run on the CUDA cores
-  const int64_t ld = tc_split_ld(K);
-  const size_t abytes = (size_t)alloc_bytes(a_rows * ld * 4);
-  const size_t bbytes = (size_t)alloc_bytes(b_rows * ld * 4);
+  const size_t abytes = (size_t)alloc_bytes(tc_operand_floats(a_rows, K) * 4);
+  const size_t bbytes = (size_t)alloc_bytes(tc_operand_floats(b_rows, K) * 4);
   const size_t wbytes = (size_t)alloc_bytes(tc_words(a_rows, b_rows, K) * 4);
   sc->work_floats = tc_work_floats(a_rows, b_rows, K, p->sms);
   const size_t bytes = abytes + bbytes + wbytes + (size_t)sc->work_floats * 4;
@@ -1500,9 +1499,9 @@ static linview_status iter_create(linview_program* p, const void* const* inputs,
     LV_TRY(dalloc(p, (size_t)2 * n * p->ldD * p->elem, &p->Dh, s));
     if (p->elem == 4 && n >= 128 && pp > kMaxFusedR) {  // products A D_{i-1} on the tensor cores
       void* t = nullptr;
-      LV_TRY(dalloc(p, (size_t)n * tc_split_ld(n) * 4, &t, s));
+      LV_TRY(dalloc(p, (size_t)tc_operand_floats(n, n) * 4, &t, s));
       p->hyA = static_cast<float*>(t);
-      LV_TRY(dalloc(p, (size_t)pp * tc_split_ld(n) * 4, &t, s));
+      LV_TRY(dalloc(p, (size_t)tc_operand_floats(pp, n) * 4, &t, s));
       p->hyB = static_cast<float*>(t);
       LV_TRY(dalloc(p, (size_t)tc_words(n, pp, n) * 4, &t, s));
       p->hyW = static_cast<unsigned*>(t);

@@ -20,8 +20,11 @@
 //    the exponent's comfortable range, or that hold infinities or NaN are found
 //    while they are split, and such a product runs on TF32 halves instead (same
 //    kernel, kind::tf32; hi = x rounded to nearest
-//    TF32, lo = x - hi rounded in turn).  Operands are K-major rows [hi | lo]
-//    (the split also transposes where the product needs the other layout).
+//    TF32, lo = x - hi rounded in turn).  Operands are stored in blocks of 128 rows x
+//    one K chunk, [hi | lo] of 16 KB each, rows of 128 bytes (the split also transposes
+//    where the product needs the other layout): a chunk of a CTA's A is one copy of
+//    32 contiguous KB (as rows [hi | lo] of length K every box line was 128 bytes 32 KB
+//    apart, and 8192 x 64 x 8192, which streams A from memory, took 57 us, 53 now; 8192 x 8192 x 1024 328 -> 316).
 //    CTA pairs (cta_group::2) compute tiles of 256 x BN outputs (BN = 256, 128 or
 //    64), each CTA holding 128 rows of A and half of B's rows, in K chunks of
 //    one 128-byte swizzle atom (64 FP16 or 32 TF32 values); a persistent grid
@@ -269,8 +272,8 @@ struct GArgs {
   unsigned* status;
 };
 
-// D (M x N, row-major, ldd) = alpha A B^T + beta C over the split rows [hi | lo]
-// (FP16: halves kp16 long; TF32: kp32 long).
+// D (M x N, row-major, ldd) = alpha A B^T + beta C over the split blocks of K = kp16
+// (FP16) or kp32 (TF32) values.
 template <int BN>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GShape<BN>::Threads, 1)
     tc_gemm_kernel(const __grid_constant__ GMaps maps, const GArgs a) {
@@ -343,18 +346,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GShape<BN>::Threads,
       while (!*abort_flag && work.next()) {
         int mb, nb;
         g_tile(work.tile, mt, nt, mb, nb);
-        const int arow = mb * kGBM + (int)rank * 128, brow = nb * BN + (int)rank * (BN / 2);
+        // 256 lines of 128 bytes per block: hi of 128 rows, then lo
+        const int aline = (mb * 2 + (int)rank) * nk * 256;
+        const int brow = nb * BN + (int)rank * (BN / 2);
+        const int bline = (brow >> 7) * nk * 256 + (brow & 127);
         for (int kc = work.kb; kc < work.ke; ++kc, ++loaded) {
           if (loaded >= S && !g_wait(&bars->empty[st], phase ^ 1u, abort_flag, status)) break;
-          const int x = chunk(kc) * kc_len;
+          const int line = chunk(kc) * 256;
           unsigned char* sb = base + st * Sh::StageBytes;
           // the first CTA's barrier counts both CTAs' bytes
           const uint32_t fb = lead_full + st * 8;
           if (rank == 0) mbar_arrive_expect_tx(&bars->full[st], 2 * Sh::StageBytes);
-          g_tma(sb, ma, x, arow, fb);
-          g_tma(sb + Sh::AHalf, ma, kp + x, arow, fb);
-          g_tma(sb + 2 * Sh::AHalf, mb_, x, brow, fb);
-          g_tma(sb + 2 * Sh::AHalf + Sh::BHalf, mb_, kp + x, brow, fb);
+          g_tma(sb, ma, 0, aline + line, fb);
+          g_tma(sb + 2 * Sh::AHalf, mb_, 0, bline + line, fb);
+          if (BN < 256) g_tma(sb + 2 * Sh::AHalf + Sh::BHalf, mb_, 0, bline + line + 128, fb);
           if (++st == S) {
             st = 0;
             phase ^= 1u;
@@ -578,8 +583,13 @@ struct SplitPair {
   unsigned* flag;
 };
 
-// FP16 halves: tiles of 64 rows x 128 k (two runs), rows of 2 kp halves [hi | lo]
-// (kp = rup(K, 64), zero past K), one pass over the operand: eight lanes hold a
+// line (of 128 bytes) of row i in the block of chunk kc of nk: its hi half; lo lies 128
+// lines on
+__device__ __forceinline__ int64_t block_line(int i, int kc, int nk) {
+  return ((int64_t)(i >> 7) * nk + kc) * 256 + (i & 127);
+}
+
+// FP16 halves: tiles of 64 rows x 128 k (two runs), zero past K (kp = rup(K, 64)), one pass over the operand: eight lanes hold a
 // run and find its largest entry by shuffles.  An entry y = 2^sh x with 0 < |y| <
 // 2^-2 has fewer than 22 bits; eight of them among 32 neighbours of a row or of a
 // column of a tile (dense data without such structure has none), a scale outside
@@ -669,9 +679,9 @@ __global__ void __launch_bounds__(256) split_f16_kernel(const __grid_constant__ 
       }
     }
     if (in) {
-      __half* d = reinterpret_cast<__half*>(o.dst) + (int64_t)i * 2 * kp + k;
+      unsigned char* d = o.dst + block_line(i, k / 64, kp / 64) * 128 + k % 64 * 2;
       *reinterpret_cast<uint4*>(d) = *reinterpret_cast<const uint4*>(hi);
-      *reinterpret_cast<uint4*>(d + kp) = *reinterpret_cast<const uint4*>(lo);
+      *reinterpret_cast<uint4*>(d + 16384) = *reinterpret_cast<const uint4*>(lo);
       if (kl % 64 == 0) o.sc[(int64_t)(k / 64) * o.pitch + i] = pow2f(-sh);
     }
   }
@@ -681,8 +691,8 @@ __global__ void __launch_bounds__(256) split_f16_kernel(const __grid_constant__ 
 }
 
 // TF32 halves, only when the flag is set (else the kernel returns at once) and
-// the buffer does not hold them already: rows of 2 kp floats [hi | lo], kp =
-// rup(K, 32).  32 x 32 tiles through shared memory, read along whichever source
+// the buffer does not hold them already (kp = rup(K, 32), zero past K).
+// 32 x 32 tiles through shared memory, read along whichever source
 // index has unit stride.
 __global__ void __launch_bounds__(256) split_tf32_kernel(const __grid_constant__ SplitPair sp) {
   griddep_wait();
@@ -715,9 +725,9 @@ __global__ void __launch_bounds__(256) split_tf32_kernel(const __grid_constant__
         // 13-bit field, then clear it; x - hi is exact
         const float hi = __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xFFFFE000u);
         const float r = x - hi;
-        float* d = reinterpret_cast<float*>(o.dst) + (int64_t)i * 2 * kp;
-        d[k] = hi;
-        d[kp + k] = __uint_as_float((__float_as_uint(r) + 0x1000u) & 0xFFFFE000u);
+        float* d = reinterpret_cast<float*>(o.dst + block_line(i, k / 32, kp / 32) * 128) + k % 32;
+        d[0] = hi;
+        d[4096] = __uint_as_float((__float_as_uint(r) + 0x1000u) & 0xFFFFE000u);
       }
     }
   }
@@ -911,8 +921,9 @@ cudaError_t launch_tc_gemm_t(const GMaps& maps, const GArgs& a, int num_sms, cud
   return launch_pdl(gemm_parts_kernel<BN>, dim3(tiles - a.dp, kGBM / 16), 256, 0, s, a, tiles);
 }
 
-// FP16 operand rows [hi | lo]: 64-value boxes (128 bytes), 128-byte swizzle
-bool make_tmap_f16(CUtensorMap* out, const void* base, int64_t cols, int64_t rows, int box_rows) {
+// A split operand as lines of 128 bytes (64 FP16 or 32 TF32 values), boxes of
+// box_lines contiguous lines, 128-byte swizzle
+bool make_tmap_lines(CUtensorMap* out, const void* base, bool f16, int64_t lines, int box_lines) {
   static const PFN_cuTensorMapEncodeTiled_v12000 encode = []() {
     cudaDriverEntryPointQueryResult q;
     void* fn = nullptr;
@@ -923,12 +934,13 @@ bool make_tmap_f16(CUtensorMap* out, const void* base, int64_t cols, int64_t row
     return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
   }();
   if (!encode) return false;
-  cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-  cuuint64_t strides[1] = {(cuuint64_t)(cols * 2)};
-  cuuint32_t box[2] = {64u, (cuuint32_t)box_rows};
+  cuuint64_t dims[2] = {f16 ? 64u : 32u, (cuuint64_t)lines};
+  cuuint64_t strides[1] = {128u};
+  cuuint32_t box[2] = {f16 ? 64u : 32u, (cuuint32_t)box_lines};
   cuuint32_t estr[2] = {1, 1};
-  return encode(out, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void*>(base), dims, strides,
-                box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+  return encode(out, f16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2,
+                const_cast<void*>(base), dims, strides, box, estr,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                 CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -985,7 +997,9 @@ void gemm_plan(int M, int N, int nk, int num_sms, int64_t work_floats, GArgs& a,
 
 }  // namespace
 
-int64_t tc_split_ld(int64_t K) { return 2 * ((K + 31) / 32 * 32); }
+int64_t tc_operand_floats(int64_t rows, int64_t K) {
+  return (rows + 127) / 128 * 128 * 2 * ((K + 31) / 32 * 32);
+}
 int64_t tc_work_floats(int64_t a_rows, int64_t b_rows, int64_t K, int num_sms) {
   const int64_t pairs = num_sms / 2, nk = (K + 63) / 64;
   int64_t most = 0;
@@ -1009,7 +1023,7 @@ cudaError_t launch_tc_split(const TcOperand* a, const TcOperand* b, unsigned* fl
   for (int w = 0; w < 2; ++w) {
     if (!in[w]) continue;
     if (in[w]->rows <= 0 || in[w]->K <= 0) return cudaErrorInvalidValue;
-    // TMA sources (rows are 128-byte multiples) and 128-bit loads of the factors
+    // TMA sources and 128-bit loads of the factors
     if ((reinterpret_cast<uintptr_t>(in[w]->buf) | reinterpret_cast<uintptr_t>(in[w]->words)) & 15)
       return cudaErrorInvalidValue;
     sp.o[w] = split_op(in[w]);
@@ -1035,15 +1049,18 @@ cudaError_t launch_tc_gemm(const TcOperand& a, const TcOperand& b, unsigned* fla
   g.M = M;
   g.N = N;
   g.kp16 = (K + 63) / 64 * 64;
-  g.kp32 = (int)(tc_split_ld(K) / 2);
+  g.kp32 = (K + 31) / 32 * 32;
   int bn = 256;
   gemm_plan(M, N, g.kp16 / 64, num_sms, work ? work_floats : 0, g, &bn);
   g.reverse = reverse ? 1 : 0;
   GMaps maps;
-  if (!make_tmap_f16(&maps.a16, a.buf, 2 * g.kp16, M, 128) ||
-      !make_tmap_f16(&maps.b16, b.buf, 2 * g.kp16, N, bn / 2) ||
-      !make_tmap_sw128(&maps.a32, a.buf, 2 * g.kp32, M, 2 * g.kp32, 128) ||
-      !make_tmap_sw128(&maps.b32, b.buf, 2 * g.kp32, N, 2 * g.kp32, bn / 2))
+  const int64_t ab = (M + 127) / 128 * 256, bb = (N + 127) / 128 * 256;  // lines per chunk
+  const int nk16 = g.kp16 / 64, nk32 = g.kp32 / 32, bl = bn == 256 ? 256 : bn / 2;
+  if (ab * nk32 > INT32_MAX || bb * nk32 > INT32_MAX) return cudaErrorInvalidValue;
+  if (!make_tmap_lines(&maps.a16, a.buf, true, ab * nk16, 256) ||
+      !make_tmap_lines(&maps.b16, b.buf, true, bb * nk16, bl) ||
+      !make_tmap_lines(&maps.a32, a.buf, false, ab * nk32, 256) ||
+      !make_tmap_lines(&maps.b32, b.buf, false, bb * nk32, bl))
     return cudaErrorInvalidValue;
   const bool c_used = C != nullptr && beta != 0.f;
   g.D = D;

@@ -134,8 +134,8 @@ cudaError_t launch_tc_update(const CUtensorMap& tmP, const CUtensorMap& tmA,
 
 // Own dense GEMMs (lv_gemm.cu).
 // A split operand of the tensor-core GEMM: element (i, k) of op(X) at X[i * rs +
-// k * cs] (rs or cs == 1), its split rows in ``buf`` (rows x tc_split_ld(K) floats,
-// 16-byte aligned; FP16 rows take half of it) and in ``words`` (tc_split_words(rows,
+// k * cs] (rs or cs == 1), its split blocks in ``buf`` (tc_operand_floats(rows,
+// K) floats, 16-byte aligned; FP16 halves take half of it) and in ``words`` (tc_split_words(rows,
 // K), 16-byte aligned) the buffer's format and the factors of its runs.  X stays
 // readable for as long as products use the split: a product that has to fall back
 // to TF32 splits it again.
@@ -146,7 +146,7 @@ struct TcOperand {
   float* buf;
   unsigned* words;
 };
-int64_t tc_split_ld(int64_t K);
+int64_t tc_operand_floats(int64_t rows, int64_t K);
 int64_t tc_split_words(int64_t rows, int64_t K);
 // floats of ``work`` below that let every product with up to these sizes cut tiles
 int64_t tc_work_floats(int64_t a_rows, int64_t b_rows, int64_t K, int num_sms);
