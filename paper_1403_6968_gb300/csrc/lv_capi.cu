@@ -143,6 +143,8 @@ struct linview_program {
   void* Ypart = nullptr;
   int64_t part_cs = 0, xp_s = 0, yp_q = 0;
   double* Cpart = nullptr;
+  double* Cpart2 = nullptr;  // exponential / skip iteration: X_j^T V_h's (its own stream)
+  void* Spart = nullptr;     // ... and the partial sums of S' U_b
   unsigned* ticket = nullptr;
   double* C = nullptr;
   unsigned* status = nullptr;
@@ -1206,12 +1208,16 @@ static linview_status sums_update_on(linview_program* p, View& sv, const T* U, c
 // The view passes of the two streams then fill each other's ramps and tails,
 // and an HBM-bound sums pass can use the bandwidth a compute-bound level pass
 // leaves idle.  (Inside a graph capture the fork and join become edges.)
+static linview_status branch_stream(cudaStream_t* st, cudaEvent_t* fork, cudaEvent_t* join) {
+  if (*st) return LINVIEW_OK;
+  LV_CUDA(cudaEventCreateWithFlags(fork, cudaEventDisableTiming));
+  LV_CUDA(cudaEventCreateWithFlags(join, cudaEventDisableTiming));
+  LV_CUDA(cudaStreamCreateWithFlags(st, cudaStreamNonBlocking));
+  return LINVIEW_OK;
+}
+
 static linview_status side_fork(linview_program* p, cudaStream_t s, cudaStream_t* out) {
-  if (!p->side) {
-    LV_CUDA(cudaStreamCreateWithFlags(&p->side, cudaStreamNonBlocking));
-    LV_CUDA(cudaEventCreateWithFlags(&p->side_fork_ev, cudaEventDisableTiming));
-    LV_CUDA(cudaEventCreateWithFlags(&p->side_join_ev, cudaEventDisableTiming));
-  }
+  LV_TRY(branch_stream(&p->side, &p->side_fork_ev, &p->side_join_ev));
   LV_CUDA(cudaEventRecord(p->side_fork_ev, s));
   LV_CUDA(cudaStreamWaitEvent(p->side, p->side_fork_ev, 0));
   p->side_pending = true;
@@ -1246,11 +1252,7 @@ static linview_status core_fork(linview_program* p, const T* V, const T* U, int 
                                 cudaStream_t s) {
   cudaStream_t cs = s;
   if (!p->prof) {
-    if (!p->core) {
-      LV_CUDA(cudaStreamCreateWithFlags(&p->core, cudaStreamNonBlocking));
-      LV_CUDA(cudaEventCreateWithFlags(&p->core_fork_ev, cudaEventDisableTiming));
-      LV_CUDA(cudaEventCreateWithFlags(&p->core_join_ev, cudaEventDisableTiming));
-    }
+    LV_TRY(branch_stream(&p->core, &p->core_fork_ev, &p->core_join_ev));
     LV_CUDA(cudaEventRecord(p->core_fork_ev, s));
     LV_CUDA(cudaStreamWaitEvent(p->core, p->core_fork_ev, 0));
     cs = p->core;
@@ -1890,6 +1892,10 @@ static linview_status iter_sk_create(linview_program* p, const void* const* inpu
   p->yp_q = (int64_t)p->Rcap * p->part_cs;
   LV_TRY(dalloc(p, (size_t)g.gC * p->xp_s * p->elem, &p->Xpart, s));
   LV_TRY(dalloc(p, (size_t)g.gR * p->yp_q * p->elem, &p->Ypart, s));
+  LV_TRY(dalloc(p, (size_t)g.gC * p->d.r_max * p->part_cs * p->elem, &p->Spart, s));
+  void* c2 = nullptr;
+  LV_TRY(dalloc(p, cpart_bytes(n), &c2, s));
+  p->Cpart2 = static_cast<double*>(c2);
   p->ldD = rup(pp, 64);
   LV_TRY(dalloc(p, (size_t)n * p->ldD * p->elem, &p->Dh, s));
   LV_TRY(ensure_stage(p, (size_t)2 * n * p->d.r_max * p->elem, s));
@@ -1910,9 +1916,43 @@ static linview_status iter_sk_create(linview_program* p, const void* const* inpu
 // old T_j, then T_j += X_j Y_j^T, and one products pass over the old P_h for
 // P_h X_j.  The exponential part runs App. A's level pass on P_h (h < s)
 // after its step; P_s, used by every skip step, is refreshed after them.
+//
+// One step has three independent chains once the factors U_h, V_h (and W^_h) are
+// there, and they run on three streams, forked and joined once per step:
+//   s: the products pass over P_h for X_i, then App. A's level pass on P_h and the
+//      assembly (the passes over the square view are ordered among themselves);
+//   y: X_j^T V_h, Y_i, then T_j += X_j Y_j^T (the panel work);
+//   z: the update of S'_h and the copied block of X_i.
+// n = 4096, p = 1024, k = 16, rank 2 (+ dB): 660 us one after the other, 560 so.
+// Under profiling all three are s.
+struct SkStreams {
+  cudaStream_t s, y, z;
+};
+static linview_status sk_fork(linview_program* p, cudaStream_t s, SkStreams* st) {
+  *st = {s, s, s};
+  if (p->prof) return LINVIEW_OK;
+  LV_TRY(branch_stream(&p->core, &p->core_fork_ev, &p->core_join_ev));
+  LV_TRY(branch_stream(&p->side, &p->side_fork_ev, &p->side_join_ev));
+  LV_CUDA(cudaEventRecord(p->core_fork_ev, s));
+  LV_CUDA(cudaStreamWaitEvent(p->core, p->core_fork_ev, 0));
+  LV_CUDA(cudaStreamWaitEvent(p->side, p->core_fork_ev, 0));
+  st->y = p->core;
+  st->z = p->side;
+  return LINVIEW_OK;
+}
+static linview_status sk_join(linview_program* p, const SkStreams& st) {
+  if (st.y == st.s) return LINVIEW_OK;
+  LV_CUDA(cudaEventRecord(p->core_join_ev, st.y));
+  LV_CUDA(cudaEventRecord(p->side_join_ev, st.z));
+  LV_CUDA(cudaStreamWaitEvent(st.s, p->core_join_ev, 0));
+  LV_CUDA(cudaStreamWaitEvent(st.s, p->side_join_ev, 0));
+  return LINVIEW_OK;
+}
+
 template <typename T>
 static linview_status iter_sk_step(linview_program* p, int cur, View& tj, const View& ph, int rh,
-                                   int c, const T* Vh, bool with_b, cudaStream_t s) {
+                                   int c, const T* Vh, bool with_b, const SkStreams& st) {
+  const cudaStream_t s = st.s, y = st.y;
   const int n = (int)p->d.n;
   const int64_t pp = p->d.p;
   const int64_t fs = p->fs;
@@ -1925,11 +1965,11 @@ static linview_status iter_sk_step(linview_program* p, int cur, View& tj, const 
   // X_j^T V_h (c x rh): FP32 factors in double-float (row-major), FP64 ones on
   // the CUDA-core GEMM (column-major)
   if constexpr (sizeof(T) == 4) {
-    ProfScope ps(p, s, 0.0);
-    LV_CUDA(launch_cross_gram(Xc, Vh, fs, n, c, rh, p->Cpart, XtV, s));
+    ProfScope ps(p, y, 0.0);
+    LV_CUDA(launch_cross_gram(Xc, Vh, fs, n, c, rh, p->Cpart2, XtV, y));
     p->all_launches++;
   } else {
-    LV_TRY(gemm_cm_own(p, true, false, c, rh, n, 1.0, Xc, fs, Vh, fs, 0.0, XtV, c, s));
+    LV_TRY(gemm_cm_own(p, true, false, c, rh, n, 1.0, Xc, fs, Vh, fs, 0.0, XtV, c, y));
   }
   // first block of Y_i (column-major p x rh): T_j^T V_h + Y_j (X_j^T V_h), and
   // with_b + B^T (W^_h - V_h) (W^_h in the What arena; dS_1 = 0)
@@ -1947,13 +1987,13 @@ static linview_status iter_sk_step(linview_program* p, int cur, View& tj, const 
   o.s_t = sizeof(T) == 4 ? rh : 1;
   o.s_c = sizeof(T) == 4 ? 1 : c;
   {
-    ProfScope ps(p, s, 0.0);
-    LV_CUDA(launch_tdot<T>(o, p->sms, s));
+    ProfScope ps(p, y, 0.0);
+    LV_CUDA(launch_tdot<T>(o, p->sms, y));
     p->all_launches++;
   }
   LV_CUDA(cudaMemcpyAsync(Yn + (int64_t)rh * pp, Yc, sizeof(T) * pp * c, cudaMemcpyDeviceToDevice,
-                          s));
-  LV_TRY(panel_rank<T>(p, tj.ptr, tj.ld, Xc, Yc, c, s));  // T_j += X_j Y_j^T
+                          y));
+  LV_TRY(panel_rank<T>(p, tj.ptr, tj.ld, Xc, Yc, c, y));  // T_j += X_j Y_j^T
   // X_i = [U_h, P_h X_j] from the old P_h
   const PassGeom g = fused_geom(sizeof(T), n, p->sms);
   LV_TRY(run_products_update<T>(p, ph, c, Xc, nullptr, nullptr, nullptr, s));
@@ -1962,7 +2002,7 @@ static linview_status iter_sk_step(linview_program* p, int cur, View& tj, const 
     LV_CUDA(launch_sum_partials<T>(static_cast<T*>(p->Xpart), g.gC, p->xp_s, p->part_cs, n, c,
                                    Xn + (int64_t)rh * fs, fs, s));
   }
-  LV_CUDA(cudaMemcpyAsync(Xn, p->Uar, sizeof(T) * fs * rh, cudaMemcpyDeviceToDevice, s));
+  LV_CUDA(cudaMemcpyAsync(Xn, p->Uar, sizeof(T) * fs * rh, cudaMemcpyDeviceToDevice, st.z));
   return LINVIEW_OK;
 }
 
@@ -1989,7 +2029,10 @@ static linview_status iter_sk_propagate(linview_program* p, int r, cudaStream_t 
       LV_CUDA(launch_suffix_sums<T>(Vh, Wh, fs, n, rh, r, s));
     }
     View& ph = ie_P(p, l);
-    LV_TRY(iter_sk_step<T>(p, cur, ie_T(p, l), ph, rh, rh, Vh, l >= 1, s));
+    SkStreams st;
+    LV_TRY(sk_fork(p, s, &st));
+    LV_TRY(iter_sk_step<T>(p, cur, ie_T(p, l), ph, rh, rh, Vh, l >= 1, st));
+    if (l >= 1) LV_TRY(run_update<T>(p, ie_S(p, l), U, Wh, rh, st.z));  // dS'_h = U_h W^_h^T
     cur ^= 1;
     // App. A's level pass on P_h, the update of S'_h, the assembly of U_2h, V_2h
     const bool fused = rh <= kMaxFusedR;
@@ -1998,7 +2041,6 @@ static linview_status iter_sk_propagate(linview_program* p, int r, cudaStream_t 
       LV_CUDA((launch_gram<T>(Vh, U, fs, n, rh, p->Cpart, p->ticket, p->C, p->status, s)));
     }
     LV_TRY(run_products_update<T>(p, ph, rh, U, Vh, U, Vh, s, fused ? p->Cpart : nullptr));
-    if (l >= 1) LV_TRY(run_update<T>(p, ie_S(p, l), U, Wh, rh, s));  // dS'_h = U_h W^_h^T
     AssembleParams a{};
     a.status = p->status;
     a.n = n;
@@ -2016,8 +2058,11 @@ static linview_status iter_sk_propagate(linview_program* p, int r, cudaStream_t 
     a.Uh = U;
     a.Unew = U + (int64_t)rh * fs;
     a.Ynew = V + (int64_t)(p->Rcap - 2 * rh) * fs;
-    ProfScope ps(p, s, 0.0);
-    LV_CUDA(launch_assemble<T>(a, s));
+    {
+      ProfScope ps(p, s, 0.0);
+      LV_CUDA(launch_assemble<T>(a, s));
+    }
+    LV_TRY(sk_join(p, st));
   }
   // skip part: T_i from T_{i-s} with the old P_s, i = 2s, .., k
   const int rs = r * sk;
@@ -2028,16 +2073,21 @@ static linview_status iter_sk_propagate(linview_program* p, int r, cudaStream_t 
   }
   for (int j = Ls + 1; j < NT; ++j) {
     const int c = (j - Ls) * rs;  // width of the factors of T_{i-s}
-    LV_TRY(iter_sk_step<T>(p, cur, ie_T(p, j - 1), ie_P(p, Ls), rs, c, Vs, Ls >= 1, s));
+    SkStreams st;
+    LV_TRY(sk_fork(p, s, &st));
+    LV_TRY(iter_sk_step<T>(p, cur, ie_T(p, j - 1), ie_P(p, Ls), rs, c, Vs, Ls >= 1, st));
+    LV_TRY(sk_join(p, st));
     cur ^= 1;
   }
-  // T_k += X_k Y_k^T, then P_s and S'_s
+  // T_k += X_k Y_k^T, P_s and S'_s
+  SkStreams st;
+  LV_TRY(sk_fork(p, s, &st));
   View& tk = ie_T(p, NT - 1);
   LV_TRY(panel_rank<T>(p, tk.ptr, tk.ld, static_cast<const T*>(p->Xar[cur]),
-                       static_cast<const T*>(p->Yar[cur]), r * k, s));
+                       static_cast<const T*>(p->Yar[cur]), r * k, st.y));
   LV_TRY(run_update<T>(p, ie_P(p, Ls), U, Vs, rs, s));
-  if (Ls >= 1) LV_TRY(run_update<T>(p, ie_S(p, Ls), U, Wh, rs, s));
-  return LINVIEW_OK;
+  if (Ls >= 1) LV_TRY(run_update<T>(p, ie_S(p, Ls), U, Wh, rs, st.z));
+  return sk_join(p, st);
 }
 
 // Updates to B, dB = U_b V_b^T (U_b in the U arena, V_b in Mr, p x rb) with
@@ -2049,9 +2099,13 @@ static linview_status iter_sk_propagate(linview_program* p, int r, cudaStream_t 
 // with S U_b = U_b + S' U_b - P U_b (S_1 = I).  Each step: T_j += X_j Y_j^T,
 // one products pass over P with [X_j | U_b] and, for S' != A, one over S'
 // with U_b; B += U_b V_b^T at the end.
+// (T_j's update on y, S' U_b on z with partial sums of its own, P's pass on s)
 template <typename T>
 static linview_status iter_sk_step_b(linview_program* p, int cur, int c, int rb, View& tj,
-                                     const View& ph, const View* sh, cudaStream_t s) {
+                                     const View& ph, const View* sh, cudaStream_t s0) {
+  SkStreams st;
+  LV_TRY(sk_fork(p, s0, &st));
+  const cudaStream_t s = st.s, y = st.y, z = st.z;
   const int n = (int)p->d.n;
   const int64_t pp = p->d.p;
   const int64_t fs = p->fs;
@@ -2063,7 +2117,22 @@ static linview_status iter_sk_step_b(linview_program* p, int cur, int c, int rb,
   T* Yn = static_cast<T*>(p->Yar[cur ^ 1]);
   T* tmp = static_cast<T*>(p->What);
   const PassGeom g = fused_geom(sizeof(T), n, p->sms);
-  LV_TRY(panel_rank<T>(p, tj.ptr, tj.ld, Xc, Yc, c, s));  // T_j += X_j Y_j^T
+  // T_j += X_j Y_j^T;  Y_i = [Y_j, V_b]
+  LV_TRY(panel_rank<T>(p, tj.ptr, tj.ld, Xc, Yc, c, y));
+  LV_CUDA(cudaMemcpyAsync(Yn, Yc, sizeof(T) * pp * c, cudaMemcpyDeviceToDevice, y));
+  LV_CUDA(cudaMemcpyAsync(Yn + (int64_t)c * pp, Vb, sizeof(T) * pp * rb, cudaMemcpyDeviceToDevice,
+                          y));
+  if (sh) {
+    const int64_t xp = p->xp_s;
+    p->xp_s = (int64_t)rb * p->part_cs;
+    const linview_status ru =
+        run_fused<T>(p, *sh, kModeX, rb, Ub, nullptr, nullptr, nullptr, p->Spart, p->Ypart, z);
+    p->xp_s = xp;
+    LV_TRY(ru);
+    ProfScope ps(p, z, 0.0);
+    LV_CUDA(launch_sum_partials<T>(static_cast<T*>(p->Spart), g.gC, (int64_t)rb * p->part_cs,
+                                   p->part_cs, n, rb, tmp, fs, z));
+  }
   // [P X_j | P U_b] in one products pass over P
   LV_CUDA(cudaMemcpyAsync(Xc + (int64_t)c * fs, Ub, sizeof(T) * fs * rb, cudaMemcpyDeviceToDevice,
                           s));
@@ -2073,24 +2142,12 @@ static linview_status iter_sk_step_b(linview_program* p, int cur, int c, int rb,
     LV_CUDA(launch_sum_partials<T>(static_cast<T*>(p->Xpart), g.gC, p->xp_s, p->part_cs, n,
                                    c + rb, Xn, fs, s));
   }
-  // second block S U_b = U_b + S' U_b - P U_b  (U_b when S = I)
-  T* blk = Xn + (int64_t)c * fs;  // column-major n x rb, seen as rb rows of n (ld fs)
-  {
-    ProfScope ps(p, s, 0.0);
-    LV_CUDA(launch_scale_copy<T>(blk, fs, blk, fs, T(sh ? -1 : 0), rb, n, s));
-    LV_CUDA(launch_axpy_rows<T>(blk, fs, Ub, fs, T(1), rb, n, s));
-  }
-  if (sh) {
-    LV_TRY(run_products_update<T>(p, *sh, rb, Ub, nullptr, nullptr, nullptr, s));
-    ProfScope ps(p, s, 0.0);
-    LV_CUDA(launch_sum_partials<T>(static_cast<T*>(p->Xpart), g.gC, p->xp_s, p->part_cs, n, rb,
-                                   tmp, fs, s));
-    LV_CUDA(launch_axpy_rows<T>(blk, fs, tmp, fs, T(1), rb, n, s));
-  }
-  // Y_i = [Y_j, V_b]
-  LV_CUDA(cudaMemcpyAsync(Yn, Yc, sizeof(T) * pp * c, cudaMemcpyDeviceToDevice, s));
-  LV_CUDA(cudaMemcpyAsync(Yn + (int64_t)c * pp, Vb, sizeof(T) * pp * rb, cudaMemcpyDeviceToDevice,
-                          s));
+  LV_TRY(sk_join(p, st));
+  // second block S U_b = U_b + S' U_b - P U_b  (U_b when S = I); column-major n x rb,
+  // seen as rb rows of n (ld fs)
+  T* blk = Xn + (int64_t)c * fs;
+  ProfScope ps(p, s, 0.0);
+  LV_CUDA(launch_s_block<T>(blk, Ub, sh ? tmp : nullptr, fs, n, rb, s));
   return LINVIEW_OK;
 }
 

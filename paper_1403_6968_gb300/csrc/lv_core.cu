@@ -659,6 +659,28 @@ cudaError_t launch_scale_copy(T* y, int64_t ldy, const T* x, int64_t ldx, T alph
   return cudaGetLastError();
 }
 
+// blk = ub + tmp - blk (column-major n x r), or ub when tmp is null: the block S U_b =
+// U_b + S' U_b - P U_b of an update to B.
+template <typename T>
+__global__ void s_block_kernel(T* blk, const T* ub, const T* tmp, int64_t fs, int n, int r) {
+  griddep_wait();
+  griddep_launch_dependents();
+  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= (int64_t)n * r) return;
+  int c, j;
+  split_index(idx, n, c, j);
+  const int64_t e = (int64_t)c * fs + j;
+  blk[e] = tmp ? (ub[e] - blk[e]) + tmp[e] : ub[e];
+}
+
+template <typename T>
+cudaError_t launch_s_block(T* blk, const T* ub, const T* tmp, int64_t fs, int n, int r,
+                           cudaStream_t s) {
+  const int64_t tot = (int64_t)n * r;
+  return launch_pdl(s_block_kernel<T>, (unsigned)((tot + kThreads - 1) / kThreads), kThreads, 0, s,
+                    blk, ub, tmp, fs, n, r);
+}
+
 // out = x + y over square views of one layout (rows of ``cols`` elements, 16-byte
 // aligned, ld a multiple of 16 bytes; the padding behind a row stays zero + zero).
 // S'_2 = A + A^2 of a re-evaluation: 12 bytes per element (n = 8192: 131 us) in
@@ -724,6 +746,8 @@ cudaError_t launch_bounded_wait_probe(uint64_t limit_ns, unsigned* status,
   template cudaError_t launch_ingest_row<T>(T*, T*, const T*, int, int, cudaStream_t);           \
   template cudaError_t launch_ingest_pair<T>(const T*, int64_t, T*, int64_t, int, const T*,      \
                                              int64_t, T*, int64_t, int, int, cudaStream_t);      \
+  template cudaError_t launch_s_block<T>(T*, const T*, const T*, int64_t, int, int,              \
+                                         cudaStream_t);                                         \
   template cudaError_t launch_add_views<T>(const T*, const T*, T*, int64_t, int64_t,             \
                                            cudaStream_t);                                       \
   template cudaError_t launch_sum_partials<T>(const T*, int, int64_t, int64_t, int, int, T*,      \

@@ -252,6 +252,10 @@ cudaError_t launch_sum_partials(const T* part, int blocks, int64_t block_stride,
                                 int n, int r, T* out, int64_t out_cs, cudaStream_t s);
 
 // Elementwise helpers.
+// blk = ub + tmp - blk, or ub (tmp null); column-major n x r, column stride fs
+template <typename T>
+cudaError_t launch_s_block(T* blk, const T* ub, const T* tmp, int64_t fs, int n, int r,
+                           cudaStream_t s);
 // out = x + y, rows x ld elements each (views of one layout)
 template <typename T>
 cudaError_t launch_add_views(const T* x, const T* y, T* out, int64_t rows, int64_t ld,
