@@ -67,7 +67,7 @@ struct PassParams {
   int64_t xp_s;
   int64_t yp_q;
   int gC, gR;         // column strips x row ranges; grid = gC * gR
-  int rows_per_cta;   // multiple of kBatch
+  int rows_per_cta;   // multiple of kBatch (FP64 also 2 or 4)
   unsigned* status;   // device status word
   double* Cpart;      // fused XYU pass: per-row-range V^T U partials [gR][r*r] (or null)
   int suffix_rin;     // update pass: >0 applies block suffix sums (block width) to Wu

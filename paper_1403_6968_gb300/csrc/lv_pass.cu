@@ -171,8 +171,7 @@ __global__ void __launch_bounds__(kThreads, 2)
     if (do_core) {
       const int c1 = ecore / r, c2 = ecore % r;
       double acc = Csh[tid];
-#pragma unroll
-      for (int j = 0; j < kBatch; ++j)
+      for (int j = 0; j < nb; ++j)
         acc = fma((double)Vs[j * R + c1], (double)Us[j * R + c2], acc);
       Csh[tid] = acc;
     }
@@ -250,8 +249,10 @@ __global__ void __launch_bounds__(kThreads, 2)
       const int c = lane % R;
       const int ts = lane / R;
       T sum = T(0);
+      if (w < nb) {
 #pragma unroll 4
-      for (int t = ts; t < 128; t += L) sum += Xbuf[(w * R + c) * XS + t];
+        for (int t = ts; t < 128; t += L) sum += Xbuf[(w * R + c) * XS + t];
+      }
 #pragma unroll
       for (int off = R; off < 32; off <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
       if (ts == 0 && w < nb && c < r) {
@@ -469,10 +470,26 @@ __global__ void __launch_bounds__(kThreads, 2)
 // ---------------------------------------------------------------------------
 static int round_up(int a, int b) { return (a + b - 1) / b * b; }
 
-static PassGeom geom_for_strip(int strip, int n, int num_sms) {
+// FP64 passes of a small view: ranges of fewer rows than a batch (the rows of the box
+// past the range are loaded and ignored), as long as the grid stays within one CTA per
+// SM.  The FP64 pipe does two FMAs per clock and SM, so the pass takes as long as its
+// rows per SM: n = 256, 4 columns 32 CTAs of 8 rows 11.9 us, 128 of 2 rows 6.4 us.
+static int short_rows(int elem_bytes, int gC, int n, int num_sms) {
+  int rows = kBatch;
+  while (elem_bytes == 8 && rows > 2 && (int64_t)gC * ((n + rows / 2 - 1) / (rows / 2)) <= num_sms)
+    rows /= 2;
+  return rows;
+}
+
+static PassGeom geom_for_strip(int elem_bytes, int strip, int n, int num_sms) {
   PassGeom g;
   g.strip = strip;
   g.gC = (n + strip - 1) / strip;
+  if (const int rows = short_rows(elem_bytes, g.gC, n, num_sms); rows < kBatch) {
+    g.rows_per_cta = rows;
+    g.gR = (n + rows - 1) / rows;
+    return g;
+  }
   const int target = 2 * num_sms;  // two resident CTAs per SM, one wave
   int gR = target / g.gC;
   const int max_gR = (n + kBatch - 1) / kBatch;
@@ -484,7 +501,7 @@ static PassGeom geom_for_strip(int strip, int n, int num_sms) {
 }
 
 PassGeom fused_geom(int elem_bytes, int n, int num_sms) {
-  return geom_for_strip(128 * (16 / elem_bytes), n, num_sms);
+  return geom_for_strip(elem_bytes, 128 * (16 / elem_bytes), n, num_sms);
 }
 
 static int update_cols(int elem_bytes, int R) {
@@ -493,7 +510,7 @@ static int update_cols(int elem_bytes, int R) {
 }
 
 PassGeom update_geom(int elem_bytes, int R, int n, int num_sms) {
-  return geom_for_strip(kThreads * update_cols(elem_bytes, R), n, num_sms);
+  return geom_for_strip(elem_bytes, kThreads * update_cols(elem_bytes, R), n, num_sms);
 }
 
 bool make_tmap(CUtensorMap* out, const void* base, int elem_bytes, int64_t cols, int64_t rows,
