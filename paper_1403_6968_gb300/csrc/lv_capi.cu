@@ -730,15 +730,17 @@ static linview_status tc_scratch(linview_program* p, TcScratch* sc, int64_t a_ro
   sc->a_rows = a_rows;
   sc->b_rows = b_rows;
   sc->K = K;
-  LV_CUDA(cudaMemsetAsync(sc->words, 0, sizeof(unsigned), s));  // no operand needs TF32 yet
+  // no operand needs TF32 yet (the second word serves linview_gemm as its status)
+  LV_CUDA(cudaMemsetAsync(sc->words, 0, 4 * sizeof(unsigned), s));
   return LINVIEW_OK;
 }
 
 // Products that go to the tensor cores (FP32, dense enough to fill tiles);
 // the rest run on the CUDA cores.
+static bool tc_shape(int64_t M, int64_t N, int64_t K) { return M >= 128 && N >= 8 && K >= 128; }
 static bool tc_eligible(const linview_program* p, const TcScratch* sc, int64_t M, int64_t N,
                         int64_t K) {
-  return p->elem == 4 && sc && sc->a && M >= 128 && N >= 8 && K >= 128 && M <= sc->a_rows &&
+  return p->elem == 4 && sc && sc->a && tc_shape(M, N, K) && M <= sc->a_rows &&
          N <= sc->b_rows && K <= sc->K;
 }
 
@@ -3314,24 +3316,25 @@ linview_status linview_gemm(int precision, int ta, int tb, int64_t M, int64_t N,
   LV_TRY(check_dev_ptr(B, tmp.device, "B"));
   LV_TRY(check_dev_ptr(C, tmp.device, "C"));
   cudaDeviceGetAttribute(&tmp.sms, cudaDevAttrMultiProcessorCount, tmp.device);
-  void* work = nullptr;
-  LV_TRY(talloc(&tmp, kGemmWorkBytes + 256, &work, s));
-  tmp.status = static_cast<unsigned*>(work);
-  tmp.gwork = static_cast<char*>(work) + 256;
-  tmp.gwork_elems = (int64_t)kGemmWorkBytes / tmp.elem;
-  cudaError_t ce = cudaMemsetAsync(work, 0, 256, s);
-  linview_status st = ce == cudaSuccess ? LINVIEW_OK : fail(LINVIEW_EDEVICE, "memset failed");
-  if (st == LINVIEW_OK) {
-    TcScratch sc;
-    st = tc_scratch(&tmp, &sc, M, N, K, s);
-    // op(A) rows; op(B)^T rows (op(B) is K x N)
-    const Opnd a = ta ? cols_of(A, lda) : rows_of(A, lda);
-    const Opnd b = tb ? rows_of(B, ldb) : cols_of(B, ldb);
-    if (st == LINVIEW_OK) st = gemm_ab(&tmp, M, N, K, alpha, a, b, beta, C, ldc, C, ldc, s, &sc);
-  }
+  // op(A) rows; op(B)^T rows (op(B) is K x N)
+  const Opnd a = ta ? cols_of(A, lda) : rows_of(A, lda);
+  const Opnd b = tb ? rows_of(B, ldb) : cols_of(B, ldb);
   unsigned hs = 0;
-  cudaMemcpyAsync(&hs, tmp.status, sizeof(unsigned), cudaMemcpyDeviceToHost, s);
-  tfree(&tmp, work, kGemmWorkBytes + 256, s);
+  linview_status st = LINVIEW_OK;
+  if (tmp.elem == 4 && tc_shape(M, N, K)) {  // one block holds everything
+    TcScratch sc;
+    LV_TRY(tc_scratch(&tmp, &sc, M, N, K, s));
+    tmp.status = sc.words + 1;
+    st = gemm_ab(&tmp, M, N, K, alpha, a, b, beta, C, ldc, C, ldc, s, &sc);
+    cudaMemcpyAsync(&hs, tmp.status, sizeof(unsigned), cudaMemcpyDeviceToHost, s);
+  } else {
+    void* work = nullptr;
+    LV_TRY(talloc(&tmp, kGemmWorkBytes, &work, s));
+    tmp.gwork = work;
+    tmp.gwork_elems = (int64_t)kGemmWorkBytes / tmp.elem;
+    st = gemm_ab(&tmp, M, N, K, alpha, a, b, beta, C, ldc, C, ldc, s, nullptr);
+    tfree(&tmp, work, kGemmWorkBytes, s);
+  }
   LV_CUDA(cudaStreamSynchronize(s));
   if (st == LINVIEW_OK && (hs & kStatusTimeout)) st = fail(LINVIEW_ETIMEOUT, "bounded wait expired");
   return st;
