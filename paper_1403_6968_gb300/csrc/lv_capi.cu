@@ -692,7 +692,8 @@ struct TcScratch {
   float* b = nullptr;
   float* work = nullptr;
   int64_t work_floats = 0;
-  unsigned* words = nullptr;  // [flag (4 words) | words of A | words of B]
+  unsigned* words = nullptr;  // [flags (4 words) | words of A | words of B]
+  int cur = 0;                // words[cur], 0 or 2: the flag of the next product
   int64_t a_rows = 0, b_rows = 0, K = 0;
   void* block = nullptr;  // temporary block owned by this scratch (null: borrowed)
   size_t bytes = 0;
@@ -748,13 +749,17 @@ static bool tc_eligible(const linview_program* p, const TcScratch* sc, int64_t M
 // ldc; may be D; beta == 0 ignores it), with a = rows of op(A) (M x K) and b =
 // rows of op(B)^T (N x K).  FP32 with scratch: split operands on the tensor cores
 // (a_ready / b_ready: the scratch already holds that operand's split rows;
-// reverse: visit K from its end, for every other product with the same A);
+// reverse: visit K from its end, for every other product with the same A;
+// d_split: the next product's second operand is D's columns, b = cols_of(D), with
+// the same inner length K = M: split them into the scratch in this call where the
+// GEMM can, *d_split tells);
 // otherwise the CUDA-core GEMM in the program's arithmetic.
 static linview_status gemm_ab(linview_program* p, int64_t M, int64_t N, int64_t K, double alpha,
                               Opnd a, Opnd b, double beta, const void* C, int64_t ldc, void* D,
                               int64_t ldd, cudaStream_t s, TcScratch* sc = nullptr,
                               bool a_ready = false, bool b_ready = false,
-                              bool reverse = false) {
+                              bool reverse = false, bool* d_split = nullptr) {
+  if (d_split) *d_split = false;
   if (M <= 0 || N <= 0) return LINVIEW_OK;
   const int e = p->elem;
   if (tc_eligible(p, sc, M, N, K)) {
@@ -762,13 +767,21 @@ static linview_status gemm_ab(linview_program* p, int64_t M, int64_t N, int64_t 
                        sc->words + 4};
     const TcOperand tb{static_cast<const float*>(b.p), b.rs, b.cs, (int)N, (int)K, sc->b,
                        sc->words + 4 + tc_split_words(sc->a_rows, sc->K)};
+    const TcOperand td{static_cast<const float*>(D), 1, ldd, (int)N, (int)M, sc->b,
+                       sc->words + 4 + tc_split_words(sc->a_rows, sc->K)};
     if (!a_ready || !b_ready) {
-      LV_CUDA(launch_tc_split(a_ready ? nullptr : &ta, b_ready ? nullptr : &tb, sc->words, s));
+      LV_CUDA(launch_tc_split(a_ready ? nullptr : &ta, b_ready ? nullptr : &tb,
+                              sc->words + sc->cur, s));
       p->all_launches += 2;
     }
-    LV_CUDA(launch_tc_gemm(ta, tb, sc->words, static_cast<float*>(D), ldd,
+    const bool next = d_split && M == K;
+    LV_CUDA(launch_tc_gemm(ta, tb, sc->words + sc->cur, static_cast<float*>(D), ldd,
                            static_cast<const float*>(C), ldc, (float)alpha, (float)beta, p->sms,
-                           p->status, s, sc->work, sc->work_floats, reverse));
+                           p->status, s, sc->work, sc->work_floats, reverse,
+                           next ? &td : nullptr, d_split, sc->words + (sc->cur ^ 2)));
+    // a kernel still reads this product's flag while it splits D, so the next
+    // product has the other one
+    if (next && *d_split) sc->cur ^= 2;
     p->all_launches += 2;
     return LINVIEW_OK;
   }
@@ -1430,6 +1443,7 @@ static linview_status iter_reeval(linview_program* p, cudaStream_t s) {
   View& a = p->views[0];
   char* T = static_cast<char*>(p->Tpanel);
   TcScratch sc;
+  bool t_split = false;  // T_{i-1}'s columns are split already
   if (!library_mode(mode) && !(p->elem == 4 && view_panel_fits<float>(p, a, (int)pp)))
     LV_TRY(tc_scratch(p, &sc, n, pp, n, s));
   for (int i = 1; i <= k; ++i) {
@@ -1447,7 +1461,7 @@ static linview_status iter_reeval(linview_program* p, cudaStream_t s) {
                                        static_cast<float*>(ti), p->ldT, s));
     } else {  // T_i = A T_{i-1} + B, A's rows split once
       LV_TRY(gemm_ab(p, n, pp, n, 1.0, rows_of(a.ptr, a.ld), cols_of(tp, p->ldT), 1.0, p->Bm,
-                     p->ldB, ti, p->ldT, s, &sc, i > 1, false, i % 2 == 0));
+                     p->ldB, ti, p->ldT, s, &sc, i > 1, t_split, i % 2 == 0, &t_split));
     }
   }
   return LINVIEW_OK;
@@ -1583,7 +1597,8 @@ static linview_status iter_propagate(linview_program* p, int r, cudaStream_t s) 
   View& a = p->views[0];
   const PassGeom g = fused_geom(sizeof(T), n, p->sms);
   // M_i = T_i^T V (old T_i), stored at block k-1-i so that [M_{i-1} .. M_0]
-  // is one contiguous p x (i r) slab: one pass over the T panel
+  // is one contiguous p x (i r) slab: one pass over the T panel (beside the
+  // Krylov passes it takes their bandwidth: 708 us against 706 us, so in line)
   LV_TRY(panel_tdot<T>(p, reinterpret_cast<const T*>(Tp), p->ldT, V1, r, k, M, s));
   if (k >= 2) {
     LV_TRY(core_fork<T>(p, V1, K, r, s));
@@ -3179,6 +3194,7 @@ static linview_status adjoint_iteration(linview_program* p, const void* Gk, int6
     const View& t0 = p->views[p->ie_NT + 2];
     LV_CUDA(cudaMemcpy2DAsync(T, ldT * e, t0.ptr, t0.ld * e, pp * e, n, cudaMemcpyDeviceToDevice,
                               s));
+    bool t_split = false;  // T_{i-1}'s columns are split already
     for (int i = 1; i <= k; ++i) {
       char* tp = T + (size_t)(i - 1) * pp * e;
       char* ti = T + (size_t)i * pp * e;
@@ -3188,7 +3204,7 @@ static linview_status adjoint_iteration(linview_program* p, const void* Gk, int6
                                          reinterpret_cast<float*>(ti), ldT, s));
       else
         LV_TRY(gemm_ab(p, n, pp, n, 1.0, rows_of(a.ptr, a.ld), cols_of(tp, ldT), 1.0, p->Bm,
-                       p->ldB, ti, ldT, s, &sc, i > 1, false, i % 2 == 0));
+                       p->ldB, ti, ldT, s, &sc, i > 1, t_split, i % 2 == 0, &t_split));
     }
   }
   // G_k = seed; G_i = A^T G_{i+1}
@@ -3204,8 +3220,9 @@ static linview_status adjoint_iteration(linview_program* p, const void* Gk, int6
                                       static_cast<const double*>(src), lds, Gk ? 1.0 : 2.0,
                                       (int)n, (int)pp, s));
   p->all_launches++;
-  // the rows of A^T are split once for all the products A^T G
-  bool at_split = false;
+  // the rows of A^T are split once for all the products A^T G, and G_i's columns by
+  // the product that makes G_i where that works out
+  bool at_split = false, g_split = false;
   for (int i = k - 1; i >= 1; --i) {
     void* gi = G + (size_t)(i - 1) * pp * e;
     void* gn = G + (size_t)i * pp * e;
@@ -3214,7 +3231,7 @@ static linview_status adjoint_iteration(linview_program* p, const void* Gk, int6
                                        nullptr, 0, static_cast<float*>(gi), p->ldG, s));
     } else {
       LV_TRY(gemm_ab(p, n, pp, n, 1.0, cols_of(a.ptr, a.ld), cols_of(gn, p->ldG), 0.0, nullptr,
-                     0, gi, p->ldG, s, &sc, at_split, false, i % 2 == 0));
+                     0, gi, p->ldG, s, &sc, at_split, g_split, i % 2 == 0, &g_split));
       at_split = true;
     }
   }
@@ -3226,7 +3243,7 @@ static linview_status adjoint_iteration(linview_program* p, const void* Gk, int6
                                        ld_dT0, s));
     else
       LV_TRY(gemm_ab(p, n, pp, n, 1.0, cols_of(a.ptr, a.ld), cols_of(G, p->ldG), 0.0, nullptr, 0,
-                     dT0, ld_dT0, s, &sc, at_split));
+                     dT0, ld_dT0, s, &sc, at_split, g_split));
   }
   if (dB) {
     if (e == 4)

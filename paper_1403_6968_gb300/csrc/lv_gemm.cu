@@ -589,11 +589,45 @@ __device__ __forceinline__ int64_t block_line(int i, int kc, int nk) {
   return ((int64_t)(i >> 7) * nk + kc) * 256 + (i & 127);
 }
 
-// FP16 halves: tiles of 64 rows x 128 k (two runs), zero past K (kp = rup(K, 64)), one pass over the operand: eight lanes hold a
-// run and find its largest entry by shuffles.  An entry y = 2^sh x with 0 < |y| <
-// 2^-2 has fewer than 22 bits; eight of them among 32 neighbours of a row or of a
-// column of a tile (dense data without such structure has none), a scale outside
-// 2^-60 .. 2^60 or a non-finite entry sets the flag that sends the product to TF32.
+// Values k .. k + 7 of row i (a run of 64 belongs to eight neighbouring lanes; all lanes
+// of the warp take part): scale, split, store (``in``: inside the operand).  ``small`` is
+// called for the entries with fewer than 22 bits.  Returns whether the run's scale is out
+// of range or an entry is not finite.
+template <typename F>
+__device__ __forceinline__ bool split_run(const float (&x)[8], const SplitOp& o, int i, int k,
+                                          bool in, int kp, F small) {
+  unsigned mx = 0;
+#pragma unroll
+  for (int e = 0; e < 8; ++e) mx = max(mx, __float_as_uint(x[e]) & 0x7fffffffu);
+#pragma unroll
+  for (int d = 1; d < 8; d <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, d));
+  int sh = mx ? 14 - ((int)(mx >> 23) - 127) : 0;
+  const bool bad = sh > 60 || sh < -60;  // (non-finite: sh = -114)
+  sh = min(60, max(-60, sh));
+  const float sc = pow2f(sh);
+  __align__(16) __half hi[8], lo[8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    const float y = x[e] * sc;
+    hi[e] = __float2half_rn(y);
+    lo[e] = __float2half_rn(y - __half2float(hi[e]));
+    if (y != 0.f && fabsf(y) < 0.25f) small(e);
+  }
+  if (in) {
+    unsigned char* d = o.dst + block_line(i, k / 64, kp / 64) * 128 + k % 64 * 2;
+    *reinterpret_cast<uint4*>(d) = *reinterpret_cast<const uint4*>(hi);
+    *reinterpret_cast<uint4*>(d + 16384) = *reinterpret_cast<const uint4*>(lo);
+    if (k % 64 == 0) o.sc[(int64_t)(k / 64) * o.pitch + i] = pow2f(-sh);
+  }
+  return bad;
+}
+
+// FP16 halves: tiles of 64 rows x 128 k (two runs), zero past K (kp = rup(K, 64)), one
+// pass over the operand: eight lanes hold a run and find its largest entry by shuffles.
+// An entry y = 2^sh x with 0 < |y| < 2^-2 has fewer than 22 bits; eight of them among 32
+// neighbours of a row or of a column of a tile (dense data without such structure has
+// none), a scale outside 2^-60 .. 2^60 or a non-finite entry sets the flag that sends
+// the product to TF32.
 // 8192 x 8192: 101 us transposed, 93 us not, 4 bytes read and 4 written per entry
 // (floor 79); TF32 halves (8 written) took 196 us.
 constexpr int kSpR = 64, kSpK = 128, kSmallCount = 8;
@@ -658,32 +692,10 @@ __global__ void __launch_bounds__(256) split_f16_kernel(const __grid_constant__ 
 #pragma unroll
       for (int e = 0; e < 8; ++e) x[e] = tile[kl + e][il];  // zeros past the operand
     }
-    unsigned mx = 0;
-#pragma unroll
-    for (int e = 0; e < 8; ++e) mx = max(mx, __float_as_uint(x[e]) & 0x7fffffffu);
-#pragma unroll
-    for (int d = 1; d < 8; d <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, d));
-    int sh = mx ? 14 - ((int)(mx >> 23) - 127) : 0;
-    bad |= sh > 60 || sh < -60;  // (non-finite: sh = -114)
-    sh = min(60, max(-60, sh));
-    const float sc = pow2f(sh);
-    __align__(16) __half hi[8], lo[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const float y = x[e] * sc;
-      hi[e] = __float2half_rn(y);
-      lo[e] = __float2half_rn(y - __half2float(hi[e]));
-      if (y != 0.f && fabsf(y) < 0.25f) {
-        atomicAdd(&rowcnt[il][(kl + e) / 32], 1);
-        atomicAdd(&colcnt[il / 32][kl + e], 1);
-      }
-    }
-    if (in) {
-      unsigned char* d = o.dst + block_line(i, k / 64, kp / 64) * 128 + k % 64 * 2;
-      *reinterpret_cast<uint4*>(d) = *reinterpret_cast<const uint4*>(hi);
-      *reinterpret_cast<uint4*>(d + 16384) = *reinterpret_cast<const uint4*>(lo);
-      if (kl % 64 == 0) o.sc[(int64_t)(k / 64) * o.pitch + i] = pow2f(-sh);
-    }
+    bad |= split_run(x, o, i, k, in, kp, [&](int e) {
+      atomicAdd(&rowcnt[il][(kl + e) / 32], 1);
+      atomicAdd(&colcnt[il / 32][kl + e], 1);
+    });
   }
   __syncthreads();
   bad |= (&rowcnt[0][0])[tid] >= kSmallCount || (&colcnt[0][0])[tid] >= kSmallCount;
@@ -856,14 +868,23 @@ __global__ void gemm_reduce_kernel(int M, int N, int splits, int batch, T alpha,
   }
 }
 
-// D = alpha (pieces) + beta C for the tiles cut along K: a CTA adds 16 rows of one
-// tile, the pieces in their order along K.
-template <int BN>
-__global__ void __launch_bounds__(256) gemm_parts_kernel(const GArgs a, int tiles) {
+// D = alpha (pieces) + beta C for the tiles cut along K: a CTA adds ROWS rows of one
+// tile, the pieces in their order along K.  SPLIT (ROWS = 64 = BN, every tile cut): D's
+// columns also go to the split operand ``nx``, a run of 64 rows per CTA and column.
+// Bound by the latency of its few CTAs (128 at 8192 rows x 64 columns: 2 MB of D, 8 MB of
+// pieces from L2); the split inside it saves the launches of a split of its own: the
+// adjoint of 16 rounds at 8192 x 64 1445 -> 1394 us.
+template <int BN, int ROWS, bool SPLIT>
+__global__ void __launch_bounds__(256) gemm_parts_kernel(const GArgs a, int tiles,
+                                                         const __grid_constant__ SplitOp nx,
+                                                         unsigned* nx_flag) {
+  __shared__ float tile[SPLIT ? ROWS : 1][SPLIT ? BN + 1 : 1];
+  __shared__ int rowcnt[SPLIT ? BN : 1][2], colcnt[2][SPLIT ? ROWS : 1];
   griddep_wait();
   griddep_launch_dependents();
   const int r = blockIdx.x;
-  const int nk = *a.flag == 0u ? a.kp16 / 64 : a.kp32 / 32;
+  const bool f16 = *a.flag == 0u;
+  const int nk = f16 ? a.kp16 / 64 : a.kp32 / 32;
   const long long W = (long long)(tiles - a.dp) * nk, lo = (long long)r * nk, hi = lo + nk;
   // ranges that meet the tile: W c / cut < hi and W (c + 1) / cut > lo
   int c0 = (int)(lo * a.cut / W), c1;
@@ -871,35 +892,73 @@ __global__ void __launch_bounds__(256) gemm_parts_kernel(const GArgs a, int tile
   while (W * (c0 + 1) / a.cut <= lo) ++c0;
   c1 = c0;
   while (W * (c1 + 1) / a.cut < hi) ++c1;
-  if (c0 == c1) return;  // computed whole
+  const bool whole = c0 == c1;  // computed by one range: D is complete
+  if (whole && !SPLIT) return;
   int mb, nb;
   g_tile(a.dp + r, (a.M + kGBM - 1) / kGBM, (a.N + BN - 1) / BN, mb, nb);
-  for (int e = threadIdx.x; e < 16 * BN / 4; e += 256) {
-    const int row = blockIdx.y * 16 + e / (BN / 4), col = e % (BN / 4) * 4;
+  const int row0 = blockIdx.y * ROWS;
+  for (int e = threadIdx.x; e < ROWS * BN / 4; e += 256) {
+    const int row = row0 + e / (BN / 4), col = e % (BN / 4) * 4;
     const int m = mb * kGBM + row, n = nb * BN + col;
-    if (m >= a.M || n >= a.N) continue;
-    const float* w = a.work + ((int64_t)(c0 + r) * kGBM + row) * BN + col;
-    float4 s = *reinterpret_cast<const float4*>(w);
+    float v[4] = {0.f, 0.f, 0.f, 0.f};
+    if (m < a.M && n < a.N) {
+      if (!whole) {
+        const float* w = a.work + ((int64_t)(c0 + r) * kGBM + row) * BN + col;
+        float4 s = *reinterpret_cast<const float4*>(w);
 #pragma unroll 4
-    for (int c = c0 + 1; c <= c1; ++c) {
-      const float4 x =
-          *reinterpret_cast<const float4*>(w + (int64_t)(c - c0) * kGBM * BN);
-      s.x += x.x;
-      s.y += x.y;
-      s.z += x.z;
-      s.w += x.w;
+        for (int c = c0 + 1; c <= c1; ++c) {
+          const float4 x =
+              *reinterpret_cast<const float4*>(w + (int64_t)(c - c0) * kGBM * BN);
+          s.x += x.x;
+          s.y += x.y;
+          s.z += x.z;
+          s.w += x.w;
+        }
+        v[0] = s.x; v[1] = s.y; v[2] = s.z; v[3] = s.w;
+        for (int j = 0; j < 4 && n + j < a.N; ++j) {
+          float o = a.alpha * v[j];
+          if (a.C && a.beta != 0.f) o += a.beta * a.C[(int64_t)m * a.ldc + n + j];
+          a.D[(int64_t)m * a.ldd + n + j] = o;
+          v[j] = o;
+        }
+      } else {
+        for (int j = 0; j < 4 && n + j < a.N; ++j) v[j] = a.D[(int64_t)m * a.ldd + n + j];
+      }
     }
-    const float v[4] = {s.x, s.y, s.z, s.w};
-    for (int j = 0; j < 4 && n + j < a.N; ++j) {
-      float o = a.alpha * v[j];
-      if (a.C && a.beta != 0.f) o += a.beta * a.C[(int64_t)m * a.ldc + n + j];
-      a.D[(int64_t)m * a.ldd + n + j] = o;
+    if constexpr (SPLIT) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) tile[e / (BN / 4)][col + j] = n + j < a.N ? v[j] : 0.f;
     }
+  }
+  if constexpr (SPLIT) {
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *nx.fmt = 0u;
+    if (threadIdx.x < BN * 2) (&rowcnt[0][0])[threadIdx.x] = 0;
+    if (threadIdx.x < ROWS * 2) (&colcnt[0][0])[threadIdx.x] = 0;
+    __syncthreads();
+    const int kp = (nx.K + 63) / 64 * 64, k0 = mb * kGBM + row0;
+    bool bad = false;
+#pragma unroll
+    for (int u = 0; u < BN * ROWS / (8 * 256); ++u) {
+      const int idx = u * 256 + threadIdx.x;
+      const int i = idx / (ROWS / 8), kl = idx % (ROWS / 8) * 8, k = k0 + kl;
+      float x[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) x[e] = tile[kl + e][i];  // zeros past D
+      bad |= split_run(x, nx, i, k, i < nx.rows && k < kp, kp, [&](int e) {
+        atomicAdd(&rowcnt[i][(kl + e) / 32], 1);
+        atomicAdd(&colcnt[i / 32][kl + e], 1);
+      });
+    }
+    __syncthreads();
+    if (threadIdx.x < BN * 2) bad |= (&rowcnt[0][0])[threadIdx.x] >= kSmallCount;
+    if (threadIdx.x < ROWS * 2) bad |= (&colcnt[0][0])[threadIdx.x] >= kSmallCount;
+    if (__syncthreads_or(bad || !f16) && threadIdx.x == 0) atomicOr(nx_flag, 1u);
   }
 }
 
 template <int BN>
-cudaError_t launch_tc_gemm_t(const GMaps& maps, const GArgs& a, int num_sms, cudaStream_t s) {
+cudaError_t launch_tc_gemm_t(const GMaps& maps, const GArgs& a, const SplitOp* next, bool* did,
+                             unsigned* next_flag, int num_sms, cudaStream_t s) {
   using Sh = GShape<BN>;
   static const cudaError_t configured = [] {
     cudaFuncAttributes at;
@@ -918,7 +977,15 @@ cudaError_t launch_tc_gemm_t(const GMaps& maps, const GArgs& a, int num_sms, cud
   const cudaError_t e =
       launch_pdl(tc_gemm_kernel<BN>, 2 * pairs, Sh::Threads, Sh::SmemBytes, s, maps, a);
   if (e != cudaSuccess || tiles == a.dp) return e;
-  return launch_pdl(gemm_parts_kernel<BN>, dim3(tiles - a.dp, kGBM / 16), 256, 0, s, a, tiles);
+  if constexpr (BN == 64) {
+    if (next && a.dp == 0 && a.N <= BN) {
+      *did = true;
+      return launch_pdl(gemm_parts_kernel<BN, 64, true>, dim3(tiles, kGBM / 64), 256, 0, s, a,
+                        tiles, *next, next_flag);
+    }
+  }
+  return launch_pdl(gemm_parts_kernel<BN, 16, false>, dim3(tiles - a.dp, kGBM / 16), 256, 0, s, a,
+                    tiles, SplitOp{}, nullptr);
 }
 
 // A split operand as lines of 128 bytes (64 FP16 or 32 TF32 values), boxes of
@@ -1036,7 +1103,8 @@ cudaError_t launch_tc_split(const TcOperand* a, const TcOperand* b, unsigned* fl
 cudaError_t launch_tc_gemm(const TcOperand& a, const TcOperand& b, unsigned* flag, float* D,
                            int64_t ldd, const float* C, int64_t ldc, float alpha, float beta,
                            int num_sms, unsigned* status, cudaStream_t s, float* work,
-                           int64_t work_floats, bool reverse) {
+                           int64_t work_floats, bool reverse, const TcOperand* next,
+                           bool* next_split, unsigned* next_flag) {
   const int M = a.rows, N = b.rows, K = a.K;
   if (M <= 0 || N <= 0 || K <= 0 || b.K != K) return cudaErrorInvalidValue;
   SplitPair sp{};
@@ -1080,9 +1148,11 @@ cudaError_t launch_tc_gemm(const TcOperand& a, const TcOperand& b, unsigned* fla
   g.fmtb = b.words;
   g.flag = flag;
   g.status = status;
-  if (bn == 256) return launch_tc_gemm_t<256>(maps, g, num_sms, s);
-  if (bn == 128) return launch_tc_gemm_t<128>(maps, g, num_sms, s);
-  return launch_tc_gemm_t<64>(maps, g, num_sms, s);
+  const SplitOp nx = split_op(next);
+  const SplitOp* np = next ? &nx : nullptr;
+  if (bn == 256) return launch_tc_gemm_t<256>(maps, g, np, next_split, next_flag, num_sms, s);
+  if (bn == 128) return launch_tc_gemm_t<128>(maps, g, np, next_split, next_flag, num_sms, s);
+  return launch_tc_gemm_t<64>(maps, g, np, next_split, next_flag, num_sms, s);
 }
 
 static int gemm_simt_splits(int M, int N, int K, int batch, int num_sms, int64_t work_elems) {

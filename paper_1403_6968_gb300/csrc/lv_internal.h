@@ -161,10 +161,16 @@ cudaError_t launch_tc_split(const TcOperand* a, const TcOperand* b, unsigned* fl
 // be null): room for the pieces of tiles that several CTA pairs share along K
 // (summed in a fixed order).  ``reverse`` visits K from its end: a product that
 // follows another one with the same A then starts on the part still in L2.
+// ``next``: D's columns as a split operand (rows N, K = M; its buffer may be b's): they
+// are split by the kernel that adds up the cut tiles when every tile is cut and one
+// tile column holds D; *next_split says whether they were, and ``next_flag`` (another word
+// than ``flag``, set when that one is) is then the flag of the product that reads them.
 cudaError_t launch_tc_gemm(const TcOperand& a, const TcOperand& b, unsigned* flag, float* D,
                            int64_t ldd, const float* C, int64_t ldc, float alpha, float beta,
                            int num_sms, unsigned* status, cudaStream_t s, float* work = nullptr,
-                           int64_t work_floats = 0, bool reverse = false);
+                           int64_t work_floats = 0, bool reverse = false,
+                           const TcOperand* next = nullptr, bool* next_split = nullptr,
+                           unsigned* next_flag = nullptr);
 // C (M x N) = alpha A B + beta C on the CUDA cores, A(m, k) = A[m a_rs + k a_cs],
 // B(k, n) = B[k b_rs + n b_cs], C(m, n) = C[m c_rs + n c_cs]; long inner
 // dimensions are split over ``work`` (work_elems elements, may be null) and

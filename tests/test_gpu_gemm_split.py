@@ -115,3 +115,58 @@ def test_tf32_split_reused():
     assert rel_frob(dB.cpu().numpy() * scale, rB * scale) <= 5 * TOL
     assert rel_frob(dA.cpu().numpy() * scale / s, rA * scale / s) <= 5 * TOL
     prog.close()
+
+
+@pytest.mark.parametrize("model", ["linear", "exp"])
+@pytest.mark.parametrize("n,p", [(128, 8), (300, 33), (1000, 64), (513, 65), (1537, 17)])
+def test_chain_split(n, p, model):
+    """Chains T_i = A T_{i-1} + B and G_i = A^T G_{i+1}: the kernel that finishes a
+    product (p <= 64: tile remainders, rows past the last run, one row past a tile)
+    also splits it for the next one.  k rounds of 3e-7 each: 5 x the tolerance."""
+    from oracle import iteration as oi
+    import linview_inputs as li
+    from paper_1403_6968_gb300 import Program
+    k = 4
+    a, b, t0 = (x.astype(np.float32) for x in li.iteration_inputs(n, p, seed=n + p))
+    prog = Program("iteration", [torch.from_numpy(x).cuda() for x in (a, b, t0)], k=k, r_max=1,
+                   model=model)
+    A, B, T = (x.astype(np.float64) for x in (a, b, t0))
+    ts = oi.reeval(A, B, T, k)
+    if model == "linear":
+        assert rel_frob(prog.read_view(k).cpu().numpy(), ts[k]) <= 5 * TOL
+    seed = np.random.default_rng(8).standard_normal((n, p)).astype(np.float32)
+    dA, dB = torch.empty(n, n, device="cuda"), torch.empty(n, p, device="cuda")
+    dT0 = torch.empty(n, p, device="cuda")
+    prog.adjoint_iteration_seed(torch.from_numpy(seed).cuda(), dA=dA, dB=dB, dT0=dT0)
+    prog.sync()
+    G, rA, rB = seed.astype(np.float64), 0.0, 0.0
+    for i in range(k, 0, -1):
+        rA, rB, G = rA + G @ ts[i - 1].T, rB + G, A.T @ G
+    for got, ref in ((dA, rA), (dB, rB), (dT0, G)):
+        assert rel_frob(got.cpu().numpy(), ref) <= 5 * TOL
+    prog.close()
+
+
+def test_chain_split_turns_to_tf32():
+    """The first product of the chain has FP16 halves, its result (rows over eight
+    decades) needs TF32: the flag that a product leaves for the next one, while other
+    blocks of the same launch still go by its own."""
+    from oracle import iteration as oi
+    import linview_inputs as li
+    from paper_1403_6968_gb300 import Program
+    n, p, k = 1000, 48, 4
+    a, b, t0 = li.iteration_inputs(n, p, seed=9)
+    s = 10.0 ** np.random.default_rng(10).uniform(-4, 4, n)
+    a, b, t0 = (x.astype(np.float32) for x in (a * s, 0 * b, t0))
+    prog = Program("iteration", [torch.from_numpy(x).cuda() for x in (a, b, t0)], k=k, r_max=1)
+    seed = np.random.default_rng(11).standard_normal((n, p)).astype(np.float32)
+    dB, dT0 = torch.empty(n, p, device="cuda"), torch.empty(n, p, device="cuda")
+    dA = torch.empty(n, n, device="cuda")
+    prog.adjoint_iteration_seed(torch.from_numpy(seed).cuda(), dA=dA, dB=dB, dT0=dT0)
+    prog.sync()
+    G, rB = seed.astype(np.float64), 0.0
+    for i in range(k, 0, -1):
+        rB, G = rB + G, a.astype(np.float64).T @ G
+    assert rel_frob(dT0.cpu().numpy() / s[:, None], G / s[:, None]) <= 5 * TOL
+    assert rel_frob(dB.cpu().numpy() / s[:, None], rB / s[:, None]) <= 5 * TOL
+    prog.close()
