@@ -24,7 +24,7 @@
 //    one K chunk, [hi | lo] of 16 KB each, rows of 128 bytes (the split also transposes
 //    where the product needs the other layout): a chunk of a CTA's A is one copy of
 //    32 contiguous KB (as rows [hi | lo] of length K every box line was 128 bytes 32 KB
-//    apart, and 8192 x 64 x 8192, which streams A from memory, took 57 us, 53 now; 8192 x 8192 x 1024 328 -> 316).
+//    apart, and 8192 x 64 x 8192, which streams A from memory, took 57 us, 53 now).
 //    CTA pairs (cta_group::2) compute tiles of 256 x BN outputs (BN = 256, 128 or
 //    64), each CTA holding 128 rows of A and half of B's rows, in K chunks of
 //    one 128-byte swizzle atom (64 FP16 or 32 TF32 values); a persistent grid
@@ -77,8 +77,10 @@ struct GShape {
   static constexpr uint32_t TmemCols = 512;
   static constexpr int CW = BN < 128 ? BN : 128;              // columns per epilogue thread
   static constexpr int NE = 4 * (BN / CW);                    // epilogue warps
-  static constexpr uint32_t OffScale = OffBar + 512;          // [NE][CW] column factors of a chunk
-  static constexpr uint32_t SmemBytes = OffScale + NE * CW * 4 + 1024;  // + alignment slack
+  // 4 KB per epilogue warp: the CW column factors of a chunk; after a tile's last
+  // chunk 32 rows x 32 columns on their way to D
+  static constexpr uint32_t OffStage = OffBar + 512;
+  static constexpr uint32_t SmemBytes = OffStage + NE * 4096 + 1024;  // + alignment slack
   // warps 0-3: copies, MMAs, two idle; then the epilogue
   static constexpr int Threads = 128 + 32 * NE;
   // With eight epilogue warps (BN = 256) a thread has 168 registers, too few for
@@ -447,7 +449,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GShape<BN>::Threads,
     const int quarter = warp & 3;     // tensor-memory lanes 32*quarter .. +31
     const int cpart = ew >> 2;        // column part: columns cpart*CW .. +CW-1
     const int row = quarter * 32 + lane;
-    float* cs = reinterpret_cast<float*>(base + Sh::OffScale) + ew * CW;
+    float* cs = reinterpret_cast<float*>(base + Sh::OffStage + ew * 4096);
     const uint32_t ae = lead_bar(&bars->acc_empty[0]);
     int buf = 0;
     uint32_t aphase = 0;
@@ -517,36 +519,59 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GShape<BN>::Threads,
         }
       }
       if (!ok) break;
-      if (grow < a.M && gc0 < a.N) {
-        if (work.slot >= 0) {  // a piece of a tile, to be summed by gemm_parts_kernel
-          float4* wrow = reinterpret_cast<float4*>(
-              a.work + ((int64_t)work.slot * kGBM + rank * 128 + row) * BN + cpart * CW);
+      // A thread holds a row, memory wants lines: blocks of 32 x 32 go through shared
+      // memory (16-byte unit u of row r at u ^ (r & 7)), so that a store writes four
+      // whole lines, not 16 bytes of 32 (or, for D whose rows are not on 16-byte units,
+      // 4): 8192 x 8192 x 1024 313 -> 264 us.
+      if (gc0 < a.N) {
+        float4* stg = reinterpret_cast<float4*>(cs);
+        const int wrow0 = (int)rank * 128 + quarter * 32;
+        const int r0 = mb * kGBM + wrow0;
+        const bool add_c = a.C && a.beta != 0.f;
 #pragma unroll
-          for (int j = 0; j < CW / 4; ++j)
-            wrow[j] = make_float4(acc[2 * j].x, acc[2 * j].y, acc[2 * j + 1].x, acc[2 * j + 1].y);
-        } else {
-          float* drow = a.D + (int64_t)grow * a.ldd + gc0;
-          const float* crow = (a.C && a.beta != 0.f) ? a.C + (int64_t)grow * a.ldc + gc0 : nullptr;
-          if (a.vec_ok && gc0 + CW <= a.N) {
+        for (int q = 0; q < CW / 32; ++q) {
+          __syncwarp();
 #pragma unroll
-            for (int j = 0; j < CW / 4; ++j) {
-              float4 o = make_float4(a.alpha * acc[2 * j].x, a.alpha * acc[2 * j].y,
-                                     a.alpha * acc[2 * j + 1].x, a.alpha * acc[2 * j + 1].y);
-              if (crow) {
-                const float4 c = *reinterpret_cast<const float4*>(crow + 4 * j);
+          for (int u = 0; u < 8; ++u) {
+            const float2 x = acc[q * 16 + 2 * u], y = acc[q * 16 + 2 * u + 1];
+            stg[lane * 8 + (u ^ (lane & 7))] = make_float4(x.x, x.y, y.x, y.y);
+          }
+          __syncwarp();
+          const int col = gc0 + q * 32;
+          if (work.slot >= 0 || (a.vec_ok && col + 32 <= a.N)) {
+#pragma unroll 2
+            for (int it = 0; it < 8; ++it) {
+              const int r = it * 4 + (lane >> 3);
+              float4 o = stg[r * 8 + ((lane & 7) ^ (r & 7))];
+              if (r0 + r >= a.M) continue;
+              if (work.slot >= 0) {  // a piece of a tile, to be summed by gemm_parts_kernel
+                *reinterpret_cast<float4*>(
+                    a.work + ((int64_t)work.slot * kGBM + wrow0 + r) * BN + cpart * CW + q * 32 +
+                    4 * (lane & 7)) = o;
+                continue;
+              }
+              o.x *= a.alpha;
+              o.y *= a.alpha;
+              o.z *= a.alpha;
+              o.w *= a.alpha;
+              if (add_c) {
+                const float4 c = *reinterpret_cast<const float4*>(
+                    a.C + (int64_t)(r0 + r) * a.ldc + col + 4 * (lane & 7));
                 o.x += a.beta * c.x;
                 o.y += a.beta * c.y;
                 o.z += a.beta * c.z;
                 o.w += a.beta * c.w;
               }
-              *reinterpret_cast<float4*>(drow + 4 * j) = o;
+              *reinterpret_cast<float4*>(a.D + (int64_t)(r0 + r) * a.ldd + col + 4 * (lane & 7)) = o;
             }
           } else {
-#pragma unroll
-            for (int j = 0; j < CW; ++j) {
-              if (gc0 + j < a.N)
-                drow[j] = a.alpha * (j & 1 ? acc[j / 2].y : acc[j / 2].x) +
-                          (crow ? a.beta * crow[j] : 0.f);
+#pragma unroll 4
+            for (int r = 0; r < 32; ++r) {
+              if (r0 + r >= a.M || col + lane >= a.N) continue;
+              float o = a.alpha * reinterpret_cast<const float*>(
+                                      stg)[r * 32 + (((lane >> 2) ^ (r & 7)) << 2) + (lane & 3)];
+              if (add_c) o += a.beta * a.C[(int64_t)(r0 + r) * a.ldc + col + lane];
+              a.D[(int64_t)(r0 + r) * a.ldd + col + lane] = o;
             }
           }
         }
@@ -872,12 +897,13 @@ __global__ void gemm_reduce_kernel(int M, int N, int splits, int batch, T alpha,
 // tile, the pieces in their order along K.  SPLIT (ROWS = 64 = BN, every tile cut): D's
 // columns also go to the split operand ``nx``, a run of 64 rows per CTA and column.
 // Bound by the latency of its few CTAs (128 at 8192 rows x 64 columns: 2 MB of D, 8 MB of
-// pieces from L2); the split inside it saves the launches of a split of its own: the
-// adjoint of 16 rounds at 8192 x 64 1445 -> 1394 us.
+// pieces from L2), so a thread has four values and every piece's load in flight (four
+// times the rows per thread: 10.1 us against 7.8); the split inside it saves the launches
+// of a split of its own: the adjoint of 16 rounds at 8192 x 64 1445 -> 1394 us.
 template <int BN, int ROWS, bool SPLIT>
-__global__ void __launch_bounds__(256) gemm_parts_kernel(const GArgs a, int tiles,
-                                                         const __grid_constant__ SplitOp nx,
-                                                         unsigned* nx_flag) {
+__global__ void __launch_bounds__(ROWS * BN / 4)
+    gemm_parts_kernel(const GArgs a, int tiles, const __grid_constant__ SplitOp nx,
+                      unsigned* nx_flag) {
   __shared__ float tile[SPLIT ? ROWS : 1][SPLIT ? BN + 1 : 1];
   __shared__ int rowcnt[SPLIT ? BN : 1][2], colcnt[2][SPLIT ? ROWS : 1];
   griddep_wait();
@@ -897,38 +923,39 @@ __global__ void __launch_bounds__(256) gemm_parts_kernel(const GArgs a, int tile
   int mb, nb;
   g_tile(a.dp + r, (a.M + kGBM - 1) / kGBM, (a.N + BN - 1) / BN, mb, nb);
   const int row0 = blockIdx.y * ROWS;
-  for (int e = threadIdx.x; e < ROWS * BN / 4; e += 256) {
-    const int row = row0 + e / (BN / 4), col = e % (BN / 4) * 4;
-    const int m = mb * kGBM + row, n = nb * BN + col;
-    float v[4] = {0.f, 0.f, 0.f, 0.f};
-    if (m < a.M && n < a.N) {
-      if (!whole) {
-        const float* w = a.work + ((int64_t)(c0 + r) * kGBM + row) * BN + col;
-        float4 s = *reinterpret_cast<const float4*>(w);
-#pragma unroll 4
-        for (int c = c0 + 1; c <= c1; ++c) {
-          const float4 x =
-              *reinterpret_cast<const float4*>(w + (int64_t)(c - c0) * kGBM * BN);
-          s.x += x.x;
-          s.y += x.y;
-          s.z += x.z;
-          s.w += x.w;
-        }
-        v[0] = s.x; v[1] = s.y; v[2] = s.z; v[3] = s.w;
-        for (int j = 0; j < 4 && n + j < a.N; ++j) {
-          float o = a.alpha * v[j];
-          if (a.C && a.beta != 0.f) o += a.beta * a.C[(int64_t)m * a.ldc + n + j];
-          a.D[(int64_t)m * a.ldd + n + j] = o;
-          v[j] = o;
-        }
-      } else {
-        for (int j = 0; j < 4 && n + j < a.N; ++j) v[j] = a.D[(int64_t)m * a.ldd + n + j];
+  const int e = threadIdx.x, lrow = e / (BN / 4), col = e % (BN / 4) * 4;
+  const int row = row0 + lrow, m = mb * kGBM + row, n = nb * BN + col;
+  float v[4] = {0.f, 0.f, 0.f, 0.f};
+  if (m < a.M && n < a.N) {
+    float* d = a.D + (int64_t)m * a.ldd + n;
+    const bool vec = a.vec_ok && n + 4 <= a.N;
+    if (!whole) {
+      const float* w = a.work + ((int64_t)(c0 + r) * kGBM + row) * BN + col;
+      float4 s = *reinterpret_cast<const float4*>(w);
+#pragma unroll 8
+      for (int c = c0 + 1; c <= c1; ++c) {
+        const float4 x = *reinterpret_cast<const float4*>(w + (int64_t)(c - c0) * kGBM * BN);
+        s.x += x.x;
+        s.y += x.y;
+        s.z += x.z;
+        s.w += x.w;
       }
+      v[0] = a.alpha * s.x; v[1] = a.alpha * s.y; v[2] = a.alpha * s.z; v[3] = a.alpha * s.w;
+      if (a.C && a.beta != 0.f) {
+        const float* cp = a.C + (int64_t)m * a.ldc + n;
+        for (int j = 0; j < 4 && n + j < a.N; ++j) v[j] += a.beta * cp[j];
+      }
+      if (vec)
+        *reinterpret_cast<float4*>(d) = make_float4(v[0], v[1], v[2], v[3]);
+      else
+        for (int j = 0; j < 4 && n + j < a.N; ++j) d[j] = v[j];
+    } else {
+      for (int j = 0; j < 4 && n + j < a.N; ++j) v[j] = d[j];
     }
-    if constexpr (SPLIT) {
+  }
+  if constexpr (SPLIT) {
 #pragma unroll
-      for (int j = 0; j < 4; ++j) tile[e / (BN / 4)][col + j] = n + j < a.N ? v[j] : 0.f;
-    }
+    for (int j = 0; j < 4; ++j) tile[lrow][col + j] = n + j < a.N ? v[j] : 0.f;
   }
   if constexpr (SPLIT) {
     if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *nx.fmt = 0u;
@@ -937,16 +964,14 @@ __global__ void __launch_bounds__(256) gemm_parts_kernel(const GArgs a, int tile
     __syncthreads();
     const int kp = (nx.K + 63) / 64 * 64, k0 = mb * kGBM + row0;
     bool bad = false;
-#pragma unroll
-    for (int u = 0; u < BN * ROWS / (8 * 256); ++u) {
-      const int idx = u * 256 + threadIdx.x;
-      const int i = idx / (ROWS / 8), kl = idx % (ROWS / 8) * 8, k = k0 + kl;
+    if (e < BN * ROWS / 8) {  // whole warps
+      const int i = e / (ROWS / 8), kl = e % (ROWS / 8) * 8, k = k0 + kl;
       float x[8];
 #pragma unroll
-      for (int e = 0; e < 8; ++e) x[e] = tile[kl + e][i];  // zeros past D
-      bad |= split_run(x, nx, i, k, i < nx.rows && k < kp, kp, [&](int e) {
-        atomicAdd(&rowcnt[i][(kl + e) / 32], 1);
-        atomicAdd(&colcnt[i / 32][kl + e], 1);
+      for (int j = 0; j < 8; ++j) x[j] = tile[kl + j][i];  // zeros past D
+      bad = split_run(x, nx, i, k, i < nx.rows && k < kp, kp, [&](int j) {
+        atomicAdd(&rowcnt[i][(kl + j) / 32], 1);
+        atomicAdd(&colcnt[i / 32][kl + j], 1);
       });
     }
     __syncthreads();
@@ -980,12 +1005,13 @@ cudaError_t launch_tc_gemm_t(const GMaps& maps, const GArgs& a, const SplitOp* n
   if constexpr (BN == 64) {
     if (next && a.dp == 0 && a.N <= BN) {
       *did = true;
-      return launch_pdl(gemm_parts_kernel<BN, 64, true>, dim3(tiles, kGBM / 64), 256, 0, s, a,
-                        tiles, *next, next_flag);
+      return launch_pdl(gemm_parts_kernel<BN, 64, true>, dim3(tiles, kGBM / 64), 1024, 0, s,
+                        a, tiles, *next, next_flag);
     }
   }
-  return launch_pdl(gemm_parts_kernel<BN, 16, false>, dim3(tiles - a.dp, kGBM / 16), 256, 0, s, a,
-                    tiles, SplitOp{}, nullptr);
+  constexpr int kRows = 1024 / BN;  // four values per thread
+  return launch_pdl(gemm_parts_kernel<BN, kRows, false>, dim3(tiles - a.dp, kGBM / kRows), 256, 0,
+                    s, a, tiles, SplitOp{}, nullptr);
 }
 
 // A split operand as lines of 128 bytes (64 FP16 or 32 TF32 values), boxes of
