@@ -435,6 +435,35 @@ static linview_status run_fused(linview_program* p, const View& v, int mode, int
   return LINVIEW_OK;
 }
 
+// X (n x r, column stride xs) = P Xf as a link of a chain of products with one view: whole
+// rows at a time where the factors of a row fit the registers (FP32, r <= 4), else a pass of
+// column strips and the sum of its partial sets.  An update of the linear iteration,
+// strips -> rows: n = 8192, p = 64 rank 2 709 -> 647 us, rank 1 678 -> 659; n = 4096 rank 2
+// 214 -> 200; n = 2000 rank 4 105 -> 102; n = 1000 rank 2 63.5 -> 57.3; n = 300 rank 1 53.0
+// -> 53.3.  Four columns past n = 4096 take twice the registers and lose (n = 8192 748 ->
+// 939).  The exponential and skip models run theirs beside the panel kernels of other
+// streams, which the rows' CTAs keep off the SMs (n = 4096, p = 1024 559 -> 586 us): they
+// stay on the strips.
+template <typename T>
+static linview_status view_product(linview_program* p, const View& v, int r, const T* Xf, T* X,
+                                   int64_t xs, cudaStream_t s, bool reverse = false) {
+  const int n = (int)v.rows;
+  if constexpr (sizeof(T) == 4) {
+    if (row_products_fit(v.ptr, v.ld, n, r)) {
+      ProfScope ps(p, s, (double)n * (double)n * sizeof(T), 1);
+      LV_CUDA(launch_row_products(static_cast<const float*>(v.ptr), v.ld, Xf, p->fs, n, r, X, xs,
+                                  reverse, p->sms, p->status, s));
+      return LINVIEW_OK;
+    }
+  }
+  LV_TRY(run_fused<T>(p, v, kModeX, r, Xf, nullptr, nullptr, nullptr, p->Xpart, p->Ypart, s,
+                      nullptr, reverse));
+  ProfScope ps(p, s, 0.0);
+  LV_CUDA(launch_sum_partials<T>(static_cast<T*>(p->Xpart), fused_geom(sizeof(T), n, p->sms).gC,
+                                 p->xp_s, p->part_cs, n, r, X, xs, s));
+  return LINVIEW_OK;
+}
+
 // A view pass that follows another one over the same view (same row ranges
 // per CTA) runs in the opposite row order (reverse), so that it starts on the
 // rows that are still in L2; blocks of one update alternate in the same way.
@@ -857,21 +886,18 @@ static linview_status view_panel_product(linview_program* p, const View& v, bool
   const int64_t fs = rup(n, 64);
   T* xcm = static_cast<T*>(p->gwork);
   T* ocm = xcm + fs * nc;
-  const PassGeom g = fused_geom(sizeof(T), n, p->sms);
   const int64_t fs_prog = p->fs;
   p->fs = fs;  // the staged factor's column stride
   LV_CUDA(launch_rm_to_cm<T>(X, ldx, xcm, fs, n, nc, s));
   const linview_status st =
-      run_fused<T>(p, v, transpose ? kModeXY : kModeX, nc, xcm, transpose ? xcm : nullptr,
-                   nullptr, nullptr, p->Xpart, p->Ypart, s);
+      transpose ? run_fused<T>(p, v, kModeXY, nc, xcm, xcm, nullptr, nullptr, p->Xpart, p->Ypart, s)
+                : view_product<T>(p, v, nc, xcm, ocm, fs, s);
   p->fs = fs_prog;
   LV_TRY(st);
   if (transpose)
-    LV_CUDA(launch_sum_partials<T>(static_cast<const T*>(p->Ypart), g.gR, p->yp_q, p->part_cs, n,
-                                   nc, ocm, fs, s));
-  else
-    LV_CUDA(launch_sum_partials<T>(static_cast<const T*>(p->Xpart), g.gC, p->xp_s, p->part_cs, n,
-                                   nc, ocm, fs, s));
+    LV_CUDA(launch_sum_partials<T>(static_cast<const T*>(p->Ypart),
+                                   fused_geom(sizeof(T), n, p->sms).gR, p->yp_q, p->part_cs, n, nc,
+                                   ocm, fs, s));
   // column-major n x nc -> row-major: the transpose of an nc x n row-major block
   if (add && add == out) {  // out += op(view) X: transpose into the scratch, then add
     T* rm = ocm + fs * nc;  // row-major n x nc, ld nc
@@ -1624,11 +1650,8 @@ static linview_status iter_propagate(linview_program* p, int r, cudaStream_t s) 
     }
     // the k - 1 passes over A alternate their row order (j = 1 was forward)
     for (int j = 2; j < k; ++j) {
-      LV_TRY(run_fused<T>(p, a, kModeX, r, K + (int64_t)(j - 1) * r * fs, nullptr, nullptr,
-                          nullptr, p->Xpart, p->Ypart, s, nullptr, j % 2 == 0));
-      ProfScope ps(p, s, 0.0);
-      LV_CUDA(launch_sum_partials<T>(static_cast<T*>(p->Xpart), g.gC, p->xp_s, p->part_cs, n, r,
-                                     K + (int64_t)j * r * fs, fs, s));
+      LV_TRY(view_product<T>(p, a, r, K + (int64_t)(j - 1) * r * fs, K + (int64_t)j * r * fs, fs,
+                             s, j % 2 == 0));
     }
   } else {
     LV_TRY(run_update<T>(p, a, K, V1, r, s));
@@ -1654,16 +1677,12 @@ static linview_status iter_propagate_b(linview_program* p, int rb, cudaStream_t 
   T* M = static_cast<T*>(p->Mr);
   char* Tp = static_cast<char*>(p->Tpanel);
   View& a = p->views[0];
-  const PassGeom g = fused_geom(sizeof(T), n, p->sms);
   for (int i = 1; i < k; ++i)
     LV_CUDA(cudaMemcpyAsync(M + (int64_t)i * rb * pp, M, sizeof(T) * rb * pp,
                             cudaMemcpyDeviceToDevice, s));
   for (int j = 1; j < k; ++j) {
-    LV_TRY(run_fused<T>(p, a, kModeX, rb, K + (int64_t)(j - 1) * rb * fs, nullptr, nullptr,
-                        nullptr, p->Xpart, p->Ypart, s, nullptr, j % 2 == 0));
-    ProfScope ps(p, s, 0.0);
-    LV_CUDA(launch_sum_partials<T>(static_cast<T*>(p->Xpart), g.gC, p->xp_s, p->part_cs, n, rb,
-                                   K + (int64_t)j * rb * fs, fs, s));
+    LV_TRY(view_product<T>(p, a, rb, K + (int64_t)(j - 1) * rb * fs, K + (int64_t)j * rb * fs, fs,
+                           s, j % 2 == 0));
   }
   // T_i += [K_0 .. K_{i-1}] [V_b .. V_b]^T for every i (every M block is V_b)
   LV_TRY(panel_update<T>(p, Tp, K, M, k, rb, true, s));

@@ -197,6 +197,13 @@ template <typename T>
 cudaError_t launch_update(const PassParams& p, const CUtensorMap& tm, int R, cudaStream_t s,
                           bool programmatic = true);
 
+// X (n x r, column stride xs) = P F for an n x n FP32 view and a few columns (lv_rows.cu),
+// without partial sums.  As for the passes, the kernel launched before must not write P.
+bool row_products_fit(const void* P, int64_t ldp, int n, int r);
+cudaError_t launch_row_products(const float* P, int64_t ldp, const float* F, int64_t fs, int n,
+                                int r, float* X, int64_t xs, bool reverse, int num_sms,
+                                unsigned* status, cudaStream_t s);
+
 // Factor cores and assembly (lv_core.cu).
 // C (r x r, FP64, row-major) = V^T U over n rows; deterministic two-level
 // reduction using Cpart (grid x r*r doubles) and a ticket counter.  FP32
