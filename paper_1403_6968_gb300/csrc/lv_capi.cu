@@ -131,6 +131,7 @@ struct linview_program {
   CUtensorMap tmA, tmB;
   // a second set for the sums updates on the side stream (wide sums only)
   float* tpF = nullptr;  // split factor of the tensor-core products pass (128 x fs floats)
+  float* tpF2 = nullptr;  // ... and V's, where X and Y of a level are split together
   int xslots = 0, yslots = 0;  // partial sets Xpart / Ypart hold
   int pc_x = 0, pc_y = 0;      // partial sets the last products pass wrote
   float* tcA2 = nullptr;
@@ -230,6 +231,9 @@ struct linview_program {
   // stream of the factor cores of wide levels (core_fork)
   cudaStream_t core = nullptr;
   cudaEvent_t core_fork_ev = nullptr, core_join_ev = nullptr;
+  // stream of the Y products of a small view's wide level (level_products)
+  cudaStream_t prod = nullptr;
+  cudaEvent_t prod_fork_ev = nullptr, prod_join_ev = nullptr;
   struct Rec {
     cudaEvent_t e0, e1;
     int kind;
@@ -520,6 +524,54 @@ static linview_status run_update(linview_program* p, const View& v, const T* Uu,
   return LINVIEW_OK;
 }
 
+static linview_status branch_stream(cudaStream_t* st, cudaEvent_t* fork, cudaEvent_t* join) {
+  if (*st) return LINVIEW_OK;
+  LV_CUDA(cudaEventCreateWithFlags(fork, cudaEventDisableTiming));
+  LV_CUDA(cudaEventCreateWithFlags(join, cudaEventDisableTiming));
+  LV_CUDA(cudaStreamCreateWithFlags(st, cudaStreamNonBlocking));
+  return LINVIEW_OK;
+}
+
+// A wide level of the exponential model on the tensor cores: X = P U, Y = P^T V (in
+// ``parts`` partial sets each), then P += U V^T.  All splits of U and V are one launch.  A
+// small view's products pass has fewer CTAs than SMs (n = 1000: 56), and X and Y only read,
+// so Y then runs beside X on a stream of its own.  An update of A^16, three splits and one
+// pass after the other -> so: n = 300 rank 3 59 -> 54 us, n = 700 rank 8 117 -> 102, n = 1000
+// rank 3 75 -> 70, n = 2048 rank 8 192 -> 184; in order past n = 2688: n = 3000 rank 5 243 ->
+// 227, n = 4096 rank 4 265 -> 257, n = 8192 with sums rank 4 1148 -> 1142.
+static linview_status level_products(linview_program* p, const View& v, int r, const float* U,
+                                     const float* V, int parts, cudaStream_t s) {
+  const int n = (int)v.rows;
+  const double nn = (double)n * (double)n * sizeof(float);
+  const bool tc = p->tcA && r > kMaxProductR;  // the update's form
+  LV_CUDA(launch_level_split(U, V, p->fs, n, r, p->tpF, p->tpF2, tc ? p->tcA : nullptr,
+                             tc ? p->tcB : nullptr, s));
+  p->all_launches++;
+  cudaStream_t y = s;
+  if (!p->prof && tp_leaves_sms(n, p->sms)) {
+    LV_TRY(branch_stream(&p->prod, &p->prod_fork_ev, &p->prod_join_ev));
+    LV_CUDA(cudaEventRecord(p->prod_fork_ev, s));
+    LV_CUDA(cudaStreamWaitEvent(p->prod, p->prod_fork_ev, 0));
+    y = p->prod;
+  }
+  for (int t = 0; t < 2; ++t) {
+    ProfScope ps(p, t ? y : s, nn, 1);
+    LV_CUDA(launch_tc_products(t == 1, static_cast<const float*>(v.ptr), v.ld, nullptr, p->fs,
+                               t ? p->tpF2 : p->tpF, n, r,
+                               static_cast<float*>(t ? p->Ypart : p->Xpart), t ? p->yp_q : p->xp_s,
+                               p->part_cs, parts, p->sms, p->status, t ? y : s));
+  }
+  if (y != s) {
+    LV_CUDA(cudaEventRecord(p->prod_join_ev, y));
+    LV_CUDA(cudaStreamWaitEvent(s, p->prod_join_ev, 0));
+  }
+  if (!tc) return run_update<float>(p, v, U, V, r, s);
+  ProfScope ps(p, s, 2.0 * nn, 2);
+  LV_CUDA(launch_tc_update(v.tmap_tc, p->tmA, p->tmB, static_cast<float*>(v.ptr), v.ld, p->tcA,
+                           p->tcB, U, V, p->fs, n, r, p->sms, p->status, s, /*presplit=*/true));
+  return LINVIEW_OK;
+}
+
 // Products X = P Xf, Y = P^T Yf for any width r (chunks of kMaxProductR in
 // FP32, kMaxFusedR in FP64) into
 // the program's partial buffers (column block c0 at column offset c0), then
@@ -549,6 +601,11 @@ static linview_status run_products_update(linview_program* p, const View& v, int
     const int parts = tp_parts(n, p->sms);  // partial sets the pass writes
     if (allow_tc && p->tpF && v.square && r > tp_min_r(n) && parts <= p->xslots &&
         (!want_y || parts <= p->yslots) && (v.ld * 4) % 16 == 0 && p->fs % 64 == 0) {
+      if (p->tpF2 && want_y && Uu == Xf && Wu == Yf && r <= kMaxTcR) {
+        p->pc_x = p->pc_y = parts;
+        return level_products(p, v, r, reinterpret_cast<const float*>(Xf),
+                              reinterpret_cast<const float*>(Yf), parts, s);
+      }
       const double nn = (double)n * (double)n * sizeof(float);
       for (int c0 = 0; c0 < r; c0 += kMaxTcR) {
         const int w = (r - c0 < kMaxTcR) ? (r - c0) : kMaxTcR;
@@ -1154,7 +1211,7 @@ static int64_t powers_device_bytes(const linview_program_desc& d, int sms) {
   b += alloc_bytes(xs * half * fs * elem) + alloc_bytes(ys * half * fs * elem);
   b += alloc_bytes(2 * n * d.r_max * elem);
   if (powers_uses_tc(d)) b += alloc_bytes(tc_split_floats(n) * 4) * (powers_wide_sums(d) ? 2 : 1);
-  if (tp) b += alloc_bytes(128 * fs * 4);
+  if (tp) b += alloc_bytes(256 * fs * 4);
   return b;
 }
 
@@ -1201,8 +1258,9 @@ static linview_status powers_create(linview_program* p, const void* const* input
   LV_TRY(dalloc(p, (size_t)p->yslots * p->yp_q * p->elem, &p->Ypart, s));
   if (tp) {
     void* t = nullptr;
-    LV_TRY(dalloc(p, sizeof(float) * 128 * p->fs, &t, s));
+    LV_TRY(dalloc(p, sizeof(float) * 256 * p->fs, &t, s));
     p->tpF = static_cast<float*>(t);
+    p->tpF2 = p->tpF + 128 * p->fs;
   }
   // host-side update factors are staged here (allocated now so that an
   // update never allocates)
@@ -1249,14 +1307,6 @@ static linview_status sums_update_on(linview_program* p, View& sv, const T* U, c
 // The view passes of the two streams then fill each other's ramps and tails,
 // and an HBM-bound sums pass can use the bandwidth a compute-bound level pass
 // leaves idle.  (Inside a graph capture the fork and join become edges.)
-static linview_status branch_stream(cudaStream_t* st, cudaEvent_t* fork, cudaEvent_t* join) {
-  if (*st) return LINVIEW_OK;
-  LV_CUDA(cudaEventCreateWithFlags(fork, cudaEventDisableTiming));
-  LV_CUDA(cudaEventCreateWithFlags(join, cudaEventDisableTiming));
-  LV_CUDA(cudaStreamCreateWithFlags(st, cudaStreamNonBlocking));
-  return LINVIEW_OK;
-}
-
 static linview_status side_fork(linview_program* p, cudaStream_t s, cudaStream_t* out) {
   LV_TRY(branch_stream(&p->side, &p->side_fork_ev, &p->side_join_ev));
   LV_CUDA(cudaEventRecord(p->side_fork_ev, s));
@@ -2709,6 +2759,9 @@ void linview_destroy(linview_program* p) {
   if (p->core_fork_ev) cudaEventDestroy(p->core_fork_ev);
   if (p->core_join_ev) cudaEventDestroy(p->core_join_ev);
   if (p->core) cudaStreamDestroy(p->core);
+  if (p->prod_fork_ev) cudaEventDestroy(p->prod_fork_ev);
+  if (p->prod_join_ev) cudaEventDestroy(p->prod_join_ev);
+  if (p->prod) cudaStreamDestroy(p->prod);
   if (p->blas) cublasDestroy(p->blas);
   if (p->solver) cusolverDnDestroy(p->solver);
   delete p;

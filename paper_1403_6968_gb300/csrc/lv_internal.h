@@ -107,11 +107,18 @@ constexpr int kTpMaxParts = 8;  // K parts (partial sums) of a tensor-core produ
 // row ranges; ``parts`` = tp_parts(n, num_sms) partial sets, every one
 // written.  Partial q, factor column c, output row i lands at
 // out[q ps + c cs + i].  F column-major (column stride fs, a multiple of 64,
-// >= n); Fsplit is scratch of 128 x fs floats (the split factor).
+// >= n); Fsplit is scratch of 128 x fs floats (the split factor; F null: it is there
+// already, see launch_level_split).
 cudaError_t launch_tc_products(bool transpose, const float* P, int64_t ldp, const float* F,
                                int64_t fs, float* Fsplit, int n, int r, float* out, int64_t ps,
                                int64_t cs, int parts, int num_sms, unsigned* status,
                                cudaStream_t s);
+// The splits of a level's factors in one launch: U and V for the products passes (FU, FV,
+// 128 x fs floats each) and, where Acat is given, both for the update P += U V^T.
+cudaError_t launch_level_split(const float* U, const float* V, int64_t fs, int n, int r, float* FU,
+                               float* FV, float* Acat, float* Bcat, cudaStream_t s);
+// whether a products pass over an n x n view has fewer CTAs than the GPU has SMs
+bool tp_leaves_sms(int n, int num_sms);
 // Blocks wider than this run on the tensor-core products pass, two passes over the
 // view and two splits of the factor; narrower ones on the CUDA cores in one pass.
 // The CUDA-core pass is bound by its issue slots at 9 - 16 columns: n = 8192 145 us

@@ -403,15 +403,12 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 // or 64: the columns the variant reads), zero past r.  A block of 256
 // threads transposes 32 rows through shared memory: reads run down the
 // factor columns, writes along the rows.
-__global__ void __launch_bounds__(256) tc_split_kernel(const float* __restrict__ U,
-                                                       const float* __restrict__ W, int64_t fs,
-                                                       int n, int r, int half,
-                                                       float* __restrict__ Acat,
-                                                       float* __restrict__ Bcat) {
-  griddep_wait();
-  griddep_launch_dependents();
+__device__ __forceinline__ void tc_split_rows(int block, const float* __restrict__ U,
+                                              const float* __restrict__ W, int64_t fs, int n,
+                                              int r, int half, float* __restrict__ Acat,
+                                              float* __restrict__ Bcat) {
   __shared__ float su[64][33], sw[64][33];
-  const int row0 = blockIdx.x * 32;
+  const int row0 = block * 32;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 8 warps
   for (int c = ty; c < half; c += 8) {
     const int i = row0 + tx;
@@ -435,6 +432,16 @@ __global__ void __launch_bounds__(256) tc_split_kernel(const float* __restrict__
       b[64 + c] = w - wh;
     }
   }
+}
+
+__global__ void __launch_bounds__(256) tc_split_kernel(const float* __restrict__ U,
+                                                       const float* __restrict__ W, int64_t fs,
+                                                       int n, int r, int half,
+                                                       float* __restrict__ Acat,
+                                                       float* __restrict__ Bcat) {
+  griddep_wait();
+  griddep_launch_dependents();
+  tc_split_rows(blockIdx.x, U, W, fs, n, r, half, Acat, Bcat);
 }
 
 // ---------------------------------------------------------------------------
@@ -831,17 +838,44 @@ __global__ void __launch_bounds__(TpShape<TR, RP>::Threads, 1)
 // Factor split for the products passes: F (128 rows x fs) row c = hi(Fin
 // column c) for c < r, 0 for r <= c < rp; row 64 + c = the low part.  Fin is
 // column-major (column stride fs), n rows.
-__global__ void tp_split_kernel(const float* __restrict__ Fin, int64_t fs, int n, int r, int rp,
-                                float* __restrict__ F) {
-  griddep_wait();
-  griddep_launch_dependents();
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void tp_split_block(int block, const float* __restrict__ Fin,
+                                               int64_t fs, int n, int r, int rp,
+                                               float* __restrict__ F) {
+  const int64_t idx = (int64_t)block * blockDim.x + threadIdx.x;
   if (idx >= (int64_t)rp * n) return;
   const int c = (int)(idx / n), i = (int)(idx % n);
   const float x = c < r ? Fin[(int64_t)c * fs + i] : 0.f;
   const float h = tf32_rn(x);
   F[(int64_t)c * fs + i] = h;
   F[(int64_t)(64 + c) * fs + i] = x - h;
+}
+
+__global__ void tp_split_kernel(const float* __restrict__ Fin, int64_t fs, int n, int r, int rp,
+                                float* __restrict__ F) {
+  griddep_wait();
+  griddep_launch_dependents();
+  tp_split_block(blockIdx.x, Fin, fs, n, r, rp, F);
+}
+
+// All the splits of a level in one launch: U and V for the two products passes, then (tc > 0
+// CTAs) the update pass's form of both.  They read the same factors, and each as a launch of
+// its own was a link of the level's chain (2.5 - 4 us, three a level).
+__global__ void __launch_bounds__(256) level_split_kernel(const float* __restrict__ U,
+                                                          const float* __restrict__ V, int64_t fs,
+                                                          int n, int r, int rp, int tp, int half,
+                                                          float* __restrict__ FU,
+                                                          float* __restrict__ FV,
+                                                          float* __restrict__ Acat,
+                                                          float* __restrict__ Bcat) {
+  griddep_wait();
+  griddep_launch_dependents();
+  const int b = blockIdx.x;
+  if (b < tp)
+    tp_split_block(b, U, fs, n, r, rp, FU);
+  else if (b < 2 * tp)
+    tp_split_block(b - tp, V, fs, n, r, rp, FV);
+  else
+    tc_split_rows(b - 2 * tp, U, V, fs, n, r, half, Acat, Bcat);
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
@@ -934,16 +968,30 @@ static cudaError_t launch_tp_t(const CUtensorMap& tmP, const CUtensorMap& tmF, f
   return cudaGetLastError();
 }
 
+static int tp_width(int r) { return r <= 16 ? 16 : (r <= 32 ? 32 : 64); }
+
+cudaError_t launch_level_split(const float* U, const float* V, int64_t fs, int n, int r, float* FU,
+                               float* FV, float* Acat, float* Bcat, cudaStream_t s) {
+  if (r < 1 || r > kMaxTcR || fs % 64 || fs < n) return cudaErrorInvalidValue;
+  const int rp = tp_width(r);
+  const int tp = (int)(((int64_t)rp * n + 255) / 256), tc = Acat ? (n + 31) / 32 : 0;
+  return launch_pdl(level_split_kernel, 2 * tp + tc, 256, 0, s, U, V, fs, n, r, rp, tp,
+                    r <= 32 ? 32 : 64, FU, FV, Acat, Bcat);
+}
+
+bool tp_leaves_sms(int n, int num_sms) { return tp_grid(n, num_sms) < num_sms; }
+
 cudaError_t launch_tc_products(bool transpose, const float* P, int64_t ldp, const float* F,
                                int64_t fs, float* Fsplit, int n, int r, float* out, int64_t ps,
                                int64_t cs, int parts, int num_sms, unsigned* status,
                                cudaStream_t s) {
   if (r < 1 || r > kMaxTcR || parts != tp_parts(n, num_sms) || fs % 64 || fs < n)
     return cudaErrorInvalidValue;
-  const int rp = r <= 16 ? 16 : (r <= 32 ? 32 : 64);
+  const int rp = tp_width(r);
   const int64_t tot = (int64_t)rp * n;
-  LV_LAUNCH(launch_pdl(tp_split_kernel, (unsigned)((tot + 255) / 256), 256, 0, s, F, fs, n, r, rp,
-      Fsplit));
+  if (F)
+    LV_LAUNCH(launch_pdl(tp_split_kernel, (unsigned)((tot + 255) / 256), 256, 0, s, F, fs, n, r, rp,
+        Fsplit));
   CUtensorMap tmP, tmF;
   // P: boxes of 32 columns x 128 rows (X) or 32 x 32 (Y); F: 32 columns of
   // K x rp factor rows (hi at row 0, lo at row 64)
