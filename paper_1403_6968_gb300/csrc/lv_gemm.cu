@@ -630,14 +630,22 @@ __device__ __forceinline__ bool split_run(const float (&x)[8], const SplitOp& o,
   const bool bad = sh > 60 || sh < -60;  // (non-finite: sh = -114)
   sh = min(60, max(-60, sh));
   const float sc = pow2f(sh);
-  __align__(16) __half hi[8], lo[8];
+  // pairs: one conversion instruction per two values; the rare small entries behind one branch
+  __align__(16) __half2 hi[4], lo[4];
+  unsigned few = 0;
 #pragma unroll
-  for (int e = 0; e < 8; ++e) {
-    const float y = x[e] * sc;
-    hi[e] = __float2half_rn(y);
-    lo[e] = __float2half_rn(y - __half2float(hi[e]));
-    if (y != 0.f && fabsf(y) < 0.25f) small(e);
+  for (int e = 0; e < 4; ++e) {
+    const float y0 = x[2 * e] * sc, y1 = x[2 * e + 1] * sc;
+    hi[e] = __floats2half2_rn(y0, y1);
+    const float2 h = __half22float2(hi[e]);
+    lo[e] = __floats2half2_rn(y0 - h.x, y1 - h.y);
+    few |= (y0 != 0.f && fabsf(y0) < 0.25f ? 1u : 0u) << (2 * e);
+    few |= (y1 != 0.f && fabsf(y1) < 0.25f ? 1u : 0u) << (2 * e + 1);
   }
+  if (few)
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+      if (few >> e & 1u) small(e);
   if (in) {
     unsigned char* d = o.dst + block_line(i, k / 64, kp / 64) * 128 + k % 64 * 2;
     *reinterpret_cast<uint4*>(d) = *reinterpret_cast<const uint4*>(hi);
@@ -654,7 +662,9 @@ __device__ __forceinline__ bool split_run(const float (&x)[8], const SplitOp& o,
 // none), a scale outside 2^-60 .. 2^60 or a non-finite entry sets the flag that sends
 // the product to TF32.
 // 8192 x 8192: 101 us transposed, 93 us not, 4 bytes read and 4 written per entry
-// (floor 79); TF32 halves (8 written) took 196 us.
+// (floor 79); TF32 halves (8 written) took 196 us.  Conversions in pairs, the rare small
+// entries behind one branch and a thread's loads issued at once take 3 us off a split inside
+// the adjoint (8192 x 64, 16 rounds: 1310.3 -> 1303.9 us, 1313.8 -> 1310.5 in a second run).
 constexpr int kSpR = 64, kSpK = 128, kSmallCount = 8;
 __global__ void __launch_bounds__(256) split_f16_kernel(const __grid_constant__ SplitPair sp) {
   __shared__ float tile[kSpK][kSpR + 1];
@@ -693,31 +703,39 @@ __global__ void __launch_bounds__(256) split_f16_kernel(const __grid_constant__ 
       for (int e = 0; e < 4; ++e) tile[kl][il + e] = v[e];
     }
   }
-  __syncthreads();
-  bool bad = false;
+  constexpr int NU = kSpR * kSpK / (8 * 256);
+  float x[NU][8];
+  if (o.cs == 1) {  // all loads of a thread in flight at once
 #pragma unroll
-  for (int u = 0; u < kSpR * kSpK / (8 * 256); ++u) {
-    const int idx = u * 256 + tid;
-    const int il = idx / (kSpK / 8), kl = idx % (kSpK / 8) * 8;
-    const int i = i0 + il, k = k0 + kl;
-    const bool in = i < o.rows && k < kp;
-    float x[8];
-    if (o.cs == 1) {
+    for (int u = 0; u < NU; ++u) {
+      const int idx = u * 256 + tid;
+      const int i = i0 + idx / (kSpK / 8), k = k0 + idx % (kSpK / 8) * 8;
+      const bool in = i < o.rows && k < kp;
       const float* row = o.X + (int64_t)i * o.rs + k;
       if (in && o.vec && k + 8 <= o.K) {
         const float4 p = reinterpret_cast<const float4*>(row)[0];
         const float4 q = reinterpret_cast<const float4*>(row)[1];
-        x[0] = p.x; x[1] = p.y; x[2] = p.z; x[3] = p.w;
-        x[4] = q.x; x[5] = q.y; x[6] = q.z; x[7] = q.w;
+        x[u][0] = p.x; x[u][1] = p.y; x[u][2] = p.z; x[u][3] = p.w;
+        x[u][4] = q.x; x[u][5] = q.y; x[u][6] = q.z; x[u][7] = q.w;
       } else {
 #pragma unroll
-        for (int e = 0; e < 8; ++e) x[e] = in && k + e < o.K ? row[e] : 0.f;
+        for (int e = 0; e < 8; ++e) x[u][e] = in && k + e < o.K ? row[e] : 0.f;
       }
-    } else {
-#pragma unroll
-      for (int e = 0; e < 8; ++e) x[e] = tile[kl + e][il];  // zeros past the operand
     }
-    bad |= split_run(x, o, i, k, in, kp, [&](int e) {
+  }
+  __syncthreads();
+  bool bad = false;
+#pragma unroll
+  for (int u = 0; u < NU; ++u) {
+    const int idx = u * 256 + tid;
+    const int il = idx / (kSpK / 8), kl = idx % (kSpK / 8) * 8;
+    const int i = i0 + il, k = k0 + kl;
+    const bool in = i < o.rows && k < kp;
+    if (o.cs != 1) {
+#pragma unroll
+      for (int e = 0; e < 8; ++e) x[u][e] = tile[kl + e][il];  // zeros past the operand
+    }
+    bad |= split_run(x[u], o, i, k, in, kp, [&](int e) {
       atomicAdd(&rowcnt[il][(kl + e) / 32], 1);
       atomicAdd(&colcnt[il / 32][kl + e], 1);
     });
