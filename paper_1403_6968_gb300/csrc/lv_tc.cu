@@ -169,9 +169,11 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 
   const int nrb = (n + kBM - 1) / kBM;
   const int ncb = (n + BN - 1) / BN;
-  const long long T = (long long)nrb * ncb;
-  const long long t0 = T * blockIdx.x / gridDim.x;
-  const long long t1 = T * (blockIdx.x + 1) / gridDim.x;
+  // (32-bit: T gridDim.x < 2^32 up to the largest view that fits the memory, n = 266 K; a
+  // 64-bit division per tile is some hundred cycles of the epilogue)
+  const unsigned T = (unsigned)nrb * ncb;
+  const unsigned t0 = T * blockIdx.x / gridDim.x;
+  const unsigned t1 = T * (blockIdx.x + 1) / gridDim.x;
   const int ntile = (int)(t1 - t0);
 
   if (tid == 0) {
@@ -213,7 +215,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       int cur_rb = -1;
       int b_issued = 0, p_issued = 0, a_issued = 0;  // loads issued (for the abort drain)
       for (int i = 0; i < ntile && !*abort_flag; ++i) {
-        const long long t = t0 + i;
+        const unsigned t = t0 + i;
         const int rb = (int)(t / ncb), cb = (int)(t % ncb);
         const int buf = i & 1, use = i >> 1;
         if (rb != cur_rb) {
@@ -311,7 +313,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     // element instead, so that no column >= n (caller padding) is written.
     const bool ragged = (n & 3) != 0;
     for (int i = 0; i < ntile; ++i) {
-      const long long t = t0 + i;
+      const unsigned t = t0 + i;
       const int rb = (int)(t / ncb), cb = (int)(t % ncb);
       const int buf = i & 1, use = i >> 1;
       const int ps = i % PS, puse = i / PS;
@@ -559,19 +561,22 @@ __global__ void __launch_bounds__(TpShape<TR, RP>::Threads, 1)
   // and the CTA that ends a tile zero-fills the partials past its own.
   const int ot_n = (n + kBM - 1) / kBM;  // output tiles
   const int nkb = (n + 31) / 32;          // K chunks of 32
-  const long long C = (long long)ot_n * nkb;
-  const long long G = gridDim.x;
-  const long long c0 = C * blockIdx.x / G;
-  const long long c1 = C * (blockIdx.x + 1) / G;
+  // (32-bit: C G < 2^32 up to n = 266 K, the largest view that fits the memory.  In 64 bits
+  // the divisions before a range and the ring indices of every chunk cost A^16 at n = 2048,
+  // rank 8 187 -> 181 us, at n = 4096, rank 4 257 -> 253)
+  const unsigned C = (unsigned)ot_n * nkb;
+  const unsigned G = gridDim.x;
+  const unsigned c0 = C * blockIdx.x / G;
+  const unsigned c1 = C * (blockIdx.x + 1) / G;
   // first CTA whose range holds chunk x: the largest b with C b / G <= x
-  auto cta_of = [&](long long x) { return (int)(((x + 1) * G + C - 1) / C - 1); };
+  auto cta_of = [&](unsigned x) { return (int)(((x + 1) * G + C - 1) / C - 1); };
   // segment of the chunk range starting at chunk c: tile, K range, slot
-  auto segment = [&](long long c, int& ot, int& kb0, int& kb1, int& part) {
+  auto segment = [&](unsigned c, int& ot, int& kb0, int& kb1, int& part) {
     ot = (int)(c / nkb);
     kb0 = (int)(c % nkb);
-    const long long tile_end = (long long)(ot + 1) * nkb;
-    kb1 = (int)((c1 < tile_end ? c1 : tile_end) - (long long)ot * nkb);
-    part = (int)blockIdx.x - cta_of((long long)ot * nkb);
+    const unsigned tile_end = (unsigned)(ot + 1) * nkb;
+    kb1 = (int)((c1 < tile_end ? c1 : tile_end) - (unsigned)ot * nkb);
+    part = (int)blockIdx.x - cta_of((unsigned)ot * nkb);
   };
 
   if (tid == 0) {
@@ -608,14 +613,14 @@ __global__ void __launch_bounds__(TpShape<TR, RP>::Threads, 1)
   if (warp == 0) {
     // ---------------- producer ----------------
     if (lane == 0) {
-      long long g = 0, issued = 0;
-      for (long long c = c0; c < c1 && !*abort_flag;) {
+      unsigned g = 0, issued = 0;
+      for (unsigned c = c0; c < c1 && !*abort_flag;) {
         int ot, part, kb0, kb1;
         segment(c, ot, kb0, kb1, part);
         c += kb1 - kb0;
         for (int kb = kb0; kb < kb1 && !*abort_flag; ++kb, ++g) {
           const int st = (int)(g % R);
-          const long long use = g / R;
+          const unsigned use = g / R;
           if (use >= 1 && !tc_wait(TR ? &bars->raw_free[st] : &bars->empty[st],
                                    (uint32_t)((use - 1) & 1), abort_flag, status))
             break;
@@ -638,20 +643,20 @@ __global__ void __launch_bounds__(TpShape<TR, RP>::Threads, 1)
         }
       }
       if (*abort_flag)  // the loads issued land before the CTA exits (bounded)
-        for (long long j = (issued > R ? issued - R : 0); j < issued; ++j)
+        for (unsigned j = (issued > R ? issued - R : 0); j < issued; ++j)
           mbar_wait_bounded(&bars->full[j % R], (uint32_t)((j / R) & 1), nullptr);
     }
   } else if (TR && warp == 2 + NS + 4) {
     // ---------------- factor chunks (Y) ----------------
     if (lane == 0) {
-      long long g = 0, issued = 0;
-      for (long long c = c0; c < c1 && !*abort_flag;) {
+      unsigned g = 0, issued = 0;
+      for (unsigned c = c0; c < c1 && !*abort_flag;) {
         int ot, part, kb0, kb1;
         segment(c, ot, kb0, kb1, part);
         c += kb1 - kb0;
         for (int kb = kb0; kb < kb1 && !*abort_flag; ++kb, ++g) {
           const int st = (int)(g % S);
-          const long long use = g / S;
+          const unsigned use = g / S;
           if (use >= 1 && !tc_wait(&bars->empty[st], (uint32_t)((use - 1) & 1), abort_flag, status))
             break;
           unsigned char* bb = base + st * Sh::StageBytes + Sh::HiBytes + Sh::LoBytes;
@@ -662,20 +667,20 @@ __global__ void __launch_bounds__(TpShape<TR, RP>::Threads, 1)
         }
       }
       if (*abort_flag)
-        for (long long j = (issued > S ? issued - S : 0); j < issued; ++j)
+        for (unsigned j = (issued > S ? issued - S : 0); j < issued; ++j)
           mbar_wait_bounded(&bars->b_full[j % S], (uint32_t)((j / S) & 1), nullptr);
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer (whole warp, one elected lane issues) ----------------
     const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
     const uint64_t s00 = sw128_desc(smem_u32(base));
-    const long long chunks = c1 - c0;
+    const unsigned chunks = c1 - c0;
     int st = 0;
     uint32_t phase = 0;
-    long long g = 0;
+    unsigned g = 0;
     for (; g < chunks; ++g) {
       const int buf = (int)(g % NB);
-      const long long bu = g / NB;
+      const unsigned bu = g / NB;
       const bool ok =
           !*abort_flag && tc_wait(&bars->split[st], phase, abort_flag, status) &&
           (!TR || tc_wait(&bars->b_full[st], phase, abort_flag, status)) &&
@@ -707,15 +712,15 @@ __global__ void __launch_bounds__(TpShape<TR, RP>::Threads, 1)
       }
     }
     if (g < chunks && g > 0 && lane == 0) {
-      const long long j = g - 1;  // aborted: the MMAs issued finish before the TMEM is freed
+      const unsigned j = g - 1;  // aborted: the MMAs issued finish before the TMEM is freed
       mbar_wait_bounded(&bars->acc_full[j % NB], (uint32_t)((j / NB) & 1), nullptr);
     }
   } else if (warp < 2 + NS) {
     // ---------------- split (warps 2 .. 2 + NS - 1) ----------------
     const int st_tid = tid - 64;
-    long long g = 0;
+    unsigned g = 0;
     bool ok = true;
-    for (long long c = c0; c < c1 && ok;) {
+    for (unsigned c = c0; c < c1 && ok;) {
       int ot, part, kb0, kb1;
       segment(c, ot, kb0, kb1, part);
       c += kb1 - kb0;
@@ -783,9 +788,9 @@ __global__ void __launch_bounds__(TpShape<TR, RP>::Threads, 1)
     // ---------------- epilogue (four warps) ----------------
     const int quarter = warp & 3;  // TMEM lanes 32 quarter .. + 31
     const int row = quarter * 32 + lane;
-    long long g = 0;
+    unsigned g = 0;
     bool ok = true;
-    for (long long c = c0; c < c1 && ok;) {
+    for (unsigned c = c0; c < c1 && ok;) {
       int ot, part, kb0, kb1;
       segment(c, ot, kb0, kb1, part);
       c += kb1 - kb0;
@@ -794,7 +799,7 @@ __global__ void __launch_bounds__(TpShape<TR, RP>::Threads, 1)
       for (int c = 0; c < RP; ++c) acc[c] = 0.f;
       for (int kb = kb0; kb < kb1; ++kb, ++g) {
         const int buf = (int)(g % NB);
-        const long long bu = g / NB;
+        const unsigned bu = g / NB;
         ok = tc_wait(&bars->acc_full[buf], (uint32_t)(bu & 1), abort_flag, status);
         if (!__all_sync(0xffffffffu, ok)) { ok = false; break; }
         tc_fence_after();
