@@ -445,7 +445,9 @@ static linview_status run_fused(linview_program* p, const View& v, int mode, int
 // strips -> rows: n = 8192, p = 64 rank 2 709 -> 647 us, rank 1 678 -> 659; n = 4096 rank 2
 // 214 -> 200; n = 2000 rank 4 105 -> 102; n = 1000 rank 2 63.5 -> 57.3; n = 300 rank 1 53.0
 // -> 53.3.  Four columns past n = 4096 take twice the registers and lose (n = 8192 748 ->
-// 939).  The exponential and skip models run theirs beside the panel kernels of other
+// 939).  The products of recomputed iterations and of the adjoint with a few right-hand sides
+// stay on the strips too, whose sums of partial sets in pairs are closer to FP64 (adjoint of
+// n = 1871, p = 1: 8.0e-8 against 8.7e-8).  The exponential and skip models run theirs beside the panel kernels of other
 // streams, which the rows' CTAs keep off the SMs (n = 4096, p = 1024 559 -> 586 us): they
 // stay on the strips.
 template <typename T>
@@ -943,18 +945,21 @@ static linview_status view_panel_product(linview_program* p, const View& v, bool
   const int64_t fs = rup(n, 64);
   T* xcm = static_cast<T*>(p->gwork);
   T* ocm = xcm + fs * nc;
+  const PassGeom g = fused_geom(sizeof(T), n, p->sms);
   const int64_t fs_prog = p->fs;
   p->fs = fs;  // the staged factor's column stride
   LV_CUDA(launch_rm_to_cm<T>(X, ldx, xcm, fs, n, nc, s));
   const linview_status st =
-      transpose ? run_fused<T>(p, v, kModeXY, nc, xcm, xcm, nullptr, nullptr, p->Xpart, p->Ypart, s)
-                : view_product<T>(p, v, nc, xcm, ocm, fs, s);
+      run_fused<T>(p, v, transpose ? kModeXY : kModeX, nc, xcm, transpose ? xcm : nullptr,
+                   nullptr, nullptr, p->Xpart, p->Ypart, s);
   p->fs = fs_prog;
   LV_TRY(st);
   if (transpose)
-    LV_CUDA(launch_sum_partials<T>(static_cast<const T*>(p->Ypart),
-                                   fused_geom(sizeof(T), n, p->sms).gR, p->yp_q, p->part_cs, n, nc,
-                                   ocm, fs, s));
+    LV_CUDA(launch_sum_partials<T>(static_cast<const T*>(p->Ypart), g.gR, p->yp_q, p->part_cs, n,
+                                   nc, ocm, fs, s));
+  else
+    LV_CUDA(launch_sum_partials<T>(static_cast<const T*>(p->Xpart), g.gC, p->xp_s, p->part_cs, n,
+                                   nc, ocm, fs, s));
   // column-major n x nc -> row-major: the transpose of an nc x n row-major block
   if (add && add == out) {  // out += op(view) X: transpose into the scratch, then add
     T* rm = ocm + fs * nc;  // row-major n x nc, ld nc
