@@ -16,10 +16,12 @@ namespace {
 // registers (at most 64), so four view entries cost one 128-bit shared load and 4 R FMAs: the
 // pass is bound by reading the view.  Four rows make a
 // batch: its sums are reduced across the lanes by halving the values with each shuffle,
-// then across the warps in a fixed order.  Row pieces of 4 KB come by bulk copies into a ring
+// then across the warps in a fixed order, as FP32 pairs.  Row pieces of 4 KB come by bulk copies into a ring
 // of six 16 KB stages, which the warps refill in turn.  Two CTAs per SM: with one, its two
 // warps per scheduler left the reductions' latency in the open (n = 8192, two columns: 50 us
-// a link against 37 with two; the strips' pass and sum 41).  Rows are exact, not boxes of
+// a link against 37 with two; the strips' pass and sum 41).  A chunk's four products are
+// summed by themselves and the warps' sums as pairs, which takes 1 us more a link and keeps
+// the error against FP64 at or below the strips' (n = 8192 1.2e-7, n = 1000 1.0e-7).  Rows are exact, not boxes of
 // eight, so the CTAs' ranges differ by one row at most.
 constexpr int kRpRows = 4, kRpCols = 1024, kRpStages = 6;
 constexpr int kRpThreads = 256, kRpWarps = kRpThreads / 32;
@@ -162,11 +164,10 @@ __global__ void __launch_bounds__(kRpThreads, 2)
         for (int j = 0; j < kRpRows; ++j)
 #pragma unroll
           for (int q = 0; q < R; ++q) {
-            float& s = acc[j * R + q];
-            s = fmaf(x[j].x, u[c][0][q], s);
-            s = fmaf(x[j].y, u[c][1][q], s);
-            s = fmaf(x[j].z, u[c][2][q], s);
-            s = fmaf(x[j].w, u[c][3][q], s);
+            float t = x[j].x * u[c][0][q];
+            t = fmaf(x[j].y, u[c][1][q], t);
+            t = fmaf(x[j].z, u[c][2][q], t);
+            acc[j * R + q] += fmaf(x[j].w, u[c][3][q], t);
           }
         // the stage of the step before is refilled, by each warp in its turn
         if (step >= 1 && step % kRpWarps == warp && step - 1 + kRpStages < total) {
@@ -204,9 +205,14 @@ __global__ void __launch_bounds__(kRpThreads, 2)
     if (lane % (32 / NV) == 0) rb[warp * NV + lane / (32 / NV)] = acc[0];
     __syncthreads();
     if (tid < NV) {
-      float s = 0.f;
+      float s = rb[tid], low = 0.f;  // as a pair: these few additions are the largest
 #pragma unroll
-      for (int w = 0; w < kRpWarps; ++w) s += rb[w * NV + tid];
+      for (int w = 1; w < kRpWarps; ++w) {  // Knuth's TwoSum
+        const float v = rb[w * NV + tid], z = s + v, b1 = z - s;
+        low += (s - (z - b1)) + (v - b1);
+        s = z;
+      }
+      s += low;
       const int j = tid / R, q = tid % R;
       if (j < nr && q < r && ok) X[(int64_t)q * xs + row0 + j] = s;
     }
