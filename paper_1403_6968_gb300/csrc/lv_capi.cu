@@ -11,6 +11,7 @@
 #include <cuda_runtime.h>
 #include <cusolverDn.h>
 
+#include <algorithm>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
@@ -162,6 +163,7 @@ struct linview_program {
   void* V1 = nullptr;   // input right factor, column-major n x r_max
   void* Mr = nullptr;   // T_i^T V blocks in reverse order, p x k r_max
   void* TVpart = nullptr;  // row-block partial sums of those products
+  int64_t tv_elems = 0;    // elements of TVpart
   void* Gpanel = nullptr;
   void* Dh = nullptr;   // hybrid strategy: dense deltas D_{i-1}, D_i (2 x n x p, ld ldD)
   int64_t ldD = 0;
@@ -1585,9 +1587,12 @@ static linview_status iter_create(linview_program* p, const void* const* inputs,
   LV_TRY(dalloc(p, (size_t)p->fs * p->Rcap * p->elem, &p->Kar, s));
   LV_TRY(dalloc(p, (size_t)p->fs * p->d.r_max * p->elem, &p->V1, s));
   LV_TRY(dalloc(p, (size_t)pp * p->Rcap * p->elem, &p->Mr, s));
-  // partial sets of M_i = T_i^T V (one pass over the T panel for all views)
-  LV_TRY(dalloc(p, (size_t)tdot_work_elems((int)n, (int)(k * pp), p->d.r_max, p->sms) * p->elem,
-                &p->TVpart, s));
+  // partial sets of M_i = T_i^T V: one pass over the T panel for all views, or (hybrid) one
+  // pass per view, whose fewer columns are cut into more row blocks
+  p->tv_elems = tdot_work_elems((int)n, (int)(k * pp), p->d.r_max, p->sms);
+  if (p->d.strategy == LINVIEW_STRATEGY_HYBRID)
+    p->tv_elems = std::max(p->tv_elems, tdot_work_elems((int)n, (int)pp, p->d.r_max, p->sms));
+  LV_TRY(dalloc(p, (size_t)p->tv_elems * p->elem, &p->TVpart, s));
   const PassGeom g = fused_geom(p->elem, (int)n, p->sms);
   p->part_cs = p->fs;
   p->xp_s = (int64_t)kMaxFusedR * p->part_cs;
@@ -1618,7 +1623,7 @@ template <typename T>
 static linview_status panel_tdot(linview_program* p, const T* A, int64_t lda, const T* F, int w,
                                  int kv, T* M, cudaStream_t s) {
   TdotOp<T> o{A, lda, F, p->fs, (int)p->d.n, (int)p->d.p, kv, w, M, p->d.p,
-              static_cast<T*>(p->TVpart)};
+              static_cast<T*>(p->TVpart), p->tv_elems};
   ProfScope ps(p, s, 0.0);
   LV_CUDA(launch_tdot<T>(o, p->sms, s));
   p->all_launches++;  // the partial sums
@@ -1975,8 +1980,8 @@ static linview_status iter_sk_create(linview_program* p, const void* const* inpu
     LV_TRY(dalloc(p, (size_t)pp * ck * p->elem, &p->Yar[i], s));
   }
   LV_TRY(dalloc(p, (size_t)ck * p->Rcap * sizeof(double), &p->XtV, s));
-  LV_TRY(dalloc(p, (size_t)tdot_work_elems((int)n, (int)pp, p->Rcap, p->sms) * p->elem, &p->TVpart,
-                s));
+  p->tv_elems = tdot_work_elems((int)n, (int)pp, p->Rcap, p->sms);
+  LV_TRY(dalloc(p, (size_t)p->tv_elems * p->elem, &p->TVpart, s));
   LV_TRY(dalloc(p, (size_t)pp * p->d.r_max * p->elem, &p->Mr, s));  // V_b of an update to B
   const PassGeom g = fused_geom(p->elem, (int)n, p->sms);
   p->part_cs = p->fs;
@@ -2066,7 +2071,7 @@ static linview_status iter_sk_step(linview_program* p, int cur, View& tj, const 
   // first block of Y_i (column-major p x rh): T_j^T V_h + Y_j (X_j^T V_h), and
   // with_b + B^T (W^_h - V_h) (W^_h in the What arena; dS_1 = 0)
   TdotOp<T> o{static_cast<const T*>(tj.ptr), tj.ld, Vh, fs, n, (int)pp, 1, rh, Yn, pp,
-              static_cast<T*>(p->TVpart)};
+              static_cast<T*>(p->TVpart), p->tv_elems};
   if (with_b) {
     o.A1 = static_cast<const T*>(b.ptr);
     o.lda1 = b.ld;

@@ -290,7 +290,8 @@ cudaError_t launch_scale_copy(T* y, int64_t ldy, const T* x, int64_t ldx, T alph
 // M[((k - 1 - i) w + c) ldm + q] = sum_j A0[j lda0 + i p + q] F0[c fs + j] for
 // i < k, c < w <= 64, q < p; optionally + sum_j A1[j lda1 + i p + q] (F1 - F0)[c fs +
 // j] and + sum_{t < ny} Yc[t ldy + i p + q] S[t s_t + c s_c].  ``work`` holds
-// tdot_work_elems(n, k p, w) elements.
+// ``work_elems`` elements, tdot_work_elems(n, k p, w) for as many row blocks as fill the
+// GPU; fewer elements mean fewer blocks, and less than one block's k p w is an error.
 template <typename T>
 struct TdotOp {
   const T* A0;
@@ -301,6 +302,7 @@ struct TdotOp {
   T* M;
   int64_t ldm;
   T* work;
+  int64_t work_elems;
   const T* A1 = nullptr;
   int64_t lda1 = 0;
   const T* F1 = nullptr;

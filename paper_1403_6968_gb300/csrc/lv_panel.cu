@@ -399,7 +399,11 @@ template <typename T>
 cudaError_t launch_tdot(const TdotOp<T>& o, int num_sms, cudaStream_t s) {
   const int cols = o.k * o.p;
   if (o.n < 1 || cols < 1 || o.w < 1 || o.w > 64) return cudaErrorInvalidValue;
-  const int nb0 = tdot_blocks(o.n, cols, num_sms);
+  // no more row blocks than the work space has room for
+  const int64_t room = o.work_elems / ((int64_t)cols * o.w);
+  if (room < 1) return cudaErrorInvalidValue;
+  int nb0 = tdot_blocks(o.n, cols, num_sms);
+  if (nb0 > room) nb0 = (int)room;
   const int rows = ((o.n + nb0 - 1) / nb0 + 7) / 8 * 8;
   const int nb = (o.n + rows - 1) / rows;
   TdotArgs a{o.A0, o.F0, o.A1, o.F1, o.lda0, o.lda1, o.fs, o.n, cols, o.w, rows, o.work};
