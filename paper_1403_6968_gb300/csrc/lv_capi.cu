@@ -406,12 +406,12 @@ struct ProfScope {
 
 // X = P Xf, Y = P^T Yf (either may be skipped by mode), optional P += Uu Wu^T,
 // for a factor block of width r <= kMaxFusedR; partials land at column offset 0
-// of the given partial arrays.
+// of the given partial arrays (row-sum sets xp_s elements apart, 0: the program's stride).
 template <typename T>
 static linview_status run_fused(linview_program* p, const View& v, int mode, int r, const T* Xf,
                                 const T* Yf, const T* Uu, const T* Wu, void* Xpart, void* Ypart,
                                 cudaStream_t s, double* Cpart = nullptr,
-                                bool reverse = false) {
+                                bool reverse = false, int64_t xp_s = 0) {
   const PassGeom g = fused_geom(sizeof(T), (int)v.rows, p->sms);
   PassParams pp{};
   pp.P = v.ptr;
@@ -426,7 +426,7 @@ static linview_status run_fused(linview_program* p, const View& v, int mode, int
   pp.Xpart = Xpart;
   pp.Ypart = Ypart;
   pp.part_cs = p->part_cs;
-  pp.xp_s = p->xp_s;
+  pp.xp_s = xp_s ? xp_s : p->xp_s;
   pp.yp_q = p->yp_q;
   pp.gC = g.gC;
   pp.gR = g.gR;
@@ -577,8 +577,11 @@ static linview_status level_products(linview_program* p, const View& v, int r, c
   return LINVIEW_OK;
 }
 
-// Products X = P Xf, Y = P^T Yf for any width r (chunks of kMaxProductR in
-// FP32, kMaxFusedR in FP64) into
+// widest block of a products-only pass
+template <typename T>
+constexpr int kProductCols = sizeof(T) == 4 ? kMaxProductR : kMaxFusedR;
+
+// Products X = P Xf, Y = P^T Yf for any width r (chunks of kProductCols) into
 // the program's partial buffers (column block c0 at column offset c0), then
 // (if Uu) the in-place update.  Fused in one pass when r <= kMaxFusedR.
 // next_reverse (if given) receives the row order for a further pass over the
@@ -638,7 +641,7 @@ static linview_status run_products_update(linview_program* p, const View& v, int
       return LINVIEW_OK;
     }
   }
-  constexpr int MW = sizeof(T) == 4 ? kMaxProductR : kMaxFusedR;  // products-only width
+  constexpr int MW = kProductCols<T>;
   bool rev = false;  // consecutive passes over the view alternate their row order
   for (int c0 = 0; c0 < r; c0 += MW) {
     const int w = (r - c0 < MW) ? (r - c0) : MW;
@@ -2219,16 +2222,18 @@ static linview_status iter_sk_step_b(linview_program* p, int cur, int c, int rb,
   LV_CUDA(cudaMemcpyAsync(Yn, Yc, sizeof(T) * pp * c, cudaMemcpyDeviceToDevice, y));
   LV_CUDA(cudaMemcpyAsync(Yn + (int64_t)c * pp, Vb, sizeof(T) * pp * rb, cudaMemcpyDeviceToDevice,
                           y));
-  if (sh) {
-    const int64_t xp = p->xp_s;
-    p->xp_s = (int64_t)rb * p->part_cs;
-    const linview_status ru =
-        run_fused<T>(p, *sh, kModeX, rb, Ub, nullptr, nullptr, nullptr, p->Spart, p->Ypart, z);
-    p->xp_s = xp;
-    LV_TRY(ru);
+  if (sh) {  // in blocks of what one pass takes, each at its columns of the partial sets
+    const int64_t set = (int64_t)rb * p->part_cs;
+    T* sp = static_cast<T*>(p->Spart);
+    bool rev = false;
+    for (int c0 = 0; c0 < rb; c0 += kProductCols<T>) {
+      const int w = std::min(rb - c0, kProductCols<T>);
+      LV_TRY(run_fused<T>(p, *sh, kModeX, w, Ub + (int64_t)c0 * fs, nullptr, nullptr, nullptr,
+                          sp + (int64_t)c0 * p->part_cs, p->Ypart, z, nullptr, rev, set));
+      rev = !rev;
+    }
     ProfScope ps(p, z, 0.0);
-    LV_CUDA(launch_sum_partials<T>(static_cast<T*>(p->Spart), g.gC, (int64_t)rb * p->part_cs,
-                                   p->part_cs, n, rb, tmp, fs, z));
+    LV_CUDA(launch_sum_partials<T>(sp, g.gC, set, p->part_cs, n, rb, tmp, fs, z));
   }
   // [P X_j | P U_b] in one products pass over P
   LV_CUDA(cudaMemcpyAsync(Xc + (int64_t)c * fs, Ub, sizeof(T) * fs * rb, cudaMemcpyDeviceToDevice,
