@@ -548,9 +548,7 @@ static linview_status level_products(linview_program* p, const View& v, int r, c
                                      const float* V, int parts, cudaStream_t s) {
   const int n = (int)v.rows;
   const double nn = (double)n * (double)n * sizeof(float);
-  const bool tc = p->tcA && r > kMaxProductR;  // the update's form
-  LV_CUDA(launch_level_split(U, V, p->fs, n, r, p->tpF, p->tpF2, tc ? p->tcA : nullptr,
-                             tc ? p->tcB : nullptr, s));
+  LV_CUDA(launch_level_split(U, V, p->fs, n, r, p->tpF, p->tpF2, p->tcA, p->tcB, s));
   p->all_launches++;
   cudaStream_t y = s;
   if (!p->prof && tp_leaves_sms(n, p->sms)) {
@@ -570,7 +568,6 @@ static linview_status level_products(linview_program* p, const View& v, int r, c
     LV_CUDA(cudaEventRecord(p->prod_join_ev, y));
     LV_CUDA(cudaStreamWaitEvent(s, p->prod_join_ev, 0));
   }
-  if (!tc) return run_update<float>(p, v, U, V, r, s);
   ProfScope ps(p, s, 2.0 * nn, 2);
   LV_CUDA(launch_tc_update(v.tmap_tc, p->tmA, p->tmB, static_cast<float*>(v.ptr), v.ld, p->tcA,
                            p->tcB, U, V, p->fs, n, r, p->sms, p->status, s, /*presplit=*/true));
@@ -607,7 +604,7 @@ static linview_status run_products_update(linview_program* p, const View& v, int
     // Y = P^T V on the tensor cores, one read of P each, K split in ``parts``
     const int n = (int)v.rows;
     const int parts = tp_parts(n, p->sms);  // partial sets the pass writes
-    if (allow_tc && p->tpF && v.square && r > tp_min_r(n) && parts <= p->xslots &&
+    if (allow_tc && p->tpF && v.square && r > kMaxProductR && parts <= p->xslots &&
         (!want_y || parts <= p->yslots) && (v.ld * 4) % 16 == 0 && p->fs % 64 == 0) {
       if (p->tpF2 && want_y && Uu == Xf && Wu == Yf && r <= kMaxTcR) {
         p->pc_x = p->pc_y = parts;
@@ -1199,7 +1196,7 @@ static bool powers_uses_tc(const linview_program_desc& d) {
 // CUDA-core products pass: the tensor-core products pass
 static bool powers_uses_tp(const linview_program_desc& d) {
   return d.precision == LINVIEW_F32 && d.model == LINVIEW_MODEL_EXP &&
-         (int64_t)d.r_max * (d.k / 2) > tp_min_r(d.n);
+         (int64_t)d.r_max * (d.k / 2) > kMaxProductR;
 }
 
 // Device bytes powers_create allocates (with the buffers every program has),

@@ -40,7 +40,13 @@ constexpr int kStagesWs = 6;    // TMA ring depth of the decoupled-ring FP32 pas
 constexpr int kBoxBytes = 1024; // bytes per TMA box row (256 floats / 128 doubles)
 constexpr int kMaxAsmR = 64;    // widest factor block U_h of one assembly (= the widest Gram block)
 constexpr int kMaxFusedR = 8;   // widest factor block of the fused products pass
-constexpr int kMaxProductR = 16;  // widest factor block of an FP32 products-only pass
+// Widest factor block of an FP32 products-only pass.  Wider levels run on the tensor-core
+// products pass.  At 9 - 16 columns it would take 3 - 5 % off an update from n = 3500 on (A^16
+// rank 4 at n = 4096 259 -> 253 us, n = 8192 812 -> 776, with sums 1146 -> 1126), but its split
+// TF32 holds less of a product than FP32 FMAs: where the update makes up most of the view, the
+// error against FP64 was 1.03e-6 against 9.7e-7 (A^8, n = 3500, rank 3) and 8.4e-7 against
+// 7.4e-7 (A^4, rank 8).
+constexpr int kMaxProductR = 16;
 constexpr int kMaxUpdateR = 32;   // widest factor block of one update pass (shared-memory
                                   // broadcasts of the factor rows bound wider blocks)
 
@@ -114,18 +120,11 @@ cudaError_t launch_tc_products(bool transpose, const float* P, int64_t ldp, cons
                                int64_t cs, int parts, int num_sms, unsigned* status,
                                cudaStream_t s);
 // The splits of a level's factors in one launch: U and V for the products passes (FU, FV,
-// 128 x fs floats each) and, where Acat is given, both for the update P += U V^T.
+// 128 x fs floats each) and both for the update P += U V^T (Acat, Bcat).
 cudaError_t launch_level_split(const float* U, const float* V, int64_t fs, int n, int r, float* FU,
                                float* FV, float* Acat, float* Bcat, cudaStream_t s);
 // whether a products pass over an n x n view has fewer CTAs than the GPU has SMs
 bool tp_leaves_sms(int n, int num_sms);
-// Blocks wider than this run on the tensor-core products pass, two passes over the
-// view and two splits of the factor; narrower ones on the CUDA cores in one pass.
-// The CUDA-core pass is bound by its issue slots at 9 - 16 columns: n = 8192 145 us
-// against 59 + 59 + 4, n = 4096 43 against 19 + 19 + 4 (an update of A^16 at rank 2:
-// 217 -> 215 us, rank 4: 286 -> 277), n = 3000 27 against 12 + 12 + 3 (150 -> 153,
-// 200 -> 196), n = 2048 15 against 8 + 9 + 3 (106 -> 110, 141 -> 143).
-inline int tp_min_r(int64_t n) { return n >= 3500 ? kMaxFusedR : kMaxProductR; }
 // partial sets the products pass writes for an n x n view (<= kTpMaxParts)
 int tp_parts(int n, int num_sms);
 // Tensor-core update pass P += U W^T (FP32 view, 17 <= r <= 64 factor

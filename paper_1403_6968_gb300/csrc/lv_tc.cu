@@ -492,7 +492,7 @@ struct TpShape {
   static constexpr uint32_t LoBytes = kBM * 128;
   static constexpr uint32_t BBytes = 2 * RP * 128;         // factor chunk: hi rows, then lo rows
   static constexpr uint32_t StageBytes = HiBytes + LoBytes + BBytes;
-  static constexpr int S = TR ? 3 : (RP == 16 ? 6 : (RP == 32 ? 5 : 4));
+  static constexpr int S = TR ? 3 : (RP == 32 ? 5 : 4);
   static constexpr int R = TR ? (RP == 64 ? 4 : 6) : 0;    // raw slabs (Y)
   static constexpr uint32_t OffRaw = S * StageBytes;
   static constexpr uint32_t OffBar = OffRaw + R * PBytes;
@@ -511,8 +511,7 @@ struct TpShape {
 };
 static_assert(TpShape<false, 64>::SmemBytes <= 232448 && TpShape<true, 64>::SmemBytes <= 232448,
               "shared memory per CTA");
-static_assert(TpShape<true, 32>::SmemBytes <= 232448 && TpShape<false, 32>::SmemBytes <= 232448 &&
-                  TpShape<true, 16>::SmemBytes <= 232448 && TpShape<false, 16>::SmemBytes <= 232448,
+static_assert(TpShape<true, 32>::SmemBytes <= 232448 && TpShape<false, 32>::SmemBytes <= 232448,
               "shared memory per CTA");
 
 struct TpBars {
@@ -862,8 +861,8 @@ __global__ void tp_split_kernel(const float* __restrict__ Fin, int64_t fs, int n
   tp_split_block(blockIdx.x, Fin, fs, n, r, rp, F);
 }
 
-// All the splits of a level in one launch: U and V for the two products passes, then (tc > 0
-// CTAs) the update pass's form of both.  They read the same factors, and each as a launch of
+// All the splits of a level in one launch: U and V for the two products passes, then the
+// update pass's form of both.  They read the same factors, and each as a launch of
 // its own was a link of the level's chain (2.5 - 4 us, three a level).
 __global__ void __launch_bounds__(256) level_split_kernel(const float* __restrict__ U,
                                                           const float* __restrict__ V, int64_t fs,
@@ -973,13 +972,13 @@ static cudaError_t launch_tp_t(const CUtensorMap& tmP, const CUtensorMap& tmF, f
   return cudaGetLastError();
 }
 
-static int tp_width(int r) { return r <= 16 ? 16 : (r <= 32 ? 32 : 64); }
+static int tp_width(int r) { return r <= 32 ? 32 : 64; }
 
 cudaError_t launch_level_split(const float* U, const float* V, int64_t fs, int n, int r, float* FU,
                                float* FV, float* Acat, float* Bcat, cudaStream_t s) {
   if (r < 1 || r > kMaxTcR || fs % 64 || fs < n) return cudaErrorInvalidValue;
   const int rp = tp_width(r);
-  const int tp = (int)(((int64_t)rp * n + 255) / 256), tc = Acat ? (n + 31) / 32 : 0;
+  const int tp = (int)(((int64_t)rp * n + 255) / 256), tc = (n + 31) / 32;
   return launch_pdl(level_split_kernel, 2 * tp + tc, 256, 0, s, U, V, fs, n, r, rp, tp,
                     r <= 32 ? 32 : 64, FU, FV, Acat, Bcat);
 }
@@ -1005,8 +1004,6 @@ cudaError_t launch_tc_products(bool transpose, const float* P, int64_t ldp, cons
     return cudaErrorInvalidValue;
   auto run = [&](auto tr) {
     constexpr bool TR = decltype(tr)::value;
-    if (rp == 16)
-      return launch_tp_t<TR, 16>(tmP, tmF, out, ps, cs, n, r, parts, num_sms, status, s);
     if (rp == 32)
       return launch_tp_t<TR, 32>(tmP, tmF, out, ps, cs, n, r, parts, num_sms, status, s);
     return launch_tp_t<TR, 64>(tmP, tmF, out, ps, cs, n, r, parts, num_sms, status, s);
