@@ -2418,16 +2418,7 @@ static linview_status ols_create(linview_program* p, const void* const* inputs,
   p->part_cs = p->fs;
   const int64_t width = (kk > pp) ? kk : pp;
   p->xp_s = rup(width, kMaxFusedR) * p->part_cs;
-  // wide blocks (FP32): G = W U on the tensor cores where that is faster (32 columns:
-  // n = 4096 2 + 20 us and 6 sets to sum against 32 and 38 sets; a whole update at
-  // n = 2048 107 -> 99 us, n = 4096 112 -> 98)
-  const bool tp = p->elem == 4 && kk > kMaxProductR && n >= 2048;
-  const int64_t xsets = tp && g.gC < kTpMaxParts ? kTpMaxParts : g.gC;
-  LV_TRY(dalloc(p, (size_t)xsets * p->xp_s * p->elem, &p->Xpart, s));
-  if (tp) {
-    LV_TRY(dalloc(p, sizeof(float) * 128 * p->fs, &t, s));
-    p->tpF = static_cast<float*>(t);
-  }
+  LV_TRY(dalloc(p, (size_t)g.gC * p->xp_s * p->elem, &p->Xpart, s));
   // FP32: G = W U by column sums, up to kMaxColSumR columns per pass, one
   // partial per row block
   const int64_t ycols = p->elem == 4 ? rup(kk < kMaxColSumR ? kk : kMaxColSumR, kMaxFusedR)
@@ -2480,31 +2471,18 @@ static linview_status ols_propagate_t(linview_program* p, int kr, cudaStream_t s
     p->all_launches++;
   }
   if constexpr (sizeof(T) == 4) {
-    if (p->tpF && kk > kMaxProductR) {
-      // wide blocks: one tensor-core products pass
-      const int parts = tp_parts(n, p->sms);
-      {
-        ProfScope ps(p, s, (double)n * (double)n * sizeof(float), 1);
-        LV_CUDA(launch_tc_products(false, static_cast<const float*>(w.ptr), w.ld,
-                                   reinterpret_cast<const float*>(U), fs, p->tpF, n, kk,
-                                   static_cast<float*>(p->Xpart), p->xp_s, p->part_cs, parts,
-                                   p->sms, p->status, s));
-        p->all_launches++;  // the split kernel
-      }
+    // G = W U = W^T U (W is symmetric): column sums of a pass over W, which
+    // need no cross-lane reductions, up to 32 columns per read of W.  (On the tensor cores an
+    // update with 2k = 32 would take 97 us instead of 112 at n = 4096, 98 instead of 107 at
+    // n = 2048, but split TF32 takes bits off G: errors against FP64 grew by 0.1 - 5 % in W and
+    // by 1 - 14 % in beta.)
+    for (int c0 = 0; c0 < kk; c0 += kMaxColSumR) {
+      const int wd = (kk - c0 < kMaxColSumR) ? kk - c0 : kMaxColSumR;
+      LV_TRY(run_fused<T>(p, w, kModeY, wd, nullptr, U + (int64_t)c0 * fs, nullptr, nullptr,
+                          p->Xpart, p->Ypart, s));
       ProfScope ps(p, s, 0.0);
-      LV_CUDA(launch_sum_partials<T>(static_cast<T*>(p->Xpart), parts, p->xp_s, p->part_cs, n, kk, G,
-                                     fs, s));
-    } else {
-      // G = W U = W^T U (W is symmetric): column sums of a pass over W, which
-      // need no cross-lane reductions, up to 32 columns per read of W
-      for (int c0 = 0; c0 < kk; c0 += kMaxColSumR) {
-        const int wd = (kk - c0 < kMaxColSumR) ? kk - c0 : kMaxColSumR;
-        LV_TRY(run_fused<T>(p, w, kModeY, wd, nullptr, U + (int64_t)c0 * fs, nullptr, nullptr,
-                            p->Xpart, p->Ypart, s));
-        ProfScope ps(p, s, 0.0);
-        LV_CUDA(launch_sum_partials<T>(static_cast<T*>(p->Ypart), g.gR, p->yp_q, p->part_cs, n, wd,
-                                       G + (int64_t)c0 * fs, fs, s));
-      }
+      LV_CUDA(launch_sum_partials<T>(static_cast<T*>(p->Ypart), g.gR, p->yp_q, p->part_cs, n, wd,
+                                     G + (int64_t)c0 * fs, fs, s));
     }
   } else {
     // G = W U (row sums, one read of W per 8 columns)
