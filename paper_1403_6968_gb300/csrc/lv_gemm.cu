@@ -31,9 +31,9 @@
 //    walks the tiles in groups of 8 row blocks (the A and B chunks a wave reads
 //    stay in L2).  Per CTA: warp 0 streams its A and B chunks with TMA into an
 //    S-stage ring, one thread of the pair's first CTA issues 12 MMAs per chunk
-//    (3 products x 4 K steps of 32 bytes) into one of two BN-column FP32
-//    accumulators in tensor memory, and the epilogue warps read the other
-//    accumulator back (tcgen05.ld).  The tensor
+//    (3 products x 4 K steps of 32 bytes) into one of 512 / BN BN-column FP32
+//    accumulators in tensor memory, and the epilogue warps read the ones before
+//    it back (tcgen05.ld).  The tensor
 //    cores accumulate with round-toward-zero, a bias that grows with the number
 //    of accumulation steps (measured 7.9e-6 relative at K = 1000, ~6e-5 at
 //    K = 8192 if the whole K were accumulated in tensor memory), so the MMAs
@@ -55,6 +55,9 @@
 #include <cuda_runtime.h>
 #include <cudaTypedefs.h>
 #include <cuda_fp16.h>
+
+#include <algorithm>
+#include <type_traits>
 
 #include "lv_device.cuh"
 #include "lv_internal.h"
@@ -281,7 +284,8 @@ struct GArgs {
 
 // D (M x N, row-major, ldd) = alpha A B^T + beta C over the split blocks of K = kp16
 // (FP16) or kp32 (TF32) values.
-template <int BN>
+// HALVES: every other chunk (FP16) goes to two accumulators.
+template <int BN, bool HALVES>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GShape<BN>::Threads, 1)
     tc_gemm_kernel(const __grid_constant__ GMaps maps, const GArgs a) {
   using Sh = GShape<BN>;
@@ -337,6 +341,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GShape<BN>::Threads,
   // pair had read at another time: adjoint of 16 rounds at 8192 x 64 1313 -> 1238 us, at
   // 5000 x 30 582 -> 535, 8 rounds at 7000 x 120 733 -> 715.
   auto chunk = [&](int kc) { return a.reverse ? work.kb + work.ke - 1 - kc : kc; };
+  // accumulators that chunk kc takes
+  auto halves = [&](int kc) { return HALVES && f16 && !((kc - work.kb) & 1) ? 2 : 1; };
   if (blockIdx.x == 0 && tid == 0) {  // the buffers' format, for later products on the same split
     *a.fmta = f16 ? 0u : 1u;
     *a.fmtb = f16 ? 0u : 1u;
@@ -397,51 +403,56 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GShape<BN>::Threads,
       const uint64_t d0 = g_desc(smem_u32(base));
       bool ok = true;
       while (ok && !*abort_flag && work.next()) {
-        for (int kc = work.kb; kc < work.ke; ++kc) {
-          if ((!first_round && !g_wait(&bars->acc_empty[buf], aphase ^ 1u, abort_flag, status)) ||
-              !g_wait(&bars->full[st], phase, abort_flag, status))
-            ok = false;
-          if (!__all_sync(0xffffffffu, ok)) {
-            ok = false;
-            break;
-          }
-          g_fence_after();
-          if (elect_one()) {
-            const uint32_t d = tm + buf * BN;
-            const uint64_t a_hi = d0 + (uint32_t)st * (Sh::StageBytes >> 4);
-            const uint64_t a_lo = a_hi + (Sh::AHalf >> 4);
-            const uint64_t b_hi = a_hi + (2 * Sh::AHalf >> 4);
-            const uint64_t b_lo = b_hi + (Sh::BHalf >> 4);
-            // lo(A) hi(B), hi(A) lo(B), then hi(A) hi(B)
-            const uint64_t pa[3] = {a_lo, a_hi, a_hi};
-            const uint64_t pb[3] = {b_hi, b_lo, b_hi};
-            if (f16) {
+        for (int kc = work.kb; kc < work.ke && ok; ++kc) {
+          const uint64_t a_hi = d0 + (uint32_t)st * (Sh::StageBytes >> 4);
+          const uint64_t a_lo = a_hi + (Sh::AHalf >> 4);
+          const uint64_t b_hi = a_hi + (2 * Sh::AHalf >> 4);
+          const uint64_t b_lo = b_hi + (Sh::BHalf >> 4);
+          // lo(A) hi(B), hi(A) lo(B), then hi(A) hi(B)
+          const uint64_t pa[3] = {a_lo, a_hi, a_hi};
+          const uint64_t pb[3] = {b_hi, b_lo, b_hi};
+          ok = g_wait(&bars->full[st], phase, abort_flag, status);
+          const int nh = halves(kc);
+          for (int h = 0; h < nh; ++h) {
+            if (ok && !first_round) ok = g_wait(&bars->acc_empty[buf], aphase ^ 1u, abort_flag, status);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            g_fence_after();
+            if (elect_one()) {
+              const uint32_t d = tm + buf * BN;
+              auto issue = [&](auto kind, auto k0, auto k1) {  // K steps of 32 bytes of a row
+                constexpr bool F16 = decltype(kind)::value;
 #pragma unroll
-              for (int pr = 0; pr < 3; ++pr)
+                for (int pr = 0; pr < 3; ++pr)
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk)  // 32 bytes of a 128-byte row per MMA
-                  g_mma<true>(d, pa[pr] + kk * 2, pb[pr] + kk * 2, Sh::Idesc16,
-                              (pr != 0 || kk != 0) ? 1u : 0u);
-            } else {
-#pragma unroll
-              for (int pr = 0; pr < 3; ++pr)
-#pragma unroll
-                for (int kk = 0; kk < 4; ++kk)
-                  g_mma<false>(d, pa[pr] + kk * 2, pb[pr] + kk * 2, Sh::Idesc32,
-                               (pr != 0 || kk != 0) ? 1u : 0u);
+                  for (int kk = k0.value; kk < k1.value; ++kk)
+                    g_mma<F16>(d, pa[pr] + kk * 2, pb[pr] + kk * 2, F16 ? Sh::Idesc16 : Sh::Idesc32,
+                               (pr != 0 || kk != k0.value) ? 1u : 0u);
+              };
+              const std::integral_constant<int, 0> k0;
+              const std::integral_constant<int, 2> k2;
+              const std::integral_constant<int, 4> k4;
+              if (!f16)
+                issue(std::false_type{}, k0, k4);
+              else if (nh == 1)
+                issue(std::true_type{}, k0, k4);
+              else if (h == 0)
+                issue(std::true_type{}, k0, k2);
+              else
+                issue(std::true_type{}, k2, k4);
+              if (h == nh - 1) g_commit(&bars->empty[st]);
+              g_commit(&bars->acc_full[buf]);
             }
-            g_commit(&bars->empty[st]);
-            g_commit(&bars->acc_full[buf]);
+            __syncwarp();
+            if (++buf == NB) {
+              buf = 0;
+              aphase ^= 1u;
+              first_round = false;
+            }
           }
-          __syncwarp();
           if (++st == S) {
             st = 0;
             phase ^= 1u;
-          }
-          if (++buf == NB) {
-            buf = 0;
-            aphase ^= 1u;
-            first_round = false;
           }
         }
       }
@@ -491,41 +502,46 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GShape<BN>::Threads,
           fr_next = row_factor(kc + 1);
           fc_next = col_factors(kc + 1);
         }
-        const bool w = g_wait(&bars->acc_full[buf], aphase, abort_flag, status);
-        if (!__all_sync(0xffffffffu, w)) {  // tcgen05.ld is warp-collective
-          ok = false;
-          break;
-        }
-        g_fence_after();
-        const uint32_t ta = tmem + ((uint32_t)(quarter * 32) << 16) + buf * BN + cpart * CW;
-#pragma unroll
-        for (int q = 0; q < CW / 64; ++q) {  // 64 columns in flight
-          uint32_t v[2][32];
-          g_tmem_ld32(ta + q * 64, v[0]);
-          g_tmem_ld32(ta + q * 64 + 32, v[1]);
-          g_tmem_wait_ld();
-          if (q == CW / 64 - 1) {  // all read: the accumulator is free
-            g_fence_before();
-            __syncwarp();
-            if (lane == 0) g_arrive_lead(ae + buf * 8);
+        const int nh = halves(kc);
+#pragma unroll 1
+        for (int h = 0; h < nh; ++h) {
+          const bool w = g_wait(&bars->acc_full[buf], aphase, abort_flag, status);
+          if (!__all_sync(0xffffffffu, w)) {  // tcgen05.ld is warp-collective
+            ok = false;
+            break;
           }
+          g_fence_after();
+          const uint32_t ta = tmem + ((uint32_t)(quarter * 32) << 16) + buf * BN + cpart * CW;
 #pragma unroll
-          for (int e = 0; e < 16; ++e) {
-            // the factors are powers of two: one rounding, in the addition
-            const float4 f = reinterpret_cast<const float4*>(cs)[q * 16 + e];
-            const uint32_t* x = &v[e / 8][e % 8 * 4];
-            float2& a0 = acc[q * 32 + 2 * e];
-            float2& a1 = acc[q * 32 + 2 * e + 1];
-            a0 = __ffma2_rn(__fmul2_rn(make_float2(__uint_as_float(x[0]), __uint_as_float(x[1])),
-                                       make_float2(f.x, f.y)), fr2, a0);
-            a1 = __ffma2_rn(__fmul2_rn(make_float2(__uint_as_float(x[2]), __uint_as_float(x[3])),
-                                       make_float2(f.z, f.w)), fr2, a1);
+          for (int q = 0; q < CW / 64; ++q) {  // 64 columns in flight
+            uint32_t v[2][32];
+            g_tmem_ld32(ta + q * 64, v[0]);
+            g_tmem_ld32(ta + q * 64 + 32, v[1]);
+            g_tmem_wait_ld();
+            if (q == CW / 64 - 1) {  // all read: the accumulator is free
+              g_fence_before();
+              __syncwarp();
+              if (lane == 0) g_arrive_lead(ae + buf * 8);
+            }
+#pragma unroll
+            for (int e = 0; e < 16; ++e) {
+              // the factors are powers of two: one rounding, in the addition
+              const float4 f = reinterpret_cast<const float4*>(cs)[q * 16 + e];
+              const uint32_t* x = &v[e / 8][e % 8 * 4];
+              float2& a0 = acc[q * 32 + 2 * e];
+              float2& a1 = acc[q * 32 + 2 * e + 1];
+              a0 = __ffma2_rn(__fmul2_rn(make_float2(__uint_as_float(x[0]), __uint_as_float(x[1])),
+                                         make_float2(f.x, f.y)), fr2, a0);
+              a1 = __ffma2_rn(__fmul2_rn(make_float2(__uint_as_float(x[2]), __uint_as_float(x[3])),
+                                         make_float2(f.z, f.w)), fr2, a1);
+            }
+          }
+          if (++buf == NB) {
+            buf = 0;
+            aphase ^= 1u;
           }
         }
-        if (++buf == NB) {
-          buf = 0;
-          aphase ^= 1u;
-        }
+        if (!ok) break;
       }
       if (!ok) break;
       // A thread holds a row, memory wants lines: blocks of 32 x 32 go through shared
@@ -1008,18 +1024,18 @@ __global__ void __launch_bounds__(ROWS * BN / 4)
   }
 }
 
-template <int BN>
+template <int BN, bool HALVES>
 cudaError_t launch_tc_gemm_t(const GMaps& maps, const GArgs& a, const SplitOp* next, bool* did,
                              unsigned* next_flag, int num_sms, cudaStream_t s) {
   using Sh = GShape<BN>;
   static const cudaError_t configured = [] {
     cudaFuncAttributes at;
-    cudaError_t e = cudaFuncGetAttributes(&at, tc_gemm_kernel<BN>);
+    cudaError_t e = cudaFuncGetAttributes(&at, tc_gemm_kernel<BN, HALVES>);
     // the registers handed over must be there, or setmaxnreg would wait forever
     if (e == cudaSuccess && Sh::Rebalance && at.numRegs * Sh::Threads < 40 * 128 + 224 * 256)
       e = cudaErrorInvalidConfiguration;
     if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(tc_gemm_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    return cudaFuncSetAttribute(tc_gemm_kernel<BN, HALVES>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)Sh::SmemBytes);
   }();
   if (configured != cudaSuccess) return configured;
@@ -1027,7 +1043,7 @@ cudaError_t launch_tc_gemm_t(const GMaps& maps, const GArgs& a, const SplitOp* n
   const int busy = a.dp > a.cut ? a.dp : a.cut;
   const int pairs = busy < num_sms / 2 ? busy : num_sms / 2;
   const cudaError_t e =
-      launch_pdl(tc_gemm_kernel<BN>, 2 * pairs, Sh::Threads, Sh::SmemBytes, s, maps, a);
+      launch_pdl(tc_gemm_kernel<BN, HALVES>, 2 * pairs, Sh::Threads, Sh::SmemBytes, s, maps, a);
   if (e != cudaSuccess || tiles == a.dp) return e;
   if constexpr (BN == 64) {
     if (next && a.dp == 0 && a.N <= BN) {
@@ -1090,10 +1106,25 @@ SplitOp split_op(const TcOperand* t) {
 // 13 us), 2048^3 (256, whole: 40), 3001 x 1025 x 5003 (256, cut: 76 + 12),
 // 4096 x 128 x 4096 (128, cut: 21 + 5), 8192 x 64 x 8192 (64, cut: 57 + 6) and
 // 300 x 40 x 5000 (64, cut: 9 + 7, whole: 38).
-void gemm_plan(int M, int N, int nk, int num_sms, int64_t work_floats, GArgs& a, int* bn_out) {
+//
+// A product that leaves half of the pairs idle (at 256 columns) has time for smaller sums,
+// as the chains of such products (A^16 at n <= 1500, the rounds of an iteration) add up
+// their errors: its choices are those whose pieces add at most 16 chunks one after the
+// other, or two thirds of its chunks (all choices where there is none), and up to 32 chunks
+// every other one goes to two accumulators, which takes a fifth off the bias that the tensor
+// cores' truncation leaves (8.9e-8 of a product; a re-evaluated A^16 has 15 times that).
+// Errors against FP64, time: A^16 re-evaluated at n = 1000 1.42e-6 -> 1.19e-6, 95.5 -> 101.4 us;
+// 314 x 3654 x 2299 1.73e-7 -> 1.54e-7, 93 -> 95; adjoint of 16 rounds at 2000 x 200 3.1e-7
+// -> 2.7e-7, 529 -> 550.  (Every chunk in halves: 0.99e-6, but 103.6 us, and 16.2 -> 19.9 ms
+// for the products of n = 8192, whose epilogue then takes longer than their MMAs.)
+void gemm_plan(int M, int N, int nk, int num_sms, int64_t work_floats, GArgs& a, int* bn_out,
+               bool* halves) {
   const int pairs = num_sms / 2;
   const long long mt = (M + kGBM - 1) / kGBM;
+  const bool small = mt * ((N + 255) / 256) <= pairs / 2;
+  const int longest = small ? std::max(16, nk * 2 / 3) : nk;
   double best = 1e30;
+  bool best_short = false;
   for (int bn = 256; bn >= 64; bn /= 2) {
     const double chunk = bn == 256 ? 1.03 : (bn == 128 ? 0.62 : 0.50);
     const long long tiles = mt * ((N + bn - 1) / bn);
@@ -1105,14 +1136,18 @@ void gemm_plan(int M, int N, int nk, int num_sms, int64_t work_floats, GArgs& a,
       if (cut)
         t += (double)((left * nk + cut - 1) / cut) * chunk + 3.5 +
              (double)(left + cut) * (kGBM * bn) * 8.0 / 6e6;
-      if (t < best) {
+      const long long chain = tiles > left ? nk : (left * nk + cut - 1) / cut;
+      const bool is_short = chain <= longest;
+      if (is_short == best_short ? t < best : is_short) {
         best = t;
+        best_short = is_short;
         *bn_out = bn;
         a.dp = (int)(tiles - left);
         a.cut = cut;
       }
     }
   }
+  *halves = small && nk <= 32;
 }
 
 }  // namespace
@@ -1172,7 +1207,8 @@ cudaError_t launch_tc_gemm(const TcOperand& a, const TcOperand& b, unsigned* fla
   g.kp16 = (K + 63) / 64 * 64;
   g.kp32 = (K + 31) / 32 * 32;
   int bn = 256;
-  gemm_plan(M, N, g.kp16 / 64, num_sms, work ? work_floats : 0, g, &bn);
+  bool halves = false;
+  gemm_plan(M, N, g.kp16 / 64, num_sms, work ? work_floats : 0, g, &bn, &halves);
   g.reverse = reverse ? 1 : 0;
   GMaps maps;
   const int64_t ab = (M + 127) / 128 * 256, bb = (N + 127) / 128 * 256;  // lines per chunk
@@ -1203,9 +1239,14 @@ cudaError_t launch_tc_gemm(const TcOperand& a, const TcOperand& b, unsigned* fla
   g.status = status;
   const SplitOp nx = split_op(next);
   const SplitOp* np = next ? &nx : nullptr;
-  if (bn == 256) return launch_tc_gemm_t<256>(maps, g, np, next_split, next_flag, num_sms, s);
-  if (bn == 128) return launch_tc_gemm_t<128>(maps, g, np, next_split, next_flag, num_sms, s);
-  return launch_tc_gemm_t<64>(maps, g, np, next_split, next_flag, num_sms, s);
+  auto run = [&](auto width) {
+    constexpr int BN = decltype(width)::value;
+    return halves ? launch_tc_gemm_t<BN, true>(maps, g, np, next_split, next_flag, num_sms, s)
+                  : launch_tc_gemm_t<BN, false>(maps, g, np, next_split, next_flag, num_sms, s);
+  };
+  if (bn == 256) return run(std::integral_constant<int, 256>{});
+  if (bn == 128) return run(std::integral_constant<int, 128>{});
+  return run(std::integral_constant<int, 64>{});
 }
 
 static int gemm_simt_splits(int M, int N, int K, int batch, int num_sms, int64_t work_elems) {
