@@ -58,6 +58,7 @@
 
 #include <algorithm>
 #include <type_traits>
+#include <utility>
 
 #include "lv_device.cuh"
 #include "lv_internal.h"
@@ -705,6 +706,8 @@ __global__ void __launch_bounds__(256) split_f16_kernel(const __grid_constant__ 
   griddep_wait();
   griddep_launch_dependents();
   if (b == 0 && tid == 0) *o.fmt = 0u;
+  // one thread's reading for the CTA, which leaves as a whole
+  const unsigned flag = tid == 0 ? *const_cast<volatile unsigned*>(sp.flag) : 0u;
   (&rowcnt[0][0])[tid] = 0;
   (&colcnt[0][0])[tid] = 0;
   if (o.cs != 1) {  // transpose: 16 lanes read 64 rows of one k
@@ -748,7 +751,7 @@ __global__ void __launch_bounds__(256) split_f16_kernel(const __grid_constant__ 
       }
     }
   }
-  __syncthreads();
+  if (__syncthreads_or(flag != 0u)) return;
   bool bad = false;
 #pragma unroll
   for (int u = 0; u < NU; ++u) {
@@ -771,43 +774,78 @@ __global__ void __launch_bounds__(256) split_f16_kernel(const __grid_constant__ 
 }
 
 // TF32 halves, only when the flag is set (else the kernel returns at once) and
-// the buffer does not hold them already (kp = rup(K, 32), zero past K).
-// 32 x 32 tiles through shared memory, read along whichever source
-// index has unit stride.
-__global__ void __launch_bounds__(256) split_tf32_kernel(const __grid_constant__ SplitPair sp) {
+// the buffer does not hold them already (kp = rup(K, 32), zero past K): tiles of 32 rows x 32 k,
+// two at a time for their loads, read along whichever index has unit stride.  With one tile and
+// half the CTAs, after an FP16 split that ran to its end, a product on TF32 halves took 881 us
+// at 8192 x 64 x 8192 and 186 at 2048^3; 326 and 136 so.
+constexpr int kSt = 2;
+__global__ void __launch_bounds__(256, 4) split_tf32_kernel(const __grid_constant__ SplitPair sp) {
   griddep_wait();
   griddep_launch_dependents();
   if (*sp.flag == 0u) return;
   __shared__ float tile[32][33];
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 8 warps
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll 1
   for (int w = 0; w < 2; ++w) {
     const SplitOp& o = sp.o[w];
     if (*o.fmt != 0u) continue;
     const int kp = (o.K + 31) / 32 * 32;
-    const int kb = kp / 32;
-    const long long tiles = (long long)kb * ((o.rows + 31) / 32);
+    const int kb = kp / 32, ib = (o.rows + 31) / 32;
+    const long long tiles = (long long)kb * ib;
     const bool k_fast = o.cs == 1;
-    for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {
-      const int k0 = (int)(t % kb) * 32, i0 = (int)(t / kb) * 32;
-      __syncthreads();
-      for (int j = ty; j < 32; j += 8) {
-        const int il = k_fast ? j : tx, kl = k_fast ? tx : j;
-        const int i = i0 + il, k = k0 + kl;
-        tile[il][kl] = (i < o.rows && k < o.K) ? o.X[(int64_t)i * o.rs + (int64_t)k * o.cs] : 0.f;
+    // this thread's four values of a tile: row il, k kl .. kl + 3
+    const int il = warp * 4 + (lane >> 3), kl = (lane & 7) * 4;
+    for (long long t0 = (long long)blockIdx.x * kSt; t0 < tiles; t0 += (long long)gridDim.x * kSt) {
+      float x[kSt][4];
+#pragma unroll
+      for (int u = 0; u < kSt; ++u) {
+        const long long t = t0 + u;
+        const int i0 = (int)(k_fast ? t / kb : t % ib) * 32, k0 = (int)(k_fast ? t % kb : t / ib) * 32;
+        if (k_fast) {
+          const int i = i0 + il, k = k0 + kl;
+          const float* row = o.X + (int64_t)i * o.rs + k;
+          const bool in = t < tiles && i < o.rows;
+          if (in && o.vec && k + 4 <= o.K) {
+            const float4 v = *reinterpret_cast<const float4*>(row);
+            x[u][0] = v.x; x[u][1] = v.y; x[u][2] = v.z; x[u][3] = v.w;
+          } else {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) x[u][e] = in && k + e < o.K ? row[e] : 0.f;
+          }
+        } else {
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {  // k warp + 8 e, row lane
+            const int i = i0 + lane, k = k0 + warp + 8 * e;
+            x[u][e] = t < tiles && i < o.rows && k < o.K ? o.X[(int64_t)k * o.cs + i] : 0.f;
+          }
+        }
       }
-      __syncthreads();
-      for (int j = ty; j < 32; j += 8) {
-        const int i = i0 + j, k = k0 + tx;
+#pragma unroll
+      for (int u = 0; u < kSt; ++u) {
+        const long long t = t0 + u;
+        if (t >= tiles) break;
+        if (!k_fast) {
+          __syncthreads();
+#pragma unroll
+          for (int e = 0; e < 4; ++e) tile[warp + 8 * e][lane] = x[u][e];
+          __syncthreads();
+#pragma unroll
+          for (int e = 0; e < 4; ++e) x[u][e] = tile[kl + e][il];
+        }
+        const int i = (int)(k_fast ? t / kb : t % ib) * 32 + il, kc = (int)(k_fast ? t % kb : t / ib);
         if (i >= o.rows) continue;
-        const float x = tile[j][tx];
-        // round to nearest TF32 (ties away from zero): add half of the dropped
-        // 13-bit field, then clear it; x - hi is exact
-        const float hi = __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xFFFFE000u);
-        const float r = x - hi;
-        float* d = reinterpret_cast<float*>(o.dst + block_line(i, k / 32, kp / 32) * 128) + k % 32;
-        d[0] = hi;
-        d[4096] = __uint_as_float((__float_as_uint(r) + 0x1000u) & 0xFFFFE000u);
+        float hi[4], lo[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          // round to nearest TF32 (ties away from zero): add half of the dropped
+          // 13-bit field, then clear it; x - hi is exact
+          hi[e] = __uint_as_float((__float_as_uint(x[u][e]) + 0x1000u) & 0xFFFFE000u);
+          const float r = x[u][e] - hi[e];
+          lo[e] = __uint_as_float((__float_as_uint(r) + 0x1000u) & 0xFFFFE000u);
+        }
+        float4* d = reinterpret_cast<float4*>(o.dst + block_line(i, kc, kb) * 128) + kl / 4;
+        d[0] = make_float4(hi[0], hi[1], hi[2], hi[3]);
+        d[1024] = make_float4(lo[0], lo[1], lo[2], lo[3]);
       }
     }
   }
@@ -1185,6 +1223,8 @@ cudaError_t launch_tc_split(const TcOperand* a, const TcOperand* b, unsigned* fl
     sp.o[w].blocks = ((sp.o[w].rows + kSpR - 1) / kSpR) *
                      (((sp.o[w].K + 63) / 64 * 64 + kSpK - 1) / kSpK);
   }
+  // the smaller operand first: what it raises spares the larger one's split
+  if (sp.o[1].blocks < sp.o[0].blocks) std::swap(sp.o[0], sp.o[1]);
   return launch_pdl(split_f16_kernel, sp.o[0].blocks + sp.o[1].blocks, 256, 0, s, sp);
 }
 
@@ -1199,7 +1239,7 @@ cudaError_t launch_tc_gemm(const TcOperand& a, const TcOperand& b, unsigned* fla
   sp.flag = flag;
   sp.o[0] = split_op(&a);
   sp.o[1] = split_op(&b);
-  const cudaError_t es = launch_pdl(split_tf32_kernel, 2 * num_sms, 256, 0, s, sp);
+  const cudaError_t es = launch_pdl(split_tf32_kernel, 4 * num_sms, 256, 0, s, sp);
   if (es != cudaSuccess) return es;
   GArgs g{};
   g.M = M;
