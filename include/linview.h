@@ -385,7 +385,10 @@ linview_status linview_level_pass(int precision, int64_t n, void* P, int64_t ldp
  *  precision LINVIEW_F32: the tcgen05 split-operand GEMM (near-FP32 accuracy,
  *   three FP16 or TF32 products per operand pair, FP32 accumulation) when M >= 128,
  *   N >= 8 and K >= 128, else the CUDA-core GEMM in FP32; LINVIEW_F64: the
- *   FP64 CUDA-core GEMM.
+ *   FP64 CUDA-core GEMM.  Either kind of product leaves an error of a few 2^-22 of
+ *   sum_k |a(m, k)| |b(k, n)| per entry, whatever the entries' sizes: operands that FP16
+ *   halves cannot hold so (entries below 2^-17 of their neighbours along k that may meet
+ *   zeros and small entries only) take TF32 halves.
  * Temporary device memory (split operands, partial sums) is allocated
  * stream-ordered on ``stream`` and released before the call returns; the call
  * synchronises ``stream``.  Errors: EINVAL, ESHAPE, ENOMEM, ETIMEOUT (a

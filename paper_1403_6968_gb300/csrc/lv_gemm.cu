@@ -15,8 +15,8 @@
 //    that every entry down to 2^-17 of the run's largest keeps the 22 bits of a
 //    TF32 pair and a smaller one is off by at most 2^-40 of the largest; a run is
 //    one K chunk of the MMAs, whose result the epilogue scales back exactly as it
-//    adds it up.  Operands for which that is not enough (many small entries
-//    side by side, e.g. columns of very different scale), whose scale is out of
+//    adds it up.  Operands for which that is not enough (entries that lose bits
+//    beside runs of mostly small or zero entries, see needs_tf32), whose scale is out of
 //    the exponent's comfortable range, or that hold infinities or NaN are found
 //    while they are split, and such a product runs on TF32 halves instead (same
 //    kernel, kind::tf32; hi = x rounded to nearest
@@ -283,6 +283,21 @@ struct GArgs {
   unsigned* status;
 };
 
+// The flag word of a product: two bits per operand, kLossy where an entry keeps fewer than
+// 22 bits and kSparse where a run of an operand has more than 3/8 of its entries below 2^-7
+// of the largest (zeros among them; runs of zeros alone do not count).  Either alone does
+// no harm.  Where no run of A or of B is sparse, a quarter of a run of length L meets with
+// both entries at 2^7 or more of their 2^15, a sum of |a||b| of at least L/4 2^14, while the
+// at most 3/4 L entries that lose bits add 2^-25 2^15 each: 2^-22.4 of the sum, as much as
+// the halves of the others leave.  With kSparse on either side an entry may meet zeros and
+// small entries only, and a product is as good as that entry.  Dense data without such
+// structure has kLossy (in normal entries 2e-5 of them) and not kSparse (25 of 64 entries
+// below 2 % of a standard deviation).
+constexpr unsigned kLossy = 1u, kSparse = 2u;
+__device__ __forceinline__ bool needs_tf32(unsigned flag) {
+  return ((flag | flag >> 2) & 3u) == (kLossy | kSparse);
+}
+
 // D (M x N, row-major, ldd) = alpha A B^T + beta C over the split blocks of K = kp16
 // (FP16) or kp32 (TF32) values.
 // HALVES: every other chunk (FP16) goes to two accumulators.
@@ -330,7 +345,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GShape<BN>::Threads,
   const uint32_t tmem = bars->tmem_base;
   griddep_wait();  // the splits
   griddep_launch_dependents();
-  const bool f16 = *a.flag == 0u;
+  const bool f16 = !needs_tf32(*a.flag);
   const int kc_len = f16 ? 64 : 32;
   const int kp = f16 ? a.kp16 : a.kp32;
   const int nk = kp / kc_len;
@@ -628,6 +643,7 @@ struct SplitOp {
   unsigned* fmt;    // 0: FP16 rows, 1: TF32 rows
   int vec;          // rows of X start on 16-byte units
   int blocks;       // CTAs of this operand in the launch at hand
+  int bit;          // this operand's two bits in the flag word: 0 (A) or 2 (B)
 };
 struct SplitPair {
   SplitOp o[2];
@@ -640,61 +656,93 @@ __device__ __forceinline__ int64_t block_line(int i, int kc, int nk) {
   return ((int64_t)(i >> 7) * nk + kc) * 256 + (i & 127);
 }
 
-// Values k .. k + 7 of row i (a run of 64 belongs to eight neighbouring lanes; all lanes
-// of the warp take part): scale, split, store (``in``: inside the operand).  ``small`` is
-// called for the entries with fewer than 22 bits.  Returns whether the run's scale is out
-// of range or an entry is not finite.
-template <typename F>
-__device__ __forceinline__ bool split_run(const float (&x)[8], const SplitOp& o, int i, int k,
-                                          bool in, int kp, F small) {
-  unsigned mx = 0;
+// FP16 rows put K's values in slots 0 .. kp - 1 (kp = rup(K, 64)), zeros in the rest.  A last
+// run of 1 to 15 values is too short to say whether it is sparse, so the 16 values before it
+// move over to it: the run before ends in 16 zeros.
+__host__ __device__ __forceinline__ int slot_gap(int K) {
+  return K > 64 && K % 64 >= 1 && K % 64 < 16 ? 16 : 0;
+}
+// first slot behind the moved ones, kp for none
+__device__ __forceinline__ int slot_last(int K) {
+  return slot_gap(K) ? K / 64 * 64 : (K + 63) / 64 * 64;
+}
+// value of a slot that is a multiple of 8 (and of the seven behind it); K or more: zeros
+__device__ __forceinline__ int slot_value(int slot, int K) {
+  const int last = slot_last(K);
+  return slot >= last ? slot - slot_gap(K) : (slot_gap(K) && slot >= last - 16 ? K : slot);
+}
+// values of the run of 64 slots at ``slot``
+__device__ __forceinline__ int run_length(int slot, int K) {
+  const int run = slot / 64 * 64, last = slot_last(K);
+  if (!slot_gap(K)) return min(64, max(0, K - run));
+  return run >= last ? K - last + 16 : (run == last - 64 ? 48 : 64);
+}
+
+// Slots k .. k + 7 of row i (a run of 64 belongs to eight neighbouring lanes; all lanes
+// of the warp take part): scale, split, store (``in``: inside the operand).  Returns the run's
+// bits of the flag, both where its scale is out of range or an entry is not finite.
+__device__ __forceinline__ unsigned split_run(const float (&x)[8], const SplitOp& o, int i, int k,
+                                              bool in, int kp) {
+  unsigned mx = 0, mn = 0xffffffffu;  // mn: the least entry that is not zero, less one
 #pragma unroll
-  for (int e = 0; e < 8; ++e) mx = max(mx, __float_as_uint(x[e]) & 0x7fffffffu);
+  for (int e = 0; e < 8; ++e) {
+    const unsigned m = __float_as_uint(x[e]) & 0x7fffffffu;
+    mx = max(mx, m);
+    mn = min(mn, m - 1u);
+  }
 #pragma unroll
   for (int d = 1; d < 8; d <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, d));
   int sh = mx ? 14 - ((int)(mx >> 23) - 127) : 0;
-  const bool bad = sh > 60 || sh < -60;  // (non-finite: sh = -114)
+  unsigned bits = sh > 60 || sh < -60 ? kLossy | kSparse : 0u;  // (non-finite: sh = -114)
   sh = min(60, max(-60, sh));
   const float sc = pow2f(sh);
-  // pairs: one conversion instruction per two values; the rare small entries behind one branch
+  if (mn < ((unsigned)(125 - sh) << 23) - 1u) bits |= kLossy;  // 2^sh x below 2^-2
+  // pairs: one instruction per two values
   __align__(16) __half2 hi[4], lo[4];
-  unsigned few = 0;
+  __half2 lows = __float2half2_rn(0.f);
 #pragma unroll
   for (int e = 0; e < 4; ++e) {
     const float y0 = x[2 * e] * sc, y1 = x[2 * e + 1] * sc;
     hi[e] = __floats2half2_rn(y0, y1);
     const float2 h = __half22float2(hi[e]);
     lo[e] = __floats2half2_rn(y0 - h.x, y1 - h.y);
-    few |= (y0 != 0.f && fabsf(y0) < 0.25f ? 1u : 0u) << (2 * e);
-    few |= (y1 != 0.f && fabsf(y1) < 0.25f ? 1u : 0u) << (2 * e + 1);
+    lows = __hadd2(lows, __hlt2(__habs2(hi[e]), __float2half2_rn(128.f)));
   }
-  if (few)
+  int low = (int)(__low2float(lows) + __high2float(lows));
+  // a sparse run has four such entries in one lane
+  if (__any_sync(0xffffffffu, low >= 4)) {
 #pragma unroll
-    for (int e = 0; e < 8; ++e)
-      if (few >> e & 1u) small(e);
+    for (int d = 1; d < 8; d <<= 1) low += __shfl_xor_sync(0xffffffffu, low, d);
+    const int len = run_length(k, o.K);
+    if (mx && low - (64 - len) > len * 3 / 8) bits |= kSparse;
+  }
   if (in) {
     unsigned char* d = o.dst + block_line(i, k / 64, kp / 64) * 128 + k % 64 * 2;
     *reinterpret_cast<uint4*>(d) = *reinterpret_cast<const uint4*>(hi);
     *reinterpret_cast<uint4*>(d + 16384) = *reinterpret_cast<const uint4*>(lo);
     if (k % 64 == 0) o.sc[(int64_t)(k / 64) * o.pitch + i] = pow2f(-sh);
   }
-  return bad;
+  return bits;
+}
+
+// what the runs of a warp raise (all lanes take part)
+__device__ __forceinline__ void raise_bits(unsigned* flag, unsigned bits, const SplitOp& o) {
+  bits = __reduce_or_sync(0xffffffffu, bits) << o.bit;
+  if (bits && (threadIdx.x & 31) == 0 && bits & ~*const_cast<volatile unsigned*>(flag))
+    atomicOr(flag, bits);
 }
 
 // FP16 halves: tiles of 64 rows x 128 k (two runs), zero past K (kp = rup(K, 64)), one
 // pass over the operand: eight lanes hold a run and find its largest entry by shuffles.
-// An entry y = 2^sh x with 0 < |y| < 2^-2 has fewer than 22 bits; eight of them among 32
-// neighbours of a row or of a column of a tile (dense data without such structure has
-// none), a scale outside 2^-60 .. 2^60 or a non-finite entry sets the flag that sends
-// the product to TF32.
+// An entry y = 2^sh x with 0 < |y| < 2^-2 may have fewer than 22 bits.
 // 8192 x 8192: 101 us transposed, 93 us not, 4 bytes read and 4 written per entry
-// (floor 79); TF32 halves (8 written) took 196 us.  Conversions in pairs, the rare small
-// entries behind one branch and a thread's loads issued at once take 3 us off a split inside
-// the adjoint (8192 x 64, 16 rounds: 1310.3 -> 1303.9 us, 1313.8 -> 1310.5 in a second run).
-constexpr int kSpR = 64, kSpK = 128, kSmallCount = 8;
-__global__ void __launch_bounds__(256) split_f16_kernel(const __grid_constant__ SplitPair sp) {
+// (floor 79); TF32 halves (8 written) took 196 us.  Conversions in pairs and a thread's loads
+// issued at once take 3 us off a split inside the adjoint (8192 x 64, 16 rounds: 1310.3 ->
+// 1303.9 us, 1313.8 -> 1310.5 in a second run).  Five CTAs per SM (48 registers): with the 62
+// of a free choice 3001 and 1025 rows of 5003, read by scalars, took 47 us instead of 42.
+constexpr int kSpR = 64, kSpK = 128;
+__global__ void __launch_bounds__(256, 5) split_f16_kernel(const __grid_constant__ SplitPair sp) {
   __shared__ float tile[kSpK][kSpR + 1];
-  __shared__ int rowcnt[kSpR][kSpK / 32], colcnt[kSpR / 32][kSpK];
   const bool second = (int)blockIdx.x >= sp.o[0].blocks;
   const SplitOp& o = sp.o[second];
   const int b = blockIdx.x - (second ? sp.o[0].blocks : 0);
@@ -708,13 +756,12 @@ __global__ void __launch_bounds__(256) split_f16_kernel(const __grid_constant__ 
   if (b == 0 && tid == 0) *o.fmt = 0u;
   // one thread's reading for the CTA, which leaves as a whole
   const unsigned flag = tid == 0 ? *const_cast<volatile unsigned*>(sp.flag) : 0u;
-  (&rowcnt[0][0])[tid] = 0;
-  (&colcnt[0][0])[tid] = 0;
   if (o.cs != 1) {  // transpose: 16 lanes read 64 rows of one k
     const int il = 4 * (tid & 15);
 #pragma unroll
     for (int u = 0; u < kSpK / 16; ++u) {
-      const int kl = u * 16 + (tid >> 4), k = k0 + kl, i = i0 + il;
+      const int kl = u * 16 + (tid >> 4), i = i0 + il;
+      const int k = slot_value(k0 + u * 16, o.K) + (tid >> 4);
       float v[4] = {0.f, 0.f, 0.f, 0.f};
       if (k < o.K) {
         const float* col = o.X + (int64_t)k * o.cs + i;
@@ -737,8 +784,9 @@ __global__ void __launch_bounds__(256) split_f16_kernel(const __grid_constant__ 
 #pragma unroll
     for (int u = 0; u < NU; ++u) {
       const int idx = u * 256 + tid;
-      const int i = i0 + idx / (kSpK / 8), k = k0 + idx % (kSpK / 8) * 8;
-      const bool in = i < o.rows && k < kp;
+      const int i = i0 + idx / (kSpK / 8), slot = k0 + idx % (kSpK / 8) * 8;
+      const int k = slot_value(slot, o.K);
+      const bool in = i < o.rows && slot < kp;
       const float* row = o.X + (int64_t)i * o.rs + k;
       if (in && o.vec && k + 8 <= o.K) {
         const float4 p = reinterpret_cast<const float4*>(row)[0];
@@ -751,8 +799,8 @@ __global__ void __launch_bounds__(256) split_f16_kernel(const __grid_constant__ 
       }
     }
   }
-  if (__syncthreads_or(flag != 0u)) return;
-  bool bad = false;
+  if (__syncthreads_or(needs_tf32(flag))) return;
+  unsigned bits = 0;
 #pragma unroll
   for (int u = 0; u < NU; ++u) {
     const int idx = u * 256 + tid;
@@ -763,14 +811,9 @@ __global__ void __launch_bounds__(256) split_f16_kernel(const __grid_constant__ 
 #pragma unroll
       for (int e = 0; e < 8; ++e) x[u][e] = tile[kl + e][il];  // zeros past the operand
     }
-    bad |= split_run(x[u], o, i, k, in, kp, [&](int e) {
-      atomicAdd(&rowcnt[il][(kl + e) / 32], 1);
-      atomicAdd(&colcnt[il / 32][kl + e], 1);
-    });
+    bits |= split_run(x[u], o, i, k, in, kp);
   }
-  __syncthreads();
-  bad |= (&rowcnt[0][0])[tid] >= kSmallCount || (&colcnt[0][0])[tid] >= kSmallCount;
-  if (__syncthreads_or(bad) && tid == 0) atomicOr(sp.flag, 1u);
+  raise_bits(sp.flag, bits, o);
 }
 
 // TF32 halves, only when the flag is set (else the kernel returns at once) and
@@ -782,7 +825,7 @@ constexpr int kSt = 2;
 __global__ void __launch_bounds__(256, 4) split_tf32_kernel(const __grid_constant__ SplitPair sp) {
   griddep_wait();
   griddep_launch_dependents();
-  if (*sp.flag == 0u) return;
+  if (!needs_tf32(*sp.flag)) return;
   __shared__ float tile[32][33];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll 1
@@ -976,7 +1019,7 @@ __global__ void gemm_reduce_kernel(int M, int N, int splits, int batch, T alpha,
 
 // D = alpha (pieces) + beta C for the tiles cut along K: a CTA adds ROWS rows of one
 // tile, the pieces in their order along K.  SPLIT (ROWS = 64 = BN, every tile cut): D's
-// columns also go to the split operand ``nx``, a run of 64 rows per CTA and column.
+// columns also go to the split operand ``nx``, a run of 64 slots per CTA and column.
 // Bound by the latency of its few CTAs (128 at 8192 rows x 64 columns: 2 MB of D, 8 MB of
 // pieces from L2), so a thread has four values and every piece's load in flight (four
 // times the rows per thread: 10.1 us against 7.8); the split inside it saves the launches
@@ -986,32 +1029,37 @@ __global__ void __launch_bounds__(ROWS * BN / 4)
     gemm_parts_kernel(const GArgs a, int tiles, const __grid_constant__ SplitOp nx,
                       unsigned* nx_flag) {
   __shared__ float tile[SPLIT ? ROWS : 1][SPLIT ? BN + 1 : 1];
-  __shared__ int rowcnt[SPLIT ? BN : 1][2], colcnt[2][SPLIT ? ROWS : 1];
   griddep_wait();
   griddep_launch_dependents();
-  const int r = blockIdx.x;
-  const bool f16 = *a.flag == 0u;
+  const unsigned flag = *a.flag;
+  const bool f16 = !needs_tf32(flag);
   const int nk = f16 ? a.kp16 / 64 : a.kp32 / 32;
-  const long long W = (long long)(tiles - a.dp) * nk, lo = (long long)r * nk, hi = lo + nk;
-  // ranges that meet the tile: W c / cut < hi and W (c + 1) / cut > lo
-  int c0 = (int)(lo * a.cut / W), c1;
-  while (c0 > 0 && W * c0 / a.cut > lo) --c0;
-  while (W * (c0 + 1) / a.cut <= lo) ++c0;
-  c1 = c0;
-  while (W * (c1 + 1) / a.cut < hi) ++c1;
-  const bool whole = c0 == c1;  // computed by one range: D is complete
-  if (whole && !SPLIT) return;
-  int mb, nb;
-  g_tile(a.dp + r, (a.M + kGBM - 1) / kGBM, (a.N + BN - 1) / BN, mb, nb);
   const int row0 = blockIdx.y * ROWS;
   const int e = threadIdx.x, lrow = e / (BN / 4), col = e % (BN / 4) * 4;
-  const int row = row0 + lrow, m = mb * kGBM + row, n = nb * BN + col;
+  int r = blockIdx.x, mb, nb;
+  g_tile(a.dp + r, (a.M + kGBM - 1) / kGBM, (a.N + BN - 1) / BN, mb, nb);
+  int m = mb * kGBM + row0 + lrow;
+  const int n = nb * BN + col;
+  if constexpr (SPLIT) {  // slots; a moved row may lie in the tile before (one column: mb == r)
+    m = slot_value(m & ~15, nx.K) + (m & 15);
+    if (m < r * kGBM) r = --mb;
+  }
+  const long long W = (long long)(tiles - a.dp) * nk, lo = (long long)r * nk, hi = lo + nk;
+  // ranges that meet the tile: W c / cut < hi and W (c + 1) / cut > lo (both rounded down;
+  // multiplied out: 64-bit divisions in every warp took 1 us of 9)
+  int c0 = r * a.cut / (tiles - a.dp), c1;
+  while (c0 > 0 && W * c0 >= (lo + 1) * a.cut) --c0;
+  while (W * (c0 + 1) < (lo + 1) * a.cut) ++c0;
+  c1 = c0;
+  while (W * (c1 + 1) < hi * a.cut) ++c1;
+  const bool whole = c0 == c1;  // computed by one range: D is complete
+  if (whole && !SPLIT) return;
   float v[4] = {0.f, 0.f, 0.f, 0.f};
   if (m < a.M && n < a.N) {
     float* d = a.D + (int64_t)m * a.ldd + n;
     const bool vec = a.vec_ok && n + 4 <= a.N;
     if (!whole) {
-      const float* w = a.work + ((int64_t)(c0 + r) * kGBM + row) * BN + col;
+      const float* w = a.work + ((int64_t)(c0 + r) * kGBM + m - mb * kGBM) * BN + col;
       float4 s = *reinterpret_cast<const float4*>(w);
 #pragma unroll 8
       for (int c = c0 + 1; c <= c1; ++c) {
@@ -1040,25 +1088,19 @@ __global__ void __launch_bounds__(ROWS * BN / 4)
   }
   if constexpr (SPLIT) {
     if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *nx.fmt = 0u;
-    if (threadIdx.x < BN * 2) (&rowcnt[0][0])[threadIdx.x] = 0;
-    if (threadIdx.x < ROWS * 2) (&colcnt[0][0])[threadIdx.x] = 0;
     __syncthreads();
-    const int kp = (nx.K + 63) / 64 * 64, k0 = mb * kGBM + row0;
-    bool bad = false;
+    const int kp = (nx.K + 63) / 64 * 64, k0 = blockIdx.x * kGBM + row0;
+    unsigned bits = 0;
     if (e < BN * ROWS / 8) {  // whole warps
       const int i = e / (ROWS / 8), kl = e % (ROWS / 8) * 8, k = k0 + kl;
       float x[8];
 #pragma unroll
       for (int j = 0; j < 8; ++j) x[j] = tile[kl + j][i];  // zeros past D
-      bad = split_run(x, nx, i, k, i < nx.rows && k < kp, kp, [&](int j) {
-        atomicAdd(&rowcnt[i][(kl + j) / 32], 1);
-        atomicAdd(&colcnt[i / 32][kl + j], 1);
-      });
+      bits = split_run(x, nx, i, k, i < nx.rows && k < kp, kp);
     }
-    __syncthreads();
-    if (threadIdx.x < BN * 2) bad |= (&rowcnt[0][0])[threadIdx.x] >= kSmallCount;
-    if (threadIdx.x < ROWS * 2) bad |= (&colcnt[0][0])[threadIdx.x] >= kSmallCount;
-    if (__syncthreads_or(bad || !f16) && threadIdx.x == 0) atomicOr(nx_flag, 1u);
+    raise_bits(nx_flag, bits, nx);
+    // A goes on as it is; once on TF32 halves, the chain stays there
+    if (blockIdx.x == 0 && blockIdx.y == 0 && e == 0) atomicOr(nx_flag, f16 ? flag & 3u : flag);
   }
 }
 
@@ -1119,7 +1161,7 @@ bool make_tmap_lines(CUtensorMap* out, const void* base, bool f16, int64_t lines
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-SplitOp split_op(const TcOperand* t) {
+SplitOp split_op(const TcOperand* t, bool second) {
   SplitOp o{};
   if (!t) return o;
   o.X = t->X;
@@ -1131,6 +1173,7 @@ SplitOp split_op(const TcOperand* t) {
   o.fmt = t->words;
   o.sc = reinterpret_cast<float*>(t->words + 4);
   o.pitch = (t->rows + 3) / 4 * 4;
+  o.bit = second ? 2 : 0;
   o.vec = (t->cs == 1 ? t->rs : t->cs) % 4 == 0 && reinterpret_cast<uintptr_t>(t->X) % 16 == 0;
   return o;
 }
@@ -1219,7 +1262,7 @@ cudaError_t launch_tc_split(const TcOperand* a, const TcOperand* b, unsigned* fl
     // TMA sources and 128-bit loads of the factors
     if ((reinterpret_cast<uintptr_t>(in[w]->buf) | reinterpret_cast<uintptr_t>(in[w]->words)) & 15)
       return cudaErrorInvalidValue;
-    sp.o[w] = split_op(in[w]);
+    sp.o[w] = split_op(in[w], w == 1);
     sp.o[w].blocks = ((sp.o[w].rows + kSpR - 1) / kSpR) *
                      (((sp.o[w].K + 63) / 64 * 64 + kSpK - 1) / kSpK);
   }
@@ -1237,8 +1280,8 @@ cudaError_t launch_tc_gemm(const TcOperand& a, const TcOperand& b, unsigned* fla
   if (M <= 0 || N <= 0 || K <= 0 || b.K != K) return cudaErrorInvalidValue;
   SplitPair sp{};
   sp.flag = flag;
-  sp.o[0] = split_op(&a);
-  sp.o[1] = split_op(&b);
+  sp.o[0] = split_op(&a, false);
+  sp.o[1] = split_op(&b, true);
   const cudaError_t es = launch_pdl(split_tf32_kernel, 4 * num_sms, 256, 0, s, sp);
   if (es != cudaSuccess) return es;
   GArgs g{};
@@ -1277,7 +1320,7 @@ cudaError_t launch_tc_gemm(const TcOperand& a, const TcOperand& b, unsigned* fla
   g.fmtb = b.words;
   g.flag = flag;
   g.status = status;
-  const SplitOp nx = split_op(next);
+  const SplitOp nx = split_op(next, true);
   const SplitOp* np = next ? &nx : nullptr;
   auto run = [&](auto width) {
     constexpr int BN = decltype(width)::value;

@@ -157,8 +157,8 @@ int64_t tc_split_words(int64_t rows, int64_t K);
 // floats of ``work`` below that let every product with up to these sizes cut tiles
 int64_t tc_work_floats(int64_t a_rows, int64_t b_rows, int64_t K, int num_sms);
 // Split a and b (either may be null).  ``flag`` (one word, zeroed by the caller
-// before the first split of a scratch) is set when an operand needs TF32; it
-// stays set, so all later products on the scratch take TF32.
+// before the first split of a scratch) collects what FP16 halves would lose of either
+// operand; its bits stay set, so once a product takes TF32 all later ones on the scratch do.
 cudaError_t launch_tc_split(const TcOperand* a, const TcOperand* b, unsigned* flag,
                             cudaStream_t s);
 // D (M x N, row-major, ldd) = alpha A B^T + beta C on the tensor cores (split
@@ -170,7 +170,7 @@ cudaError_t launch_tc_split(const TcOperand* a, const TcOperand* b, unsigned* fl
 // ``next``: D's columns as a split operand (rows N, K = M; its buffer may be b's): they
 // are split by the kernel that adds up the cut tiles when every tile is cut and one
 // tile column holds D; *next_split says whether they were, and ``next_flag`` (another word
-// than ``flag``, set when that one is) is then the flag of the product that reads them.
+// than ``flag``, with its bits of a) is then the flag of the product that reads them.
 cudaError_t launch_tc_gemm(const TcOperand& a, const TcOperand& b, unsigned* flag, float* D,
                            int64_t ldd, const float* C, int64_t ldc, float alpha, float beta,
                            int num_sms, unsigned* status, cudaStream_t s, float* work = nullptr,
