@@ -169,8 +169,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 
   const int nrb = (n + kBM - 1) / kBM;
   const int ncb = (n + BN - 1) / BN;
-  // (32-bit: T gridDim.x < 2^32 up to the largest view that fits the memory, n = 266 K; a
-  // 64-bit division per tile is some hundred cycles of the epilogue)
+  // (32-bit: T gridDim.x < 2^32 up to n = 481 K, which the launcher checks; a 64-bit division
+  // per tile is some hundred cycles of the epilogue)
   const unsigned T = (unsigned)nrb * ncb;
   const unsigned t0 = T * blockIdx.x / gridDim.x;
   const unsigned t1 = T * (blockIdx.x + 1) / gridDim.x;
@@ -560,9 +560,9 @@ __global__ void __launch_bounds__(TpShape<TR, RP>::Threads, 1)
   // and the CTA that ends a tile zero-fills the partials past its own.
   const int ot_n = (n + kBM - 1) / kBM;  // output tiles
   const int nkb = (n + 31) / 32;          // K chunks of 32
-  // (32-bit: C G < 2^32 up to n = 266 K, the largest view that fits the memory.  In 64 bits
-  // the divisions before a range and the ring indices of every chunk cost A^16 at n = 2048,
-  // rank 8 187 -> 181 us, at n = 4096, rank 4 257 -> 253)
+  // (32-bit: C (G + 1) < 2^32 up to n = 339 K, which the launcher checks.  In 64 bits the
+  // divisions before a range and the ring indices of every chunk cost A^16 at n = 2048, rank 8
+  // 187 -> 181 us, at n = 4096, rank 4 257 -> 253)
   const unsigned C = (unsigned)ot_n * nkb;
   const unsigned G = gridDim.x;
   const unsigned c0 = C * blockIdx.x / G;
@@ -923,6 +923,7 @@ static cudaError_t launch_tc_t(const CUtensorMap& tmP, const CUtensorMap& tmA,
   if (configured != cudaSuccess) return configured;
   const long long T = (long long)((n + kBM - 1) / kBM) * ((n + Sh::BN - 1) / Sh::BN);
   const int grid = (int)(T < num_sms ? T : num_sms);
+  if (T * grid > UINT32_MAX) return cudaErrorInvalidValue;  // the kernel's 32-bit ranges
   LV_LAUNCH(launch_pdl(tc_update_kernel<RP>, grid, kTcThreads, Sh::SmemBytes, s, tmP, tmA, tmB, P,
       ldp, n, status));
   return cudaGetLastError();
@@ -967,6 +968,8 @@ static cudaError_t launch_tp_t(const CUtensorMap& tmP, const CUtensorMap& tmF, f
       tc_products_kernel<TR, RP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::SmemBytes);
   if (configured != cudaSuccess) return configured;
   const int grid = (int)tp_grid(n, num_sms);
+  const long long C = (long long)((n + kBM - 1) / kBM) * ((n + 31) / 32);
+  if (C * (grid + 1) > UINT32_MAX) return cudaErrorInvalidValue;  // the kernel's 32-bit ranges
   LV_LAUNCH(launch_pdl(tc_products_kernel<TR, RP>, grid, Sh::Threads, Sh::SmemBytes, s, tmP, tmF,
       out, ps, cs, n, r_out, parts, status));
   return cudaGetLastError();
