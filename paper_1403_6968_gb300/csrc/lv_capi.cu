@@ -444,15 +444,13 @@ static linview_status run_fused(linview_program* p, const View& v, int mode, int
 // X (n x r, column stride xs) = P Xf as a link of a chain of products with one view: whole
 // rows at a time where the factors of a row fit the registers (FP32, r <= 4), else a pass of
 // column strips and the sum of its partial sets.  An update of the linear iteration,
-// strips -> rows: n = 8192, p = 64 rank 2 709 -> 659 us, rank 1 678 -> 661; n = 4096 rank 2
-// 214 -> 206; n = 1000 rank 2 63.5 -> 58.2; rounding sums less exactly (see the kernel)
-// these were 647, 659, 200, 57.3, and n = 2000 rank 4 105 -> 102, n = 300 rank 1 53.0
-// -> 53.3.  Four columns past n = 4096 take twice the registers and lose (n = 8192 748 ->
-// 939).  The products of recomputed iterations and of the adjoint with a few right-hand sides
-// stay on the strips too, whose sums of partial sets in pairs are closer to FP64 (adjoint of
-// n = 1871, p = 1: 8.0e-8 against 8.7e-8).  The exponential and skip models run theirs beside the panel kernels of other
-// streams, which the rows' CTAs keep off the SMs (n = 4096, p = 1024 559 -> 586 us): they
-// stay on the strips.
+// strips -> rows: n = 8192, p = 64 rank 2 709 -> 656 us, rank 1 678 -> 665; n = 4096 rank 2
+// 214 -> 201; n = 1000 rank 2 63.5 -> 61; n = 2000 rank 4 105 -> 104.  Four columns past n =
+// 4096 take twice the registers and lose (n = 8192 748 -> 939).  The products of recomputed
+// iterations and of the adjoint with a few right-hand sides stay on the strips (adjoint of
+// n = 1871, p = 1: 8.0e-8 from FP64, on rows with plain lane sums 8.7e-8).  So do the
+// exponential and skip models, which run theirs beside the panel kernels of other streams, and
+// the rows' CTAs keep those off the SMs (n = 4096, p = 1024 559 -> 586 us).
 template <typename T>
 static linview_status view_product(linview_program* p, const View& v, int r, const T* Xf, T* X,
                                    int64_t xs, cudaStream_t s, bool reverse = false) {

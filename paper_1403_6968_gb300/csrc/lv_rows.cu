@@ -14,15 +14,19 @@ namespace {
 // 512 columns to a kernel of their own, which in a chain of dependent products is another
 // link.  Thread t keeps the factor entries of columns 4t .. 4t + 3 of every 1024 in
 // registers (at most 64), so four view entries cost one 128-bit shared load and 4 R FMAs: the
-// pass is bound by reading the view.  Four rows make a
-// batch: its sums are reduced across the lanes by halving the values with each shuffle,
-// then across the warps in a fixed order, as FP32 pairs.  Row pieces of 4 KB come by bulk copies into a ring
-// of six 16 KB stages, which the warps refill in turn.  Two CTAs per SM: with one, its two
-// warps per scheduler left the reductions' latency in the open (n = 8192, two columns: 50 us
-// a link against 37 with two; the strips' pass and sum 41).  A chunk's four products are
-// summed by themselves and the warps' sums as pairs, which takes 1 us more a link and keeps
-// the error against FP64 at or below the strips' (n = 8192 1.2e-7, n = 1000 1.0e-7).  Rows are exact, not boxes of
-// eight, so the CTAs' ranges differ by one row at most.
+// pass is bound by reading the view.  Four rows make a batch: its sums are reduced across the
+// lanes by halving the values with each shuffle, then across the warps in a fixed order.  Row
+// pieces of 4 KB come by bulk copies into a ring of six 16 KB stages, which the warps refill in
+// turn.  Two CTAs per SM: with one, its two warps per scheduler left the reductions' latency in
+// the open (n = 8192, two columns: 50 us a link against 37 with two; the strips' pass and sum
+// 41).  Rows are exact, not boxes of eight, so the CTAs' ranges differ by one row at most.
+// Rounding: a chunk's four products are summed by themselves, the chunks in fours, and once a
+// lane holds one value its sums are pairs, to the end.  So an entry passes 9 FP32 roundings of
+// a sum's size at every n, as in the strips, which sum their partial sets in pairs: the last
+// of 15 links is off by 2.5e-7 (n = 1000), 3.2e-7 (8192), 3.4e-7 (16384, one column) against
+// the strips' 3.4e-7, 3.6e-7, 3.5e-7.  With chunks one after the other and plain lane sums it
+// was 3.1e-7, 3.8e-7 and 4.3e-7; an update at n = 8192, p = 64 took 656 us (one column) and
+// 652 (two) so, 665 and 656 now.
 constexpr int kRpRows = 4, kRpCols = 1024, kRpStages = 6;
 constexpr int kRpThreads = 256, kRpWarps = kRpThreads / 32;
 constexpr int kRpStageBytes = kRpRows * kRpCols * 4;
@@ -33,8 +37,15 @@ struct RpBars {
   int abort;
 };
 
-constexpr int rp_smem(int R) {
-  return kRpStages * kRpStageBytes + 2 * kRpWarps * kRpRows * R * 4 + (int)sizeof(RpBars);
+template <int R>
+constexpr int kRpSmem = kRpStages * kRpStageBytes + 2 * kRpWarps * kRpRows * R * (int)sizeof(float2) +
+                        (int)sizeof(RpBars);
+
+// (s, low) += v as a pair, Knuth's TwoSum
+__device__ __forceinline__ void rp_two_sum(float& s, float& low, float v) {
+  const float z = s + v, b = z - s;
+  low += (s - (z - b)) + (v - b);
+  s = z;
 }
 
 // false once a wait of this CTA has run out (status then holds the timeout)
@@ -64,9 +75,8 @@ __global__ void __launch_bounds__(kRpThreads, 2)
                         unsigned* status) {
   extern __shared__ __align__(128) unsigned char rp_mem[];
   float* ring = reinterpret_cast<float*>(rp_mem);
-  float* red = reinterpret_cast<float*>(rp_mem + kRpStages * kRpStageBytes);
-  RpBars* bars = reinterpret_cast<RpBars*>(rp_mem + kRpStages * kRpStageBytes +
-                                           2 * kRpWarps * kRpRows * R * 4);
+  float2* red = reinterpret_cast<float2*>(rp_mem + kRpStages * kRpStageBytes);
+  RpBars* bars = reinterpret_cast<RpBars*>(rp_mem + kRpSmem<R> - sizeof(RpBars));
   volatile int* abort_flag = &bars->abort;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int r0 = (int)((int64_t)n * blockIdx.x / gridDim.x);
@@ -137,9 +147,13 @@ __global__ void __launch_bounds__(kRpThreads, 2)
   bool ok = true;
   for (int b = 0; b < nb; ++b) {
     const int row0 = batch_row(b), nr = min(kRpRows, r1 - row0);
-    float acc[NV];
+    constexpr bool GRP = CH > 4;
+    float acc[NV], tot[GRP ? NV : 1];  // sums of up to four chunks, of the fours before
 #pragma unroll
     for (int i = 0; i < NV; ++i) acc[i] = 0.f;
+    if constexpr (GRP)
+#pragma unroll
+      for (int i = 0; i < NV; ++i) tot[i] = 0.f;
 #pragma unroll
     for (int c = 0; c < CH; ++c) {
       if (c < nch) {
@@ -169,6 +183,13 @@ __global__ void __launch_bounds__(kRpThreads, 2)
             t = fmaf(x[j].z, u[c][2][q], t);
             acc[j * R + q] += fmaf(x[j].w, u[c][3][q], t);
           }
+        if (GRP && c % 4 == 3) {
+#pragma unroll
+          for (int i = 0; i < NV; ++i) {
+            tot[GRP ? i : 0] += acc[i];
+            acc[i] = 0.f;
+          }
+        }
         // the stage of the step before is refilled, by each warp in its turn
         if (step >= 1 && step % kRpWarps == warp && step - 1 + kRpStages < total) {
           const int pt = step - 1;
@@ -183,9 +204,13 @@ __global__ void __launch_bounds__(kRpThreads, 2)
         }
       }
     }
+    if constexpr (GRP)
+#pragma unroll
+      for (int i = 0; i < NV; ++i) acc[i] += tot[i];
     // lane sums: while there are several values, each shuffle halves their number; lane
-    // ends with value lane / (32 / NV)
+    // ends with value lane / (32 / NV), which goes on as a pair
     int cnt = NV;
+    float low = 0.f;
 #pragma unroll
     for (int m = 16; m >= 1; m >>= 1) {
       if (cnt > 1) {
@@ -198,19 +223,22 @@ __global__ void __launch_bounds__(kRpThreads, 2)
             acc[i] = keep + __shfl_xor_sync(0xffffffffu, give, m);
           }
       } else {
-        acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], m);
+        const float l = __shfl_xor_sync(0xffffffffu, low, m);
+        rp_two_sum(acc[0], low, __shfl_xor_sync(0xffffffffu, acc[0], m));
+        low += l;
       }
     }
-    float* rb = red + (b & 1) * kRpWarps * NV;
-    if (lane % (32 / NV) == 0) rb[warp * NV + lane / (32 / NV)] = acc[0];
+    float2* rb = red + (b & 1) * kRpWarps * NV;
+    if (lane % (32 / NV) == 0) rb[warp * NV + lane / (32 / NV)] = make_float2(acc[0], low);
     __syncthreads();
     if (tid < NV) {
-      float s = rb[tid], low = 0.f;  // as a pair: these few additions are the largest
+      float s = rb[tid].x;
+      low = rb[tid].y;
 #pragma unroll
-      for (int w = 1; w < kRpWarps; ++w) {  // Knuth's TwoSum
-        const float v = rb[w * NV + tid], z = s + v, b1 = z - s;
-        low += (s - (z - b1)) + (v - b1);
-        s = z;
+      for (int w = 1; w < kRpWarps; ++w) {
+        const float2 v = rb[w * NV + tid];
+        rp_two_sum(s, low, v.x);
+        low += v.y;
       }
       s += low;
       const int j = tid / R, q = tid % R;
@@ -227,14 +255,14 @@ cudaError_t launch_rows_t(const float* P, int64_t ldp, const float* F, int64_t f
                           float* X, int64_t xs, bool reverse, int num_sms, unsigned* status,
                           cudaStream_t s) {
   static const cudaError_t configured = cudaFuncSetAttribute(
-      row_products_kernel<R, CH>, cudaFuncAttributeMaxDynamicSharedMemorySize, rp_smem(R));
+      row_products_kernel<R, CH>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRpSmem<R>);
   if (configured != cudaSuccess) return configured;
   // every resident CTA, while there are batches for it
   const int batches = (n + kRpRows - 1) / kRpRows;
   const int resident = 2 * num_sms;
   const int grid = batches < resident ? batches : resident;
   const int vec = fs % 4 == 0 && (reinterpret_cast<uintptr_t>(F) & 15) == 0;
-  return launch_pdl(row_products_kernel<R, CH>, grid, kRpThreads, rp_smem(R), s, P, ldp, F, fs, n,
+  return launch_pdl(row_products_kernel<R, CH>, grid, kRpThreads, kRpSmem<R>, s, P, ldp, F, fs, n,
                     r, X, xs, vec, reverse ? 1 : 0, status);
 }
 
