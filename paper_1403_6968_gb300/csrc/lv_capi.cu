@@ -896,13 +896,10 @@ static linview_status gemm_ab(linview_program* p, int64_t M, int64_t N, int64_t 
 // alpha op(A) op(B) + beta C with A, B column-major (lda, ldb): the CUDA-core
 // GEMM with the program's split-K partials (small products of the general
 // form, captured into the propagation graphs).
-// (batch > 1: ``batch`` such products, entry b at A + b a_bs, B + b b_bs,
-// C + b c_bs elements, strides possibly negative, in one launch)
 static linview_status gemm_cm_own(linview_program* p, bool ta, bool tb, int64_t M, int64_t N,
                                   int64_t K, double alpha, const void* A, int64_t lda,
                                   const void* B, int64_t ldb, double beta, void* C, int64_t ldc,
-                                  cudaStream_t s, int batch = 1, int64_t a_bs = 0,
-                                  int64_t b_bs = 0, int64_t c_bs = 0) {
+                                  cudaStream_t s) {
   if (M <= 0 || N <= 0) return LINVIEW_OK;
   // column-major X(i, j) = X[i + j ld]; op(A)(m, k), op(B)(k, n)
   const int64_t a_rs = ta ? lda : 1, a_cs = ta ? 1 : lda;
@@ -912,13 +909,12 @@ static linview_status gemm_cm_own(linview_program* p, bool ta, bool tb, int64_t 
                                     static_cast<const float*>(A), a_rs, a_cs,
                                     static_cast<const float*>(B), b_rs, b_cs, (float)beta,
                                     static_cast<float*>(C), 1, ldc, static_cast<float*>(p->gwork),
-                                    p->gwork_elems, p->sms, s, batch, a_bs, b_bs, c_bs));
+                                    p->gwork_elems, p->sms, s));
   else
     LV_CUDA(launch_gemm_simt<double>((int)M, (int)N, (int)K, alpha, static_cast<const double*>(A),
                                      a_rs, a_cs, static_cast<const double*>(B), b_rs, b_cs, beta,
                                      static_cast<double*>(C), 1, ldc,
-                                     static_cast<double*>(p->gwork), p->gwork_elems, p->sms, s,
-                                     batch, a_bs, b_bs, c_bs));
+                                     static_cast<double*>(p->gwork), p->gwork_elems, p->sms, s));
   p->all_launches += 2;
   return LINVIEW_OK;
 }
