@@ -283,19 +283,23 @@ struct GArgs {
   unsigned* status;
 };
 
-// The flag word of a product: two bits per operand, kLossy where an entry keeps fewer than
-// 22 bits and kSparse where a run of an operand has more than 3/8 of its entries below 2^-7
-// of the largest (zeros among them; runs of zeros alone do not count).  Either alone does
-// no harm.  Where no run of A or of B is sparse, a quarter of a run of length L meets with
-// both entries at 2^7 or more of their 2^15, a sum of |a||b| of at least L/4 2^14, while the
-// at most 3/4 L entries that lose bits add 2^-25 2^15 each: 2^-22.4 of the sum, as much as
-// the halves of the others leave.  With kSparse on either side an entry may meet zeros and
-// small entries only, and a product is as good as that entry.  Dense data without such
-// structure has kLossy (in normal entries 2e-5 of them) and not kSparse (25 of 64 entries
-// below 2 % of a standard deviation).
-constexpr unsigned kLossy = 1u, kSparse = 2u;
+// The flag word of a product: three bits per operand, A's from bit 0, B's from bit 4.  kLossy:
+// entries that keep fewer than 22 bits.  kSparse, kSparser: runs of which more than 3/8 lie
+// below 512 and below 7, where the largest is 2^14 to 2^15 (below 256 and 8 in runs of fewer
+// than 48), zeros among them, runs of zeros aside.  Entries that lose bits do no harm where
+// dense runs meet: where no run of one operand is kSparse and none of the other kSparser, a
+// quarter of a run of length L meets with products of 3584 and more, a sum of |a||b| of at
+// least L/4 3584, while the at most 2 + 8 entries that lose bits add 2^-25 2^15 each: 2^-22.5
+// of the sum at L = 64 (2^-20 in a last run of 16, with at most 4 + 4), about what the halves of
+// the other entries leave.  Else such an entry may meet zeros and small entries only, and a
+// product is as good as that entry.  (Runs with more of them, zeros counted where there is one,
+// are kSparser.)  Dense data has entries that lose bits (2e-5 of normal ones) and no sparse
+// runs; a matrix with a diagonal or a few rows some hundred times the rest is kSparse along one
+// of its sides and not kSparser.
+constexpr unsigned kLossy = 1u, kSparse = 2u, kSparser = 4u, kFlagAll = 7u;
 __device__ __forceinline__ bool needs_tf32(unsigned flag) {
-  return ((flag | flag >> 2) & 3u) == (kLossy | kSparse);
+  const unsigned a = flag & kFlagAll, b = flag >> 4;
+  return ((a | b) & kLossy) && ((a & b & kSparse) || ((a | b) & kSparser));
 }
 
 // D (M x N, row-major, ldd) = alpha A B^T + beta C over the split blocks of K = kp16
@@ -643,7 +647,7 @@ struct SplitOp {
   unsigned* fmt;    // 0: FP16 rows, 1: TF32 rows
   int vec;          // rows of X start on 16-byte units
   int blocks;       // CTAs of this operand in the launch at hand
-  int bit;          // this operand's two bits in the flag word: 0 (A) or 2 (B)
+  int bit;          // first of this operand's bits in the flag word: 0 (A) or 4 (B)
 };
 struct SplitPair {
   SplitOp o[2];
@@ -680,7 +684,7 @@ __device__ __forceinline__ int run_length(int slot, int K) {
 
 // Slots k .. k + 7 of row i (a run of 64 belongs to eight neighbouring lanes; all lanes
 // of the warp take part): scale, split, store (``in``: inside the operand).  Returns the run's
-// bits of the flag, both where its scale is out of range or an entry is not finite.
+// bits of the flag, all where its scale is out of range or an entry is not finite.
 __device__ __forceinline__ unsigned split_run(const float (&x)[8], const SplitOp& o, int i, int k,
                                               bool in, int kp) {
   unsigned mx = 0, mn = 0xffffffffu;  // mn: the least entry that is not zero, less one
@@ -693,10 +697,10 @@ __device__ __forceinline__ unsigned split_run(const float (&x)[8], const SplitOp
 #pragma unroll
   for (int d = 1; d < 8; d <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, d));
   int sh = mx ? 14 - ((int)(mx >> 23) - 127) : 0;
-  unsigned bits = sh > 60 || sh < -60 ? kLossy | kSparse : 0u;  // (non-finite: sh = -114)
+  unsigned bits = sh > 60 || sh < -60 ? kFlagAll : 0u;  // (non-finite: sh = -114)
   sh = min(60, max(-60, sh));
   const float sc = pow2f(sh);
-  if (mn < ((unsigned)(125 - sh) << 23) - 1u) bits |= kLossy;  // 2^sh x below 2^-2
+  const bool lossy = mn < ((unsigned)(125 - sh) << 23) - 1u;  // 2^sh x below 2^-2
   // pairs: one instruction per two values
   __align__(16) __half2 hi[4], lo[4];
   __half2 lows = __float2half2_rn(0.f);
@@ -706,15 +710,25 @@ __device__ __forceinline__ unsigned split_run(const float (&x)[8], const SplitOp
     hi[e] = __floats2half2_rn(y0, y1);
     const float2 h = __half22float2(hi[e]);
     lo[e] = __floats2half2_rn(y0 - h.x, y1 - h.y);
-    lows = __hadd2(lows, __hlt2(__habs2(hi[e]), __float2half2_rn(128.f)));
+    lows = __hadd2(lows, __hlt2(__habs2(hi[e]), __float2half2_rn(512.f)));
   }
-  int low = (int)(__low2float(lows) + __high2float(lows));
-  // a sparse run has four such entries in one lane
-  if (__any_sync(0xffffffffu, low >= 4)) {
+  // rare in dense data (a sparse run has four such entries in one lane)
+  const bool few = __low2float(lows) + __high2float(lows) >= 4.f;
+  if (__any_sync(0xffffffffu, few || lossy)) {
+    const int len = run_length(k, o.K), most = mx ? len * 3 / 8 : 64;
+    auto below = [&](float bound) {  // entries of the run, from what its lanes hold
+      __half2 c = __float2half2_rn(0.f);
 #pragma unroll
-    for (int d = 1; d < 8; d <<= 1) low += __shfl_xor_sync(0xffffffffu, low, d);
-    const int len = run_length(k, o.K);
-    if (mx && low - (64 - len) > len * 3 / 8) bits |= kSparse;
+      for (int e = 0; e < 4; ++e) c = __hadd2(c, __hlt2(__habs2(hi[e]), __float2half2_rn(bound)));
+      int m = (int)(__low2float(c) + __high2float(c));
+#pragma unroll
+      for (int d = 1; d < 8; d <<= 1) m += __shfl_xor_sync(0xffffffffu, m, d);
+      return m - (64 - len);
+    };
+    if (below(len < 48 ? 256.f : 512.f) > most) bits |= kSparse;
+    if (below(len < 48 ? 8.f : 7.f) > most) bits |= kSparser;
+    const int lost = below(0.25f);
+    if (lossy) bits |= lost > (len < 48 ? 4 : bits & kSparse ? 8 : 2) ? kFlagAll : kLossy;
   }
   if (in) {
     unsigned char* d = o.dst + block_line(i, k / 64, kp / 64) * 128 + k % 64 * 2;
@@ -1085,7 +1099,7 @@ __global__ void __launch_bounds__(ROWS * BN / 4)
     }
     raise_bits(nx_flag, bits, nx);
     // A goes on as it is; once on TF32 halves, the chain stays there
-    if (blockIdx.x == 0 && blockIdx.y == 0 && e == 0) atomicOr(nx_flag, f16 ? flag & 3u : flag);
+    if (blockIdx.x == 0 && blockIdx.y == 0 && e == 0) atomicOr(nx_flag, f16 ? flag & kFlagAll : flag);
   }
 }
 
@@ -1158,7 +1172,7 @@ SplitOp split_op(const TcOperand* t, bool second) {
   o.fmt = t->words;
   o.sc = reinterpret_cast<float*>(t->words + 4);
   o.pitch = (t->rows + 3) / 4 * 4;
-  o.bit = second ? 2 : 0;
+  o.bit = second ? 4 : 0;
   o.vec = (t->cs == 1 ? t->rs : t->cs) % 4 == 0 && reinterpret_cast<uintptr_t>(t->X) % 16 == 0;
   return o;
 }

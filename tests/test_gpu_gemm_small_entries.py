@@ -71,6 +71,21 @@ def test_short_last_runs(K, ta, tb):
     _check(a, b, ta, tb)
 
 
+@pytest.mark.parametrize("ta,tb", [(False, False), (True, True)])
+@pytest.mark.parametrize("scale", [30, 300, 3e3, 1e5])
+@pytest.mark.parametrize("n", [256, 400, 529])
+def test_outlier_rows(n, scale, ta, tb):
+    """Rows far larger than the others, a diagonal far larger than the rest: small entries beside
+    a large one in the runs of one side, dense runs in those of the other."""
+    g = torch.Generator(device="cuda").manual_seed(n)
+    a, b = _normal(g, n, n), _normal(g, n, n)
+    a[7::61] *= scale
+    _check(a, a, ta, tb)
+    b.diagonal().mul_(scale)
+    _check(a, b, ta, tb)
+    _check(b, b, ta, tb)
+
+
 @pytest.mark.parametrize("n,p", [(256, 33), (300, 64), (1024, 17), (327, 40)])
 def test_chain(n, p):
     """G <- A^T G with a diagonal A: the product that is split for the next one by the kernel
