@@ -343,8 +343,12 @@ __global__ void __launch_bounds__(kThreads) assemble_kernel(const AssembleParams
 // to fill the GPU with one thread per (j, c), which then sums all partials
 // itself (CTA = 256 rows of one column; the C_h column is summed once per
 // CTA).  Same fixed orders as above within a thread's sums.  Small views have few
-// outputs and many row ranges (n = 1000: 127 partial sets): below n = 4096 with more
-// than 24 sets the warps of a CTA share them (n = 1000, 12 columns: 15.5 -> 7 us).
+// outputs and many row ranges (n = 1000: 127 partial sets): with more than 24 sets and
+// outputs for fewer CTAs than half of the SMs the warps of a CTA share the sets.  Updates,
+// shared sets against one thread per output: A^16 rank 2 at n = 1000 58 and 67 us, n = 2000
+// 92.0 and 92.0, n = 3000 146 and 140; A^2 .. A^4 (linear), 16 columns, at n = 1000 82 and 92
+// us, n = 1300 103 and 99, n = 3500 262 and 241.
+constexpr int kWideAssembleCtas = 76;
 template <typename T>
 __global__ void __launch_bounds__(kThreads) assemble_wide_kernel(const AssembleParams a) {
   __shared__ T Cc[kMaxAsmR];
@@ -396,8 +400,9 @@ cudaError_t launch_assemble(const AssembleParams& a, cudaStream_t s) {
   const int ro = a.r_out > 0 ? a.r_out : a.r_h;
   cudaError_t e;
   const int sets = a.gC + (a.Ypart ? a.gR : 0);
-  if (ro >= 8 && (sets <= 24 || a.n >= 4096)) {
-    const dim3 grid((unsigned)((a.n + kThreads - 1) / kThreads), (unsigned)ro);
+  const int ctas = (a.n + kThreads - 1) / kThreads;  // of 256 rows
+  if (ro >= 8 && (sets <= 24 || (int64_t)ctas * ro >= kWideAssembleCtas)) {
+    const dim3 grid((unsigned)ctas, (unsigned)ro);
     e = launch_pdl(assemble_wide_kernel<T>, grid, kThreads, 0, s, a);
   } else {
     const dim3 grid((unsigned)((a.n + 31) / 32), (unsigned)ro);
