@@ -1583,9 +1583,9 @@ static linview_status iter_create(linview_program* p, const void* const* inputs,
   LV_TRY(dalloc(p, (size_t)pp * p->Rcap * p->elem, &p->Mr, s));
   // partial sets of M_i = T_i^T V: one pass over the T panel for all views, or (hybrid) one
   // pass per view, whose fewer columns are cut into more row blocks
-  p->tv_elems = tdot_work_elems((int)n, (int)(k * pp), p->d.r_max, p->sms);
+  p->tv_elems = tdot_work_elems(p->elem, (int)n, (int)(k * pp), p->d.r_max, p->sms);
   if (p->d.strategy == LINVIEW_STRATEGY_HYBRID)
-    p->tv_elems = std::max(p->tv_elems, tdot_work_elems((int)n, (int)pp, p->d.r_max, p->sms));
+    p->tv_elems = std::max(p->tv_elems, tdot_work_elems(p->elem, (int)n, (int)pp, p->d.r_max, p->sms));
   LV_TRY(dalloc(p, (size_t)p->tv_elems * p->elem, &p->TVpart, s));
   const PassGeom g = fused_geom(p->elem, (int)n, p->sms);
   p->part_cs = p->fs;
@@ -1974,7 +1974,7 @@ static linview_status iter_sk_create(linview_program* p, const void* const* inpu
     LV_TRY(dalloc(p, (size_t)pp * ck * p->elem, &p->Yar[i], s));
   }
   LV_TRY(dalloc(p, (size_t)ck * p->Rcap * sizeof(double), &p->XtV, s));
-  p->tv_elems = tdot_work_elems((int)n, (int)pp, p->Rcap, p->sms);
+  p->tv_elems = tdot_work_elems(p->elem, (int)n, (int)pp, p->Rcap, p->sms);
   LV_TRY(dalloc(p, (size_t)p->tv_elems * p->elem, &p->TVpart, s));
   LV_TRY(dalloc(p, (size_t)pp * p->d.r_max * p->elem, &p->Mr, s));  // V_b of an update to B
   const PassGeom g = fused_geom(p->elem, (int)n, p->sms);

@@ -287,7 +287,7 @@ cudaError_t launch_scale_copy(T* y, int64_t ldy, const T* x, int64_t ldx, T alph
 // M[((k - 1 - i) w + c) ldm + q] = sum_j A0[j lda0 + i p + q] F0[c fs + j] for
 // i < k, c < w <= 64, q < p; optionally + sum_j A1[j lda1 + i p + q] (F1 - F0)[c fs +
 // j] and + sum_{t < ny} Yc[t ldy + i p + q] S[t s_t + c s_c].  ``work`` holds
-// ``work_elems`` elements, tdot_work_elems(n, k p, w) for as many row blocks as fill the
+// ``work_elems`` elements, tdot_work_elems(sizeof(T), n, k p, w) for as many row blocks as fill the
 // GPU; fewer elements mean fewer blocks, and less than one block's k p w is an error.
 template <typename T>
 struct TdotOp {
@@ -309,7 +309,7 @@ struct TdotOp {
   const double* S = nullptr;
   int64_t s_t = 0, s_c = 0;
 };
-int64_t tdot_work_elems(int n, int cols, int w, int num_sms);
+int64_t tdot_work_elems(int elem_bytes, int n, int cols, int w, int num_sms);
 template <typename T>
 cudaError_t launch_tdot(const TdotOp<T>& o, int num_sms, cudaStream_t s);
 // T_i(j, q) = T1[j ldT + (i - 1) p + q] += sum_{t < i r} K[t fs + j] M[((k - i) r + t) ldm

@@ -379,10 +379,28 @@ cudaError_t launch_outer_t(T* T1, int64_t ldT, const T* K, int64_t fs, const T* 
                     p, k, r, accumulate ? 1 : 0);
 }
 
-// row blocks of a tdot over ``cols`` columns: about two CTAs per SM (two waves
-// of one would leave the second one nearly empty), at least 64 rows each
-int tdot_blocks(int n, int cols, int num_sms) {
+// row blocks of a tdot over ``cols`` columns.  FP32: about two CTAs per SM (two waves
+// of one would leave the second one nearly empty), at least 64 rows each.  FP64 is bound by
+// its FMAs, two a clock and SM, so the blocks are those (of 16 rows and more, and some 24 rows'
+// time to start one) that leave the busiest SM the fewest rows: linear iterations of 8 steps
+// against FP32's rule at n = 300, p = 3, rank 8 114 -> 104 us, n = 777, p = 64 327 -> 321,
+// n = 1500, p = 129, rank 1 198 -> 186 (187 before these kernels).
+int tdot_blocks(int elem_bytes, int n, int cols, int num_sms) {
   const int cb = (cols + kTdCols - 1) / kTdCols;
+  if (elem_bytes == 8) {
+    int best = 1;
+    int64_t least = INT64_MAX;
+    for (int nb = 1; nb <= kTdMaxBlocks && 16 * nb < n + 16; ++nb) {
+      const int rows = ((n + nb - 1) / nb + 7) / 8 * 8;
+      const int64_t ctas = (int64_t)cb * ((n + rows - 1) / rows);
+      const int64_t busiest = (ctas + num_sms - 1) / num_sms * (rows + 24);
+      if (busiest < least) {
+        least = busiest;
+        best = nb;
+      }
+    }
+    return best;
+  }
   int nb = 2 * num_sms / cb;
   if (nb > (n + 63) / 64) nb = (n + 63) / 64;
   if (nb > kTdMaxBlocks) nb = kTdMaxBlocks;
@@ -391,8 +409,8 @@ int tdot_blocks(int n, int cols, int num_sms) {
 
 }  // namespace
 
-int64_t tdot_work_elems(int n, int cols, int w, int num_sms) {
-  return (int64_t)tdot_blocks(n, cols, num_sms) * cols * w;
+int64_t tdot_work_elems(int elem_bytes, int n, int cols, int w, int num_sms) {
+  return (int64_t)tdot_blocks(elem_bytes, n, cols, num_sms) * cols * w;
 }
 
 template <typename T>
@@ -402,7 +420,7 @@ cudaError_t launch_tdot(const TdotOp<T>& o, int num_sms, cudaStream_t s) {
   // no more row blocks than the work space has room for
   const int64_t room = o.work_elems / ((int64_t)cols * o.w);
   if (room < 1) return cudaErrorInvalidValue;
-  int nb0 = tdot_blocks(o.n, cols, num_sms);
+  int nb0 = tdot_blocks(sizeof(T), o.n, cols, num_sms);
   if (nb0 > room) nb0 = (int)room;
   const int rows = ((o.n + nb0 - 1) / nb0 + 7) / 8 * 8;
   const int nb = (o.n + rows - 1) / rows;
@@ -428,7 +446,12 @@ cudaError_t launch_outer(T* T1, int64_t ldT, const T* K, int64_t fs, const T* M,
                          int p, int k, int r, bool accumulate, int num_sms, cudaStream_t s) {
   if (n <= 0 || p <= 0 || k < 1 || r < 1) return cudaSuccess;
   if (!outer_fits(k * r, sizeof(T))) return cudaErrorInvalidValue;
-  if (outer_smem(4, k * r, sizeof(T)) <= (size_t)smem_optin_max())
+  // FP64 is bound by its FMAs, not by shared memory: tiles of 16 rows while those of 64 are few,
+  // which spread more evenly (8 steps, rank 8, p = 129: n = 300 161 -> 145 us, n = 777 415 -> 384
+  // (381 before these kernels), but n = 1000, 48 tiles of 64 rows, 411 -> 442)
+  const int64_t tiles = (int64_t)((n + 63) / 64) * ((p + 63) / 64);
+  if (!(sizeof(T) == 8 && tiles < num_sms * 3 / 10) &&
+      outer_smem(4, k * r, sizeof(T)) <= (size_t)smem_optin_max())
     return launch_outer_t<T, 4>(T1, ldT, K, fs, M, ldm, n, p, k, r, accumulate, num_sms, s);
   return launch_outer_t<T, 1>(T1, ldT, K, fs, M, ldm, n, p, k, r, accumulate, num_sms, s);
 }
