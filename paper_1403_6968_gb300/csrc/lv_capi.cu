@@ -502,7 +502,7 @@ static linview_status run_update(linview_program* p, const View& v, const T* Uu,
         continue;
       }
     }
-    const PassGeom g = update_geom(sizeof(T), w, (int)v.rows, p->sms);
+    const PassGeom g = update_geom(sizeof(T), w, (int)v.rows, p->sms, p->side && s == p->side);
     PassParams pp{};
     pp.P = v.ptr;
     pp.ldp = v.ld;

@@ -92,7 +92,8 @@ struct PassGeom {
   int strip, gC, gR, rows_per_cta;
 };
 PassGeom fused_geom(int elem_bytes, int n, int num_sms);
-PassGeom update_geom(int elem_bytes, int R, int n, int num_sms);
+// beside: the pass runs next to another one (on a side stream)
+PassGeom update_geom(int elem_bytes, int R, int n, int num_sms, bool beside = false);
 
 // Host: 2-D tensor map over a row-major matrix (rows x cols, ld elements),
 // box = (kBoxBytes / elem_bytes) columns x kBatch rows.

@@ -474,6 +474,9 @@ static int round_up(int a, int b) { return (a + b - 1) / b * b; }
 // past the range are loaded and ignored), as long as the grid stays within one CTA per
 // SM.  The FP64 pipe does two FMAs per clock and SM, so the pass takes as long as its
 // rows per SM: n = 256, 4 columns 32 CTAs of 8 rows 11.9 us, 128 of 2 rows 6.4 us.
+// Narrow updates beside another pass (``beside``, up to 4 columns) stay within half of the SMs,
+// or the other pass, which the next one waits for, goes slower: A^8 and its sums, row updates,
+// n = 200 52.6 -> 48.5 us, n = 400 63.4 -> 60.7, n = 500 73.2 -> 65.5 (64.7 without short ranges).
 static int short_rows(int elem_bytes, int gC, int n, int num_sms) {
   int rows = kBatch;
   while (elem_bytes == 8 && rows > 2 && (int64_t)gC * ((n + rows / 2 - 1) / (rows / 2)) <= num_sms)
@@ -481,11 +484,12 @@ static int short_rows(int elem_bytes, int gC, int n, int num_sms) {
   return rows;
 }
 
-static PassGeom geom_for_strip(int elem_bytes, int strip, int n, int num_sms) {
+static PassGeom geom_for_strip(int elem_bytes, int strip, int n, int num_sms, bool beside = false) {
   PassGeom g;
   g.strip = strip;
   g.gC = (n + strip - 1) / strip;
-  if (const int rows = short_rows(elem_bytes, g.gC, n, num_sms); rows < kBatch) {
+  if (const int rows = short_rows(elem_bytes, g.gC, n, beside ? num_sms / 2 : num_sms);
+      rows < kBatch) {
     g.rows_per_cta = rows;
     g.gR = (n + rows - 1) / rows;
     return g;
@@ -509,8 +513,9 @@ static int update_cols(int elem_bytes, int R) {
   return R <= 16 ? 2 : 1;
 }
 
-PassGeom update_geom(int elem_bytes, int R, int n, int num_sms) {
-  return geom_for_strip(elem_bytes, kThreads * update_cols(elem_bytes, R), n, num_sms);
+PassGeom update_geom(int elem_bytes, int R, int n, int num_sms, bool beside) {
+  return geom_for_strip(elem_bytes, kThreads * update_cols(elem_bytes, R), n, num_sms,
+                        beside && R <= 4);
 }
 
 bool make_tmap(CUtensorMap* out, const void* base, int elem_bytes, int64_t cols, int64_t rows,
