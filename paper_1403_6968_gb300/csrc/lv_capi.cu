@@ -444,7 +444,7 @@ static linview_status run_fused(linview_program* p, const View& v, int mode, int
 // X (n x r, column stride xs) = P Xf as a link of a chain of products with one view: whole
 // rows at a time where the factors of a row fit the registers (FP32, r <= 4), else a pass of
 // column strips and the sum of its partial sets.  An update of the linear iteration,
-// strips -> rows: n = 8192, p = 64 rank 2 709 -> 656 us, rank 1 678 -> 665; n = 4096 rank 2
+// strips -> rows: n = 8192, p = 64 rank 2 709 -> 656 us, rank 1 678 -> 625; n = 4096 rank 2
 // 214 -> 201; n = 1000 rank 2 63.5 -> 61; n = 2000 rank 4 105 -> 104.  Four columns past n =
 // 4096 take twice the registers and lose (n = 8192 748 -> 939).  The products of recomputed
 // iterations and of the adjoint with a few right-hand sides stay on the strips (adjoint of

@@ -25,8 +25,12 @@ namespace {
 // a sum's size at every n, as in the strips, which sum their partial sets in pairs: the last
 // of 15 links is off by 2.5e-7 (n = 1000), 3.2e-7 (8192), 3.4e-7 (16384, one column) against
 // the strips' 3.4e-7, 3.6e-7, 3.5e-7.  With chunks one after the other and plain lane sums it
-// was 3.1e-7, 3.8e-7 and 4.3e-7; an update at n = 8192, p = 64 took 656 us (one column) and
-// 652 (two) so, 665 and 656 now.
+// was 3.1e-7, 3.8e-7 and 4.3e-7; an update at n = 8192, p = 64 took 652 us (two columns) so,
+// 656 now.
+// One column up to n = 8192 has room for half of the entries (32 registers; with the 64 that
+// n = 16384 needs a link was slower than with two columns, and than a strip pass from n = 1300
+// to 4096): n = 300 57.0 -> 45.5 us an update, n = 1318 99 -> 81 (strips 98), n = 4096 205 -> 178,
+// n = 8192 665 -> 625.
 constexpr int kRpRows = 4, kRpCols = 1024, kRpStages = 6;
 constexpr int kRpThreads = 256, kRpWarps = kRpThreads / 32;
 constexpr int kRpStageBytes = kRpRows * kRpCols * 4;
@@ -277,6 +281,8 @@ cudaError_t launch_row_products(const float* P, int64_t ldp, const float* F, int
                                 int r, float* X, int64_t xs, bool reverse, int num_sms,
                                 unsigned* status, cudaStream_t s) {
   if (n < 1 || r < 1 || !row_products_fit(P, ldp, n, r)) return cudaErrorInvalidValue;
+  if (r == 1 && n <= 8 * kRpCols)
+    return launch_rows_t<1, 8>(P, ldp, F, fs, n, r, X, xs, reverse, num_sms, status, s);
   if (r == 1)
     return launch_rows_t<1, 16>(P, ldp, F, fs, n, r, X, xs, reverse, num_sms, status, s);
   if (r == 2) return launch_rows_t<2, 8>(P, ldp, F, fs, n, r, X, xs, reverse, num_sms, status, s);
