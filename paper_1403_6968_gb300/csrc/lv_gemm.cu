@@ -1189,20 +1189,23 @@ SplitOp split_op(const TcOperand* t, bool second) {
 //
 // A product that leaves half of the pairs idle (at 256 columns) has time for smaller sums,
 // as the chains of such products (A^16 at n <= 1500, the rounds of an iteration) add up
-// their errors: its choices are those whose pieces add at most 16 chunks one after the
+// their errors: its choices are those whose pieces add at most 20 chunks one after the
 // other, or two thirds of its chunks (all choices where there is none), and up to 32 chunks
 // every other one goes to two accumulators, which takes a fifth off the bias that the tensor
 // cores' truncation leaves (8.9e-8 of a product; a re-evaluated A^16 has 15 times that).
 // Errors against FP64, time: A^16 re-evaluated at n = 1000 1.42e-6 -> 1.19e-6, 95.5 -> 101.4 us;
 // 314 x 3654 x 2299 1.73e-7 -> 1.54e-7, 93 -> 95; adjoint of 16 rounds at 2000 x 200 3.1e-7
-// -> 2.7e-7, 529 -> 550.  (Every chunk in halves: 0.99e-6, but 103.6 us, and 16.2 -> 19.9 ms
+// -> 2.7e-7, 529 -> 550.  20 chunks add up to no more error than TF32 halves left (n = 1250
+// 1.562e-7 of a product against 1.571e-7); with 16 the products of n = 1050 to 1280 were cut for
+// nothing (n = 1250 153 us a re-evaluation, 137 so), with all 22 n = 1352 would be 1.598e-7
+// against 1.581e-7 (145 us, 174 so).  (Every chunk in halves: 0.99e-6, but 103.6 us, and 16.2 -> 19.9 ms
 // for the products of n = 8192, whose epilogue then takes longer than their MMAs.)
 void gemm_plan(int M, int N, int nk, int num_sms, int64_t work_floats, GArgs& a, int* bn_out,
                bool* halves) {
   const int pairs = num_sms / 2;
   const long long mt = (M + kGBM - 1) / kGBM;
   const bool small = mt * ((N + 255) / 256) <= pairs / 2;
-  const int longest = small ? std::max(16, nk * 2 / 3) : nk;
+  const int longest = small ? std::max(20, nk * 2 / 3) : nk;
   double best = 1e30;
   bool best_short = false;
   for (int bn = 256; bn >= 64; bn /= 2) {
